@@ -125,6 +125,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   return true;
 }
+// True for exactly one thread of a converged warp.  The threads that issue TMA loads, MMAs and commits are chosen with it:
+// those instructions take their operands from uniform registers, and only behind elect.sync does the compiler know that one
+// thread is active and issue them directly; behind `lane == 0` it wraps each in a loop over the active threads.  Measured:
+// eight expect-and-copy pairs are issued in 92 cycles against 474; 1024-row responses of 784-4096-4096-2048 take 2561 us
+// against 2782 (33 chunks), a step of 512-1024-768-512 (bf16, batch 512) 54.3 us against 61.2.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -684,7 +694,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0; uint32_t phase = 0;
       int fills = 0;                     // stages filled so far, counted up to the ring's depth: the first pass waits for nothing
       bool ok = true;
@@ -719,7 +729,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       // instruction descriptor: fp32 accumulate, operand format, operand majors, N, M
       constexpr uint32_t fmt = TF32 ? 2u : 1u;
       constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((A_MN ? 1u : 0u) << 15) |
@@ -921,7 +931,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   // free; bytes of B that land before the announcement only take the barrier's byte count below zero for a while
   // (the phase cannot complete before the announcing arrival).
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0; uint32_t phase = 0;
       for (int kb = kb_begin; kb < kb_end; ++kb) {
         // the first pass over the ring finds every stage free: no wait (a wait that passes at once still costs a
@@ -941,7 +951,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t fmt = TF32 ? 2u : 1u;
       constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((A_MN ? 1u : 0u) << 15) |
                                  ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(BLOCK_N >> 3) << 17) |
@@ -974,7 +984,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     }
   } else {
     // ---------------- epilogue warps: reduce-scatter across the cluster, then the usual epilogue ------------
-    if (warp == 2 && lane == 0) {                          // first: the B tiles of the main loop (see above)
+    if (warp == 2 && elect_one()) {                        // first: the B tiles of the main loop (see above)
       int stage = 0; uint32_t phase = 0;
       for (int kb = kb_begin; kb < kb_end; ++kb) {
         // the first pass over the ring finds every stage free: no wait (a wait that passes at once still costs a
@@ -1180,7 +1190,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs; completion on the even CTA's barrier) ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0; uint32_t phase = 0;
       int fills = 0;                     // as in the single-CTA kernel: no wait on the first pass over the ring
       bool ok = true;
@@ -1217,7 +1227,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: the even CTA only ----------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       constexpr uint32_t fmt = TF32 ? 2u : 1u;
       constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((A_MN ? 1u : 0u) << 15) |
                                  ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(PAIR_TILE_N >> 3) << 17) |
