@@ -52,9 +52,10 @@ int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
 // Position of the caller-supplied pointers in the parameter list of the kernel that takes them in: the input
 // staging kernel (see elementwise.cu), or the first kernel of a small segment's two-launch step.
-struct StageArgs { int count, x, cls, gather, loss; };
-constexpr StageArgs kStageInputsArgs = {19, 3, 9, 14, 15};
-constexpr StageArgs kSmallStepArgs = {5, 1, 2, 3, 4};
+// map: the tensor map of x, where the kernel has one (-1: it has none).
+struct StageArgs { int count, x, cls, gather, loss, map; };
+constexpr StageArgs kStageInputsArgs = {19, 3, 9, 14, 15, -1};
+constexpr StageArgs kSmallStepArgs = {10, 1, 2, 3, 4, 7};
 
 }  // namespace
 
@@ -110,9 +111,13 @@ struct seg_handle {
     std::vector<void*> stage_args;
     const void* cur_x = nullptr; const int32_t* cur_cls = nullptr; float* cur_loss = nullptr;   // now in the exec
     const float* cur_gather = nullptr;
+    int batch = 0;
+    uint32_t box[2] = {0, 0};        // columns and rows of the input tile, for the tensor map of x
   };
   cudaGraphNode_t cap_stage_node = nullptr;   // filled while capturing
   StageArgs cap_stage_idx{};
+  int cap_batch = 0;
+  uint32_t cap_box[2] = {0, 0};
   bool capturing = false;
   std::map<int, StepGraph> graphs; // by batch size
   std::map<std::pair<uint64_t, int>, StepGraph> recovery_graphs;   // by (right segment's uid, batch size)
@@ -428,11 +433,16 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
   seg_status st = SEG_OK;
   auto bail = [&](seg_status s) { seg_destroy(h); return s; };
 
+  {
+    const char* env = getenv("SEG_NO_SMALL_FUSED");
+    h->small_fused = h->precision == SEG_FP32 && !(env && env[0] == '1') &&
+                     small_step_supported(h->n_layers, h->widths.data()) && gemm_tc_init();
+  }
   int64_t off = 0;
   for (int l = 0; l < h->n_layers; ++l) {
     LayerInfo L;
     L.in = h->widths[l]; L.out = h->widths[l + 1];
-    L.ldw = round_up(L.in, 8);
+    L.ldw = h->small_fused ? small_weight_pitch(L.in) : round_up(L.in, 8);
     L.w_off = off; off = round_up(off + (int64_t)L.out * L.ldw, 64);
     L.b_off = off; off = round_up(off + L.out, 64);
     h->layers.push_back(L);
@@ -451,7 +461,8 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
   h->ld_act.assign(h->n_layers + 1, 0);
   h->act_dtype.assign(h->n_layers + 1, h->act_dt);
   for (int l = 0; l <= h->n_layers; ++l) {
-    h->ld_act[l] = round_up(h->widths[l], 8);
+    // a small fp32 segment keeps a column of ones behind its activations (its second kernel's bias gradient)
+    h->ld_act[l] = round_up(h->widths[l] + (h->small_fused ? 1 : 0), 8);
   }
   if (h->is_final) h->act_dtype[h->n_layers] = DT_F32;
   for (int l = 1; l <= h->n_layers; ++l) {
@@ -524,11 +535,6 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
   if ((st = dev_alloc(h, &h->loss_partials, loss_max_partials(), true)) != SEG_OK) return bail(st);
   if ((st = dev_alloc(h, &h->loss_counter, 1, true)) != SEG_OK) return bail(st);
   if ((st = dev_alloc(h, &h->dev_status, 1, true)) != SEG_OK) return bail(st);
-  {
-    const char* env = getenv("SEG_NO_SMALL_FUSED");
-    h->small_fused = h->precision == SEG_FP32 && !(env && env[0] == '1') &&
-                     small_step_supported(h->n_layers, h->widths.data());
-  }
   if (h->small_fused) {
     SmallStep& p = h->small;
     p.n_layers = h->n_layers; p.n_classes = h->n_classes; p.is_final = h->is_final ? 1 : 0;
@@ -543,12 +549,20 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
     }
     p.params = h->params; p.grads = h->grads; p.s1 = h->state1; p.s2 = h->state2;
     p.sil = h->sil; p.cls_stage = h->cls_stage;
-    p.loss_partials = h->loss_partials; p.loss_counter = h->loss_counter; p.loss_dst = h->loss_dst;
+    p.loss_partials = h->loss_partials; p.loss_dst = h->loss_dst;
     p.t = h->step_dev; p.bc = h->bc_dev; p.dev_status = h->dev_status;
     p.lr = h->lr; p.momentum = h->momentum; p.beta1 = h->beta1; p.beta2 = h->beta2; p.eps = h->eps;
-    p.wg_slots = small_step_wgrad_slots(h->n_layers, h->widths.data());
-    if ((st = dev_alloc(h, &p.wg_scratch, (size_t)p.wg_slots * kSimtTileFloats, false)) != SEG_OK) return bail(st);
-    if ((st = dev_alloc(h, &p.wg_counters, p.wg_slots, true)) != SEG_OK) return bail(st);
+    for (int l = 0; l < h->n_layers; ++l) {
+      ++h->launches;
+      if (launch_small_ones(p.act[l], p.ld_act[l], p.widths[l], h->max_batch, h->stream) != cudaSuccess) return bail(SEG_ERR_CUDA);
+    }
+    CUtensorMap maps[4 * kSmallMaxLayers];
+    CUtensorMap* dev_maps = nullptr;
+    if (!small_step_maps(p, h->max_batch, maps)) return bail(SEG_ERR_CUDA);
+    if ((st = dev_alloc(h, &dev_maps, 4 * kSmallMaxLayers, false)) != SEG_OK) return bail(st);
+    if (cudaMemcpyAsync(dev_maps, maps, sizeof(CUtensorMap) * 4 * h->n_layers, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+      return bail(SEG_ERR_CUDA);
+    p.maps = dev_maps;
   }
   if (cudaEventCreate(&h->ev_start) != cudaSuccess || cudaEventCreate(&h->ev_stop) != cudaSuccess)
     return bail(SEG_ERR_CUDA);
@@ -617,6 +631,16 @@ seg_status seg_forward(seg_handle* h, const void* x, int32_t batch, void* y) {
   if (!h || !x || !y) return SEG_ERR_INVALID_ARG;
   DeviceGuard guard(h);
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
+  if (h->small_fused) {               // small fp32 segment: all layers in one launch, the last one's output also into y
+    SmallStep p = h->small;
+    p.batch = batch;
+    Launch l(h, K_FWD);
+    SEG_TRY(h, launch_small_forward(p, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), h->stream),
+            "small-segment forward launch");
+    ++h->family_launches[FAM_SIMT];
+    h->last_batch = batch;
+    return SEG_OK;
+  }
   seg_status st = forward_impl(h, x, batch);
   if (st != SEG_OK) return st;
   return copy_out(h, y, batch);
@@ -644,17 +668,17 @@ static seg_status enqueue_step(seg_handle* h, int batch, bool forked, const void
   cudaStream_t mainst = h->stream;
   seg_status st;
   float* loss_to = loss_out ? loss_out : h->loss_slot;
-  if (h->small_fused && small_step_batch_ok(batch)) {
+  SmallStep p = h->small;
+  p.batch = batch;
+  if (h->small_fused && small_step_batch_ok(p)) {
     // small fp32 segment: staging, forward, loss and the dgrad chain in one launch, every weight and bias
     // gradient with its update in a second
-    SmallStep p = h->small;
-    p.batch = batch;
     {
       Launch lf(h, K_FWD_BWD);
-      SEG_TRY(h, launch_small_fwd_bwd(p, reinterpret_cast<const float*>(x), cls, gather, loss_to, mainst),
+      SEG_TRY(h, launch_small_fwd_bwd(p, reinterpret_cast<const float*>(x), cls, gather, loss_to, mainst, h->cap_box),
               "small-segment forward/backward launch");
     }
-    if (h->capturing) { h->cap_stage_node = last_captured_node(h); h->cap_stage_idx = kSmallStepArgs; }
+    if (h->capturing) { h->cap_stage_node = last_captured_node(h); h->cap_stage_idx = kSmallStepArgs; h->cap_batch = batch; }
     {
       Launch lw(h, K_WGRAD_UPDATE);
       SEG_TRY(h, launch_small_wgrad_update(p, mainst), "small-segment weight-gradient/update launch");
@@ -764,6 +788,8 @@ static bool adopt_captured_graph(seg_handle* h, seg_handle::StepGraph& g, cudaGr
   if (!h->cap_stage_node) return false;
   g.stage_node = h->cap_stage_node;
   g.stage_idx = h->cap_stage_idx;
+  g.batch = h->cap_batch;
+  g.box[0] = h->cap_box[0]; g.box[1] = h->cap_box[1];
   if (cudaGraphKernelNodeGetParams(g.stage_node, &g.stage_params) != cudaSuccess) return false;
   g.stage_args.assign(g.stage_params.kernelParams, g.stage_params.kernelParams + g.stage_idx.count);
   if (cudaGraphInstantiate(&g.exec, graph, 0) != cudaSuccess) { g.exec = nullptr; return false; }
@@ -778,6 +804,13 @@ static seg_status replay_graph(seg_handle* h, seg_handle::StepGraph& g, const vo
     g.stage_args[g.stage_idx.cls] = (void*)&cls;
     g.stage_args[g.stage_idx.gather] = (void*)&gather;
     g.stage_args[g.stage_idx.loss] = (void*)&loss_to;
+    CUtensorMap map;
+    if (g.stage_idx.map >= 0 && small_input_by_tensor(reinterpret_cast<const float*>(x), gather, h->widths[0])) {
+      SmallStep p = h->small;
+      p.batch = g.batch;
+      if (!small_input_map(p, reinterpret_cast<const float*>(x), g.box[0], g.box[1], &map)) return SEG_ERR_CUDA;
+      g.stage_args[g.stage_idx.map] = (void*)&map;
+    }
     cudaKernelNodeParams sp = g.stage_params;
     sp.kernelParams = g.stage_args.data();
     SEG_TRY(h, cudaGraphExecKernelNodeSetParams(g.exec, g.stage_node, &sp), "graph parameter update");

@@ -2,19 +2,29 @@
 // segment's layers, loss against the intermediate labels of the samples' classes or, in the final
 // segment, against the class labels, backward, update; Section 3: layers of 80, 60 and 47 units).
 //
-// A segment whose layers are at most kSmallMaxWidth wide runs ten or more dependent launches of a few
-// microseconds each when every product, the loss and every update is a kernel of its own.  Here
-//   1. small_fwd_bwd_kernel gives every CTA a slice of R rows of the batch and carries it through the
-//      whole chain: input staging (class clamp, gather of label rows), all forward products with bias
-//      and ReLU, the loss and dZ of the last layer, and the dgrad chain.  Activations and dZ of the slice
-//      stay in shared memory (stored k-major, so that a thread reads its rows with 16-byte loads); the
-//      weights of all products of the chain arrive as one stream of 64-row tiles through a cp.async ring.
-//      Every activation and dZ also goes to global memory, where the second kernel (and
-//      seg_get_activation) reads it.
-//   2. small_wgrad_update_kernel forms dW_l = dZ_l^T A_{l-1} of all layers in one grid of 64 x 64 tiles,
-//      the batch split over several CTAs per tile; the bias gradient is the column a ones-vector appended
-//      to A_{l-1} yields.  The last CTA of a tile to arrive adds the partial tiles in split order (a fixed
-//      order: bit-reproducible), stores the gradient and applies the optimizer to its elements.
+// A segment whose layers are at most kSmallMaxWidth wide is a chain of small dependent products: what bounds it
+// is not arithmetic but how few SMs and warps a chain keeps busy, how many instructions a link issues and how long
+// every link takes.
+//   1. small_fwd_bwd_kernel: a cluster of C CTAs owns a block of C * R rows of the batch.  A wide first layer is
+//      split over K: CTA r contracts its slice of the features, at most 132 of them, for all rows of the block and
+//      sends every row's partial sums to the CTA that owns the row (bulk copies through distributed shared
+//      memory).  From there each CTA carries its own R rows through the rest of the chain - the other forward
+//      products, the loss with dZ of the last layer, the dgrad products - with everything it needs already on its
+//      way into shared memory by a handful of bulk and tensor copies; each weight matrix is loaded once for both
+//      directions.  A link of the chain takes one barrier: a warp owns a block of output columns and half of the
+//      rows, its lanes split the contraction in four, and the four shares meet in a shuffle reduce-scatter (a fixed
+//      order: bit-reproducible).  Activations, dZ and the staged input also go to global memory for the second
+//      kernel.  Forward-only calls (seg_forward) run the same kernel up to the last layer's output.
+//   2. small_wgrad_update_kernel: tiles of (all outputs) x NT inputs of dW_l = dZ_l^T [A_{l-1} | 1] for all layers
+//      in one grid; a cluster of S CTAs splits the batch of one tile, tensor copies bring 32 rows of both operands
+//      per stage, threads hold 8 x NT/8 register tiles, the partial tiles are combined as a reduce-scatter through
+//      distributed shared memory (fixed order), and every CTA applies the optimizer to the rows it received.  The
+//      column of ones, which yields the bias gradient, is kept in the padding of the activation buffers.
+// Register tiles: a 16-byte shared-memory load costs the SM 2 cycles when neighbouring lanes share the address and 4
+// when they do not (measured), so r rows x c columns cost 2 r + 4 c cycles of loads per r c cycles of FFMA issue and
+// four k.
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 
@@ -23,526 +33,960 @@
 namespace segk {
 namespace {
 
-constexpr int SS_THREADS = 256;
-constexpr int SS_KT = 64;                                   // contraction rows per staged weight tile
-constexpr int SS_STAGES = 3;                                // weight tiles in flight (cp.async groups)
-constexpr int SS_KF_LD = SS_KT + 4;                         // k-fast tile [128 n][68]: a lane reads 4 k with one conflict-free 16-byte load
-constexpr int SS_NF_LD = kSmallMaxWidth + 4;                // n-fast tile [64 k][132]
-constexpr int SS_STAGE_FLOATS = kSmallMaxWidth * SS_KF_LD;  // the larger of the two layouts
-constexpr int SS_CHUNKS = kSmallMaxWidth * SS_KT / 4 / SS_THREADS;   // 16-byte chunks of a tile per thread
-static_assert(SS_STAGE_FLOATS >= SS_KT * SS_NF_LD, "stage size");
-static_assert(kSmallMaxWidth == 128 && SS_THREADS == 256 && SS_KT == 64, "thread mappings below");
+constexpr int SS_THREADS = 256, SS_WARPS = SS_THREADS / 32;
+constexpr size_t SS_SMEM_LIMIT = 226 * 1024;                // dynamic shared memory; the static part is below 1 KiB
+constexpr uint64_t SS_WAIT_LIMIT_NS = 2000000000ull;
 
-__device__ __forceinline__ void cp_async16(float* smem_dst, const float* src, bool valid) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  const int bytes = valid ? 16 : 0;                         // 0: nothing is read, the 16 bytes are zero-filled
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+// ---- copies, barriers, clusters ---------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// One matrix product of the chain, seen from the weight side: out[r][n] = sum_k left[k][r] * Wmat(k, n) with
-// Wmat(k, n) = W[n * ldw + k] (k_fast: a forward product, A W^T) or W[k * ldw + n] (dgrad, dZ W).
-struct Phase { const float* W; int ldw, K, N; bool k_fast; };
-
-__device__ __forceinline__ Phase phase_of(const SmallStep& p, int ph) {
-  Phase q;
-  const int L = p.n_layers;
-  const int l = ph < L ? ph : 2 * L - 1 - ph;               // forward 0 .. L-1, then dgrad L-1 .. 1
-  q.k_fast = ph < L;
-  q.W = p.params + p.w_off[l]; q.ldw = (int)p.ldw[l];
-  q.K = q.k_fast ? p.widths[l] : p.widths[l + 1];
-  q.N = q.k_fast ? p.widths[l + 1] : p.widths[l];
-  return q;
+__device__ __forceinline__ void bar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count));
 }
-
-// The stream of weight tiles of the whole chain (all forward products, then the dgrad chain): the weights depend
-// on nothing the kernel computes, so the tiles of a later product are in flight while an earlier one finishes.
-// A tile is rows k0 .. k0+63 of Wmat, copied asynchronously, 8 chunks of 16 bytes per thread.  Rows of W are 16-byte
-// aligned and their pitch is a multiple of 8 floats, so a chunk never crosses a row's allocation; what it carries
-// beyond K or N is never read by the arithmetic.  Per phase every thread keeps the source and destination of its
-// first chunk; the others follow at fixed strides (k-fast: thread -> 4 k of row n = tid / 16 + 16 i; n-fast:
-// 4 n of row k = tid / 32 + 8 i).
-struct TileStream {
-  const SmallStep& p;
-  float* stages;
-  int n_phases, ph = 0, k0 = 0, stage = 0;
-  Phase q;
-  const float* src = nullptr;
-  int c4 = 0, r0 = 0, r_step = 0, dst = 0, dst_step = 0, src_step = 0;
-  __device__ TileStream(const SmallStep& pp, float* st) : p(pp), stages(st), n_phases(2 * pp.n_layers - 1) { load_phase(); }
-  __device__ __forceinline__ void load_phase() {
-    q = phase_of(p, ph);
-    const int tid = threadIdx.x;
-    if (q.k_fast) { c4 = 4 * (tid & 15); r0 = tid >> 4; r_step = 16; dst = r0 * SS_KF_LD + c4; dst_step = 16 * SS_KF_LD; }
-    else { c4 = 4 * (tid & 31); r0 = tid >> 5; r_step = 8; dst = r0 * SS_NF_LD + c4; dst_step = 8 * SS_NF_LD; }
-    src = q.W + (int64_t)r0 * q.ldw + c4;
-    src_step = r_step * q.ldw;
-  }
-  __device__ __forceinline__ void issue_next() {           // always commits a group, so that the group count is uniform
-    if (ph < n_phases) {
-      float* d = stages + stage * SS_STAGE_FLOATS + dst;
-      if (q.k_fast) {
-        const bool col_ok = k0 + c4 < q.ldw;
-        const float* s0 = src + k0;
-#pragma unroll
-        for (int i = 0; i < SS_CHUNKS; ++i) {
-          const bool ok = col_ok && r0 + r_step * i < q.N;
-          cp_async16(d + i * dst_step, ok ? s0 + i * src_step : q.W, ok);
-        }
-      } else {
-        const bool col_ok = c4 < q.ldw;
-        const float* s0 = src + (int64_t)k0 * q.ldw;
-#pragma unroll
-        for (int i = 0; i < SS_CHUNKS; ++i) {
-          const bool ok = col_ok && k0 + r0 + r_step * i < q.K;
-          cp_async16(d + i * dst_step, ok ? s0 + i * src_step : q.W, ok);
-        }
-      }
-      k0 += SS_KT;
-      if (k0 >= q.K) {
-        ++ph; k0 = 0;
-        if (ph < n_phases) load_phase();
-      }
+__device__ __forceinline__ void bar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+// Bounded wait: past the limit it records DEV_TIMEOUT and returns (what follows computes garbage, but ends).
+__device__ __forceinline__ void bar_wait(uint64_t* bar, uint32_t parity, int* dev_status) {
+  const uint32_t a = smem_addr(bar);
+  uint32_t spins = 0;
+  uint64_t t0 = 0;
+  for (;;) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+    if (ok) return;
+    if ((++spins & 0xFFu) == 0u) {
+      uint64_t now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > SS_WAIT_LIMIT_NS) { atomicOr(dev_status, (int)DEV_TIMEOUT); return; }
     }
-    cp_async_commit();
-    stage = stage + 1 == SS_STAGES ? 0 : stage + 1;
   }
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void tensor_load(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+               ::"r"(smem_addr(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void tensor_store(const CUtensorMap* map, const void* src, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(src)), "r"(c0), "r"(c1) : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void store_wait_source() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t in_cta(uint32_t local, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void bulk_send(uint32_t dst_cluster, const void* src, uint32_t bytes, uint32_t bar_cluster) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst_cluster), "r"(smem_addr(src)), "r"(bytes), "r"(bar_cluster) : "memory");
+}
+__device__ __forceinline__ void store_cluster4(uint32_t addr, const float4& v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
+
+__host__ __device__ constexpr int up(int v, int m) { return (v + m - 1) / m * m; }
+__host__ __device__ constexpr int pitch_of(int K) { return small_weight_pitch(K); }
+
+// ---- first kernel -----------------------------------------------------------------------------------
+// Shared-memory layout and work split of one launch (offsets in floats; filled by layout_small).
+struct SmallPlan {
+  int C, R;                    // CTAs per cluster, rows of the batch per CTA
+  int ks;                      // features per CTA (C > 1) or the input width rounded up to 4 (C = 1): row pitch of the x tile
+  int late;                    // chain weights share the x and W_0 tiles' memory and are loaded once the first layer is done
+  int streamed;                // chain weights go through two slots instead of one slot each
+  int forward_only;
+  int off_x, off_w0, off_send, off_recv, off_bias, off_tgt, off_dz[2];
+  int off_act[kSmallMaxLayers + 1], off_slot[kSmallMaxLayers];
+  int floats;
 };
 
-// acc[j] += sum_k left[k][rg * RPT + j] * Wmat(k, n) for this thread's column n and its RPT rows; left is the
-// slice's left operand in shared memory, k-major with R rows per k.  All threads of the CTA call it; `cstage` is the
-// stage the next tile to consume sits in.
-template <int R, int RPT>
-__device__ __forceinline__ void rows_times_weights(float (&acc)[RPT], const float* left, const Phase& q, TileStream& ts,
-                                                   int& cstage, int rg, int n) {
-  for (int k0 = 0; k0 < q.K; k0 += SS_KT) {
-    cp_async_wait<SS_STAGES - 2>();      // this tile's group has landed (for this thread's copies) ...
-    __syncthreads();                     // ... and for everyone's; all threads are done with the previous tile
-    ts.issue_next();                     // refills the stage the previous tile occupied
-    const float* stage = ts.stages + cstage * SS_STAGE_FLOATS;
-    cstage = cstage + 1 == SS_STAGES ? 0 : cstage + 1;
-    const int kmax = min(SS_KT, q.K - k0);
-    if (n < q.N) {
-      const float* ap = left + (size_t)k0 * R + rg * RPT;
-      auto fma_row = [&](int kk, float w) {
+// Sum over the SL lane groups (consecutive groups of 32 / SL lanes) of v[0 .. V): afterwards a lane of group b holds, in
+// v[0 .. H), the complete sums of the elements b * H + i, where H = VP / SL and VP = V rounded up to a multiple of SL.
+template <int V, int SL>
+__device__ __forceinline__ void reduce_scatter(float (&v)[(V + SL - 1) / SL * SL], int lane) {
+  constexpr int VP = (V + SL - 1) / SL * SL;
 #pragma unroll
-        for (int u = 0; u < RPT / 4; ++u) {
-          const float4 a = *reinterpret_cast<const float4*>(ap + kk * R + 4 * u);
-          acc[4 * u + 0] = fmaf(a.x, w, acc[4 * u + 0]);
-          acc[4 * u + 1] = fmaf(a.y, w, acc[4 * u + 1]);
-          acc[4 * u + 2] = fmaf(a.z, w, acc[4 * u + 2]);
-          acc[4 * u + 3] = fmaf(a.w, w, acc[4 * u + 3]);
-        }
-      };
-      if (q.k_fast) {
-        const float* ws = stage + n * SS_KF_LD;
-        int kk = 0;
-#pragma unroll 4
-        for (; kk + 4 <= kmax; kk += 4) {
-          const float4 w = *reinterpret_cast<const float4*>(ws + kk);
-          fma_row(kk, w.x); fma_row(kk + 1, w.y); fma_row(kk + 2, w.z); fma_row(kk + 3, w.w);
-        }
-        for (; kk < kmax; ++kk) fma_row(kk, ws[kk]);
-      } else {
-#pragma unroll 4
-        for (int kk = 0; kk < kmax; ++kk) fma_row(kk, stage[kk * SS_NF_LD + n]);
+  for (int len = VP, bit = 16; len > VP / SL; len /= 2, bit /= 2) {
+    const bool hi = (lane & bit) != 0;
+#pragma unroll
+    for (int i = 0; i < VP / 2; ++i) {
+      if (i < len / 2) {
+        const float give = hi ? v[i] : v[i + len / 2];
+        const float keep = hi ? v[i + len / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, bit);
+      }
+    }
+  }
+}
+// The element a lane holds after reduce_scatter, as (row, column index) of an RT x CT tile: element e = b * H + i.
+template <int CT, int H, int SL>
+__device__ __forceinline__ void element_of(int i, int b, int& row, int& col) {
+  row = i / CT; col = i % CT;                               // compile-time alternatives, chosen by the lane group
+#pragma unroll
+  for (int s = 1; s < SL; ++s)
+    if (b == s) { row = (s * H + i) / CT; col = (s * H + i) % CT; }
+}
+
+// v[r * CT + j] += sum over this lane's chunks c (four k each) of A[r][4c ..] . W[n_j][4c ..]; A rows `pa` apart, wp[j] the
+// row of column n_j.
+template <int RT, int CT, int VP>
+__device__ __forceinline__ void dot_rows(float (&v)[VP], const float* A, int pa, const float* const (&wp)[CT], int c0, int c1, int step) {
+#pragma unroll 2
+  for (int c = c0; c < c1; c += step) {
+    float4 w[CT];
+#pragma unroll
+    for (int j = 0; j < CT; ++j) w[j] = lds4(wp[j] + 4 * c);
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+      const float4 a = lds4(A + r * pa + 4 * c);
+#pragma unroll
+      for (int j = 0; j < CT; ++j) {
+        float t = v[r * CT + j];
+        t = fmaf(a.x, w[j].x, t); t = fmaf(a.y, w[j].y, t); t = fmaf(a.z, w[j].z, t); t = fmaf(a.w, w[j].w, t);
+        v[r * CT + j] = t;
       }
     }
   }
 }
 
-// Shared-memory floats of small_fwd_bwd_kernel: weight stages, two dZ buffers, one activation buffer per layer boundary.
-size_t fwd_bwd_smem_floats(const SmallStep& p, int R) {
-  size_t f = (size_t)SS_STAGES * SS_STAGE_FLOATS + 2 * (size_t)kSmallMaxWidth * R;
-  for (int l = 0; l <= p.n_layers; ++l) f += (size_t)p.widths[l] * R;
-  return f;
+// A forward link for R rows: emit(row, n, value) receives every element n < N of A W^T (columns up to N rounded up to 4 are
+// emitted too).  Warp = (half of the rows, block of 8 * CT columns), lane = (column, quarter of the contraction).
+template <int R, int CT, typename Emit>
+__device__ __forceinline__ void link_forward(const float* A, int pa, const float* W, int pw, int K, int N, const Emit& emit) {
+  constexpr int RP = R >= 4 ? 2 : 1, RT = R / RP, V = RT * CT, VP = (V + 3) / 4 * 4, H = VP / 4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sl = lane >> 3;
+  const int rp = warp % RP, n0 = warp / RP * 8 * CT + (lane & 7);
+  if (warp / RP * 8 * CT >= N) return;
+  float v[VP];
+#pragma unroll
+  for (int i = 0; i < VP; ++i) v[i] = 0.f;
+  const float* wp[CT];
+#pragma unroll
+  for (int j = 0; j < CT; ++j) wp[j] = W + min(n0 + 8 * j, N - 1) * pw;
+  dot_rows<RT, CT, VP>(v, A + rp * RT * pa, pa, wp, sl, (K + 3) >> 2, 4);
+  reduce_scatter<V, 4>(v, lane);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    int r, j;
+    element_of<CT, H, 4>(i, sl, r, j);
+    const int n = n0 + 8 * j;
+    if (r < RT && n < up(N, 4)) emit(rp * RT + r, n, v[i]);
+  }
 }
 
-template <int R>
-__global__ void __launch_bounds__(SS_THREADS)
+// A dgrad link: emit(row, k, value) for every element of dZ W (k < K rounded up to 4); lane = (CT consecutive k, quarter of n).
+template <int R, int CT, typename Emit>
+__device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float* W, int pw, int N, int K, const Emit& emit) {
+  constexpr int RP = R >= 4 ? 2 : 1, RT = R / RP, V = RT * CT, VP = (V + 3) / 4 * 4, H = VP / 4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sl = lane >> 3;
+  const int rp = warp % RP, k0 = warp / RP * 8 * CT + (lane & 7) * CT;
+  if (warp / RP * 8 * CT >= K) return;
+  float v[VP];
+#pragma unroll
+  for (int i = 0; i < VP; ++i) v[i] = 0.f;
+  const float* wk = W + min(k0, pw - CT);                   // lanes beyond the row read its end and are not emitted
+  const float* A = dZ + rp * RT * pz;
+  for (int c = sl; c < (N + 3) >> 2; c += 4) {
+    float w[4][CT];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float* row = wk + min(4 * c + i, N - 1) * pw;   // beyond N: dZ is zero there
+      if constexpr (CT == 4) { const float4 t = lds4(row); w[i][0] = t.x; w[i][1] = t.y; w[i][2] = t.z; w[i][3] = t.w; }
+      else if constexpr (CT == 2) { const float2 t = *reinterpret_cast<const float2*>(row); w[i][0] = t.x; w[i][1] = t.y; }
+      else w[i][0] = row[0];
+    }
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+      const float4 a = lds4(A + r * pz + 4 * c);
+#pragma unroll
+      for (int j = 0; j < CT; ++j) {
+        float t = v[r * CT + j];
+        t = fmaf(a.x, w[0][j], t); t = fmaf(a.y, w[1][j], t); t = fmaf(a.z, w[2][j], t); t = fmaf(a.w, w[3][j], t);
+        v[r * CT + j] = t;
+      }
+    }
+  }
+  reduce_scatter<V, 4>(v, lane);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    int r, j;
+    element_of<CT, H, 4>(i, sl, r, j);
+    if (r < RT && k0 + j < up(K, 4)) emit(rp * RT + r, k0 + j, v[i]);
+  }
+}
+
+// Columns per lane of a link with N columns: the smallest for which the warps cover them in one pass.
+template <int R, typename F1, typename F2, typename F4>
+__device__ __forceinline__ void by_width(int N, const F1& f1, const F2& f2, const F4& f4) {
+  constexpr int blocks = SS_WARPS / (R >= 4 ? 2 : 1);
+  if (N <= 8 * blocks) f1();
+  else if (N <= 16 * blocks) f2();
+  else f4();
+}
+
+// CT0: columns per lane in the split first layer (16 lanes along the columns); 0: the first layer is an ordinary link (C = 1).
+template <int R, int CT0>
+__global__ void __launch_bounds__(SS_THREADS, 1)
 small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restrict__ x, const int32_t* __restrict__ cls,
-                     const float* __restrict__ gather, float* loss_to) {
-  constexpr int RPT = R / 2;
-  extern __shared__ __align__(16) float ss_smem[];
-  __shared__ int cls_s[R];
-  __shared__ float red[32];
+                     const float* __restrict__ gather, float* loss_to, const __grid_constant__ SmallPlan q, float* y,
+                     const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w0,
+                     const __grid_constant__ CUtensorMap map_stage) {
+  constexpr bool SPLIT = CT0 > 0;
+  extern __shared__ __align__(128) float sm[];
+  __shared__ uint64_t bars[3 + kSmallMaxLayers];            // x (and W_0) tiles; biases; received sums; weights of layer l
+  __shared__ int cls_s[128];                                // classes of the cluster's rows (C * R <= 128)
+  __shared__ float red[SS_WARPS];
+  uint64_t *bar_x = bars, *bar_bias = bars + 1, *bar_recv = bars + 2, *bar_w = bars + 3;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, L = p.n_layers;
+  const int C = SPLIT ? q.C : 1, rank = SPLIT ? (int)cluster_rank() : 0;
+  const int RB = C * R;                                     // rows of the cluster's block
+  const int rb0 = (int)blockIdx.x / C * RB;
+  const int row0 = rb0 + rank * R, nv = max(0, min(R, p.batch - row0));
+  const int nvb = min(RB, p.batch - rb0);                   // valid rows of the block
+  constexpr int first = SPLIT ? 1 : 0;                      // first layer whose weights sit in a slot
+  const int n0 = p.widths[0], NL = p.widths[L], N1 = p.widths[1];
+  const bool train = !q.forward_only;
+  const int k0 = SPLIT ? rank * q.ks : 0;                   // first feature of this CTA's slice
+  float* xs = sm + q.off_x;
+  float* bias_s = sm + q.off_bias;
+  auto act_s = [&](int l) { return sm + q.off_act[l]; };
+  auto slot = [&](int l) { return sm + q.off_slot[l]; };
+  const float* xsrc = gather != nullptr ? gather : x;
+  const bool x_tensor = small_input_by_tensor(x, gather, n0);       // the host built map_x under the same condition
+  const bool stage = train && k0 < n0;
+  const uint32_t recv_bytes = SPLIT ? (uint32_t)(SS_WARPS / C * R * up(N1, 4) * 4) : 0u;   // from each CTA of the cluster
+
+  if (tid == 0) {
+    for (int i = 0; i < 3 + kSmallMaxLayers; ++i) bar_init(bars + i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async();
+    if (SPLIT) bar_expect(bar_recv, (uint32_t)(C - 1) * recv_bytes);
+  }
+  __syncthreads();
+  if (SPLIT) cluster_arrive_release();                      // "my barriers exist"; waited for before the first send
   pdl_wait();
   pdl_trigger();
-  const int tid = threadIdx.x, n = tid & (kSmallMaxWidth - 1), rg = tid >> 7;
-  const int L = p.n_layers;
-  const int row0 = blockIdx.x * R;
-  const int nv = min(R, p.batch - row0);
-  float* dzT[2] = {ss_smem + SS_STAGES * SS_STAGE_FLOATS, ss_smem + SS_STAGES * SS_STAGE_FLOATS + kSmallMaxWidth * R};
-  float* aT0 = dzT[1] + kSmallMaxWidth * R;
-  auto aT = [&](int l) {               // activation of layer boundary l (0: the segment's input), [widths[l]][R]
-    float* q = aT0;
-    for (int i = 0; i < l; ++i) q += p.widths[i] * R;
-    return q;
-  };
-  TileStream ts(p, ss_smem);
-  int cstage = 0;
-#pragma unroll
-  for (int i = 0; i < SS_STAGES - 1; ++i) ts.issue_next();
 
-  // step counter, Adam's bias corrections, where the loss goes; class indices of the slice (clamped)
-  if (blockIdx.x == 0 && tid == 0) {
-    const unsigned long long step = *p.t + 1ull;
-    *p.t = step;
-    if (p.optimizer == SEG_ADAM) {      // the only reader of the bias corrections; two double-precision powers cost over a microsecond
-      p.bc[0] = (float)(1.0 - pow((double)p.beta1, (double)step));
-      p.bc[1] = (float)(1.0 - pow((double)p.beta2, (double)step));
+  auto load_weight = [&](int l) {                           // by the issuing thread: the whole matrix, rows at their global pitch
+    const uint32_t bytes = (uint32_t)p.widths[l + 1] * (uint32_t)p.ldw[l] * 4u;
+    bar_expect(bar_w + l, bytes);
+    bulk_load(slot(l), p.params + p.w_off[l], bytes, bar_w + l);
+  };
+  auto load_chain = [&]() {
+    const int last = q.streamed ? min(L, first + 2) : L;
+    for (int l = first; l < last; ++l) load_weight(l);
+  };
+  if (warp == 0) {
+    if (elect_one()) {
+      const uint32_t xb = x_tensor ? (uint32_t)(RB * q.ks * 4) : 0u, wb = SPLIT ? (uint32_t)(N1 * q.ks * 4) : 0u;
+      bar_expect(bar_x, xb + wb);
+      if (SPLIT) tensor_load(sm + q.off_w0, &map_w0, k0, 0, bar_x);
+      if (x_tensor) tensor_load(xs, &map_x, k0, rb0, bar_x);
+      uint32_t bb = 0;
+      for (int l = 0; l < L; ++l) bb += (uint32_t)up(p.widths[l + 1], 4) * 4u;
+      bar_expect(bar_bias, bb);
+      for (int l = 0; l < L; ++l)
+        bulk_load(bias_s + l * kSmallMaxWidth, p.params + p.b_off[l], (uint32_t)up(p.widths[l + 1], 4) * 4u, bar_bias);
+      if (!q.late) load_chain();
     }
-    *p.loss_dst = loss_to;
   }
-  if (tid < R) {
+  // classes of the block's rows, clamped
+  if (train && tid < RB) {
     int c = 0;
-    if (tid < nv) {
-      c = cls[row0 + tid];
+    if (tid < nvb) {
+      c = cls[rb0 + tid];
       if (c < 0 || c >= p.n_classes) {
-        atomicOr(p.dev_status, (int)DEV_BAD_CLASS);
+        if (rank == 0) atomicOr(p.dev_status, (int)DEV_BAD_CLASS);
         c = min(max(c, 0), p.n_classes - 1);
       }
-      p.cls_stage[row0 + tid] = c;
+      if (rank == 0) p.cls_stage[rb0 + tid] = c;
     }
     cls_s[tid] = c;
   }
-  __syncthreads();
-
-  // the slice's input rows: the caller's batch, or the previous cut's label rows gathered by class
-  {
-    const int n0 = p.widths[0];
-    for (int k = tid; k < n0; k += SS_THREADS) {
-      float v[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        v[r] = 0.f;
-        if (r < nv) {
-          const float* src = gather ? gather + (int64_t)cls_s[r] * n0 : x + (int64_t)(row0 + r) * n0;
-          v[r] = src[k];
-        }
+  // step counter, Adam's bias corrections, where the loss goes
+  if (train && blockIdx.x == 0 && tid == SS_THREADS - 32) {
+    const unsigned long long step = *p.t + 1ull;
+    *p.t = step;
+    if (p.optimizer == SEG_ADAM) {                          // beta^t by repeated squaring, in double precision
+      double r1 = 1.0, r2 = 1.0, b1 = (double)p.beta1, b2 = (double)p.beta2;
+      for (unsigned long long e = step; e != 0; e >>= 1) {
+        if (e & 1ull) { r1 *= b1; r2 *= b2; }
+        b1 *= b1; b2 *= b2;
       }
+      p.bc[0] = (float)(1.0 - r1);
+      p.bc[1] = (float)(1.0 - r2);
+    }
+    *p.loss_dst = loss_to;
+  }
+  __syncthreads();                                          // cls_s
+  if (!x_tensor) {
+    // label rows gathered by class, or a batch whose rows are not whole 16-byte groups: plain loads, a row per warp.  The
+    // column of ones is put down as well: the staging store clips whole 16-byte groups only (its weights are zero)
+    for (int r = warp; r < RB; r += SS_WARPS) {
+      const float* src = gather != nullptr ? gather + (int64_t)cls_s[r] * n0 : xsrc + (int64_t)(rb0 + min(r, nvb - 1)) * n0;
+      for (int k = lane; k < q.ks; k += 32) xs[r * q.ks + k] = (r < nvb && k0 + k < n0) ? src[k0 + k] : (k0 + k == n0 ? 1.f : 0.f);
+    }
+    fence_async();                                          // the staging store below reads them through the async proxy
+    __syncthreads();
+  }
+  // the loss targets of the CTA's rows, in flight during the forward pass
+  const int NL4 = up(NL, 4);
+  float tgt_v[(R * kSmallMaxWidth + SS_THREADS - 1) / SS_THREADS];
+  const bool want_targets = train && !p.is_final;
+  if (want_targets) {
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        if (r < nv) p.act[0][(int64_t)(row0 + r) * p.ld_act[0] + k] = v[r];
-#pragma unroll
-      for (int u = 0; u < R / 4; ++u)
-        *reinterpret_cast<float4*>(aT0 + (size_t)k * R + 4 * u) = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+    for (int i = 0; i < (R * kSmallMaxWidth + SS_THREADS - 1) / SS_THREADS; ++i) {
+      const int e = tid + i * SS_THREADS, r = e >> 7, n = e & 127;
+      tgt_v[i] = (r < nv && n < NL) ? __ldg(p.sil + (int64_t)cls_s[rank * R + r] * NL + n) : 0.f;
     }
   }
 
-  // forward:  A_l = act(A_{l-1} W_l^T + b_l)   (the first wait of every product orders the shared-memory
-  // writes of the step before it)
-  for (int l = 0; l < L; ++l) {
-    const Phase q = phase_of(p, l);
-    float acc[RPT];
-#pragma unroll
-    for (int j = 0; j < RPT; ++j) acc[j] = 0.f;
-    const float b = n < q.N ? p.params[p.b_off[l] + n] : 0.f;      // in flight during the product
-    rows_times_weights<R, RPT>(acc, aT(l), q, ts, cstage, rg, n);
-    if (n < q.N) {
-      const bool relu = (l < L - 1) || p.last_relu;
-      float* an = aT(l + 1) + (size_t)n * R + rg * RPT;
-#pragma unroll
-      for (int j = 0; j < RPT; ++j) {
-        float v = acc[j] + b;
-        if (relu) v = fmaxf(v, 0.f);
-        an[j] = v;
-        const int r = rg * RPT + j;
-        if (r < nv) p.act[l + 1][(int64_t)(row0 + r) * p.ld_act[l + 1] + n] = v;
-      }
-    }
-  }
-  __syncthreads();
-
-  // loss and dZ of the last layer
-  const int NL = p.widths[L];
-  const float* zT = aT(L);
-  float* dz_cur = dzT[0];
-  float* dz_g = p.dz[L - 1];
-  const int64_t ld_dzL = p.ld_act[L];
+  // output of layer l, element (r, n): bias, ReLU, shared and global memory; on the last layer of a non-final segment
+  // also the loss  mean (a - t)^2  and  dZ = 2 (a - t) / (B N_P) * [a > 0]
   float lsum = 0.f;
-  if (!p.is_final) {
-    // mean squared error against the label row of the sample's class:  dZ = 2 (a - t) / (B N_P) * [a > 0]
-    const float gscale = 2.0f / (float)((int64_t)p.batch * NL);
-    if (n < NL) {
-      float tgt[RPT];
-#pragma unroll
-      for (int j = 0; j < RPT; ++j) tgt[j] = rg * RPT + j < nv ? __ldg(p.sil + (int64_t)cls_s[rg * RPT + j] * NL + n) : 0.f;
-#pragma unroll
-      for (int j = 0; j < RPT; ++j) {
-        const int r = rg * RPT + j;
-        float g = 0.f;
-        if (r < nv) {
-          const float a = zT[(size_t)n * R + r];
-          const float d = a - tgt[j];
-          lsum = fmaf(d, d, lsum);
-          g = d * gscale;
-          if (p.last_relu && !(a > 0.f)) g = 0.f;
-          dz_g[(int64_t)(row0 + r) * ld_dzL + n] = g;
-        }
-        dz_cur[(size_t)n * R + r] = g;
+  const float gscale = 2.0f / (float)((int64_t)p.batch * NL);
+  float* dz_cur = sm + q.off_dz[0];
+  auto emit_forward = [&](int l, int r, int n, float v) {
+    const int N = p.widths[l + 1];
+    const bool last = l == L - 1;
+    v += bias_s[l * kSmallMaxWidth + n];
+    if (!last || p.last_relu) v = fmaxf(v, 0.f);
+    if (n >= N) v = 0.f;
+    const bool store = r < nv && n < N;
+    if (store) p.act[l + 1][(int64_t)(row0 + r) * p.ld_act[l + 1] + n] = v;
+    if (last && store && y != nullptr) y[(int64_t)(row0 + r) * N + n] = v;
+    if (last && want_targets) {
+      float g = 0.f;
+      if (store) {
+        const float d = v - sm[q.off_tgt + r * NL4 + n];
+        lsum = fmaf(d, d, lsum);
+        g = (p.last_relu && !(v > 0.f)) ? 0.f : d * gscale;
+        p.dz[L - 1][(int64_t)(row0 + r) * p.ld_act[L] + n] = g;
       }
+      dz_cur[r * kSmallMaxWidth + n] = g;
+    } else {
+      act_s(l + 1)[r * up(N, 4) + n] = v;
+    }
+  };
+  auto put_targets = [&]() {
+    if (!want_targets) return;
+#pragma unroll
+    for (int i = 0; i < (R * kSmallMaxWidth + SS_THREADS - 1) / SS_THREADS; ++i) {
+      const int e = tid + i * SS_THREADS, r = e >> 7, n = e & 127;
+      if (r < R && n < NL4) sm[q.off_tgt + r * NL4 + n] = tgt_v[i];
+    }
+  };
+
+  // ---- first layer, split over the cluster --------------------------------------------------------
+  if constexpr (SPLIT) {
+    const int N4 = up(N1, 4);
+    constexpr int V = R * CT0, VP = (V + 1) / 2 * 2, H = VP / 2;
+    const int KW = SS_WARPS / C, owner = warp % C, kw = warp / C;    // a warp contracts for one owner's rows; KW warps share its k
+    float v[VP];
+#pragma unroll
+    for (int i = 0; i < VP; ++i) v[i] = 0.f;
+    const float* wp[CT0];
+#pragma unroll
+    for (int j = 0; j < CT0; ++j) wp[j] = sm + q.off_w0 + min((lane & 15) + 16 * j, N1 - 1) * q.ks;
+    bar_wait(bar_x, 0, p.dev_status);
+    if (warp == 0 && stage) {                               // the staged input of the second kernel
+      if (elect_one()) tensor_store(&map_stage, xs, k0, rb0);
+    }
+    const int kc = max(0, min(q.ks, n0 - k0) + 3) >> 2;     // 16-byte groups that hold features
+    dot_rows<R, CT0, VP>(v, xs + owner * R * q.ks, q.ks, wp, 2 * kw + (lane >> 4), kc, 2 * KW);
+    reduce_scatter<V, 2>(v, lane);
+    // [owner][kw][row][column] in the send buffer, the own rows' share straight into the receive buffer
+    float* out = owner == rank ? sm + q.off_recv + (size_t)(rank * KW + kw) * R * N4 : sm + q.off_send + (size_t)(owner * KW + kw) * R * N4;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      int r, j;
+      element_of<CT0, H, 2>(i, lane >> 4, r, j);
+      const int n = (lane & 15) + 16 * j;
+      if (r < R && n < N4) out[r * N4 + n] = v[i];
+    }
+    fence_async();
+    cluster_wait_acquire();                                 // every peer's receive barrier exists
+    __syncthreads();
+    if (warp == 0) {
+      if (elect_one()) {
+        for (int d = 1; d < C; ++d) {
+          const int dest = (rank + d) & (C - 1);
+          bulk_send(in_cta(smem_addr(sm + q.off_recv), (uint32_t)dest) + (uint32_t)rank * recv_bytes,
+                    reinterpret_cast<const char*>(sm + q.off_send) + (size_t)dest * recv_bytes, recv_bytes,
+                    in_cta(smem_addr(bar_recv), (uint32_t)dest));
+        }
+      }
+      if (q.late) {                                         // the x and W_0 tiles are free once the staging store has read them
+        if (stage) store_wait_source();
+        __syncwarp();
+        if (elect_one()) load_chain();
+      }
+    }
+    put_targets();
+    bar_wait(bar_bias, 0, p.dev_status);
+    bar_wait(bar_recv, 0, p.dev_status);
+    cluster_arrive_release();                               // "I have received everything"; waited for at the very end
+    if (L == 1) __syncthreads();                            // the targets
+    const int G = N4 / 4;
+    for (int e = tid; e < R * G; e += SS_THREADS) {
+      const int r = e / G, g = e - r * G;
+      const float* src = sm + q.off_recv + r * N4 + 4 * g;
+      float4 s[SS_WARPS];
+#pragma unroll
+      for (int u = 0; u < SS_WARPS; ++u) s[u] = lds4(src + u * R * N4);
+      float4 t = s[0];
+#pragma unroll
+      for (int u = 1; u < SS_WARPS; ++u) add4(t, s[u]);
+      emit_forward(0, r, 4 * g, t.x); emit_forward(0, r, 4 * g + 1, t.y);
+      emit_forward(0, r, 4 * g + 2, t.z); emit_forward(0, r, 4 * g + 3, t.w);
     }
   } else {
-    // softmax cross-entropy, one warp per row:  dZ = (softmax(z) - onehot) / B
-    const int lane = tid & 31, warp = tid >> 5;
-    const float inv_b = 1.0f / (float)p.batch;
-    for (int r = warp; r < R; r += SS_THREADS / 32) {
-      float v[kSmallMaxWidth / 32];
-      float mx = -INFINITY;
-#pragma unroll
-      for (int j = 0; j < kSmallMaxWidth / 32; ++j) {
-        const int i = lane + 32 * j;
-        v[j] = i < NL ? zT[(size_t)i * R + r] : -INFINITY;
-        mx = fmaxf(mx, v[j]);
-      }
-      mx = warp_max(mx);
-      float se = 0.f;
-#pragma unroll
-      for (int j = 0; j < kSmallMaxWidth / 32; ++j)
-        if (lane + 32 * j < NL) se += expf(v[j] - mx);
-      se = warp_sum(se);
-      const float inv_se = 1.0f / se;
-      const int c = cls_s[r];
-      float zc = 0.f;
-#pragma unroll
-      for (int j = 0; j < kSmallMaxWidth / 32; ++j) {
-        const int i = lane + 32 * j;
-        if (i < NL) {
-          float g = 0.f;
-          if (r < nv) {
-            g = (expf(v[j] - mx) * inv_se - (i == c ? 1.f : 0.f)) * inv_b;
-            if (p.last_relu && !(v[j] > 0.f)) g = 0.f;
-            dz_g[(int64_t)(row0 + r) * ld_dzL + i] = g;
-            if (i == c) zc = v[j];
-          }
-          dz_cur[(size_t)i * R + r] = g;
-        }
-      }
-      zc = warp_sum(zc);
-      if (lane == 0 && r < nv) lsum += logf(se) - (zc - mx);
+    put_targets();
+    bar_wait(bar_bias, 0, p.dev_status);
+    if (x_tensor) bar_wait(bar_x, 0, p.dev_status);
+    if (warp == 0 && stage) {
+      if (elect_one()) tensor_store(&map_stage, xs, 0, rb0);
     }
   }
 
-  // dgrad chain:  dZ_{l-1} = (dZ_l W_l) * [A_{l-1} > 0]
-  for (int l = L - 1; l >= 1; --l) {
-    const Phase q = phase_of(p, 2 * L - 1 - l);
-    float acc[RPT];
+  // ---- the forward chain ------------------------------------------------------------------------------
+  for (int l = first; l < L; ++l) {
+    __syncthreads();                                        // the layer's input is complete
+    bar_wait(bar_w + l, 0, p.dev_status);
+    const int K = p.widths[l], N = p.widths[l + 1];
+    const float* A = l == 0 ? xs : act_s(l);
+    const int pa = l == 0 ? q.ks : up(K, 4), pw = (int)p.ldw[l];
+    auto emit = [&](int r, int n, float v) { emit_forward(l, r, n, v); };
+    by_width<R>(N, [&]() { link_forward<R, 1>(A, pa, slot(l), pw, K, N, emit); },
+                [&]() { link_forward<R, 2>(A, pa, slot(l), pw, K, N, emit); },
+                [&]() { link_forward<R, 4>(A, pa, slot(l), pw, K, N, emit); });
+    if (q.streamed && l + 2 < L) {                          // two slots: refill this one for the layer after the next
+      __syncthreads();
+      if (warp == 0) { if (elect_one()) { fence_async(); load_weight(l + 2); } }
+    }
+  }
+  if (!train) {
+    if (SPLIT) cluster_wait_acquire();
+    return;
+  }
+  __syncthreads();
+
+  // ---- softmax cross-entropy of a final segment, 16 lanes per row:  dZ = (softmax(z) - onehot) / B -------
+  if (p.is_final) {
+    constexpr int M = kSmallMaxWidth / 16;
+    const int r = tid >> 4, i0 = tid & 15;
+    const float inv_b = 1.0f / (float)p.batch;
+    const float* z = act_s(L) + min(r, R - 1) * NL4;
+    float v[M], mx = -INFINITY;
 #pragma unroll
-    for (int j = 0; j < RPT; ++j) acc[j] = 0.f;
-    rows_times_weights<R, RPT>(acc, dz_cur, q, ts, cstage, rg, n);
-    float* dz_next = (dz_cur == dzT[0]) ? dzT[1] : dzT[0];
-    if (n < q.N) {
-      const float* al = aT(l) + (size_t)n * R + rg * RPT;
+    for (int j = 0; j < M; ++j) {
+      v[j] = i0 + 16 * j < NL ? z[i0 + 16 * j] : -INFINITY;
+      mx = fmaxf(mx, v[j]);
+    }
 #pragma unroll
-      for (int j = 0; j < RPT; ++j) {
-        const int r = rg * RPT + j;
-        float g = acc[j];
-        if (!(al[j] > 0.f)) g = 0.f;
-        dz_next[(size_t)n * R + r] = g;
-        if (r < nv) p.dz[l - 1][(int64_t)(row0 + r) * p.ld_act[l] + n] = g;
+    for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    float ex[M], se = 0.f, zc = 0.f;
+    const int c = cls_s[rank * R + min(r, R - 1)];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      ex[j] = 0.f;
+      if (16 * j < NL) ex[j] = i0 + 16 * j < NL ? expf(v[j] - mx) : 0.f;
+      se += ex[j];
+      if (i0 + 16 * j == c) zc = v[j];
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) { se += __shfl_xor_sync(0xFFFFFFFFu, se, o); zc += __shfl_xor_sync(0xFFFFFFFFu, zc, o); }
+    const float inv_se = 1.0f / se;
+    if (r < R) {
+#pragma unroll
+      for (int j = 0; j < M; ++j) {
+        const int i = i0 + 16 * j;
+        if (i < NL4) {
+          float g = 0.f;
+          if (r < nv && i < NL) {
+            g = (ex[j] * inv_se - (i == c ? 1.f : 0.f)) * inv_b;
+            if (p.last_relu && !(v[j] > 0.f)) g = 0.f;
+            p.dz[L - 1][(int64_t)(row0 + r) * p.ld_act[L] + i] = g;
+          }
+          dz_cur[r * kSmallMaxWidth + i] = g;
+        }
       }
+      if (i0 == 0 && r < nv) lsum = logf(se) - (zc - mx);
+    }
+  }
+  lsum = warp_sum(lsum);
+  if (lane == 0) red[warp] = lsum;
+  __syncthreads();
+  if (tid == SS_THREADS - 32) {                             // the CTA's share of the batch loss; the second kernel adds them up
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < SS_WARPS; ++w) t += red[w];
+    p.loss_partials[blockIdx.x] = t;
+  }
+
+  // ---- dgrad chain:  dZ_{l-1} = (dZ_l W_l) * [A_{l-1} > 0] -----------------------------------------------
+  for (int l = L - 1; l >= 1; --l) {
+    const int K = p.widths[l], K4 = up(K, 4), N = p.widths[l + 1], pw = (int)p.ldw[l];
+    if (q.streamed && l + 2 < L) bar_wait(bar_w + l, 1, p.dev_status);   // loaded a second time
+    float* dz_next = dz_cur == sm + q.off_dz[0] ? sm + q.off_dz[1] : sm + q.off_dz[0];
+    const float* al = act_s(l);
+    auto emit = [&](int r, int k, float v) {
+      if (!(al[r * K4 + k] > 0.f)) v = 0.f;                 // columns beyond the width hold 0: masked as well
+      dz_next[r * kSmallMaxWidth + k] = v;
+      if (r < nv && k < K) p.dz[l - 1][(int64_t)(row0 + r) * p.ld_act[l] + k] = v;
+    };
+    by_width<R>(K, [&]() { link_dgrad<R, 1>(dz_cur, kSmallMaxWidth, slot(l), pw, N, K, emit); },
+                [&]() { link_dgrad<R, 2>(dz_cur, kSmallMaxWidth, slot(l), pw, N, K, emit); },
+                [&]() { link_dgrad<R, 4>(dz_cur, kSmallMaxWidth, slot(l), pw, N, K, emit); });
+    __syncthreads();
+    if (q.streamed && l - 2 >= 1) {
+      if (warp == 0) { if (elect_one()) { fence_async(); load_weight(l - 2); } }
     }
     dz_cur = dz_next;
   }
-  cp_async_wait<0>();
-
-  const float bt = block_sum(lsum, red);
-  const float scale = p.is_final ? 1.0f / (float)p.batch : 1.0f / (float)((int64_t)p.batch * NL);
-  finish_loss(bt, p.loss_partials, p.loss_counter, loss_to, nullptr, scale, red);
+  if (warp == 0 && stage) store_wait_all();                 // (a no-op for the threads that issued no store)
+  if (SPLIT) cluster_wait_acquire();                        // the peers have read what this CTA sent
 }
 
 // ---- weight gradients of all layers, bias gradients and the update ---------------------------------
-constexpr int WT = 64, WK = 32, WPAD = 4;
+constexpr int WK = 32, W_STAGES = 6;                        // batch rows per stage, stages at most
 
-__host__ __device__ inline int wgrad_tiles(int in, int out) { return ((out + WT - 1) / WT) * ((in + 1 + WT - 1) / WT); }
+__host__ __device__ inline int wgrad_tiles(int in, int nt) { return (in + 1 + nt - 1) / nt; }
 
-template <int OPT>
-__global__ void __launch_bounds__(SS_THREADS)
-small_wgrad_update_kernel(SmallStep p, int splits, int k_per_split) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ bool is_last;
-  __shared__ __align__(16) float As[WK][WT + WPAD];
-  __shared__ __align__(16) float Bs[WK][WT + WPAD];
-  const int tile = blockIdx.x / splits, z = blockIdx.x - tile * splits;
-  int l = 0, t = tile;
+// Floats of dynamic shared memory: the operand ring, which also holds the thread groups' partial tiles, and the received slices.
+__host__ __device__ inline int wgrad_ring_floats(int mt, int nt, int stages) {
+  const int ring = stages * WK * (mt + nt), parts = (SS_THREADS / mt) * mt * nt;
+  return ring > parts ? ring : parts;
+}
+
+template <int OPT, int NT>
+__global__ void __launch_bounds__(SS_THREADS, 2)
+small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_per_cta, int n_partials, int stages) {
+  constexpr int CN = NT / 8;                                // columns per thread
+  constexpr int CPR = NT / 4;                               // 16-byte groups per row of B
+  extern __shared__ __align__(128) float sm[];
+  __shared__ uint64_t full[W_STAGES], empty[W_STAGES];
+  __shared__ float red[32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = S > 1 ? (int)cluster_rank() : 0;
+  int l = 0, t = (int)blockIdx.x / S;
   for (; l < p.n_layers - 1; ++l) {
-    const int nt = wgrad_tiles(p.widths[l], p.widths[l + 1]);
+    const int nt = wgrad_tiles(p.widths[l], NT);
     if (t < nt) break;
     t -= nt;
   }
-  const int in = p.widths[l], out = p.widths[l + 1];
-  const int tiles_n = (in + 1 + WT - 1) / WT;
-  const int m0 = (t / tiles_n) * WT, n0 = (t % tiles_n) * WT;
-  const float* __restrict__ dz = p.dz[l];            // (m = o, k = b) at dz[b * ld_dz + o]
-  const float* __restrict__ ap = p.act[l];           // (k = b, n = i) at ap[b * ld_a + i];  column `in` is all ones
-  const int64_t ld_dz = p.ld_act[l + 1], ld_a = p.ld_act[l];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int k_begin = z * k_per_split, k_end = min(p.batch, k_begin + k_per_split);
-  // A k-step of each operand is 32 rows of 64 floats = 512 groups of 4: two per thread.  A group inside the
-  // buffer's pitch is one 16-byte load (rows are 32-byte aligned; what lies between the width and the pitch is
-  // zero, and products with it are never stored); the group of A_{l-1} that holds column `in` (the ones) or
-  // crosses the width is put together element by element.
-  constexpr int LD = WT * WK / 4 / SS_THREADS;
-  float4 ra[LD], rb[LD];
-  float acc[4][4] = {};
-  auto fetch = [&](int k0) {
+  const int in = p.widths[l], out = p.widths[l + 1], MT = up(out, 8), n0 = t * NT;
+  const int items = MT;                                     // (MT / 8) x 8 threads hold the tile
+  const int G = SS_THREADS / items, grp = tid / items, it = tid - grp * items;
+  const int tx = it & 7, ty = it >> 3;
+  const int k_begin = rank * rows_per_cta, k_end = min(p.batch, k_begin + rows_per_cta);
+  const int rows = max(0, k_end - k_begin), steps = (rows + WK - 1) / WK;
+  float* ringA = sm;                                        // [stage][WK][MT]
+  float* ringB = sm + stages * WK * MT;                     // [stage][WK][NT]
+  float* recv = sm + wgrad_ring_floats(MT, NT, stages);     // [source CTA][MT / S rows][NT]
+  const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(p.maps) + 4 * l;
+  const CUtensorMap* map_a = maps;                          // (m = o, k = b) at dz[b * ld + o]
+  const CUtensorMap* map_b = maps + (NT == 64 ? 1 : NT == 32 ? 2 : 3);   // (k = b, n = i) at act[b * ld + i]; column `in` holds ones
+  const uint32_t stage_bytes = (uint32_t)(WK * (MT + NT) * 4);
+  auto load = [&](int step) {                               // by the issuing thread
+    const int s = step % stages;
+    bar_expect(full + s, stage_bytes);
+    tensor_load(ringA + s * WK * MT, map_a, 0, k_begin + step * WK, full + s);
+    tensor_load(ringB + s * WK * NT, map_b, n0, k_begin + step * WK, full + s);
+  };
+  if (tid == 0) {
+    for (int i = 0; i < stages; ++i) { bar_init(full + i, 1); bar_init(empty + i, SS_WARPS); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async();
+  }
+  __syncthreads();
+  if (S > 1) cluster_arrive_release();
+  pdl_wait();
+  pdl_trigger();
+  if (warp == 0) {
+    if (elect_one())
+      for (int s = 0; s < min(stages, steps); ++s) load(s);
+  }
+  float lpart = 0.f;                                        // the batch loss: the first block adds the first kernel's shares
+  if (blockIdx.x == 0)
+    for (int i = tid; i < n_partials; i += SS_THREADS) lpart += p.loss_partials[i];
+
+  float acc[8][CN];
 #pragma unroll
-    for (int i = 0; i < LD; ++i) {
-      const int idx = threadIdx.x + SS_THREADS * i;
-      const int c = (idx & 15) * 4, k = k0 + (idx >> 4);
-      ra[i] = make_float4(0.f, 0.f, 0.f, 0.f); rb[i] = ra[i];
-      if (k < k_end) {
-        if (m0 + c + 3 < ld_dz) ra[i] = *reinterpret_cast<const float4*>(dz + (int64_t)k * ld_dz + m0 + c);
-        if (n0 + c + 3 < in) {
-          rb[i] = *reinterpret_cast<const float4*>(ap + (int64_t)k * ld_a + n0 + c);
-        } else {
-          float t[4];
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int cc = n0 + c + j;
-            t[j] = cc < in ? ap[(int64_t)k * ld_a + cc] : (cc == in ? 1.0f : 0.f);
-          }
-          rb[i] = make_float4(t[0], t[1], t[2], t[3]);
+    for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+  struct Frag { float a[8], b[CN]; };
+  auto fetch_frag = [&](const float* a_s, const float* b_s, int k, Frag& f) {
+    const float4 a0 = lds4(a_s + k * MT), a1 = lds4(a_s + k * MT + 4);
+    f.a[0] = a0.x; f.a[1] = a0.y; f.a[2] = a0.z; f.a[3] = a0.w; f.a[4] = a1.x; f.a[5] = a1.y; f.a[6] = a1.z; f.a[7] = a1.w;
+    if constexpr (CN == 8) {
+      const float4 b0 = lds4(b_s + k * NT + 4 * tx), b1 = lds4(b_s + k * NT + 32 + 4 * tx);
+      f.b[0] = b0.x; f.b[1] = b0.y; f.b[2] = b0.z; f.b[3] = b0.w; f.b[4] = b1.x; f.b[5] = b1.y; f.b[6] = b1.z; f.b[7] = b1.w;
+    } else if constexpr (CN == 4) {
+      const float4 b0 = lds4(b_s + k * NT + 4 * tx);
+      f.b[0] = b0.x; f.b[1] = b0.y; f.b[2] = b0.z; f.b[3] = b0.w;
+    } else {
+      const float2 b0 = *reinterpret_cast<const float2*>(b_s + k * NT + 2 * tx);
+      f.b[0] = b0.x; f.b[1] = b0.y;
+    }
+  };
+  auto mul = [&](const Frag& f) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < CN; ++j) acc[i][j] = fmaf(f.a[i], f.b[j], acc[i][j]);
+  };
+  for (int step = 0; step < steps; ++step) {
+    const int s = step % stages;
+    bar_wait(full + s, (uint32_t)(step / stages) & 1u, p.dev_status);
+    if (grp < G) {
+      const float* a_s = ringA + s * WK * MT + ty * 8;
+      const float* b_s = ringB + s * WK * NT;
+      const int kmax = min(WK, rows - step * WK);           // rows beyond this CTA's share are never multiplied
+      // two fragments in turn: the loads of the next k are in flight during the arithmetic of this one
+      Frag f0, f1;
+      int k = grp;
+      if (k < kmax) fetch_frag(a_s, b_s, k, f0);
+      for (; k < kmax; k += 2 * G) {
+        if (k + G < kmax) fetch_frag(a_s, b_s, k + G, f1);
+        mul(f0);
+        if (k + 2 * G < kmax) fetch_frag(a_s, b_s, k + 2 * G, f0);
+        if (k + G < kmax) mul(f1);
+      }
+    }
+    if (step + stages < steps) {                            // the stage is needed again
+      __syncwarp();
+      if (lane == 0) bar_arrive(empty + s);
+      if (warp == 0) {
+        if (elect_one()) {
+          bar_wait(empty + s, (uint32_t)(step / stages) & 1u, p.dev_status);
+          load(step + stages);
         }
       }
     }
-  };
-  if (k_begin < k_end) fetch(k_begin);
-  for (int k0 = k_begin; k0 < k_end; k0 += WK) {
-#pragma unroll
-    for (int i = 0; i < LD; ++i) {
-      const int idx = threadIdx.x + SS_THREADS * i;
-      *reinterpret_cast<float4*>(&As[idx >> 4][(idx & 15) * 4]) = ra[i];
-      *reinterpret_cast<float4*>(&Bs[idx >> 4][(idx & 15) * 4]) = rb[i];
-    }
-    __syncthreads();
-    if (k0 + WK < k_end) fetch(k0 + WK);
-#pragma unroll
-    for (int k = 0; k < WK; ++k) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    __syncthreads();
   }
-  if (splits > 1) {
-    float* slot = p.wg_scratch + ((size_t)tile * splits + z) * kSimtTileFloats;
+  __syncthreads();                                          // the ring is free: partial tiles [group][MT][NT] take its place
+  if (grp < G) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      *reinterpret_cast<float4*>(slot + (ty * 4 + i) * WT + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(p.wg_counters + tile, 1u) == (unsigned)splits - 1u);
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    const float* base = p.wg_scratch + (size_t)tile * splits * kSimtTileFloats;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    // four partial tiles are loaded before any is added (the loads of one round overlap; a round past the last split
-    // adds zeros); the order of the additions stays split by split
-    auto part = [&](int s, int i) {
-      return __ldcg(reinterpret_cast<const float4*>(base + (size_t)s * kSimtTileFloats + (ty * 4 + i) * WT + tx * 4));
-    };
-    for (int s = 0; s < splits; s += 4) {
-      float4 q[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) q[u][i] = s + u < splits ? part(s + u, i) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i][0] += q[u][i].x; acc[i][1] += q[u][i].y; acc[i][2] += q[u][i].z; acc[i][3] += q[u][i].w;
-        }
+    for (int i = 0; i < 8; ++i) {
+      float* d = sm + (grp * MT + ty * 8 + i) * NT;
+      if constexpr (CN == 8) {
+        *reinterpret_cast<float4*>(d + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        *reinterpret_cast<float4*>(d + 32 + 4 * tx) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+      } else if constexpr (CN == 4) {
+        *reinterpret_cast<float4*>(d + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      } else {
+        *reinterpret_cast<float2*>(d + 2 * tx) = make_float2(acc[i][0], acc[i][1]);
+      }
     }
-    if (threadIdx.x == 0) p.wg_counters[tile] = 0u;
   }
-  float inv_bc1 = 1.0f, inv_bc2 = 1.0f;
-  if constexpr (OPT == SEG_ADAM) { inv_bc1 = 1.0f / __ldg(p.bc); inv_bc2 = 1.0f / __ldg(p.bc + 1); }
-  // this thread's 16 elements (4 rows of 4 consecutive columns): all loads first (they do not depend on one
-  // another), then the arithmetic and the stores.  A row segment that lies wholly inside the weight matrix moves
-  // with 16-byte accesses (rows of W are 32-byte aligned and the segment starts at a multiple of 4 columns); the
-  // ragged segment at the matrix edge, which also carries the bias element, goes element by element.
-  int64_t e[4][4];
-  bool wide[4];
-  float w[4][4], m[4][4], v[4][4];
-  const int c0 = n0 + tx * 4;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int o = m0 + ty * 4 + i;
-    wide[i] = o < out && c0 + 3 < in;
+  const int slice = MT / S;                                 // rows each CTA of the cluster ends up with
+  // four consecutive columns of one row per thread and pass.  A group that lies wholly inside the weight matrix moves with
+  // 16-byte accesses; the ragged group at the matrix edge, which also carries the bias element, goes element by element.
+  struct Item { int64_t e[4]; bool wide, any; float w[4], m[4], v[4]; };
+  auto fetch = [&](int e, Item& q) {
+    const int o = rank * slice + e / CPR, c0 = n0 + 4 * (e % CPR);
+    q.any = e < slice * CPR && o < out && c0 <= in;
+    q.wide = q.any && c0 + 3 < in;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int c = c0 + j;
-      e[i][j] = (o >= out || c > in) ? -1 : (c < in ? p.w_off[l] + (int64_t)o * p.ldw[l] + c : p.b_off[l] + o);
-      w[i][j] = 0.f; m[i][j] = 0.f; v[i][j] = 0.f;
+      q.e[j] = !q.any || c > in ? -1 : (c < in ? p.w_off[l] + (int64_t)o * p.ldw[l] + c : p.b_off[l] + o);
+      q.w[j] = q.m[j] = q.v[j] = 0.f;
     }
-    if (wide[i]) {
-      const float4 q = *reinterpret_cast<const float4*>(p.params + e[i][0]);
-      w[i][0] = q.x; w[i][1] = q.y; w[i][2] = q.z; w[i][3] = q.w;
+    if (q.wide) {
+      const float4 a = *reinterpret_cast<const float4*>(p.params + q.e[0]);
+      q.w[0] = a.x; q.w[1] = a.y; q.w[2] = a.z; q.w[3] = a.w;
       if constexpr (OPT != SEG_SGD) {
-        const float4 t = *reinterpret_cast<const float4*>(p.s1 + e[i][0]);
-        m[i][0] = t.x; m[i][1] = t.y; m[i][2] = t.z; m[i][3] = t.w;
+        const float4 b = *reinterpret_cast<const float4*>(p.s1 + q.e[0]);
+        q.m[0] = b.x; q.m[1] = b.y; q.m[2] = b.z; q.m[3] = b.w;
       }
       if constexpr (OPT == SEG_ADAM) {
-        const float4 t = *reinterpret_cast<const float4*>(p.s2 + e[i][0]);
-        v[i][0] = t.x; v[i][1] = t.y; v[i][2] = t.z; v[i][3] = t.w;
+        const float4 b = *reinterpret_cast<const float4*>(p.s2 + q.e[0]);
+        q.v[0] = b.x; q.v[1] = b.y; q.v[2] = b.z; q.v[3] = b.w;
       }
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (e[i][j] < 0) continue;
-        w[i][j] = p.params[e[i][j]];
-        if constexpr (OPT != SEG_SGD) m[i][j] = p.s1[e[i][j]];
-        if constexpr (OPT == SEG_ADAM) v[i][j] = p.s2[e[i][j]];
+        if (q.e[j] < 0) continue;
+        q.w[j] = p.params[q.e[j]];
+        if constexpr (OPT != SEG_SGD) q.m[j] = p.s1[q.e[j]];
+        if constexpr (OPT == SEG_ADAM) q.v[j] = p.s2[q.e[j]];
+      }
+    }
+  };
+  Item q;
+  fetch(tid, q);                                            // in flight during the exchange
+  float inv_bc1 = 1.0f, inv_bc2 = 1.0f;
+  if constexpr (OPT == SEG_ADAM) { inv_bc1 = 1.0f / __ldg(p.bc); inv_bc2 = 1.0f / __ldg(p.bc + 1); }
+  if (S > 1) cluster_wait_acquire();                        // every peer has started: its shared memory may be written
+  __syncthreads();
+  const uint32_t inv_slice = (65536u + (uint32_t)slice - 1u) / (uint32_t)slice;     // row / slice for row < 128, exactly
+  for (int e0 = tid; e0 < MT * CPR; e0 += 4 * SS_THREADS) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * SS_THREADS;
+      if (e < MT * CPR) {
+        v[u] = lds4(sm + 4 * e);
+        for (int g = 1; g < G; ++g) add4(v[u], lds4(sm + g * MT * NT + 4 * e));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * SS_THREADS;
+      if (e < MT * CPR) {
+        const int row = e / CPR, c = e % CPR, owner = (int)(((uint32_t)row * inv_slice) >> 16);
+        const uint32_t off = 4u * (uint32_t)((rank * slice + row - owner * slice) * NT + 4 * c);
+        if (S > 1) store_cluster4(in_cta(smem_addr(recv), (uint32_t)owner) + off, v[u]);
+        else *reinterpret_cast<float4*>(recv + off / 4) = v[u];
       }
     }
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  if (S > 1) { cluster_arrive_release(); cluster_wait_acquire(); } else __syncthreads();
+  for (int e = tid; e < slice * CPR; e += SS_THREADS) {
+    if (e != tid) fetch(e, q);
+    if (!q.any) continue;
+    float4 g4 = lds4(recv + 4 * e);
+    for (int s = 1; s < S; ++s) add4(g4, lds4(recv + s * slice * NT + 4 * e));
+    const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (e[i][j] >= 0) opt_step<OPT>(w[i][j], acc[i][j], m[i][j], v[i][j], p, inv_bc1, inv_bc2);
-    if (wide[i]) {
-      *reinterpret_cast<float4*>(p.grads + e[i][0]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-      if constexpr (OPT != SEG_SGD) *reinterpret_cast<float4*>(p.s1 + e[i][0]) = make_float4(m[i][0], m[i][1], m[i][2], m[i][3]);
-      if constexpr (OPT == SEG_ADAM) *reinterpret_cast<float4*>(p.s2 + e[i][0]) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
-      *reinterpret_cast<float4*>(p.params + e[i][0]) = make_float4(w[i][0], w[i][1], w[i][2], w[i][3]);
+      if (q.e[j] >= 0) opt_step<OPT>(q.w[j], gv[j], q.m[j], q.v[j], p, inv_bc1, inv_bc2);
+    if (q.wide) {
+      *reinterpret_cast<float4*>(p.grads + q.e[0]) = g4;
+      if constexpr (OPT != SEG_SGD) *reinterpret_cast<float4*>(p.s1 + q.e[0]) = make_float4(q.m[0], q.m[1], q.m[2], q.m[3]);
+      if constexpr (OPT == SEG_ADAM) *reinterpret_cast<float4*>(p.s2 + q.e[0]) = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]);
+      *reinterpret_cast<float4*>(p.params + q.e[0]) = make_float4(q.w[0], q.w[1], q.w[2], q.w[3]);
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (e[i][j] < 0) continue;
-        p.grads[e[i][j]] = acc[i][j];
-        if constexpr (OPT != SEG_SGD) p.s1[e[i][j]] = m[i][j];
-        if constexpr (OPT == SEG_ADAM) p.s2[e[i][j]] = v[i][j];
-        p.params[e[i][j]] = w[i][j];
+        if (q.e[j] < 0) continue;
+        p.grads[q.e[j]] = gv[j];
+        if constexpr (OPT != SEG_SGD) p.s1[q.e[j]] = q.m[j];
+        if constexpr (OPT == SEG_ADAM) p.s2[q.e[j]] = q.v[j];
+        p.params[q.e[j]] = q.w[j];
       }
+    }
+  }
+  if (blockIdx.x == 0) {
+    const float total = block_sum(lpart, red);
+    if (tid == 0) {
+      const int NL = p.widths[p.n_layers];
+      const float scale = p.is_final ? 1.0f / (float)p.batch : 1.0f / (float)((int64_t)p.batch * NL);
+      float* dst = *p.loss_dst;
+      if (dst) *dst = total * scale;
     }
   }
 }
 
-// CTAs the second kernel aims at: two per SM, so that short tiles of different layers overlap.
-constexpr int kWgradTargetCtas = 296;
-
-int total_wgrad_tiles(int n_layers, const int* widths) {
-  int t = 0;
-  for (int l = 0; l < n_layers; ++l) t += wgrad_tiles(widths[l], widths[l + 1]);
-  return t;
+__global__ void small_ones_kernel(float* a, int64_t ld, int col, int rows) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += gridDim.x * blockDim.x) a[(int64_t)i * ld + col] = 1.0f;
 }
 
-std::atomic<bool> g_smem_attr_set[2][64];    // [R == 16][device]
+// ---- host side -------------------------------------------------------------------------------------
+// Clusters of C CTAs the GPU runs at once with one CTA per SM (cudaOccupancyMaxActiveClusters on a B200: 148, 74, 33, 15 - a
+// cluster lives inside one GPC, and what a GPC has beyond a multiple of C stays idle).
+int resident_clusters(int C) { return C == 1 ? 148 : C == 2 ? 74 : C == 4 ? 33 : 15; }
+
+constexpr int kRowChoices[] = {1, 2, 4, 6, 8, 10, 12, 16};
+int split_columns(int N1) { return N1 <= 32 ? 2 : N1 <= 64 ? 4 : N1 <= 80 ? 5 : 8; }   // columns per lane in the split first layer
+
+// Lays out one launch with R rows per CTA; false when it does not fit into shared memory.
+bool layout_small(const SmallStep& p, int R, SmallPlan* q) {
+  const int L = p.n_layers, n0 = p.widths[0], N1 = p.widths[1];
+  q->R = R;
+  q->C = n0 <= 128 ? 1 : n0 <= 256 ? 2 : n0 <= 512 ? 4 : 8;        // at most 128 features per CTA
+  const int first = q->C > 1 ? 1 : 0, n_slots = L - first;
+  q->ks = q->C > 1 ? pitch_of((n0 + q->C - 1) / q->C) : up(n0, 4);
+  int slot_max = 0, slot_sum = 0;
+  for (int l = first; l < L; ++l) {
+    const int f = up(p.widths[l + 1] * (int)p.ldw[l], 32);
+    slot_max = std::max(slot_max, f); slot_sum += f;
+  }
+  const int t_x = up(q->C * R * q->ks, 32), t_w = q->C > 1 ? up(N1 * q->ks, 32) : 0;
+  const int exch = q->C > 1 ? SS_WARPS * R * up(N1, 4) : 0;         // sums sent / received: one share per warp and row
+  for (int mode = 0; mode < 4; ++mode) {                            // own slots, two slots; the same in the first layer's tiles
+    q->late = mode >= 2; q->streamed = mode & 1;
+    if (q->streamed && n_slots <= 2) continue;
+    if (q->late && q->C == 1) continue;
+    const int slots = q->streamed ? 2 * slot_max : slot_sum;
+    q->off_x = 0; q->off_w0 = t_x;
+    int so = q->late ? 0 : t_x + t_w;
+    int off = q->late ? std::max(t_x + t_w, slots) : t_x + t_w + slots;
+    for (int l = first; l < L; ++l) {
+      if (q->streamed) q->off_slot[l] = so + ((l - first) & 1) * slot_max;
+      else { q->off_slot[l] = so; so += up(p.widths[l + 1] * (int)p.ldw[l], 32); }
+    }
+    q->off_send = off; off += exch;
+    q->off_recv = off; off += exch;
+    for (int l = 1; l <= L; ++l) { q->off_act[l] = off; off += R * up(p.widths[l], 4); }
+    for (int i = 0; i < 2; ++i) { q->off_dz[i] = off; off += R * kSmallMaxWidth; }
+    q->off_bias = off; off += L * kSmallMaxWidth;
+    q->off_tgt = off; off += p.is_final ? 0 : R * up(p.widths[L], 4);
+    q->floats = off;
+    if ((size_t)off * sizeof(float) <= SS_SMEM_LIMIT) return true;
+  }
+  return false;
+}
+
+// Rows per CTA: the split with the smallest estimate of waves x time of a CTA.  A link costs its fixed latency, the pass
+// over the weights in shared memory, and arithmetic in proportion to the rows; the first layer's share grows with the
+// cluster's rows (cycles, fitted to clock stamps inside the kernel).
+bool plan_small(const SmallStep& p, SmallPlan* best) {
+  double best_t = 1e30;
+  for (int R : kRowChoices) {
+    SmallPlan q{};
+    if (!layout_small(p, R, &q)) continue;
+    const int clusters = (p.batch + q.C * R - 1) / (q.C * R);
+    const int waves = (clusters + resident_clusters(q.C) - 1) / resident_clusters(q.C);
+    double links = 0;
+    for (int l = q.C > 1 ? 1 : 0; l < p.n_layers; ++l)
+      links += (l > 0 ? 2 : 1) * (600.0 + p.widths[l] * p.widths[l + 1] * (0.04 + 0.012 * R));
+    const double t0 = q.C > 1 ? 2500.0 + (double)up(q.C * R, 8) * p.widths[1] * q.ks / 90.0 : 0.0;
+    const double t = waves * (3000.0 + t0 + links);
+    if (t < best_t) { best_t = t; *best = q; }
+  }
+  return best_t < 1e30;
+}
+
+int chain_grid(const SmallStep& p, const SmallPlan& q) { return (p.batch + q.C * q.R - 1) / (q.C * q.R) * q.C; }
+
+template <typename Kern>
+cudaError_t launch_clustered(Kern kern, int grid, int cluster, size_t smem, cudaStream_t s, void** args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(SS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (g_use_pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), args);
+}
+
+// Allows a kernel its largest dynamic shared memory, once per device.
+cudaError_t allow_smem(const void* kern, size_t bytes, std::atomic<bool>* flags) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (flags[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) flags[dev].store(true, std::memory_order_release);
+  return e;
+}
+
+struct ChainArgs {
+  SmallStep p; SmallPlan q;
+  const float* x; const int32_t* cls; const float* gather; float* loss_to; float* y;
+  CUtensorMap map_x, map_w0, map_stage;
+};
+
+template <int R, int CT0>
+cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
+  static std::atomic<bool> allowed[64];
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(small_fwd_bwd_kernel<R, CT0>), SS_SMEM_LIMIT, allowed);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a.p, &a.x, &a.cls, &a.gather, &a.loss_to, &a.q, &a.y, &a.map_x, &a.map_w0, &a.map_stage};
+  return launch_clustered(small_fwd_bwd_kernel<R, CT0>, chain_grid(a.p, a.q), a.q.C, (size_t)a.q.floats * sizeof(float), s, args);
+}
+
+template <int R>
+cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
+  if (a.q.C == 1) return launch_chain<R, 0>(a, s);
+  switch (split_columns(a.p.widths[1])) {
+    case 2: return launch_chain<R, 2>(a, s);
+    case 4: return launch_chain<R, 4>(a, s);
+    case 5: return launch_chain<R, 5>(a, s);
+    default: return launch_chain<R, 8>(a, s);
+  }
+}
+
+cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
+  const SmallStep& p = a.p;
+  const SmallPlan& q = a.q;
+  const uint32_t rows = (uint32_t)(q.C * q.R), bw = (uint32_t)q.ks;
+  // x_stage: clipped to the input width and the batch, so that the column of ones behind the width stays
+  if (!make_map_f32(&a.map_stage, p.act[0], (uint64_t)p.widths[0], (uint64_t)p.batch, (uint64_t)p.ld_act[0] * 4, bw, rows))
+    return cudaErrorInvalidValue;
+  a.map_w0 = a.map_stage;
+  if (q.C > 1 && !make_map_f32(&a.map_w0, p.params + p.w_off[0], (uint64_t)p.widths[0], (uint64_t)p.widths[1],
+                               (uint64_t)p.ldw[0] * 4, bw, (uint32_t)p.widths[1]))
+    return cudaErrorInvalidValue;
+  a.map_x = a.map_stage;
+  if (small_input_by_tensor(a.x, a.gather, p.widths[0]) && !small_input_map(p, a.x, bw, rows, &a.map_x)) return cudaErrorInvalidValue;
+  switch (q.R) {
+    case 1: return launch_chain<1>(a, s);
+    case 2: return launch_chain<2>(a, s);
+    case 4: return launch_chain<4>(a, s);
+    case 6: return launch_chain<6>(a, s);
+    case 8: return launch_chain<8>(a, s);
+    case 10: return launch_chain<10>(a, s);
+    case 12: return launch_chain<12>(a, s);
+    case 16: return launch_chain<16>(a, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int OPT, int NT>
+cudaError_t launch_wgrad(const SmallStep& p, int tiles, int S, int rows, int n_partials, cudaStream_t s) {
+  static std::atomic<bool> allowed[64];
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(small_wgrad_update_kernel<OPT, NT>), SS_SMEM_LIMIT, allowed);
+  if (e != cudaSuccess) return e;
+  // all of a CTA's rows in flight at once where the stages allow it; two CTAs on an SM where the grid needs them
+  int stages = std::max(1, std::min((rows + WK - 1) / WK, W_STAGES));
+  auto bytes = [&](int st) {
+    size_t b = 0;
+    for (int l = 1; l <= p.n_layers; ++l) {
+      const int mt = up(p.widths[l], 8);
+      b = std::max(b, (size_t)(wgrad_ring_floats(mt, NT, st) + mt * NT) * sizeof(float));
+    }
+    return b;
+  };
+  if (tiles > resident_clusters(S)) while (stages > 2 && bytes(stages) > 112 * 1024) --stages;
+  SmallStep pp = p;
+  void* args[] = {&pp, &S, &rows, &n_partials, &stages};
+  return launch_clustered(small_wgrad_update_kernel<OPT, NT>, tiles * S, S, bytes(stages), s, args);
+}
+
+template <int OPT>
+cudaError_t launch_wgrad(const SmallStep& p, int nt, int tiles, int S, int rows, int n_partials, cudaStream_t s) {
+  if (nt == 64) return launch_wgrad<OPT, 64>(p, tiles, S, rows, n_partials, s);
+  if (nt == 32) return launch_wgrad<OPT, 32>(p, tiles, S, rows, n_partials, s);
+  return launch_wgrad<OPT, 16>(p, tiles, S, rows, n_partials, s);
+}
 
 }  // namespace
 
@@ -553,58 +997,76 @@ bool small_step_supported(int n_layers, const int* widths) {
   return true;
 }
 
-// Rows of the batch per CTA of the first kernel: 8 while that fills the GPU at most once, 16 beyond.
-int small_step_rows(int batch) { return batch <= 148 * 8 ? 8 : 16; }
-
-bool small_step_batch_ok(int batch) {
-  const int R = small_step_rows(batch);
-  return (batch + R - 1) / R <= loss_max_partials();
+bool small_step_batch_ok(const SmallStep& p) {
+  SmallPlan q;
+  return plan_small(p, &q) && chain_grid(p, q) <= loss_max_partials();
 }
 
-int small_step_wgrad_slots(int n_layers, const int* widths) {
-  const int tiles = total_wgrad_tiles(n_layers, widths);
-  return tiles * std::max(1, kWgradTargetCtas / tiles);
+bool small_input_map(const SmallStep& p, const float* x, uint32_t box_cols, uint32_t box_rows, CUtensorMap* map) {
+  return make_map_f32(map, x, (uint64_t)p.widths[0], (uint64_t)p.batch, (uint64_t)p.widths[0] * 4, box_cols, box_rows);
+}
+
+bool small_step_maps(const SmallStep& p, int max_batch, CUtensorMap* maps) {
+  for (int l = 0; l < p.n_layers; ++l) {
+    CUtensorMap* m = maps + 4 * l;
+    const uint32_t mt = (uint32_t)up(p.widths[l + 1], 8);
+    if (!make_map_f32(m, p.dz[l], mt, (uint64_t)max_batch, (uint64_t)p.ld_act[l + 1] * 4, mt, WK)) return false;
+    const uint32_t nts[3] = {64, 32, 16};
+    for (int i = 0; i < 3; ++i)
+      if (!make_map_f32(m + 1 + i, p.act[l], (uint64_t)p.widths[l] + 1, (uint64_t)max_batch, (uint64_t)p.ld_act[l] * 4, nts[i], WK)) return false;
+  }
+  return true;
+}
+
+cudaError_t launch_small_ones(float* act, int64_t ld, int col, int rows, cudaStream_t s) {
+  small_ones_kernel<<<std::min((rows + 255) / 256, 148), 256, 0, s>>>(act, ld, col, rows);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_small_fwd_bwd(const SmallStep& p, const float* x, const int32_t* cls, const float* gather,
-                                 float* loss_to, cudaStream_t s) {
-  const int R = small_step_rows(p.batch);
-  const size_t smem = fwd_bwd_smem_floats(p, R) * sizeof(float);
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::atomic<bool>& flag = g_smem_attr_set[R == 16][dev];
-  if (!flag.load(std::memory_order_acquire)) {
-    // the largest footprint any supported segment has, so that the attribute is set once per device
-    const size_t max_floats = (size_t)SS_STAGES * SS_STAGE_FLOATS + 2 * (size_t)kSmallMaxWidth * R +
-                              ((size_t)kSmallMaxInput + (size_t)kSmallMaxLayers * kSmallMaxWidth) * R;
-    e = R == 16 ? cudaFuncSetAttribute(small_fwd_bwd_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_floats * 4))
-                : cudaFuncSetAttribute(small_fwd_bwd_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_floats * 4));
-    if (e != cudaSuccess) return e;
-    flag.store(true, std::memory_order_release);
-  }
-  const int grid = (p.batch + R - 1) / R;
-  if (R == 16) launch_k(small_fwd_bwd_kernel<16>, dim3(grid), dim3(SS_THREADS), smem, s, p, x, cls, gather, loss_to);
-  else launch_k(small_fwd_bwd_kernel<8>, dim3(grid), dim3(SS_THREADS), smem, s, p, x, cls, gather, loss_to);
-  return cudaGetLastError();
+                                 float* loss_to, cudaStream_t s, uint32_t* box) {
+  ChainArgs a{};
+  a.p = p; a.x = x; a.cls = cls; a.gather = gather; a.loss_to = loss_to;
+  if (!plan_small(p, &a.q)) return cudaErrorInvalidValue;
+  if (box) { box[0] = (uint32_t)a.q.ks; box[1] = (uint32_t)(a.q.C * a.q.R); }
+  return launch_chain(a, s);
+}
+
+cudaError_t launch_small_forward(const SmallStep& p, const float* x, float* y, cudaStream_t s) {
+  ChainArgs a{};
+  a.p = p; a.x = x; a.y = y;
+  if (!plan_small(p, &a.q)) return cudaErrorInvalidValue;
+  a.q.forward_only = 1;
+  return launch_chain(a, s);
 }
 
 cudaError_t launch_small_wgrad_update(const SmallStep& p, cudaStream_t s) {
-  const int tiles = total_wgrad_tiles(p.n_layers, p.widths);
-  // split the batch while that adds CTAs the GPU has room for and leaves every split at least two k-steps
-  int splits = std::min(std::min(kWgradTargetCtas / tiles, p.wg_slots / tiles), p.batch / (2 * WK));
-  if (splits < 1) splits = 1;
-  int k_per_split = ((p.batch + splits - 1) / splits + WK - 1) / WK * WK;
-  splits = (p.batch + k_per_split - 1) / k_per_split;
-  const int grid = tiles * splits;
+  SmallPlan q;
+  if (!plan_small(p, &q)) return cudaErrorInvalidValue;
+  const int n_partials = chain_grid(p, q);
+  // tile width and batch split with the smallest estimate: a wave of CTAs costs its fixed latencies once per CTA an SM has
+  // to run, its arithmetic at the rate the register tile reaches (8 x 8 best, 8 x 2 bound by shared-memory loads)
+  int best_nt = 64, best_s = 1, best_tiles = 1;
+  double best_t = 1e30;
+  for (int nt : {64, 32, 16}) {
+    int tiles = 0, mt = 8;
+    for (int l = 0; l < p.n_layers; ++l) { tiles += wgrad_tiles(p.widths[l], nt); mt = std::max(mt, up(p.widths[l + 1], 8)); }
+    const double rate = nt == 64 ? 90.0 : nt == 32 ? 80.0 : 60.0;      // multiply-adds per cycle and SM
+    for (int S : {1, 2, 4, 8}) {
+      if (S > 1 && p.batch < 8 * S) continue;
+      const int rows = (p.batch + S - 1) / S;
+      const int load = (tiles + resident_clusters(S) - 1) / resident_clusters(S);
+      const double t = (S > 1 ? 1500.0 : 500.0) + load * (1500.0 + rows * (double)mt * nt / rate + mt * nt / 8.0 * (1.0 + 1.0 / S));
+      if (t < best_t) { best_t = t; best_nt = nt; best_s = S; best_tiles = tiles; }
+    }
+  }
+  const int rows = (p.batch + best_s - 1) / best_s;
   switch (p.optimizer) {
-    case SEG_SGD: launch_k(small_wgrad_update_kernel<SEG_SGD>, dim3(grid), dim3(SS_THREADS), 0, s, p, splits, k_per_split); break;
-    case SEG_SGD_MOMENTUM: launch_k(small_wgrad_update_kernel<SEG_SGD_MOMENTUM>, dim3(grid), dim3(SS_THREADS), 0, s, p, splits, k_per_split); break;
-    case SEG_ADAM: launch_k(small_wgrad_update_kernel<SEG_ADAM>, dim3(grid), dim3(SS_THREADS), 0, s, p, splits, k_per_split); break;
+    case SEG_SGD: return launch_wgrad<SEG_SGD>(p, best_nt, best_tiles, best_s, rows, n_partials, s);
+    case SEG_SGD_MOMENTUM: return launch_wgrad<SEG_SGD_MOMENTUM>(p, best_nt, best_tiles, best_s, rows, n_partials, s);
+    case SEG_ADAM: return launch_wgrad<SEG_ADAM>(p, best_nt, best_tiles, best_s, rows, n_partials, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace segk
