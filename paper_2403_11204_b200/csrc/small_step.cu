@@ -152,32 +152,51 @@ __device__ __forceinline__ void element_of(int i, int b, int& row, int& col) {
     if (b == s) { row = (s * H + i) / CT; col = (s * H + i) % CT; }
 }
 
-// v[r * CT + j] += sum over this lane's chunks c (four k each) of A[r][4c ..] . W[n_j][4c ..]; A rows `pa` apart, wp[j] the
-// row of column n_j.
+// v[r * CT + j] += sum over this lane's chunks (four k each) of A[r][4c ..] . W[n_j][4c ..]; A rows `pa` apart, wp[j] the row
+// of column n_j.  The lanes' chunks are c0, c0 + step, ...; all lanes make the same number of rounds (a lane without a chunk
+// left multiplies by zero), so that a warp never splits.
 template <int RT, int CT, int VP>
-__device__ __forceinline__ void dot_rows(float (&v)[VP], const float* A, int pa, const float* const (&wp)[CT], int c0, int c1, int step) {
-#pragma unroll 2
-  for (int c = c0; c < c1; c += step) {
-    float4 w[CT];
+__device__ __forceinline__ void dot_chunk(float (&v)[VP], const float* A, int pa, const float4 (&w)[CT]) {
 #pragma unroll
-    for (int j = 0; j < CT; ++j) w[j] = lds4(wp[j] + 4 * c);
+  for (int r = 0; r < RT; ++r) {
+    const float4 a = lds4(A + r * pa);
 #pragma unroll
-    for (int r = 0; r < RT; ++r) {
-      const float4 a = lds4(A + r * pa + 4 * c);
-#pragma unroll
-      for (int j = 0; j < CT; ++j) {
-        float t = v[r * CT + j];
-        t = fmaf(a.x, w[j].x, t); t = fmaf(a.y, w[j].y, t); t = fmaf(a.z, w[j].z, t); t = fmaf(a.w, w[j].w, t);
-        v[r * CT + j] = t;
-      }
+    for (int j = 0; j < CT; ++j) {
+      float t = v[r * CT + j];
+      t = fmaf(a.x, w[j].x, t); t = fmaf(a.y, w[j].y, t); t = fmaf(a.z, w[j].z, t); t = fmaf(a.w, w[j].w, t);
+      v[r * CT + j] = t;
     }
   }
 }
+template <int RT, int CT, int VP>
+__device__ __forceinline__ void dot_rows(float (&v)[VP], const float* A, int pa, const float* const (&wp)[CT], int c0, int chunks, int step) {
+  const int full = chunks / step;
+  int c = c0;
+#pragma unroll 2
+  for (int i = 0; i < full; ++i, c += step) {
+    float4 w[CT];
+#pragma unroll
+    for (int j = 0; j < CT; ++j) w[j] = lds4(wp[j] + 4 * c);
+    dot_chunk<RT, CT, VP>(v, A + 4 * c, pa, w);
+  }
+  if (full * step < chunks) {
+    const bool ok = c < chunks;
+    c = min(c, chunks - 1);
+    float4 w[CT];
+#pragma unroll
+    for (int j = 0; j < CT; ++j) {
+      w[j] = lds4(wp[j] + 4 * c);
+      if (!ok) w[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    dot_chunk<RT, CT, VP>(v, A + 4 * c, pa, w);
+  }
+}
 
-// A forward link for R rows: emit(row, n, value) receives every element n < N of A W^T (columns up to N rounded up to 4 are
-// emitted too).  Warp = (half of the rows, block of 8 * CT columns), lane = (column, quarter of the contraction).
-template <int R, int CT, typename Emit>
-__device__ __forceinline__ void link_forward(const float* A, int pa, const float* W, int pw, int K, int N, const Emit& emit) {
+// A forward link for R rows: every element n < N (rounded up to 4) of A W^T.  Warp = (half of the rows, block of 8 * CT columns),
+// lane = (column, quarter of the contraction).  side(r, n) is what the element's epilogue needs from shared memory, fetched
+// ahead of the arithmetic; emit(r, n, value, side) finishes the element.
+template <int R, int CT, typename Side, typename Emit>
+__device__ __forceinline__ void link_forward(const float* A, int pa, const float* W, int pw, int K, int N, const Side& side, const Emit& emit) {
   constexpr int RP = R >= 4 ? 2 : 1, RT = R / RP, V = RT * CT, VP = (V + 3) / 4 * 4, H = VP / 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sl = lane >> 3;
   const int rp = warp % RP, n0 = warp / RP * 8 * CT + (lane & 7);
@@ -188,20 +207,28 @@ __device__ __forceinline__ void link_forward(const float* A, int pa, const float
   const float* wp[CT];
 #pragma unroll
   for (int j = 0; j < CT; ++j) wp[j] = W + min(n0 + 8 * j, N - 1) * pw;
+  const int N4 = up(N, 4);
+  int er[H], en[H];
+  float2 es[H];
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    int j;
+    element_of<CT, H, 4>(i, sl, er[i], j);
+    en[i] = n0 + 8 * j;
+    if (er[i] >= RT || en[i] >= N4) en[i] = -1;
+    er[i] += rp * RT;
+    if (en[i] >= 0) es[i] = side(er[i], en[i]);
+  }
   dot_rows<RT, CT, VP>(v, A + rp * RT * pa, pa, wp, sl, (K + 3) >> 2, 4);
   reduce_scatter<V, 4>(v, lane);
 #pragma unroll
-  for (int i = 0; i < H; ++i) {
-    int r, j;
-    element_of<CT, H, 4>(i, sl, r, j);
-    const int n = n0 + 8 * j;
-    if (r < RT && n < up(N, 4)) emit(rp * RT + r, n, v[i]);
-  }
+  for (int i = 0; i < H; ++i)
+    if (en[i] >= 0) emit(er[i], en[i], v[i], es[i]);
 }
 
-// A dgrad link: emit(row, k, value) for every element of dZ W (k < K rounded up to 4); lane = (CT consecutive k, quarter of n).
-template <int R, int CT, typename Emit>
-__device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float* W, int pw, int N, int K, const Emit& emit) {
+// A dgrad link: every element k < K (rounded up to 4) of dZ W; lane = (CT consecutive k, quarter of n).
+template <int R, int CT, typename Side, typename Emit>
+__device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float* W, int pw, int N, int K, const Side& side, const Emit& emit) {
   constexpr int RP = R >= 4 ? 2 : 1, RT = R / RP, V = RT * CT, VP = (V + 3) / 4 * 4, H = VP / 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sl = lane >> 3;
   const int rp = warp % RP, k0 = warp / RP * 8 * CT + (lane & 7) * CT;
@@ -211,18 +238,36 @@ __device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float*
   for (int i = 0; i < VP; ++i) v[i] = 0.f;
   const float* wk = W + min(k0, pw - CT);                   // lanes beyond the row read its end and are not emitted
   const float* A = dZ + rp * RT * pz;
-  for (int c = sl; c < (N + 3) >> 2; c += 4) {
+  const int K4 = up(K, 4);
+  int er[H], ek[H];
+  float2 es[H];
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    int j;
+    element_of<CT, H, 4>(i, sl, er[i], j);
+    ek[i] = k0 + j;
+    if (er[i] >= RT || ek[i] >= K4) ek[i] = -1;
+    er[i] += rp * RT;
+    if (ek[i] >= 0) es[i] = side(er[i], ek[i]);
+  }
+  // chunks of four n in rounds of four lane groups, as in dot_rows: in the last round a lane beyond N multiplies by zero
+  const int chunks = (N + 3) >> 2;
+  auto round = [&](int c, bool ok) {
     float w[4][CT];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float* row = wk + min(4 * c + i, N - 1) * pw;   // beyond N: dZ is zero there
-      if constexpr (CT == 4) { const float4 t = lds4(row); w[i][0] = t.x; w[i][1] = t.y; w[i][2] = t.z; w[i][3] = t.w; }
-      else if constexpr (CT == 2) { const float2 t = *reinterpret_cast<const float2*>(row); w[i][0] = t.x; w[i][1] = t.y; }
-      else w[i][0] = row[0];
+    for (int u = 0; u < 4; ++u) {
+      const float* row = wk + min(4 * c + u, N - 1) * pw;
+      if constexpr (CT == 4) { const float4 t = lds4(row); w[u][0] = t.x; w[u][1] = t.y; w[u][2] = t.z; w[u][3] = t.w; }
+      else if constexpr (CT == 2) { const float2 t = *reinterpret_cast<const float2*>(row); w[u][0] = t.x; w[u][1] = t.y; }
+      else w[u][0] = row[0];
+      if (!ok) {
+#pragma unroll
+        for (int j = 0; j < CT; ++j) w[u][j] = 0.f;
+      }
     }
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
-      const float4 a = lds4(A + r * pz + 4 * c);
+      const float4 a = lds4(A + r * pz + 4 * c);            // zero between N and the end of the chunk
 #pragma unroll
       for (int j = 0; j < CT; ++j) {
         float t = v[r * CT + j];
@@ -230,14 +275,15 @@ __device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float*
         v[r * CT + j] = t;
       }
     }
-  }
+  };
+  const int full = chunks >> 2;
+#pragma unroll 2
+  for (int i = 0; i < full; ++i) round(4 * i + sl, true);
+  if (full * 4 < chunks) round(min(4 * full + sl, chunks - 1), 4 * full + sl < chunks);
   reduce_scatter<V, 4>(v, lane);
 #pragma unroll
-  for (int i = 0; i < H; ++i) {
-    int r, j;
-    element_of<CT, H, 4>(i, sl, r, j);
-    if (r < RT && k0 + j < up(K, 4)) emit(rp * RT + r, k0 + j, v[i]);
-  }
+  for (int i = 0; i < H; ++i)
+    if (ek[i] >= 0) emit(er[i], ek[i], v[i], es[i]);
 }
 
 // Columns per lane of a link with N columns: the smallest for which the warps cover them in one pass.
@@ -315,21 +361,22 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
       if (!q.late) load_chain();
     }
   }
-  // classes of the block's rows, clamped
-  if (train && tid < RB) {
+  // classes of the block's rows, clamped (by the upper half of the threads: the first warp is issuing copies)
+  const int crow = tid - SS_THREADS / 2;
+  if (train && crow >= 0 && crow < RB) {
     int c = 0;
-    if (tid < nvb) {
-      c = cls[rb0 + tid];
+    if (crow < nvb) {
+      c = cls[rb0 + crow];
       if (c < 0 || c >= p.n_classes) {
         if (rank == 0) atomicOr(p.dev_status, (int)DEV_BAD_CLASS);
         c = min(max(c, 0), p.n_classes - 1);
       }
-      if (rank == 0) p.cls_stage[rb0 + tid] = c;
+      if (rank == 0) p.cls_stage[rb0 + crow] = c;
     }
-    cls_s[tid] = c;
+    cls_s[crow] = c;
   }
   // step counter, Adam's bias corrections, where the loss goes
-  if (train && blockIdx.x == 0 && tid == SS_THREADS - 32) {
+  if (train && blockIdx.x == 0 && tid == 32) {
     const unsigned long long step = *p.t + 1ull;
     *p.t = step;
     if (p.optimizer == SEG_ADAM) {                          // beta^t by repeated squaring, in double precision
@@ -346,10 +393,11 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
   __syncthreads();                                          // cls_s
   if (!x_tensor) {
     // label rows gathered by class, or a batch whose rows are not whole 16-byte groups: plain loads, a row per warp.  The
-    // column of ones is put down as well: the staging store clips whole 16-byte groups only (its weights are zero)
+    // column of ones is put down as well where it shares a 16-byte group with the last features: the staging store clips
+    // whole groups only (the weights of that column are zero)
     for (int r = warp; r < RB; r += SS_WARPS) {
       const float* src = gather != nullptr ? gather + (int64_t)cls_s[r] * n0 : xsrc + (int64_t)(rb0 + min(r, nvb - 1)) * n0;
-      for (int k = lane; k < q.ks; k += 32) xs[r * q.ks + k] = (r < nvb && k0 + k < n0) ? src[k0 + k] : (k0 + k == n0 ? 1.f : 0.f);
+      for (int k = lane; k < q.ks; k += 32) xs[r * q.ks + k] = (r < nvb && k0 + k < n0) ? src[k0 + k] : (k0 + k == n0 && (n0 & 3) != 0 ? 1.f : 0.f);
     }
     fence_async();                                          // the staging store below reads them through the async proxy
     __syncthreads();
@@ -371,26 +419,39 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
   float lsum = 0.f;
   const float gscale = 2.0f / (float)((int64_t)p.batch * NL);
   float* dz_cur = sm + q.off_dz[0];
-  auto emit_forward = [&](int l, int r, int n, float v) {
-    const int N = p.widths[l + 1];
-    const bool last = l == L - 1;
-    v += bias_s[l * kSmallMaxWidth + n];
-    if (!last || p.last_relu) v = fmaxf(v, 0.f);
-    if (n >= N) v = 0.f;
-    const bool store = r < nv && n < N;
-    if (store) p.act[l + 1][(int64_t)(row0 + r) * p.ld_act[l + 1] + n] = v;
-    if (last && store && y != nullptr) y[(int64_t)(row0 + r) * N + n] = v;
-    if (last && want_targets) {
+  const float* tgt_s = sm + q.off_tgt;
+  struct Out { int N, pa; bool last, relu; float *a_s, *a_g, *y_g, *dz_g; int64_t ld, ld_y; };
+  auto out_of = [&](int l) {                                // where layer l's output goes
+    Out o;
+    o.N = p.widths[l + 1]; o.pa = up(o.N, 4);
+    o.last = l == L - 1; o.relu = !o.last || p.last_relu;
+    o.a_s = act_s(l + 1);
+    o.ld = p.ld_act[l + 1]; o.a_g = p.act[l + 1] + (int64_t)row0 * o.ld;
+    o.ld_y = o.N; o.y_g = (o.last && y != nullptr) ? y + (int64_t)row0 * o.N : nullptr;
+    o.dz_g = p.dz[l] + (int64_t)row0 * o.ld;
+    return o;
+  };
+  auto side_forward = [&](const Out& o, int l, int r, int n) {      // bias and, on the last layer, the loss target
+    return make_float2(bias_s[l * kSmallMaxWidth + n], (o.last && want_targets) ? tgt_s[r * NL4 + n] : 0.f);
+  };
+  auto emit_forward = [&](const Out& o, int r, int n, float v, const float2& sd) {
+    v += sd.x;
+    if (o.relu) v = fmaxf(v, 0.f);
+    if (n >= o.N) v = 0.f;
+    const bool store = r < nv && n < o.N;
+    if (store) o.a_g[r * o.ld + n] = v;
+    if (store && o.y_g != nullptr) o.y_g[r * o.ld_y + n] = v;
+    if (o.last && want_targets) {
       float g = 0.f;
       if (store) {
-        const float d = v - sm[q.off_tgt + r * NL4 + n];
+        const float d = v - sd.y;
         lsum = fmaf(d, d, lsum);
         g = (p.last_relu && !(v > 0.f)) ? 0.f : d * gscale;
-        p.dz[L - 1][(int64_t)(row0 + r) * p.ld_act[L] + n] = g;
+        o.dz_g[r * o.ld + n] = g;
       }
       dz_cur[r * kSmallMaxWidth + n] = g;
     } else {
-      act_s(l + 1)[r * up(N, 4) + n] = v;
+      o.a_s[r * o.pa + n] = v;
     }
   };
   auto put_targets = [&]() {
@@ -453,17 +514,21 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
     cluster_arrive_release();                               // "I have received everything"; waited for at the very end
     if (L == 1) __syncthreads();                            // the targets
     const int G = N4 / 4;
+    const Out o = out_of(0);
     for (int e = tid; e < R * G; e += SS_THREADS) {
       const int r = e / G, g = e - r * G;
       const float* src = sm + q.off_recv + r * N4 + 4 * g;
       float4 s[SS_WARPS];
 #pragma unroll
       for (int u = 0; u < SS_WARPS; ++u) s[u] = lds4(src + u * R * N4);
+      float2 sd[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sd[j] = side_forward(o, 0, r, 4 * g + j);
       float4 t = s[0];
 #pragma unroll
       for (int u = 1; u < SS_WARPS; ++u) add4(t, s[u]);
-      emit_forward(0, r, 4 * g, t.x); emit_forward(0, r, 4 * g + 1, t.y);
-      emit_forward(0, r, 4 * g + 2, t.z); emit_forward(0, r, 4 * g + 3, t.w);
+      emit_forward(o, r, 4 * g, t.x, sd[0]); emit_forward(o, r, 4 * g + 1, t.y, sd[1]);
+      emit_forward(o, r, 4 * g + 2, t.z, sd[2]); emit_forward(o, r, 4 * g + 3, t.w, sd[3]);
     }
   } else {
     put_targets();
@@ -476,15 +541,17 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
 
   // ---- the forward chain ------------------------------------------------------------------------------
   for (int l = first; l < L; ++l) {
+    const int K = p.widths[l], N = p.widths[l + 1];
+    const float *A = l == 0 ? xs : act_s(l), *W = slot(l);
+    const int pa = l == 0 ? q.ks : up(K, 4), pw = (int)p.ldw[l];
+    const Out o = out_of(l);
     __syncthreads();                                        // the layer's input is complete
     bar_wait(bar_w + l, 0, p.dev_status);
-    const int K = p.widths[l], N = p.widths[l + 1];
-    const float* A = l == 0 ? xs : act_s(l);
-    const int pa = l == 0 ? q.ks : up(K, 4), pw = (int)p.ldw[l];
-    auto emit = [&](int r, int n, float v) { emit_forward(l, r, n, v); };
-    by_width<R>(N, [&]() { link_forward<R, 1>(A, pa, slot(l), pw, K, N, emit); },
-                [&]() { link_forward<R, 2>(A, pa, slot(l), pw, K, N, emit); },
-                [&]() { link_forward<R, 4>(A, pa, slot(l), pw, K, N, emit); });
+    auto side = [&](int r, int n) { return side_forward(o, l, r, n); };
+    auto emit = [&](int r, int n, float v, const float2& sd) { emit_forward(o, r, n, v, sd); };
+    by_width<R>(N, [&]() { link_forward<R, 1>(A, pa, W, pw, K, N, side, emit); },
+                [&]() { link_forward<R, 2>(A, pa, W, pw, K, N, side, emit); },
+                [&]() { link_forward<R, 4>(A, pa, W, pw, K, N, side, emit); });
     if (q.streamed && l + 2 < L) {                          // two slots: refill this one for the layer after the next
       __syncthreads();
       if (warp == 0) { if (elect_one()) { fence_async(); load_weight(l + 2); } }
@@ -542,7 +609,7 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
   lsum = warp_sum(lsum);
   if (lane == 0) red[warp] = lsum;
   __syncthreads();
-  if (tid == SS_THREADS - 32) {                             // the CTA's share of the batch loss; the second kernel adds them up
+  if (tid == 0) {                                           // the CTA's share of the batch loss; the second kernel adds them up
     float t = 0.f;
 #pragma unroll
     for (int w = 0; w < SS_WARPS; ++w) t += red[w];
@@ -554,16 +621,19 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
     const int K = p.widths[l], K4 = up(K, 4), N = p.widths[l + 1], pw = (int)p.ldw[l];
     if (q.streamed && l + 2 < L) bar_wait(bar_w + l, 1, p.dev_status);   // loaded a second time
     float* dz_next = dz_cur == sm + q.off_dz[0] ? sm + q.off_dz[1] : sm + q.off_dz[0];
-    const float* al = act_s(l);
-    auto emit = [&](int r, int k, float v) {
-      if (!(al[r * K4 + k] > 0.f)) v = 0.f;                 // columns beyond the width hold 0: masked as well
+    const float *al = act_s(l), *W = slot(l);
+    const int64_t ld = p.ld_act[l];
+    float* dz_g = p.dz[l - 1] + (int64_t)row0 * ld;
+    auto side = [&](int r, int k) { return make_float2(al[r * K4 + k], 0.f); };
+    auto emit = [&](int r, int k, float v, const float2& sd) {
+      if (!(sd.x > 0.f)) v = 0.f;                           // columns beyond the width hold 0: masked as well
       dz_next[r * kSmallMaxWidth + k] = v;
-      if (r < nv && k < K) p.dz[l - 1][(int64_t)(row0 + r) * p.ld_act[l] + k] = v;
+      if (r < nv && k < K) dz_g[r * ld + k] = v;
     };
-    by_width<R>(K, [&]() { link_dgrad<R, 1>(dz_cur, kSmallMaxWidth, slot(l), pw, N, K, emit); },
-                [&]() { link_dgrad<R, 2>(dz_cur, kSmallMaxWidth, slot(l), pw, N, K, emit); },
-                [&]() { link_dgrad<R, 4>(dz_cur, kSmallMaxWidth, slot(l), pw, N, K, emit); });
-    __syncthreads();
+    by_width<R>(K, [&]() { link_dgrad<R, 1>(dz_cur, kSmallMaxWidth, W, pw, N, K, side, emit); },
+                [&]() { link_dgrad<R, 2>(dz_cur, kSmallMaxWidth, W, pw, N, K, side, emit); },
+                [&]() { link_dgrad<R, 4>(dz_cur, kSmallMaxWidth, W, pw, N, K, side, emit); });
+    if (l > 1) __syncthreads();
     if (q.streamed && l - 2 >= 1) {
       if (warp == 0) { if (elect_one()) { fence_async(); load_weight(l - 2); } }
     }
@@ -641,43 +711,32 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
-  struct Frag { float a[8], b[CN]; };
-  auto fetch_frag = [&](const float* a_s, const float* b_s, int k, Frag& f) {
-    const float4 a0 = lds4(a_s + k * MT), a1 = lds4(a_s + k * MT + 4);
-    f.a[0] = a0.x; f.a[1] = a0.y; f.a[2] = a0.z; f.a[3] = a0.w; f.a[4] = a1.x; f.a[5] = a1.y; f.a[6] = a1.z; f.a[7] = a1.w;
-    if constexpr (CN == 8) {
-      const float4 b0 = lds4(b_s + k * NT + 4 * tx), b1 = lds4(b_s + k * NT + 32 + 4 * tx);
-      f.b[0] = b0.x; f.b[1] = b0.y; f.b[2] = b0.z; f.b[3] = b0.w; f.b[4] = b1.x; f.b[5] = b1.y; f.b[6] = b1.z; f.b[7] = b1.w;
-    } else if constexpr (CN == 4) {
-      const float4 b0 = lds4(b_s + k * NT + 4 * tx);
-      f.b[0] = b0.x; f.b[1] = b0.y; f.b[2] = b0.z; f.b[3] = b0.w;
-    } else {
-      const float2 b0 = *reinterpret_cast<const float2*>(b_s + k * NT + 2 * tx);
-      f.b[0] = b0.x; f.b[1] = b0.y;
-    }
-  };
-  auto mul = [&](const Frag& f) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < CN; ++j) acc[i][j] = fmaf(f.a[i], f.b[j], acc[i][j]);
-  };
   for (int step = 0; step < steps; ++step) {
     const int s = step % stages;
     bar_wait(full + s, (uint32_t)(step / stages) & 1u, p.dev_status);
     if (grp < G) {
-      const float* a_s = ringA + s * WK * MT + ty * 8;
-      const float* b_s = ringB + s * WK * NT;
       const int kmax = min(WK, rows - step * WK);           // rows beyond this CTA's share are never multiplied
-      // two fragments in turn: the loads of the next k are in flight during the arithmetic of this one
-      Frag f0, f1;
-      int k = grp;
-      if (k < kmax) fetch_frag(a_s, b_s, k, f0);
-      for (; k < kmax; k += 2 * G) {
-        if (k + G < kmax) fetch_frag(a_s, b_s, k + G, f1);
-        mul(f0);
-        if (k + 2 * G < kmax) fetch_frag(a_s, b_s, k + 2 * G, f0);
-        if (k + G < kmax) mul(f1);
+      const float* a_s = ringA + (s * WK + grp) * MT + ty * 8;
+      const float* b_s = ringB + (s * WK + grp) * NT + (CN == 2 ? 2 : 4) * tx;
+#pragma unroll 4
+      for (int k = grp; k < kmax; k += G, a_s += G * MT, b_s += G * NT) {
+        const float4 a0 = lds4(a_s), a1 = lds4(a_s + 4);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        float b[CN];
+        if constexpr (CN == 8) {
+          const float4 b0 = lds4(b_s), b1 = lds4(b_s + 32);
+          b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
+        } else if constexpr (CN == 4) {
+          const float4 b0 = lds4(b_s);
+          b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
+        } else {
+          const float2 b0 = *reinterpret_cast<const float2*>(b_s);
+          b[0] = b0.x; b[1] = b0.y;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < CN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
       }
     }
     if (step + stages < steps) {                            // the stage is needed again
