@@ -50,12 +50,10 @@ enum Kind { K_FWD = 0, K_DGRAD, K_WGRAD, K_LOSS, K_WGRAD_UPDATE, K_UPDATE, K_COP
 
 int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
-// Position of the caller-supplied pointers in the parameter list of the kernel that takes them in: the input
-// staging kernel (see elementwise.cu), or the first kernel of a small segment's two-launch step.
-// map: the tensor map of x, where the kernel has one (-1: it has none).
-struct StageArgs { int count, x, cls, gather, loss, map; };
-constexpr StageArgs kStageInputsArgs = {19, 3, 9, 14, 15, -1};
-constexpr StageArgs kSmallStepArgs = {10, 1, 2, 3, 4, 7};
+// Position of the caller-supplied pointers in the parameter list of the kernel that takes them in, the input
+// staging kernel (see elementwise.cu).
+struct StageArgs { int count, x, cls, gather, loss; };
+constexpr StageArgs kStageInputsArgs = {19, 3, 9, 14, 15};
 
 }  // namespace
 
@@ -111,14 +109,11 @@ struct seg_handle {
     std::vector<void*> stage_args;
     const void* cur_x = nullptr; const int32_t* cur_cls = nullptr; float* cur_loss = nullptr;   // now in the exec
     const float* cur_gather = nullptr;
-    int batch = 0;
-    uint32_t box[2] = {0, 0};        // columns and rows of the input tile, for the tensor map of x
   };
   cudaGraphNode_t cap_stage_node = nullptr;   // filled while capturing
   StageArgs cap_stage_idx{};
-  int cap_batch = 0;
-  uint32_t cap_box[2] = {0, 0};
   bool capturing = false;
+  cudaStream_t capture_stream = nullptr;      // a step of a handle on the legacy default stream is captured on this one
   std::map<int, StepGraph> graphs; // by batch size
   std::map<std::pair<uint64_t, int>, StepGraph> recovery_graphs;   // by (right segment's uid, batch size)
   uint64_t uid = 0;                // unique per handle of the process (a reused address is not the same segment)
@@ -126,7 +121,8 @@ struct seg_handle {
   bool fuse_loss = true;           // take the intermediate-label loss in the last forward product's epilogue where possible
   bool fork_enabled = true;        // run the gradient and update branches on their own streams
   bool small_fused = false;        // small fp32 segment: the whole step runs as two launches (SEG_NO_SMALL_FUSED=1: off)
-  SmallStep small{};               // its description, filled by seg_create (batch is set per step)
+  SmallStep small{};               // its description, filled by seg_create (batch is set per launch)
+  std::map<int, SmallPrepared*> small_by_batch;
   bool fuse_update = false;        // SEG_FUSED_UPDATE=1: apply the optimizer inside the weight-gradient product where the
                                    // kernel can (measured slower than the separate update launch, see gemm_tc.cu)
   float* sil = nullptr;
@@ -358,6 +354,39 @@ seg_status refresh_operand_copy(seg_handle* h, int64_t off, int64_t n) {
   char* dst = reinterpret_cast<char*>(h->params_op) + off * elem_size(h->op_dt);
   SEG_TRY(h, launch_copy2d(dst, h->op_dt, n, h->params + off, DT_F32, n, 1, n, h->op_round,
                            h->stream), "operand copy refresh");
+  return SEG_OK;
+}
+
+// The prepared launches of a small fp32 segment for this batch size; nullptr: the segment runs layer by layer.
+SmallPrepared* small_for(seg_handle* h, int batch) {
+  if (!h->small_fused) return nullptr;
+  SmallPrepared*& w = h->small_by_batch[batch];
+  if (!w) {
+    SmallStep p = h->small;
+    p.batch = batch;
+    w = small_prepare(p);
+  }
+  return w;
+}
+
+// Small fp32 segment: staging, forward, loss and the dgrad chain in one launch, every weight and bias gradient with its
+// update in a second.  The two are launched as they are, without a captured graph: a graph's launch and its parameter
+// update take the GPU about 2.5 us longer a step than two launches chained across steps (784-128-128-64 at batch 64:
+// 18.6 against 15.9 us), and the host needs less than either.
+seg_status small_step(seg_handle* h, SmallPrepared& w, int batch, const void* x, const int32_t* cls, float* loss_to,
+                      const float* gather) {
+  {
+    Launch lf(h, K_FWD_BWD);
+    SEG_TRY(h, launch_small_fwd_bwd(w, reinterpret_cast<const float*>(x), cls, gather, loss_to, h->stream),
+            "small-segment forward/backward launch");
+  }
+  {
+    Launch lw(h, K_WGRAD_UPDATE);
+    SEG_TRY(h, launch_small_wgrad_update(w, h->stream), "small-segment weight-gradient/update launch");
+  }
+  h->family_launches[FAM_SIMT] += 2;
+  ++h->fused_updates;
+  h->last_batch = batch;
   return SEG_OK;
 }
 
@@ -601,12 +630,14 @@ seg_status seg_destroy(seg_handle* h) {
   for (cudaEvent_t e : h->ev_done) if (e) cudaEventDestroy(e);
   for (cudaStream_t ls : h->lstream) if (ls) cudaStreamDestroy(ls);
   for (void* p : h->allocations) cudaFree(p);
+  for (auto& kv : h->small_by_batch) if (kv.second) small_release(kv.second);
   if (h->host_loss) cudaFreeHost(h->host_loss);
   for (int i = 0; i < 2; ++i) {
     if (h->ev_copied[i]) cudaEventDestroy(h->ev_copied[i]);
     if (h->ev_consumed[i]) cudaEventDestroy(h->ev_consumed[i]);
   }
   if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
+  if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   if (h->ev_start) cudaEventDestroy(h->ev_start);
   if (h->ev_stop) cudaEventDestroy(h->ev_stop);
@@ -631,11 +662,9 @@ seg_status seg_forward(seg_handle* h, const void* x, int32_t batch, void* y) {
   if (!h || !x || !y) return SEG_ERR_INVALID_ARG;
   DeviceGuard guard(h);
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
-  if (h->small_fused) {               // small fp32 segment: all layers in one launch, the last one's output also into y
-    SmallStep p = h->small;
-    p.batch = batch;
+  if (SmallPrepared* w = small_for(h, batch)) {   // small fp32 segment: all layers in one launch, the last one's output also into y
     Launch l(h, K_FWD);
-    SEG_TRY(h, launch_small_forward(p, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), h->stream),
+    SEG_TRY(h, launch_small_forward(*w, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), h->stream),
             "small-segment forward launch");
     ++h->family_launches[FAM_SIMT];
     h->last_batch = batch;
@@ -668,26 +697,6 @@ static seg_status enqueue_step(seg_handle* h, int batch, bool forked, const void
   cudaStream_t mainst = h->stream;
   seg_status st;
   float* loss_to = loss_out ? loss_out : h->loss_slot;
-  SmallStep p = h->small;
-  p.batch = batch;
-  if (h->small_fused && small_step_batch_ok(p)) {
-    // small fp32 segment: staging, forward, loss and the dgrad chain in one launch, every weight and bias
-    // gradient with its update in a second
-    {
-      Launch lf(h, K_FWD_BWD);
-      SEG_TRY(h, launch_small_fwd_bwd(p, reinterpret_cast<const float*>(x), cls, gather, loss_to, mainst, h->cap_box),
-              "small-segment forward/backward launch");
-    }
-    if (h->capturing) { h->cap_stage_node = last_captured_node(h); h->cap_stage_idx = kSmallStepArgs; h->cap_batch = batch; }
-    {
-      Launch lw(h, K_WGRAD_UPDATE);
-      SEG_TRY(h, launch_small_wgrad_update(p, mainst), "small-segment weight-gradient/update launch");
-    }
-    h->family_launches[FAM_SIMT] += 2;
-    ++h->fused_updates;
-    h->last_batch = batch;
-    return SEG_OK;
-  }
   {
     // fixed staging buffers: rounds x in TF32 mode, pads the pitch, keeps every later pointer constant;
     // the same launch advances the device-side step counter and Adam's bias corrections and records
@@ -788,8 +797,6 @@ static bool adopt_captured_graph(seg_handle* h, seg_handle::StepGraph& g, cudaGr
   if (!h->cap_stage_node) return false;
   g.stage_node = h->cap_stage_node;
   g.stage_idx = h->cap_stage_idx;
-  g.batch = h->cap_batch;
-  g.box[0] = h->cap_box[0]; g.box[1] = h->cap_box[1];
   if (cudaGraphKernelNodeGetParams(g.stage_node, &g.stage_params) != cudaSuccess) return false;
   g.stage_args.assign(g.stage_params.kernelParams, g.stage_params.kernelParams + g.stage_idx.count);
   if (cudaGraphInstantiate(&g.exec, graph, 0) != cudaSuccess) { g.exec = nullptr; return false; }
@@ -804,13 +811,6 @@ static seg_status replay_graph(seg_handle* h, seg_handle::StepGraph& g, const vo
     g.stage_args[g.stage_idx.cls] = (void*)&cls;
     g.stage_args[g.stage_idx.gather] = (void*)&gather;
     g.stage_args[g.stage_idx.loss] = (void*)&loss_to;
-    CUtensorMap map;
-    if (g.stage_idx.map >= 0 && small_input_by_tensor(reinterpret_cast<const float*>(x), gather, h->widths[0])) {
-      SmallStep p = h->small;
-      p.batch = g.batch;
-      if (!small_input_map(p, reinterpret_cast<const float*>(x), g.box[0], g.box[1], &map)) return SEG_ERR_CUDA;
-      g.stage_args[g.stage_idx.map] = (void*)&map;
-    }
     cudaKernelNodeParams sp = g.stage_params;
     sp.kernelParams = g.stage_args.data();
     SEG_TRY(h, cudaGraphExecKernelNodeSetParams(g.exec, g.stage_node, &sp), "graph parameter update");
@@ -827,16 +827,23 @@ static seg_status replay_graph(seg_handle* h, seg_handle::StepGraph& g, const vo
   return SEG_OK;
 }
 
-// Runs one step through its captured graph: the first call with this graph slot runs eagerly (it sets
-// kernel attributes), the second captures the same enqueue into a graph, later ones replay it with the
-// caller's pointers written into the staging node.  enqueue(forked) enqueues the whole step; peer is a
+// Eager runs of a step before it is captured, on a handle that uses the legacy default stream.  Capture and instantiation cost
+// about 0.4 ms, a replayed step of 784-1024-1024-512 (TF32, batch 256) saves the GPU 5 us over an eager one: a short pass
+// over a new handle, or the partial batch at the end of a few epochs, is not worth a graph.
+constexpr int kLegacyEagerRuns = 24;
+
+// Runs one step through its captured graph: the first call with this graph slot (the first kLegacyEagerRuns calls on the
+// legacy default stream) runs eagerly (it sets kernel attributes), the next captures the same enqueue into a graph, later ones
+// replay it with the caller's pointers written into the staging node.  enqueue(forked) enqueues the whole step; peer is a
 // second handle whose kernels the step launches (the frozen right segment of a recovery step) or null.
 static seg_status run_step_captured(seg_handle* h, seg_handle::StepGraph& g, seg_handle* peer,
                                     const std::function<seg_status(bool)>& enqueue,
                                     const void* x, const int32_t* cls, float* loss_to, const float* gather) {
   if (g.exec != nullptr) return replay_graph(h, g, x, cls, loss_to, gather);
-  if (g.eager_runs == 0) {
-    g.eager_runs = 1;
+  const cudaStream_t user_stream = h->stream;
+  const bool legacy = user_stream == nullptr || user_stream == cudaStreamLegacy;
+  if (g.eager_runs < (legacy ? kLegacyEagerRuns : 1)) {
+    ++g.eager_runs;
     return enqueue(h->fork_enabled);
   }
   const uint64_t before = h->launches, before_peer = peer ? peer->launches : 0;
@@ -853,15 +860,27 @@ static seg_status run_step_captured(seg_handle* h, seg_handle::StepGraph& g, seg
     }
   };
   cudaGraph_t graph = nullptr;
-  if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+  // the legacy default stream cannot be captured (a graph can be launched into it all the same): the step is then recorded
+  // on a stream of the handle's own
+  if (legacy && !h->capture_stream &&
+      cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    h->capture_stream = nullptr;
+  }
+  const cudaStream_t record_on = legacy && h->capture_stream ? h->capture_stream : user_stream;
+  if (cudaStreamBeginCapture(record_on, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
     h->graphs_enabled = false;
     return enqueue(h->fork_enabled);
   }
   h->capturing = true; h->cap_stage_node = nullptr;
+  h->stream = record_on;
+  if (peer) peer->stream = record_on;
   seg_status st = enqueue(h->fork_enabled);
+  h->stream = user_stream;
+  if (peer) peer->stream = user_stream;
   h->capturing = false;
-  cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
+  cudaError_t e = cudaStreamEndCapture(record_on, &graph);
   if (st == SEG_OK && e == cudaSuccess && graph != nullptr && adopt_captured_graph(h, g, graph)) {
     g.kernels = h->launches - before;
     for (int f = 0; f < FAM_COUNT; ++f) g.family[f] = h->family_launches[f] - fam_before[f];
@@ -910,7 +929,10 @@ static seg_status train_step_impl(seg_handle* h, const void* x, const int32_t* c
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
   if (!h->is_final && !h->have_labels) return SEG_ERR_STATE;
   seg_status st = SEG_OK;
-  if (h->profile || !h->graphs_enabled) {
+  SmallPrepared* small = small_for(h, batch);
+  if (small && small_can_train(*small)) {
+    st = small_step(h, *small, batch, x, cls, loss_out ? loss_out : h->loss_slot, gather);
+  } else if (h->profile || !h->graphs_enabled) {
     st = enqueue_step(h, batch, !h->profile && h->fork_enabled, x, cls, loss_out, gather);
   } else {
     auto enqueue = [&](bool forked) { return enqueue_step(h, batch, forked, x, cls, loss_out, gather); };

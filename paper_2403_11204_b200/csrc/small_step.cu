@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <new>
 
 #include "common.cuh"
 
@@ -973,6 +974,18 @@ struct ChainArgs {
   CUtensorMap map_x, map_w0, map_stage;
 };
 
+}  // namespace
+
+// Everything about a launch that depends on the batch size only: split, shared-memory layout, tensor maps of the handle's
+// own buffers, tiles of the second kernel.
+struct SmallPrepared {
+  ChainArgs a;
+  int nt, S, tiles, rows, stages;
+  size_t wgrad_smem;
+};
+
+namespace {
+
 template <int R, int CT0>
 cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
   static std::atomic<bool> allowed[64];
@@ -996,16 +1009,9 @@ cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
 cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
   const SmallStep& p = a.p;
   const SmallPlan& q = a.q;
-  const uint32_t rows = (uint32_t)(q.C * q.R), bw = (uint32_t)q.ks;
-  // x_stage: clipped to the input width and the batch, so that the column of ones behind the width stays
-  if (!make_map_f32(&a.map_stage, p.act[0], (uint64_t)p.widths[0], (uint64_t)p.batch, (uint64_t)p.ld_act[0] * 4, bw, rows))
+  if (small_input_by_tensor(a.x, a.gather, p.widths[0]) &&
+      !make_map_f32(&a.map_x, a.x, (uint64_t)p.widths[0], (uint64_t)p.batch, (uint64_t)p.widths[0] * 4, (uint32_t)q.ks, (uint32_t)(q.C * q.R)))
     return cudaErrorInvalidValue;
-  a.map_w0 = a.map_stage;
-  if (q.C > 1 && !make_map_f32(&a.map_w0, p.params + p.w_off[0], (uint64_t)p.widths[0], (uint64_t)p.widths[1],
-                               (uint64_t)p.ldw[0] * 4, bw, (uint32_t)p.widths[1]))
-    return cudaErrorInvalidValue;
-  a.map_x = a.map_stage;
-  if (small_input_by_tensor(a.x, a.gather, p.widths[0]) && !small_input_map(p, a.x, bw, rows, &a.map_x)) return cudaErrorInvalidValue;
   switch (q.R) {
     case 1: return launch_chain<1>(a, s);
     case 2: return launch_chain<2>(a, s);
@@ -1019,32 +1025,54 @@ cudaError_t launch_chain(ChainArgs& a, cudaStream_t s) {
   }
 }
 
+size_t wgrad_smem_bytes(const SmallStep& p, int nt, int stages) {
+  size_t b = 0;
+  for (int l = 1; l <= p.n_layers; ++l) {
+    const int mt = up(p.widths[l], 8);
+    b = std::max(b, (size_t)(wgrad_ring_floats(mt, nt, stages) + mt * nt) * sizeof(float));
+  }
+  return b;
+}
+
+// Tile width and batch split of the second kernel with the smallest estimate: a wave of CTAs costs its fixed latencies once
+// per CTA an SM has to run, its arithmetic at the rate the register tile reaches (8 x 8 best, 8 x 2 bound by shared-memory loads).
+void plan_wgrad(SmallPrepared* w) {
+  const SmallStep& p = w->a.p;
+  double best_t = 1e30;
+  for (int nt : {64, 32, 16}) {
+    int tiles = 0, mt = 8;
+    for (int l = 0; l < p.n_layers; ++l) { tiles += wgrad_tiles(p.widths[l], nt); mt = std::max(mt, up(p.widths[l + 1], 8)); }
+    const double rate = nt == 64 ? 90.0 : nt == 32 ? 80.0 : 60.0;      // multiply-adds per cycle and SM
+    for (int S : {1, 2, 4, 8}) {
+      if (S > 1 && p.batch < 8 * S) continue;
+      const int rows = (p.batch + S - 1) / S;
+      const int load = (tiles + resident_clusters(S) - 1) / resident_clusters(S);
+      const double t = (S > 1 ? 1500.0 : 500.0) + load * (1500.0 + rows * (double)mt * nt / rate + mt * nt / 8.0 * (1.0 + 1.0 / S));
+      if (t < best_t) { best_t = t; w->nt = nt; w->S = S; w->tiles = tiles; w->rows = rows; }
+    }
+  }
+  // all of a CTA's rows in flight at once where the stages allow it; two CTAs on an SM where the grid needs them
+  w->stages = std::max(1, std::min((w->rows + WK - 1) / WK, W_STAGES));
+  if (w->tiles > resident_clusters(w->S))
+    while (w->stages > 2 && wgrad_smem_bytes(p, w->nt, w->stages) > 112 * 1024) --w->stages;
+  w->wgrad_smem = wgrad_smem_bytes(p, w->nt, w->stages);
+}
+
 template <int OPT, int NT>
-cudaError_t launch_wgrad(const SmallStep& p, int tiles, int S, int rows, int n_partials, cudaStream_t s) {
+cudaError_t launch_wgrad(SmallPrepared& w, cudaStream_t s) {
   static std::atomic<bool> allowed[64];
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(small_wgrad_update_kernel<OPT, NT>), SS_SMEM_LIMIT, allowed);
   if (e != cudaSuccess) return e;
-  // all of a CTA's rows in flight at once where the stages allow it; two CTAs on an SM where the grid needs them
-  int stages = std::max(1, std::min((rows + WK - 1) / WK, W_STAGES));
-  auto bytes = [&](int st) {
-    size_t b = 0;
-    for (int l = 1; l <= p.n_layers; ++l) {
-      const int mt = up(p.widths[l], 8);
-      b = std::max(b, (size_t)(wgrad_ring_floats(mt, NT, st) + mt * NT) * sizeof(float));
-    }
-    return b;
-  };
-  if (tiles > resident_clusters(S)) while (stages > 2 && bytes(stages) > 112 * 1024) --stages;
-  SmallStep pp = p;
-  void* args[] = {&pp, &S, &rows, &n_partials, &stages};
-  return launch_clustered(small_wgrad_update_kernel<OPT, NT>, tiles * S, S, bytes(stages), s, args);
+  int n_partials = chain_grid(w.a.p, w.a.q);
+  void* args[] = {&w.a.p, &w.S, &w.rows, &n_partials, &w.stages};
+  return launch_clustered(small_wgrad_update_kernel<OPT, NT>, w.tiles * w.S, w.S, w.wgrad_smem, s, args);
 }
 
 template <int OPT>
-cudaError_t launch_wgrad(const SmallStep& p, int nt, int tiles, int S, int rows, int n_partials, cudaStream_t s) {
-  if (nt == 64) return launch_wgrad<OPT, 64>(p, tiles, S, rows, n_partials, s);
-  if (nt == 32) return launch_wgrad<OPT, 32>(p, tiles, S, rows, n_partials, s);
-  return launch_wgrad<OPT, 16>(p, tiles, S, rows, n_partials, s);
+cudaError_t launch_wgrad(SmallPrepared& w, cudaStream_t s) {
+  if (w.nt == 64) return launch_wgrad<OPT, 64>(w, s);
+  if (w.nt == 32) return launch_wgrad<OPT, 32>(w, s);
+  return launch_wgrad<OPT, 16>(w, s);
 }
 
 }  // namespace
@@ -1056,14 +1084,30 @@ bool small_step_supported(int n_layers, const int* widths) {
   return true;
 }
 
-bool small_step_batch_ok(const SmallStep& p) {
-  SmallPlan q;
-  return plan_small(p, &q) && chain_grid(p, q) <= loss_max_partials();
+SmallPrepared* small_prepare(const SmallStep& p) {
+  SmallPrepared* w = new (std::nothrow) SmallPrepared();
+  if (!w) return nullptr;
+  ChainArgs& a = w->a;
+  a.p = p;
+  bool ok = plan_small(p, &a.q);
+  if (ok) {
+    const SmallPlan& q = a.q;
+    // x_stage: clipped to the input width and the batch, so that the column of ones behind the width stays
+    ok = make_map_f32(&a.map_stage, p.act[0], (uint64_t)p.widths[0], (uint64_t)p.batch, (uint64_t)p.ld_act[0] * 4, (uint32_t)q.ks,
+                      (uint32_t)(q.C * q.R));
+    a.map_x = a.map_w0 = a.map_stage;
+    if (ok && q.C > 1)
+      ok = make_map_f32(&a.map_w0, p.params + p.w_off[0], (uint64_t)p.widths[0], (uint64_t)p.widths[1], (uint64_t)p.ldw[0] * 4,
+                        (uint32_t)q.ks, (uint32_t)p.widths[1]);
+  }
+  if (!ok) { delete w; return nullptr; }
+  plan_wgrad(w);
+  return w;
 }
 
-bool small_input_map(const SmallStep& p, const float* x, uint32_t box_cols, uint32_t box_rows, CUtensorMap* map) {
-  return make_map_f32(map, x, (uint64_t)p.widths[0], (uint64_t)p.batch, (uint64_t)p.widths[0] * 4, box_cols, box_rows);
-}
+void small_release(SmallPrepared* w) { delete w; }
+
+bool small_can_train(const SmallPrepared& w) { return chain_grid(w.a.p, w.a.q) <= loss_max_partials(); }
 
 bool small_step_maps(const SmallStep& p, int max_batch, CUtensorMap* maps) {
   for (int l = 0; l < p.n_layers; ++l) {
@@ -1082,48 +1126,26 @@ cudaError_t launch_small_ones(float* act, int64_t ld, int col, int rows, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_small_fwd_bwd(const SmallStep& p, const float* x, const int32_t* cls, const float* gather,
-                                 float* loss_to, cudaStream_t s, uint32_t* box) {
-  ChainArgs a{};
-  a.p = p; a.x = x; a.cls = cls; a.gather = gather; a.loss_to = loss_to;
-  if (!plan_small(p, &a.q)) return cudaErrorInvalidValue;
-  if (box) { box[0] = (uint32_t)a.q.ks; box[1] = (uint32_t)(a.q.C * a.q.R); }
+cudaError_t launch_small_fwd_bwd(SmallPrepared& w, const float* x, const int32_t* cls, const float* gather, float* loss_to,
+                                 cudaStream_t s) {
+  ChainArgs& a = w.a;
+  a.x = x; a.cls = cls; a.gather = gather; a.loss_to = loss_to; a.y = nullptr;
+  a.q.forward_only = 0;
   return launch_chain(a, s);
 }
 
-cudaError_t launch_small_forward(const SmallStep& p, const float* x, float* y, cudaStream_t s) {
-  ChainArgs a{};
-  a.p = p; a.x = x; a.y = y;
-  if (!plan_small(p, &a.q)) return cudaErrorInvalidValue;
+cudaError_t launch_small_forward(SmallPrepared& w, const float* x, float* y, cudaStream_t s) {
+  ChainArgs& a = w.a;
+  a.x = x; a.cls = nullptr; a.gather = nullptr; a.loss_to = nullptr; a.y = y;
   a.q.forward_only = 1;
   return launch_chain(a, s);
 }
 
-cudaError_t launch_small_wgrad_update(const SmallStep& p, cudaStream_t s) {
-  SmallPlan q;
-  if (!plan_small(p, &q)) return cudaErrorInvalidValue;
-  const int n_partials = chain_grid(p, q);
-  // tile width and batch split with the smallest estimate: a wave of CTAs costs its fixed latencies once per CTA an SM has
-  // to run, its arithmetic at the rate the register tile reaches (8 x 8 best, 8 x 2 bound by shared-memory loads)
-  int best_nt = 64, best_s = 1, best_tiles = 1;
-  double best_t = 1e30;
-  for (int nt : {64, 32, 16}) {
-    int tiles = 0, mt = 8;
-    for (int l = 0; l < p.n_layers; ++l) { tiles += wgrad_tiles(p.widths[l], nt); mt = std::max(mt, up(p.widths[l + 1], 8)); }
-    const double rate = nt == 64 ? 90.0 : nt == 32 ? 80.0 : 60.0;      // multiply-adds per cycle and SM
-    for (int S : {1, 2, 4, 8}) {
-      if (S > 1 && p.batch < 8 * S) continue;
-      const int rows = (p.batch + S - 1) / S;
-      const int load = (tiles + resident_clusters(S) - 1) / resident_clusters(S);
-      const double t = (S > 1 ? 1500.0 : 500.0) + load * (1500.0 + rows * (double)mt * nt / rate + mt * nt / 8.0 * (1.0 + 1.0 / S));
-      if (t < best_t) { best_t = t; best_nt = nt; best_s = S; best_tiles = tiles; }
-    }
-  }
-  const int rows = (p.batch + best_s - 1) / best_s;
-  switch (p.optimizer) {
-    case SEG_SGD: return launch_wgrad<SEG_SGD>(p, best_nt, best_tiles, best_s, rows, n_partials, s);
-    case SEG_SGD_MOMENTUM: return launch_wgrad<SEG_SGD_MOMENTUM>(p, best_nt, best_tiles, best_s, rows, n_partials, s);
-    case SEG_ADAM: return launch_wgrad<SEG_ADAM>(p, best_nt, best_tiles, best_s, rows, n_partials, s);
+cudaError_t launch_small_wgrad_update(SmallPrepared& w, cudaStream_t s) {
+  switch (w.a.p.optimizer) {
+    case SEG_SGD: return launch_wgrad<SEG_SGD>(w, s);
+    case SEG_SGD_MOMENTUM: return launch_wgrad<SEG_SGD_MOMENTUM>(w, s);
+    case SEG_ADAM: return launch_wgrad<SEG_ADAM>(w, s);
     default: return cudaErrorInvalidValue;
   }
 }

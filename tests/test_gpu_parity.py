@@ -505,3 +505,49 @@ def test_handles_created_and_used_from_two_threads():
         assert len(r) == 1, "a thread did not finish"
         for a, b in zip(r[0], ref[0]):
             assert bits_equal(a, b)
+
+
+@pytest.mark.parametrize("widths,precision,batch", [([72, 200, 136, 64], "tf32", 96), ([200, 160, 96], "fp32", 50)])
+def test_default_stream_step_is_captured_and_replayed(widths, precision, batch):
+    """A handle on the legacy default stream, whose step is captured on a stream of the handle's own after a number of eager
+    runs, must end with the bits of a handle on an ordinary stream; batch size, input and loss address change on the way."""
+    import torch
+    from paper_2403_11204_b200.binding import Segment
+    w = wl.WORKLOADS["tiny"]
+    x, cls = batch_arrays(w, 4 * batch, widths[0])
+    xt, ct = to_device(x, cls, precision)
+    results = []
+    for stream in (None, torch.cuda.Stream()):
+        seg = Segment(widths, 47, False, precision=precision, optimizer="adam", lr=1e-3, max_batch=batch, stream=stream)
+        seg.gen_labels(wl.LABEL_SEED, "normal")
+        loss = torch.zeros(70, device="cuda")
+        torch.cuda.synchronize()
+        for i in range(70):
+            lo, n = (i % 4) * batch, batch - 7 * (i % 2)
+            seg.train_step(xt[lo:lo + n], ct[lo:lo + n], loss[i:i + 1])
+        seg.poll()
+        out = [loss.cpu().numpy()] + [t.cpu().numpy() for l in range(len(widths) - 1) for t in seg.params(l)]
+        results.append(out)
+        seg.close()
+    for a, b in zip(*results):
+        assert bits_equal(a, b)
+
+
+@pytest.mark.parametrize("widths,final", [([784, 128, 128, 128, 47], True), ([1024, 128, 128, 128, 128], False),
+                                          ([128, 128, 128, 128, 128], False), ([129, 1, 47], True), ([300, 81, 33], False),
+                                          ([513, 97, 128, 5], False), ([260, 17, 128], False), ([1, 1], False)])
+@pytest.mark.parametrize("batch", [1, 7, 200, 1411])
+def test_small_segment_shapes(widths, final, batch):
+    """Edges of the two-launch step: weights that pass through two slots or wait for the first layer's tiles, first layers
+    split over 2, 4 and 8 CTAs and not at all, rows per CTA from 1 up, features that are no whole 16-byte groups, forward alone."""
+    w = wl.WORKLOADS["tiny"]
+    gpu, ora = make_pair(widths, 47, final, "fp32", "momentum", 0.01, batch)
+    x, cls = batch_arrays(w, batch, widths[0])
+    xt, _ = to_device(x, cls, "fp32")
+    y = gpu.forward(xt)
+    gpu.poll()
+    assert rel_err(y.cpu().numpy(), ora.forward(x)[-1]) < 1e-4
+    compare_step(gpu, ora, x, cls, "fp32", TOL["fp32"])
+    x2, cls2 = batch_arrays(w, batch, widths[0], seed=3)
+    compare_step(gpu, ora, x2, cls2, "fp32", TOL["fp32"])
+    gpu.close()
