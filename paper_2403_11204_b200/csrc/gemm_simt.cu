@@ -7,8 +7,16 @@
 // split over gridDim.z CTAs per tile: every CTA stores its partial tile to a workspace, the last one
 // to arrive adds the partials in split order (a fixed order: bit-reproducible), applies the epilogue
 // and leaves the arrival counter at zero.
+//
+// gemm_ffma_kernel is the fp32 path proper: tiles of 64 x 64, both operands brought by tensor copies into a ring of shared-memory
+// stages, 8 x 8 outputs per thread.  The 64 threads that hold a tile exist four times in a CTA (each group takes a quarter of
+// every stage's K) and S CTAs of a cluster split K again, so that few tiles still fill the GPU; the partial tiles meet in
+// shared memory and, as a reduce-scatter, in distributed shared memory, in a fixed order.  gemm_simt_kernel serves what tensor
+// copies cannot take (rows that are no whole 16-byte groups) and bf16 operands on the FFMA backend.
 #include <algorithm>
+#include <atomic>
 
+#include "async_copy.cuh"
 #include "common.cuh"
 
 namespace segk {
@@ -131,6 +139,299 @@ gemm_simt_kernel(GemmDesc g, int k_per_split) {
   }
 }
 
+// ---- fp32 products by tensor copies and packed FFMA ------------------------------------------------------
+// What bounds it: FFMA issue.  The packed form (fma.rn.f32x2, two multiply-adds per issue slot) leaves issue slots for the
+// shared-memory loads; a plain 8 x 8 loop measures 60-64 % of the FFMA peak, the packed one 64-71 %.
+enum Form : int { FORM_NT = 0, FORM_NN = 1, FORM_TN = 2 };   // operands k-fast / k-fast, k-fast / n-fast, m-fast / n-fast
+constexpr int FT = 64, FK = 32;                             // tile edge, k per stage
+constexpr int FGROUPS = 4, FTHREADS = 64 * FGROUPS + 32;    // four k groups of 64 threads, one copying warp
+constexpr int FSTAGES = 6, FSTAGE_FLOATS = 2 * FT * FK;     // 16 KiB per stage
+constexpr int FPART = FT + 8;                               // row pitch of a partial tile: conflict-free stores in every form
+constexpr int FRING_FLOATS = FSTAGES * FSTAGE_FLOATS;
+constexpr size_t FSMEM = 1024 + (size_t)(FRING_FLOATS + FT * FT) * sizeof(float);
+static_assert(FGROUPS * FT * FPART <= FRING_FLOATS, "the partial tiles take the ring's place");
+
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
+
+struct FfmaEpi { void* C; int64_t ldc, ldmask; int c_round, epi, relu; const float* bias; const float* mask; };
+
+template <int FORM>
+__global__ void __launch_bounds__(FTHREADS, 1)
+gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N, int K, int S,
+                 int k_per_cta, FfmaEpi e, int* dev_status) {
+  extern __shared__ uint8_t raw[];
+  float* sm = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+  float* recv = sm + FRING_FLOATS;                          // [source CTA][64 / S rows][64]
+  __shared__ uint64_t full[FSTAGES], empty[FSTAGES];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = S > 1 ? (int)cluster_rank() : 0;
+  const int tile = (int)blockIdx.x / S, tiles_m = (M + FT - 1) / FT;
+  const int m0 = tile % tiles_m * FT, n0 = tile / tiles_m * FT;
+  const int k0 = rank * k_per_cta, k1 = min(K, k0 + k_per_cta), steps = k1 > k0 ? (k1 - k0 + FK - 1) / FK : 0;
+  if (tid == 0) {
+    for (int i = 0; i < FSTAGES; ++i) { bar_init(full + i, 1); bar_init(empty + i, 2 * FGROUPS); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async();
+  }
+  __syncthreads();
+  if (S > 1) cluster_arrive_release();
+  pdl_wait();
+  pdl_trigger();
+  const int grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+  f32x2 acc[8][4];                                          // NN, TN: pairs of columns
+  float accf[8][8];                                         // NT
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) accf[i][j] = 0.f;
+  }
+  if (warp == 2 * FGROUPS) {
+    // ---------------- copies ----------------
+    if (elect_one()) {
+      for (int s = 0; s < steps; ++s) {
+        const int st = s % FSTAGES, k = k0 + s * FK;
+        if (s >= FSTAGES) bar_wait(empty + st, (uint32_t)(s / FSTAGES - 1) & 1u, dev_status);
+        float* a = sm + st * FSTAGE_FLOATS;
+        float* b = a + FT * FK;
+        bar_expect(full + st, FSTAGE_FLOATS * 4);
+        if constexpr (FORM == FORM_TN) tensor_load(a, &map_a, m0, k, full + st); else tensor_load(a, &map_a, k, m0, full + st);
+        if constexpr (FORM == FORM_NT) tensor_load(b, &map_b, k, n0, full + st); else tensor_load(b, &map_b, n0, k, full + st);
+      }
+    }
+  } else {
+    // ---------------- arithmetic: this group's 8 of every stage's 32 k ----------------
+    for (int s = 0; s < steps; ++s) {
+      const int st = s % FSTAGES;
+      const float* a_s = sm + st * FSTAGE_FLOATS;
+      const float* b_s = a_s + FT * FK;
+      bar_wait(full + st, (uint32_t)(s / FSTAGES) & 1u, dev_status);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = 2 * grp + h;                          // four k: c * 4 ..
+        if constexpr (FORM == FORM_NT) {
+          // k-fast tiles: rows of 32 k, 128-byte swizzle (16-byte group c of row r at c ^ (r & 7)).  Plain FFMA: pairs along k would
+          // need twice the accumulators, more than the 168 registers nine warps leave a thread
+          float4 a[8];
+          const float* ar = a_s + ty * FK + ((c ^ ty) << 2);
+          const float* br = b_s + tx * FK + ((c ^ tx) << 2);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) a[i] = lds4(ar + i * 8 * FK);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float4 b = lds4(br + j * 8 * FK);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              accf[i][j] = fmaf(a[i].x, b.x, accf[i][j]);
+              accf[i][j] = fmaf(a[i].y, b.y, accf[i][j]);
+              accf[i][j] = fmaf(a[i].z, b.z, accf[i][j]);
+              accf[i][j] = fmaf(a[i].w, b.w, accf[i][j]);
+            }
+          }
+        } else {
+          // n-fast B: rows of 64 n; packed multiply-adds over pairs of columns 4 tx .. and 32 + 4 tx ..
+          float4 a[8];                                      // NN: [row i] four k;  TN: [2 k' + half] four rows
+          if constexpr (FORM == FORM_NN) {
+            const float* ar = a_s + ty * FK + ((c ^ ty) << 2);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(ar + i * 8 * FK);
+          } else {
+            const float* ar = a_s + 4 * c * FT + 4 * ty;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              a[2 * k] = *reinterpret_cast<const float4*>(ar + k * FT);
+              a[2 * k + 1] = *reinterpret_cast<const float4*>(ar + k * FT + 32);
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float* br = b_s + (4 * c + k) * FT + 4 * tx;
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(br), b1 = *reinterpret_cast<const ulonglong2*>(br + 32);
+            const f32x2 b[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              float av;
+              if constexpr (FORM == FORM_NN) av = k == 0 ? a[i].x : k == 1 ? a[i].y : k == 2 ? a[i].z : a[i].w;
+              else { const float4 t = a[2 * k + (i >> 2)]; av = (i & 3) == 0 ? t.x : (i & 3) == 1 ? t.y : (i & 3) == 2 ? t.z : t.w; }
+              const f32x2 aa = pack2(av, av);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) fma2(acc[i][j], aa, b[j]);
+            }
+          }
+        }
+      }
+      if (s + FSTAGES < steps) {
+        __syncwarp();
+        if (lane == 0) bar_arrive(empty + st);
+      }
+    }
+  }
+  __syncthreads();                                          // the ring is free: partial tiles [group][64][72] take its place
+  if (warp < 2 * FGROUPS) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int m = FORM == FORM_TN ? (i >> 2) * 32 + 4 * ty + (i & 3) : ty + 8 * i;
+      float* d = sm + (grp * FT + m) * FPART;
+      if constexpr (FORM == FORM_NT) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d[tx + 8 * j] = accf[i][j];
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float4 v;
+          unpack2(acc[i][2 * h], v.x, v.y);
+          unpack2(acc[i][2 * h + 1], v.z, v.w);
+          *reinterpret_cast<float4*>(d + 32 * h + 4 * tx) = v;
+        }
+      }
+    }
+  }
+  const int slice = FT / S;                                 // rows each CTA of the cluster finishes
+  if (S > 1) cluster_wait_acquire();                        // every peer has started: its shared memory may be written
+  __syncthreads();
+  auto group_sum = [&](int row, int c) {
+    float4 v = lds4(sm + row * FPART + 4 * c);
+#pragma unroll
+    for (int g = 1; g < FGROUPS; ++g) add4(v, lds4(sm + (g * FT + row) * FPART + 4 * c));
+    return v;
+  };
+  if (S > 1) {
+    if (tid < 64 * FGROUPS) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int row = (tid >> 4) + 16 * u, c = tid & 15, owner = row / slice;
+        const uint32_t off = 4u * (uint32_t)((rank * slice + row - owner * slice) * FT + 4 * c);
+        store_cluster4(in_cta(smem_addr(recv), (uint32_t)owner) + off, group_sum(row, c));
+      }
+    }
+    cluster_arrive_release();
+    cluster_wait_acquire();
+  }
+  if (tid >= 64 * FGROUPS) return;
+  float* C = reinterpret_cast<float*>(e.C);
+  const bool wide = (e.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0;
+  const bool mask_wide = (e.ldmask & 3) == 0 && (reinterpret_cast<uintptr_t>(e.mask) & 15u) == 0;
+  for (int r = tid >> 4; r < slice; r += 16) {
+    const int c = tid & 15, m = m0 + rank * slice + r, n = n0 + 4 * c;
+    if (m >= M || n >= N) continue;
+    float4 v4;
+    if (S > 1) {
+      v4 = lds4(recv + r * FT + 4 * c);
+      for (int s = 1; s < S; ++s) add4(v4, lds4(recv + (s * slice + r) * FT + 4 * c));
+    } else {
+      v4 = group_sum(r, c);
+    }
+    float v[4] = {v4.x, v4.y, v4.z, v4.w};
+    const bool whole = n + 3 < N;
+    if (e.epi == EPI_BIAS_ACT) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (n + j < N) v[j] += __ldg(e.bias + n + j);
+        if (e.relu) v[j] = fmaxf(v[j], 0.f);
+      }
+    } else if (e.epi == EPI_MASK) {
+      const float* mr = e.mask + (int64_t)m * e.ldmask + n;
+      if (whole && mask_wide) {
+        const float4 q = *reinterpret_cast<const float4*>(mr);
+        if (!(q.x > 0.f)) v[0] = 0.f;
+        if (!(q.y > 0.f)) v[1] = 0.f;
+        if (!(q.z > 0.f)) v[2] = 0.f;
+        if (!(q.w > 0.f)) v[3] = 0.f;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (n + j < N && !(mr[j] > 0.f)) v[j] = 0.f;
+      }
+    }
+    if (e.c_round == RND_TF32) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = round_tf32_rne(v[j]);
+    }
+    float* cr = C + (int64_t)m * e.ldc + n;
+    if (whole && wide) *reinterpret_cast<float4*>(cr) = make_float4(v[0], v[1], v[2], v[3]);
+    else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) if (n + j < N) cr[j] = v[j];
+    }
+  }
+}
+
+// CTAs that split K of one tile.  A CTA pays about 3000 cycles of latencies (start, first stage, exchange, epilogue) and 46
+// cycles per k (64 x 64 multiply-adds at 70 % of the FFMA rate); clusters of 2, 4 and 8 leave 148, 132 and 120 SMs to fill.
+int ffma_split(int tiles, int K) {
+  int best = 1;
+  double best_t = 1e30;
+  for (int S : {1, 2, 4, 8}) {
+    const int resident = S == 1 ? 148 : S == 2 ? 74 : S == 4 ? 33 : 15;
+    const int kp = ((K + S - 1) / S + FK - 1) / FK * FK;
+    if (S > 1 && kp * (S - 1) >= K) continue;               // a CTA would have nothing to do
+    const double t = (double)((tiles + resident - 1) / resident) * ((S > 1 ? 4000.0 : 3000.0) + 46.0 * kp);
+    if (t < best_t) { best_t = t; best = S; }
+  }
+  return best;
+}
+
+template <int FORM>
+cudaError_t launch_ffma(const CUtensorMap& ma, const CUtensorMap& mb, const GemmDesc& g, int* dev_status, cudaStream_t s) {
+  static std::atomic<bool> allowed[64];
+  auto kern = gemm_ffma_kernel<FORM>;
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!allowed[dev].load(std::memory_order_acquire)) {
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FSMEM);
+    if (err != cudaSuccess) return err;
+    allowed[dev].store(true, std::memory_order_release);
+  }
+  const int tiles = ((g.M + FT - 1) / FT) * ((g.N + FT - 1) / FT);
+  const int S = ffma_split(tiles, g.K);
+  const int kp = ((g.K + S - 1) / S + FK - 1) / FK * FK;
+  FfmaEpi e{};
+  e.C = g.C; e.ldc = g.ldc; e.ldmask = g.ldmask; e.c_round = g.c_round; e.epi = g.epi; e.relu = g.relu;
+  e.bias = g.bias; e.mask = reinterpret_cast<const float*>(g.mask);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(tiles * S)); cfg.blockDim = dim3(FTHREADS); cfg.dynamicSmemBytes = FSMEM; cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (g_use_pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (S > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)S; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, ma, mb, g.M, g.N, g.K, S, kp, e, dev_status);
+}
+
+// cudaErrorNotSupported: operands that tensor copies cannot take (the strided kernel serves them).
+cudaError_t try_ffma(const GemmDesc& g, int* dev_status, cudaStream_t s) {
+  if (g.a_dt != DT_F32 || g.b_dt != DT_F32 || g.c_dt != DT_F32 || g.M <= 0 || g.N <= 0 || g.K <= 0 || g.c_round == RND_BF16)
+    return cudaErrorNotSupported;
+  const bool a_k = g.a_sk == 1, b_k = g.b_sk == 1 && g.b_sn != 1;
+  const int64_t a_pitch = a_k ? g.a_sm : g.a_sk, b_pitch = b_k ? g.b_sn : g.b_sk;
+  if ((!a_k && g.a_sm != 1) || (!b_k && g.b_sn != 1) || (!a_k && b_k)) return cudaErrorNotSupported;
+  if ((a_pitch & 3) || (b_pitch & 3) || ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.B)) & 15u)) return cudaErrorNotSupported;
+  CUtensorMap ma, mb;
+  bool ok = a_k ? make_map_f32(&ma, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)a_pitch * 4, FK, FT, true)
+                : make_map_f32(&ma, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)a_pitch * 4, FT, FK, false);
+  ok = ok && (b_k ? make_map_f32(&mb, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)b_pitch * 4, FK, FT, true)
+                  : make_map_f32(&mb, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)b_pitch * 4, FT, FK, false));
+  if (!ok) return cudaErrorNotSupported;
+  if (a_k && b_k) return launch_ffma<FORM_NT>(ma, mb, g, dev_status, s);
+  if (a_k) return launch_ffma<FORM_NN>(ma, mb, g, dev_status, s);
+  return launch_ffma<FORM_TN>(ma, mb, g, dev_status, s);
+}
+
 }  // namespace
 
 // Partial tiles the split of an M x N x K product would use with an unlimited workspace (0: no split).
@@ -141,9 +442,10 @@ int gemm_simt_slots(int M, int N, int K) {
   return splits > 1 ? tiles * splits : 0;
 }
 
-cudaError_t launch_gemm_simt(const GemmDesc& g, cudaStream_t s) {
+cudaError_t launch_gemm_simt(const GemmDesc& g, int* dev_status, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   if (g.a_dt != g.b_dt) return cudaErrorInvalidValue;
+  if (cudaError_t e = try_ffma(g, dev_status, s); e != cudaErrorNotSupported) return e;
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
   // split K while that adds CTAs the GPU has room for and leaves every split at least 4 k-steps
   const int tiles = (int)(grid.x * grid.y);

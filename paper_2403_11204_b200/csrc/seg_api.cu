@@ -241,7 +241,7 @@ seg_status run_gemm(seg_handle* h, const GemmDesc& g_in, int kind, cudaStream_t 
       return SEG_ERR_UNSUPPORTED;
     }
   }
-  SEG_TRY(h, launch_gemm_simt(g, stream), "FFMA product launch");
+  SEG_TRY(h, launch_gemm_simt(g, h->dev_status, stream), "FFMA product launch");
   ++h->family_launches[FAM_SIMT];
   return SEG_OK;
 }
@@ -453,6 +453,7 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
   h->widths.assign(cfg->widths, cfg->widths + cfg->n_layers + 1);
   if (h->precision == SEG_BF16) { h->act_dt = DT_BF16; h->act_round = RND_BF16; h->op_dt = DT_BF16; h->op_round = RND_BF16; }
   if (h->precision == SEG_TF32) { h->act_round = RND_TF32; h->op_round = RND_TF32; }
+  gemm_tc_init();                  // the fp32 products use tensor maps too (without them: the strided FFMA kernel)
   h->use_tc = (h->precision != SEG_FP32) && (cfg->gemm_backend != SEG_GEMM_SIMT);
   if (h->use_tc && !gemm_tc_init()) {
     if (cfg->gemm_backend == SEG_GEMM_TCGEN05) { delete h; return SEG_ERR_UNSUPPORTED; }
