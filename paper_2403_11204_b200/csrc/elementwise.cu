@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kLossThreads)
 mse_loss_kernel(const TOut* __restrict__ out, int64_t ld_out, const int32_t* __restrict__ cls,
                 const float* __restrict__ sil, int n_classes, int n_p, int batch, int relu_mask,
                 TDz* __restrict__ dz, int dz_round, int64_t ld_dz, float* partials,
-                unsigned int* counter, float* loss_out, float* const* loss_dst) {
+                unsigned int* counter, float* loss_out) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
@@ -86,7 +86,8 @@ mse_loss_kernel(const TOut* __restrict__ out, int64_t ld_out, const int32_t* __r
     }
   }
   const float bt = block_sum(acc, red);
-  finish_loss(bt, partials, counter, loss_out, loss_dst, 1.0f / (float)((int64_t)batch * n_p), red);
+  if (counter != nullptr) finish_loss(bt, partials, counter, loss_out, 1.0f / (float)((int64_t)batch * n_p), red);
+  else if (threadIdx.x == 0) partials[blockIdx.x] = bt;    // a training step: its last update launch adds the partials up
 }
 
 // Final segment: one warp per sample;  p = softmax(z) with the row maximum subtracted,
@@ -97,8 +98,7 @@ template <typename TDz, bool IN_REGS>
 __global__ void __launch_bounds__(kLossThreads)
 softmax_ce_kernel(const float* __restrict__ logits, int64_t ld, const int32_t* __restrict__ cls,
                   int n_classes, int batch, int relu_mask, TDz* __restrict__ dz, int dz_round,
-                  int64_t ld_dz, float* partials, unsigned int* counter, float* loss_out,
-                  float* const* loss_dst) {
+                  int64_t ld_dz, float* partials) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
@@ -161,7 +161,7 @@ softmax_ce_kernel(const float* __restrict__ logits, int64_t ld, const int32_t* _
     }
   }
   const float bt = block_sum(acc, red);
-  finish_loss(bt, partials, counter, loss_out, loss_dst, inv_b, red);
+  if (threadIdx.x == 0) partials[blockIdx.x] = bt;
 }
 
 // The update of one layer in one launch.  Parameters, gradients and optimizer state share one flat
@@ -169,13 +169,26 @@ softmax_ce_kernel(const float* __restrict__ logits, int64_t ld, const int32_t* _
 //   blocks [0, bias_blocks): each forms the bias gradient of 8 or 32 columns, db[n] = sum_b dZ[b][n]
 //     (32 or 8 row lanes per column, then the lanes in index order: one fixed order, bit-reproducible),
 //     stores it and applies the optimizer to those bias elements;
-//   the other blocks stream over the weight range, whose gradient the weight-gradient product wrote.
+//   the other blocks stream over the weight range, whose gradient the weight-gradient product wrote;
+//   with loss partials to add up, one more block does that.
 // Both parts refresh the reduced-precision operand copy.
 template <int OPT, int OPDT>
 __global__ void __launch_bounds__(256)
 update_kernel(UpdateArgs u, int bias_blocks, int bias_cols) {
   pdl_wait();
   pdl_trigger();
+  const int stream_blocks = (int)gridDim.x - bias_blocks - (u.n_loss > 0 ? 1 : 0);
+  if ((int)blockIdx.x == bias_blocks + stream_blocks) {
+    __shared__ float red[32];
+    float v = 0.f;
+    for (int i = threadIdx.x; i < u.n_loss; i += blockDim.x) v += u.loss_partials[i];
+    const float total = block_sum(v, red);
+    if (threadIdx.x == 0) {
+      float* dst = *u.loss_dst;
+      if (dst) *dst = total * u.loss_scale;
+    }
+    return;
+  }
   float inv_bc1 = 1.0f, inv_bc2 = 1.0f;
   if constexpr (OPT == SEG_ADAM) { inv_bc1 = 1.0f / __ldg(u.bc); inv_bc2 = 1.0f / __ldg(u.bc + 1); }
   if ((int)blockIdx.x < bias_blocks) {
@@ -225,7 +238,7 @@ update_kernel(UpdateArgs u, int bias_blocks, int bias_cols) {
   const float4* __restrict__ g4 = reinterpret_cast<const float4*>(u.g);
   float4* __restrict__ s14 = reinterpret_cast<float4*>(u.s1);
   float4* __restrict__ s24 = reinterpret_cast<float4*>(u.s2);
-  const int64_t stride = (int64_t)(gridDim.x - bias_blocks) * blockDim.x;
+  const int64_t stride = (int64_t)stream_blocks * blockDim.x;
   for (int64_t i = (int64_t)(blockIdx.x - bias_blocks) * blockDim.x + threadIdx.x; i < n4; i += stride) {
     const float4 p = p4[i];
     const float4 g = g4[i];
@@ -383,13 +396,13 @@ bool mse_wide(const void* out, int64_t ld_out, const void* dz, int64_t ld_dz, co
 cudaError_t launch_mse_loss(const void* out, int out_dt, int64_t ld_out, const int32_t* cls,
                             const float* sil, int n_classes, int n_p, int batch, int relu_mask, void* dz,
                             int dz_dt, int dz_round, int64_t ld_dz, float* partials,
-                            unsigned int* counter, float* const* loss_dst, cudaStream_t s) {
-  float* const loss_out = nullptr;
+                            int* n_partials, cudaStream_t s) {
   const bool wide = mse_wide(out, ld_out, dz, ld_dz, sil, n_p);
   const int grid = grid_for((int64_t)batch * n_p, kLossThreads * (wide ? 16 : 4), kMaxLossBlocks);
+  *n_partials = grid;
 #define SEGK_MSE(TO, TD, V)                                                                              \
   launch_k(mse_loss_kernel<TO, TD, V>, dim3(grid), dim3(kLossThreads), 0, s, (const TO*)out, ld_out, cls, \
-           sil, n_classes, n_p, batch, relu_mask, (TD*)dz, dz_round, ld_dz, partials, counter, loss_out, loss_dst)
+           sil, n_classes, n_p, batch, relu_mask, (TD*)dz, dz_round, ld_dz, partials, nullptr, nullptr)
   if (out_dt == DT_BF16 && dz_dt == DT_BF16) {
     if (wide) SEGK_MSE(__nv_bfloat16, __nv_bfloat16, 8); else SEGK_MSE(__nv_bfloat16, __nv_bfloat16, 1);
   } else if (out_dt == DT_F32 && dz_dt == DT_F32) {
@@ -403,15 +416,14 @@ cudaError_t launch_mse_loss(const void* out, int out_dt, int64_t ld_out, const i
 
 cudaError_t launch_softmax_ce_loss(const float* logits, int64_t ld_logits, const int32_t* cls,
                                    int n_classes, int batch, int relu_mask, void* dz, int dz_dt,
-                                   int dz_round, int64_t ld_dz, float* partials,
-                                   unsigned int* counter, float* const* loss_dst, cudaStream_t s) {
-  float* const loss_out = nullptr;
+                                   int dz_round, int64_t ld_dz, float* partials, int* n_partials, cudaStream_t s) {
   const int warps = kLossThreads / 32;
   const int grid = grid_for(batch, warps, kMaxLossBlocks);
+  *n_partials = grid;
   const bool in_regs = n_classes <= 32 * CE_REGS;
 #define SEGK_CE(TD, R)                                                                                         \
   launch_k(softmax_ce_kernel<TD, R>, dim3(grid), dim3(kLossThreads), 0, s, logits, ld_logits, cls, n_classes, \
-           batch, relu_mask, (TD*)dz, dz_round, ld_dz, partials, counter, loss_out, loss_dst)
+           batch, relu_mask, (TD*)dz, dz_round, ld_dz, partials)
   if (dz_dt == DT_BF16) {
     if (in_regs) SEGK_CE(__nv_bfloat16, true); else SEGK_CE(__nv_bfloat16, false);
   } else {
@@ -425,10 +437,10 @@ cudaError_t launch_update(const UpdateArgs& u, cudaStream_t s) {
   if (u.n & 3) return cudaErrorInvalidValue;
   const int bias_cols = (u.batch <= 1024 || u.n_bias <= 256) ? 8 : 32;   // narrow layers: few blocks either way, keep the walk short
   const int bias_blocks = (u.dz != nullptr && u.n_bias > 0) ? (u.n_bias + bias_cols - 1) / bias_cols : 0;
-  if (u.n == 0 && bias_blocks == 0) return cudaSuccess;
+  if (u.n == 0 && bias_blocks == 0 && u.n_loss == 0) return cudaSuccess;
   // two rounds of resident blocks (8 per SM): measured 5.6 TB/s against 4.9 with one round on the 67 M-element
   // momentum update, no difference for Adam; streaming (evict-first) loads and stores measured no better
-  const int grid = bias_blocks + (u.n > 0 ? grid_for(u.n >> 2, 256, 148 * 16) : 0);
+  const int grid = bias_blocks + (u.n > 0 ? grid_for(u.n >> 2, 256, 148 * 16) : 0) + (u.n_loss > 0 ? 1 : 0);
   const bool bf = (u.p_op != nullptr && u.op_dt == DT_BF16);
 #define SEGK_UPD(OPT)                                                      \
   if (bf) launch_k(update_kernel<OPT, DT_BF16>, dim3(grid), dim3(256), 0, s, u, bias_blocks, bias_cols);             \
@@ -521,10 +533,10 @@ extern "C" SEG_API seg_status seg_label_loss_noalloc(const float* out, const int
   const int grid = grid_for((int64_t)batch * n_p, kLossThreads * (wide ? 16 : 4), kMaxLossBlocks);
   if (wide)
     mse_loss_kernel<float, float, 8><<<grid, kLossThreads, 0, s>>>(out, n_p, cls, sil, n_classes, n_p, batch, relu_mask ? 1 : 0,
-                                                                  dz, RND_NONE, n_p, partials, counter, loss_out, nullptr);
+                                                                  dz, RND_NONE, n_p, partials, counter, loss_out);
   else
     mse_loss_kernel<float, float, 1><<<grid, kLossThreads, 0, s>>>(out, n_p, cls, sil, n_classes, n_p, batch, relu_mask ? 1 : 0,
-                                                                  dz, RND_NONE, n_p, partials, counter, loss_out, nullptr);
+                                                                  dz, RND_NONE, n_p, partials, counter, loss_out);
   if (cudaGetLastError() != cudaSuccess) return SEG_ERR_CUDA;
   return SEG_OK;
 }

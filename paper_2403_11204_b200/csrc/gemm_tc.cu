@@ -67,6 +67,8 @@ constexpr int UPDATE_WARPS = 8;                        // fused-update variants:
 constexpr int NUM_THREADS_FUSED = NUM_THREADS + 32 * UPDATE_WARPS;
 constexpr int SMEM_BUDGET = 192 * 1024;                // operand ring
 constexpr int SMEM_EXTRA = 2048;                       // alignment slack + barriers
+constexpr int HALF_SM_MAX_KB = 16;                     // k-blocks up to which the persistent kernel gives up ring depth for it
+constexpr int HALF_SM_SMEM = 113 * 1024;               // two CTAs of this size fit on an SM (228 KiB, 1 KiB of it per CTA reserved)
 // Output staging of the persistent kernels: every epilogue warp owns two buffers of 32 rows x 64 bytes (32 bf16 or 16
 // fp32 columns), written with the shared-memory swizzle of the output tensor map and drained by bulk tensor stores, so
 // that global memory sees whole 64-byte row segments instead of 32 separate 16-byte pieces.  16 KiB in all, taken out
@@ -234,6 +236,7 @@ struct EpilogueArgs {
   const void* mask;
   int64_t ldmask;
   int staged;               // persistent kernels: store C through shared memory and bulk tensor stores
+  int b_early;              // B may be loaded before the preceding kernel is complete (GemmDesc::b_early)
   LossFuse loss;
   FusedUpdate upd;
 };
@@ -495,38 +498,18 @@ __device__ __forceinline__ void epilogue_store_mse(const EpilogueArgs& e, float 
 }
 
 // End of a CTA's epilogue: the four epilogue warps leave their loss sums in shared memory; the last
-// warp to arrive adds them in warp order and publishes the CTA's partial; the last CTA of the grid
-// adds all partials in index order (a fixed order: bit-reproducible) and writes the batch loss.
-// No barrier is used, so a warp that gave up a bounded wait cannot block the others.
+// warp to arrive adds them in warp order and publishes the CTA's partial (the step's last update launch adds the
+// partials in index order: bit-reproducible).  No barrier is used, so a warp that gave up a bounded wait cannot block the others.
 __device__ __forceinline__ void loss_finish(const LossFuse& l, float lacc, int quarter, int lane, volatile float* slots,
                                             unsigned int* warp_counter) {
   const float w = warp_sum_f(lacc);
-  unsigned int prev = 0;
   if (lane == 0) {
     slots[quarter] = w;
     __threadfence_block();
-    prev = atomicAdd(warp_counter, 1u);
-  }
-  prev = __shfl_sync(0xFFFFFFFFu, prev, 0);
-  if (prev != 3u) return;
-  __threadfence_block();
-  unsigned int done = 0;
-  if (lane == 0) {
-    const float block_total = ((slots[0] + slots[1]) + slots[2]) + slots[3];
-    l.partials[blockIdx.x] = block_total;
-    __threadfence();
-    done = atomicAdd(l.counter, 1u);
-  }
-  done = __shfl_sync(0xFFFFFFFFu, done, 0);
-  if (done != gridDim.x - 1) return;
-  __threadfence();
-  float part = 0.f;
-  for (unsigned int i = lane; i < gridDim.x; i += 32) part += __ldcg(l.partials + i);
-  const float total = warp_sum_f(part);
-  if (lane == 0) {
-    float* dst = *l.loss_dst;
-    if (dst) *dst = total * l.loss_scale;
-    *l.counter = 0u;
+    if (atomicAdd(warp_counter, 1u) == 3u) {
+      __threadfence_block();
+      l.partials[blockIdx.x] = ((slots[0] + slots[1]) + slots[2]) + slots[3];
+    }
   }
 }
 
@@ -689,6 +672,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   const int num_k = (K + BLOCK_K - 1) / BLOCK_K;
   int first_m = 0, first_n = 0;
   if ((int)blockIdx.x < n_tiles) tile_coords((int)blockIdx.x, tiles_m, tiles_n, group_m, first_m, first_n);
+  auto load_b = [&](int st, int n0, int k0) {
+    const uint32_t b_dst = smem_u32(smem_b + st * L::B_TILE_BYTES);
+    if constexpr (B_MN) {
+#pragma unroll
+      for (int c = 0; c < BLOCK_N / CHUNK; ++c)
+        tma_load_2d(b_dst + c * MN_CHUNK_BYTES, &map_b, n0 + c * CHUNK, k0, full_bar(st));
+    } else {
+      tma_load_2d(b_dst, &map_b, k0, n0, full_bar(st));
+    }
+  };
+  // stages whose B tiles are under way before the preceding kernel has finished
+  const int early = (epi.b_early && (int)blockIdx.x < n_tiles) ? min(STAGES, num_k) : 0;
+  if (warp == 0 && early > 0) {
+    if (elect_one()) {
+      for (int kb = 0; kb < early; ++kb) {
+        mbar_arrive_expect_tx(full_bar(kb), (uint32_t)L::STAGE_BYTES);
+        load_b(kb, first_n * BLOCK_N, kb * BLOCK_K);
+      }
+    }
+  }
   pdl_wait();                         // everything above overlapped the previous kernel's tail
   pdl_trigger();
 
@@ -697,6 +700,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (elect_one()) {
       int stage = 0; uint32_t phase = 0;
       int fills = 0;                     // stages filled so far, counted up to the ring's depth: the first pass waits for nothing
+      int ahead = early;
       bool ok = true;
       for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
         int m_idx, n_idx;
@@ -705,9 +709,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         for (int kb = 0; kb < num_k; ++kb) {
           if (fills < STAGES) ++fills;
           else if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, dev_status)) { ok = false; break; }
-          mbar_arrive_expect_tx(full_bar(stage), (uint32_t)L::STAGE_BYTES);
+          const bool b_under_way = ahead > 0;
+          if (b_under_way) --ahead;
+          else mbar_arrive_expect_tx(full_bar(stage), (uint32_t)L::STAGE_BYTES);
           const uint32_t a_dst = smem_u32(smem_a + stage * A_TILE_BYTES);
-          const uint32_t b_dst = smem_u32(smem_b + stage * L::B_TILE_BYTES);
           const int k0 = kb * BLOCK_K;
           if constexpr (A_MN) {
 #pragma unroll
@@ -716,13 +721,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           } else {
             tma_load_2d(a_dst, &map_a, k0, m0, full_bar(stage));
           }
-          if constexpr (B_MN) {
-#pragma unroll
-            for (int c = 0; c < BLOCK_N / CHUNK; ++c)
-              tma_load_2d(b_dst + c * MN_CHUNK_BYTES, &map_b, n0 + c * CHUNK, k0, full_bar(stage));
-          } else {
-            tma_load_2d(b_dst, &map_b, k0, n0, full_bar(stage));
-          }
+          if (!b_under_way) load_b(stage, n0, k0);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
@@ -852,10 +851,14 @@ __device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster_addr, uin
                ::"r"(dst_cluster_addr), "r"(src_local_addr), "r"(bytes), "r"(bar_cluster_addr) : "memory");
 }
 constexpr int SPLITK_BLOCK_N = 64;
-constexpr int SPLITK_STAGES = 6;
+// Three stages, and the send buffer takes the ring's place once the accumulator is complete: 106 KiB per CTA, so that two CTAs
+// share an SM.  What that buys is not this kernel's own time but its neighbours': the next kernel's prologue runs beside it, and
+// a weight gradient on another branch no longer keeps the dgrad chain's clusters waiting for whole SMs.
+constexpr int SPLITK_STAGES = 3;
 constexpr int SPLITK_STAGE_BYTES = A_TILE_BYTES + SPLITK_BLOCK_N * TILE_ROW_BYTES;       // 24 KiB
 constexpr int SPLITK_RECV_BYTES = 8 * (SPLITK_BLOCK_N / 8) * BLOCK_M * 4;                // [src][col in slice][row] fp32, 32 KiB
-constexpr int SPLITK_SMEM = SPLITK_STAGES * SPLITK_STAGE_BYTES + 2 * SPLITK_RECV_BYTES + SMEM_EXTRA;   // + send buffer
+constexpr int SPLITK_SMEM = SPLITK_STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES + SMEM_EXTRA;
+static_assert(SPLITK_STAGES * SPLITK_STAGE_BYTES >= SPLITK_RECV_BYTES, "the send buffer fits into the ring");
 
 // One 128 x 64 output tile per cluster; CTA r of the cluster contracts k-blocks [r*kpc, (r+1)*kpc).
 template <bool TF32, bool A_MN, bool B_MN, int SPLIT, bool LOSS = false>
@@ -879,8 +882,8 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   uint8_t* smem_a = smem;
   uint8_t* smem_b = smem + STAGES * A_TILE_BYTES;
   float* recv = reinterpret_cast<float*>(smem + STAGES * SPLITK_STAGE_BYTES);                      // [src][col in slice][row]
-  float* send = reinterpret_cast<float*>(smem + STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES);  // [dest][col in slice][row]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * SPLITK_STAGE_BYTES + 2 * SPLITK_RECV_BYTES);
+  float* send = reinterpret_cast<float*>(smem);                        // [dest][col in slice][row], in the ring's place
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES);
   // bars[0..S) full, [S..2S) empty, [2S] accumulator complete, [2S+1] partial slices received
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -922,6 +925,21 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   const int kpc = (num_k + split - 1) / split;
   const int kb_begin = min(num_k, (int)rank * kpc), kb_end = min(num_k, kb_begin + kpc);
   const int my_k = kb_end - kb_begin;     // may be 0 for the last ranks: they contribute zeros
+  auto load_b = [&](int st, int kb) {
+    const uint32_t b_dst = smem_u32(smem_b + st * B_TILE_BYTES);
+    if constexpr (B_MN) {
+#pragma unroll
+      for (int c = 0; c < BLOCK_N / CHUNK; ++c)
+        tma_load_2d(b_dst + c * MN_CHUNK_BYTES, &map_b, n0 + c * CHUNK, kb * BLOCK_K, full_bar(st));
+    } else {
+      tma_load_2d(b_dst, &map_b, kb * BLOCK_K, n0, full_bar(st));
+    }
+  };
+  const int early = epi.b_early ? min(STAGES, my_k) : 0;   // B tiles under way before the preceding kernel has finished
+  if (warp == 2 && early > 0) {
+    if (elect_one())
+      for (int i = 0; i < early; ++i) load_b(i, kb_begin + i);
+  }
   pdl_wait();
   pdl_trigger();
 
@@ -990,15 +1008,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         // the first pass over the ring finds every stage free: no wait (a wait that passes at once still costs a
         // couple of hundred cycles of the issuing thread)
         if (kb - kb_begin >= STAGES && !mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, dev_status)) break;
-        const uint32_t b_dst = smem_u32(smem_b + stage * B_TILE_BYTES);
-        const int k0 = kb * BLOCK_K;
-        if constexpr (B_MN) {
-#pragma unroll
-          for (int c = 0; c < BLOCK_N / CHUNK; ++c)
-            tma_load_2d(b_dst + c * MN_CHUNK_BYTES, &map_b, n0 + c * CHUNK, k0, full_bar(stage));
-        } else {
-          tma_load_2d(b_dst, &map_b, k0, n0, full_bar(stage));
-        }
+        if (kb - kb_begin >= early) load_b(stage, kb);
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
@@ -1440,7 +1450,13 @@ cudaError_t launch_variant(const CUtensorMap& ma, const CUtensorMap& mb, const C
   const int grid = tiles < num_sms() ? tiles : num_sms();
   const int group_m = pick_group_m((g.M + BLOCK_M - 1) / BLOCK_M, (g.N + BLOCK_N - 1) / BLOCK_N, grid, BLOCK_M, BLOCK_N, g.K,
                                    TF32 ? 4 : 2);
-  const int n_stages = e.staged ? L::STAGES_STAGED : L::STAGES;
+  int n_stages = e.staged ? L::STAGES_STAGED : L::STAGES;
+  // A product of one 64-column tile per CTA over a short contraction is latency-bound and runs beside others: at most half of an
+  // SM's shared memory, so that the next kernel's CTAs are resident, with their weights on the way, before this one ends.  The
+  // main loop itself wants the deep ring (1024x2048x4096 in 128-column tiles: 44 us with two stages, 23 us with five).
+  constexpr int BLOCK_K = TF32 ? 32 : 64;
+  if (BLOCK_N == 64 && tiles <= num_sms() && g.K <= HALF_SM_MAX_KB * BLOCK_K)
+    n_stages = std::min(n_stages, (HALF_SM_SMEM - (e.staged ? STAGE_OUT_BYTES : 0) - SMEM_EXTRA) / L::STAGE_BYTES);
   const int smem_bytes = n_stages * L::STAGE_BYTES + (e.staged ? STAGE_OUT_BYTES : 0) + SMEM_EXTRA;
   return launch_k(kern, dim3(grid), dim3(FUSED ? NUM_THREADS_FUSED : NUM_THREADS), smem_bytes, s, ma, mb, mc, g.M, g.N, g.K,
                   e, dev_status, group_m, n_stages);
@@ -1667,9 +1683,10 @@ cudaError_t launch_wait_selftest(int* dev_status, uint64_t limit_ns, cudaStream_
 // rows, lanes over the classes (slower still: 32 dependent reduction chains per warp), and one thread
 // per row with short loops over its row in shared memory (about the cost of the launch it saves, and
 // it gives up the split over K) - and stays a launch of its own.
-bool gemm_tc_can_fuse_loss(int M, int N, int K, bool tf32) {
-  if (!g_init_ok || !g_allow_splitk) return false;
-  return pick_split(M, N, K, tf32) > 1;
+int gemm_tc_fused_loss_partials(int M, int N, int K, bool tf32) {
+  if (!g_init_ok || !g_allow_splitk) return 0;
+  const int split = pick_split(M, N, K, tf32);
+  return split > 1 ? split * ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N) : 0;
 }
 
 // The fused update lives in the persistent kernels (one CTA or a CTA pair per tile); products small enough to
@@ -1710,8 +1727,8 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   if (a_pitch * (int64_t)esz >= (1ll << 40) || b_pitch * (int64_t)esz >= (1ll << 40)) return cudaErrorNotSupported;
 
   const bool fuse_loss = (g.epi == EPI_BIAS_ACT) && g.loss.enabled != 0;
-  if (fuse_loss && (a_mn || b_mn || !gemm_tc_can_fuse_loss(g.M, g.N, g.K, tf32)))
-    return cudaErrorInvalidValue;                           // the caller asks gemm_tc_can_fuse_loss first
+  if (fuse_loss && (a_mn || b_mn || gemm_tc_fused_loss_partials(g.M, g.N, g.K, tf32) == 0))
+    return cudaErrorInvalidValue;                           // the caller asks gemm_tc_fused_loss_partials first
   const bool throughput = g.off_critical_path != 0;
   const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 1;
   const Choice choice = pick_kernel(g.M, g.N, g.K, tf32, throughput);
@@ -1729,7 +1746,7 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
 
   EpilogueArgs e;
   e.C = g.C; e.ldc = g.ldc; e.c_dt = g.c_dt; e.c_round = g.c_round; e.epi = g.epi; e.relu = g.relu;
-  e.bias = g.bias; e.mask = g.mask; e.ldmask = g.ldmask;
+  e.bias = g.bias; e.mask = g.mask; e.ldmask = g.ldmask; e.b_early = g.b_early;
   e.loss = g.loss; e.loss.enabled = fuse_loss ? 1 : 0;
   e.upd = g.upd;
   e.staged = (g_staged_epilogue && !e.upd.enabled) ? 1 : 0;

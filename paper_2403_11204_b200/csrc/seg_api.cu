@@ -128,7 +128,7 @@ struct seg_handle {
   float* sil = nullptr;
   bool have_labels = false;
   float* loss_partials = nullptr;
-  unsigned int* loss_counter = nullptr;
+  int n_loss_partials = 0;         // partials the last enqueued loss wrote
   int* dev_status = nullptr;
   void* host_x = nullptr;          // device staging of seg_train_step_host
   int32_t* host_cls = nullptr;
@@ -271,34 +271,32 @@ seg_status prepare_input(seg_handle* h, const void* x, int batch, const void** x
 }
 
 // Description of a non-final segment's loss for fusion into its last forward product.
-LossFuse loss_fuse_desc(seg_handle* h, int batch, const int32_t* cls, float* const* loss_dst) {
+LossFuse loss_fuse_desc(seg_handle* h, int batch, const int32_t* cls) {
   const int L = h->n_layers;
   LossFuse f{};
   f.enabled = 1;
   f.cls = cls; f.sil = h->sil;
   f.dz = h->dzbuf[L - 1]; f.ld_dz = h->ld_act[L]; f.dz_dt = h->act_dt; f.dz_round = h->act_round;
   f.relu_mask = h->last_relu ? 1 : 0;
-  const double count = (double)batch * h->widths[L];
   f.gscale = 2.0f / (float)((int64_t)batch * h->widths[L]);
-  f.loss_scale = (float)(1.0 / count);
-  f.partials = h->loss_partials; f.counter = h->loss_counter; f.loss_dst = loss_dst;
+  f.partials = h->loss_partials;
   return f;
 }
 
 // The segment's loss as a launch of its own (the final segment's softmax cross-entropy always; the
 // intermediate-label loss when the last forward product could not take it).
-seg_status launch_loss(seg_handle* h, int batch, const int32_t* cls, float* const* loss_dst) {
+seg_status launch_loss(seg_handle* h, int batch, const int32_t* cls) {
   const int L = h->n_layers;
   Launch l(h, K_LOSS, h->stream);
   void* dz_L = h->dzbuf[L - 1];
   if (h->is_final) {
     SEG_TRY(h, launch_softmax_ce_loss((const float*)h->act[L], h->ld_act[L], cls, h->n_classes, batch,
                                       h->last_relu ? 1 : 0, dz_L, h->act_dt, h->act_round, h->ld_act[L],
-                                      h->loss_partials, h->loss_counter, loss_dst, h->stream), "softmax-CE loss");
+                                      h->loss_partials, &h->n_loss_partials, h->stream), "softmax-CE loss");
   } else {
     SEG_TRY(h, launch_mse_loss(h->act[L], h->act_dtype[L], h->ld_act[L], cls, h->sil, h->n_classes, h->widths[L], batch,
                                h->last_relu ? 1 : 0, dz_L, h->act_dt, h->act_round, h->ld_act[L],
-                               h->loss_partials, h->loss_counter, loss_dst, h->stream), "MSE loss");
+                               h->loss_partials, &h->n_loss_partials, h->stream), "MSE loss");
   }
   return SEG_OK;
 }
@@ -306,8 +304,9 @@ seg_status launch_loss(seg_handle* h, int batch, const int32_t* cls, float* cons
 // Forward products of all layers, reading layer 0's input from (a_prev, ld_prev).  With loss_cls not
 // null the segment's loss follows: inside the last product's epilogue where the tensor-core path can
 // take it, as a separate launch otherwise.
-seg_status forward_layers(seg_handle* h, const void* a_prev, int64_t ld_prev, int batch,
-                          const int32_t* loss_cls = nullptr, float* const* loss_dst = nullptr) {
+// first_early: the kernel enqueued before does not write layer 0's weights (an input staging, another segment's product).
+seg_status forward_layers(seg_handle* h, const void* a_prev, int64_t ld_prev, int batch, bool first_early,
+                          const int32_t* loss_cls = nullptr) {
   for (int l = 0; l < h->n_layers; ++l) {
     const LayerInfo& L = h->layers[l];
     const bool last = (l == h->n_layers - 1);
@@ -319,14 +318,16 @@ seg_status forward_layers(seg_handle* h, const void* a_prev, int64_t ld_prev, in
     g.c_round = (last && h->is_final) ? RND_NONE : h->act_round;
     g.epi = EPI_BIAS_ACT; g.relu = (!last || h->last_relu) ? 1 : 0;
     g.bias = h->params + L.b_off;
+    g.b_early = (l > 0 || first_early) ? 1 : 0;
     const bool want_loss = last && loss_cls != nullptr;
-    if (want_loss && !h->is_final && h->use_tc && h->fuse_loss &&
-        gemm_tc_can_fuse_loss(g.M, g.N, g.K, h->precision == SEG_TF32))
-      g.loss = loss_fuse_desc(h, batch, loss_cls, loss_dst);
+    if (want_loss && !h->is_final && h->use_tc && h->fuse_loss) {
+      const int n = gemm_tc_fused_loss_partials(g.M, g.N, g.K, h->precision == SEG_TF32);
+      if (n > 0 && n <= loss_max_partials()) { g.loss = loss_fuse_desc(h, batch, loss_cls); h->n_loss_partials = n; }
+    }
     bool used_tc = false;
     seg_status st = run_gemm(h, g, K_FWD, h->stream, &used_tc);
     if (st != SEG_OK) return st;
-    if (want_loss && !(used_tc && g.loss.enabled) && (st = launch_loss(h, batch, loss_cls, loss_dst)) != SEG_OK) return st;
+    if (want_loss && !(used_tc && g.loss.enabled) && (st = launch_loss(h, batch, loss_cls)) != SEG_OK) return st;
     a_prev = h->act[l + 1]; ld_prev = h->ld_act[l + 1];
   }
   h->last_batch = batch;
@@ -337,7 +338,7 @@ seg_status forward_impl(seg_handle* h, const void* x, int batch) {
   const void* a_prev; int64_t ld_prev;
   seg_status st = prepare_input(h, x, batch, &a_prev, &ld_prev);
   if (st != SEG_OK) return st;
-  return forward_layers(h, a_prev, ld_prev, batch);
+  return forward_layers(h, a_prev, ld_prev, batch, a_prev == h->x_stage);
 }
 
 seg_status copy_out(seg_handle* h, void* y, int batch) {
@@ -563,7 +564,6 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
   if (!h->is_final &&
       (st = dev_alloc(h, &h->sil, (size_t)h->n_classes * h->widths[h->n_layers], true)) != SEG_OK) return bail(st);
   if ((st = dev_alloc(h, &h->loss_partials, loss_max_partials(), true)) != SEG_OK) return bail(st);
-  if ((st = dev_alloc(h, &h->loss_counter, 1, true)) != SEG_OK) return bail(st);
   if ((st = dev_alloc(h, &h->dev_status, 1, true)) != SEG_OK) return bail(st);
   if (h->small_fused) {
     SmallStep& p = h->small;
@@ -691,7 +691,7 @@ static cudaGraphNode_t last_captured_node(seg_handle* h) {
   return deps[0];
 }
 
-static seg_status enqueue_backward(seg_handle* h, int batch, bool forked);
+static seg_status enqueue_backward(seg_handle* h, int batch, bool forked, const seg_handle* loss_of);
 
 static seg_status enqueue_step(seg_handle* h, int batch, bool forked, const void* x, const int32_t* cls,
                                float* loss_out, const float* gather) {
@@ -708,8 +708,8 @@ static seg_status enqueue_step(seg_handle* h, int batch, bool forked, const void
                                    gather, loss_to, h->loss_dst, h->n_classes, h->dev_status, mainst), "input staging");
   }
   if (h->capturing) { h->cap_stage_node = last_captured_node(h); h->cap_stage_idx = kStageInputsArgs; }
-  if ((st = forward_layers(h, h->x_stage, h->ld_act[0], batch, h->cls_stage, h->loss_dst)) != SEG_OK) return st;
-  return enqueue_backward(h, batch, forked);
+  if ((st = forward_layers(h, h->x_stage, h->ld_act[0], batch, true, h->cls_stage)) != SEG_OK) return st;
+  return enqueue_backward(h, batch, forked, h);
 }
 
 // Backward pass and update of every layer, starting from dZ of the last layer in dzbuf[L-1].
@@ -718,7 +718,8 @@ static seg_status enqueue_step(seg_handle* h, int batch, bool forked, const void
 // gradient starts as soon as dZ_l exists, its update (which also forms the bias gradient) follows
 // once dgrad(l), the last reader of the old W_l, is done.  The branches of the upper layers thereby
 // finish beside the dgrad chain, and what is left after the last dgrad is two kernels.
-static seg_status enqueue_backward(seg_handle* h, int batch, bool forked) {
+// loss_of: the segment whose loss kernel ran; layer 0's update, the last launch of the step, adds its partials up.
+static seg_status enqueue_backward(seg_handle* h, int batch, bool forked, const seg_handle* loss_of) {
   const int L = h->n_layers;
   cudaStream_t mainst = h->stream;
   seg_status st;
@@ -739,6 +740,7 @@ static seg_status enqueue_backward(seg_handle* h, int batch, bool forked) {
       d.C = h->dzbuf[l - 1]; d.ldc = h->ld_act[l]; d.c_dt = h->act_dt; d.c_round = h->act_round;
       d.M = batch; d.N = Ly.in; d.K = Ly.out; d.epi = EPI_MASK;
       d.mask = h->act[l]; d.ldmask = h->ld_act[l];
+      d.b_early = 1;
       if ((st = run_gemm(h, d, K_DGRAD, mainst)) != SEG_OK) return st;
       if (forked) SEG_TRY(h, cudaEventRecord(h->ev_dz[l - 1], mainst), "event record");
     }
@@ -749,6 +751,7 @@ static seg_status enqueue_backward(seg_handle* h, int batch, bool forked) {
     w.B = a_prev; w.b_sk = ld_prev; w.b_sn = 1; w.b_dt = h->act_dt;
     w.C = h->grads + Ly.w_off; w.ldc = Ly.ldw; w.c_dt = DT_F32; w.c_round = RND_NONE;
     w.M = Ly.out; w.N = Ly.in; w.K = batch; w.epi = EPI_PLAIN;
+    w.b_early = 1;               // the input activations: at least two kernels old
     w.off_critical_path = l > 0;  // the upper layers' weight gradients run beside the dgrad chain and each other
     const int64_t lo = Ly.w_off;
     // Opt-in (SEG_FUSED_UPDATE=1; measured slower): where the persistent tensor-core kernels run the product, they also
@@ -783,6 +786,10 @@ static seg_status enqueue_backward(seg_handle* h, int batch, bool forked) {
     u.bias_off = Ly.b_off - lo; u.g_bias = h->grads + Ly.b_off;
     u.lr = h->lr; u.momentum = h->momentum; u.beta1 = h->beta1; u.beta2 = h->beta2; u.eps = h->eps;
     u.bc = h->bc_dev;
+    if (l == 0) {
+      u.loss_partials = loss_of->loss_partials; u.n_loss = loss_of->n_loss_partials; u.loss_dst = h->loss_dst;
+      u.loss_scale = loss_of->is_final ? 1.0f / (float)batch : 1.0f / (float)((int64_t)batch * loss_of->widths[loss_of->n_layers]);
+    }
     {
       Launch lu(h, K_UPDATE, ls);
       SEG_TRY(h, launch_update(u, ls), "optimizer update");
@@ -959,9 +966,9 @@ static seg_status enqueue_recovery(seg_handle* h, seg_handle* r, int batch, bool
                                    nullptr, loss_to, h->loss_dst, h->n_classes, h->dev_status, s), "input staging");
   }
   if (h->capturing) { h->cap_stage_node = last_captured_node(h); h->cap_stage_idx = kStageInputsArgs; }
-  if ((st = forward_layers(h, h->x_stage, h->ld_act[0], batch)) != SEG_OK) return st;
+  if ((st = forward_layers(h, h->x_stage, h->ld_act[0], batch, true)) != SEG_OK) return st;
   // the joined network's loss: the right segment's softmax cross-entropy on the class labels
-  if ((st = forward_layers(r, h->act[Ll], h->ld_act[Ll], batch, h->cls_stage, h->loss_dst)) != SEG_OK) return st;
+  if ((st = forward_layers(r, h->act[Ll], h->ld_act[Ll], batch, true, h->cls_stage)) != SEG_OK) return st;
   // through the frozen right segment: dgrad only, down to its input, which is the left segment's output
   for (int l = Lr - 1; l >= 0; --l) {
     const LayerInfo& Ly = r->layers[l];
@@ -969,6 +976,7 @@ static seg_status enqueue_recovery(seg_handle* h, seg_handle* r, int batch, bool
     d.A = r->dzbuf[l]; d.a_sm = r->ld_act[l + 1]; d.a_sk = 1; d.a_dt = r->act_dt;
     d.B = weights_op(r, l); d.b_sk = Ly.ldw; d.b_sn = 1; d.b_dt = r->op_dt;
     d.M = batch; d.N = Ly.in; d.K = Ly.out; d.c_dt = r->act_dt; d.c_round = r->act_round;
+    d.b_early = 1;
     if (l > 0) {
       d.C = r->dzbuf[l - 1]; d.ldc = r->ld_act[l];
       d.epi = EPI_MASK; d.mask = r->act[l]; d.ldmask = r->ld_act[l];
@@ -979,7 +987,7 @@ static seg_status enqueue_recovery(seg_handle* h, seg_handle* r, int batch, bool
     }
     if ((st = run_gemm(r, d, K_DGRAD, s)) != SEG_OK) return st;
   }
-  return enqueue_backward(h, batch, forked);
+  return enqueue_backward(h, batch, forked, r);
 }
 
 seg_status seg_recovery_step(seg_handle* left, seg_handle* right, const void* x, const int32_t* cls,
