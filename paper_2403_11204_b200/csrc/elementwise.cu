@@ -283,6 +283,44 @@ copy2d_kernel(void* dst, int dst_dt, int64_t ld_dst, const void* src, int src_dt
   }
 }
 
+// The same copy between matrices of one element type: a warp per row segment, 16 bytes per lane and access where both sides allow
+// it (no division per element).  seg is the number of elements a warp copies at a time.
+template <typename T, bool WIDE>
+__global__ void __launch_bounds__(256)
+copy_rows_kernel(T* __restrict__ dst, int64_t ld_dst, const T* __restrict__ src, int64_t ld_src, int64_t rows, int64_t cols, int seg,
+                 int segs_per_row, int round) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5), total = rows * segs_per_row;
+  for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < total; w += warps) {
+    const int64_t r = segs_per_row == 1 ? w : w / segs_per_row;
+    const int64_t c0 = (w - r * segs_per_row) * seg, c1 = min(cols, c0 + seg);
+    const T* s = src + r * ld_src;
+    T* d = dst + r * ld_dst;
+    if constexpr (WIDE) {
+      constexpr int V = 16 / (int)sizeof(T);
+#pragma unroll 4
+      for (int64_t c = c0 + lane * V; c < c1; c += 32 * V) {
+        uint4 q = *reinterpret_cast<const uint4*>(s + c);
+        if (sizeof(T) == 4 && round == RND_TF32) {
+          q.x = __float_as_uint(round_tf32_rne(__uint_as_float(q.x)));
+          q.y = __float_as_uint(round_tf32_rne(__uint_as_float(q.y)));
+          q.z = __float_as_uint(round_tf32_rne(__uint_as_float(q.z)));
+          q.w = __float_as_uint(round_tf32_rne(__uint_as_float(q.w)));
+        }
+        *reinterpret_cast<uint4*>(d + c) = q;
+      }
+    } else {
+#pragma unroll 4
+      for (int64_t c = c0 + lane; c < c1; c += 32) {
+        if constexpr (sizeof(T) == 4) d[c] = apply_round(s[c], round);
+        else d[c] = s[c];
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256)
 stage_inputs_kernel(void* dst, int dt, int64_t ld_dst, const void* src, int64_t ld_src, int rows, int cols,
                     int round, int32_t* cls_dst, const int32_t* cls_src, unsigned long long* t, float* bc,
@@ -470,6 +508,21 @@ cudaError_t launch_stage_inputs(void* dst, int dt, int64_t ld_dst, const void* s
 cudaError_t launch_copy2d(void* dst, int dst_dt, int64_t ld_dst, const void* src, int src_dt,
                           int64_t ld_src, int64_t rows, int64_t cols, int round, cudaStream_t s) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
+  if (src_dt == dst_dt && (round == RND_NONE || (round == RND_TF32 && dst_dt == DT_F32) || (round == RND_BF16 && dst_dt == DT_BF16))) {
+    if (ld_src == cols && ld_dst == cols) { cols *= rows; rows = 1; ld_src = ld_dst = cols; }      // contiguous on both sides
+    const int esz = dst_dt == DT_BF16 ? 2 : 4, v = 16 / esz;
+    const bool wide = ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15u) == 0 && cols % v == 0 &&
+                      (rows == 1 || (ld_src % v == 0 && ld_dst % v == 0));
+    // a warp takes up to 2 KiB (four accesses of a lane) of a row at a time
+    const int seg = wide ? 4 * 32 * v : 4 * 32;
+    const int segs = (int)((cols + seg - 1) / seg);
+    const int grid = grid_for(rows * segs, 8, 148 * 8);
+#define SEGK_COPY(T, W) launch_k(copy_rows_kernel<T, W>, dim3(grid), dim3(256), 0, s, (T*)dst, ld_dst, (const T*)src, ld_src, rows, cols, seg, segs, round)
+    if (esz == 2) { if (wide) SEGK_COPY(unsigned short, true); else SEGK_COPY(unsigned short, false); }
+    else { if (wide) SEGK_COPY(float, true); else SEGK_COPY(float, false); }
+#undef SEGK_COPY
+    return cudaGetLastError();
+  }
   const int grid = grid_for(rows * cols, 256 * 4, 148 * 8);
   launch_k(copy2d_kernel, dim3(grid), dim3(256), 0, s, dst, dst_dt, ld_dst, src, src_dt, ld_src, rows, cols, round);
   return cudaGetLastError();

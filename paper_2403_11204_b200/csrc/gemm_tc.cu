@@ -1058,6 +1058,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     } else {
       cluster_wait();
     }
+    cluster_arrive();                   // "I have received everything": completes under the epilogue, waited for at the end
     if (ok) {
 #pragma unroll
       for (int cs = 0; cs < W; ++cs) own[cs] = send[((int)rank * w + cs) * BLOCK_M + row_in_tile];
@@ -1079,13 +1080,15 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   if (*abort_flag) {
     for (int i = 0; i < 64; ++i) __nanosleep(20000);
   }
-  if (warp < 2) cluster_wait();       // the producer and MMA warps complete the first cluster phase here
+  if (warp < 2) {                     // the producer and MMA warps complete the first cluster phase and arrive for the second here
+    cluster_wait();
+    cluster_arrive();
+  }
   tc_fence_before();
   __syncthreads();
-  cluster_arrive();                   // no CTA leaves while a peer may still read its send buffer or write
-  cluster_wait();                     // into its receive buffer
   tc_fence_after();
   if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
+  cluster_wait();                     // no CTA leaves before its peers have what it sent them
 }
 
 
