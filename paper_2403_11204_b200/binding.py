@@ -255,6 +255,11 @@ class Segment:
             raise SegError(status, detail)
 
     def _empty(self, *shape, dtype=None):
+        # on the segment's own device and stream, as the caching allocator wants it; the contexts cost more than the
+        # allocation, so they are entered only where they change something
+        cuda = self._torch.cuda
+        if cuda.current_device() == self.device and cuda.current_stream() == self.stream:
+            return self._torch.empty(*shape, dtype=dtype or self._torch.float32, device="cuda")
         with self._torch.cuda.device(self.device), self._torch.cuda.stream(self.stream):
             return self._torch.empty(*shape, dtype=dtype or self._torch.float32, device="cuda")
 

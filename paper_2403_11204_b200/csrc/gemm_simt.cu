@@ -365,7 +365,7 @@ gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 
 // CTAs that split K of one tile.  A CTA pays about 3000 cycles of latencies (start, first stage, exchange, epilogue) and 46
 // cycles per k (64 x 64 multiply-adds at 70 % of the FFMA rate); clusters of 2, 4 and 8 leave 148, 132 and 120 SMs to fill.
-int ffma_split(int tiles, int K) {
+int ffma_split(int tiles, int K, double* cycles = nullptr) {
   int best = 1;
   double best_t = 1e30;
   for (int S : {1, 2, 4, 8}) {
@@ -375,6 +375,7 @@ int ffma_split(int tiles, int K) {
     const double t = (double)((tiles + resident - 1) / resident) * ((S > 1 ? 4000.0 : 3000.0) + 46.0 * kp);
     if (t < best_t) { best_t = t; best = S; }
   }
+  if (cycles) *cycles = best_t;
   return best;
 }
 
@@ -433,6 +434,12 @@ cudaError_t try_ffma(const GemmDesc& g, int* dev_status, cudaStream_t s) {
 }
 
 }  // namespace
+
+double ffma_estimate_us(int M, int N, int K) {
+  double cycles = 0;
+  ffma_split(((M + FT - 1) / FT) * ((N + FT - 1) / FT), K, &cycles);
+  return cycles / 1900.0;
+}
 
 // Partial tiles the split of an M x N x K product would use with an unlimited workspace (0: no split).
 int gemm_simt_slots(int M, int N, int K) {

@@ -1686,6 +1686,10 @@ cudaError_t launch_wait_selftest(int* dev_status, uint64_t limit_ns, cudaStream_
 // rows, lanes over the classes (slower still: 32 dependent reduction chains per warp), and one thread
 // per row with short loops over its row in shared memory (about the cost of the launch it saves, and
 // it gives up the split over K) - and stays a launch of its own.
+double gemm_tc_estimate_us(int M, int N, int K, bool tf32) {
+  return 3.0 + pick_kernel(M, N, K, tf32, false).us;         // + launch, first loads and drain
+}
+
 int gemm_tc_fused_loss_partials(int M, int N, int K, bool tf32) {
   if (!g_init_ok || !g_allow_splitk) return 0;
   const int split = pick_split(M, N, K, tf32);

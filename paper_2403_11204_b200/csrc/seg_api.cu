@@ -134,6 +134,11 @@ struct seg_handle {
   int32_t* host_cls = nullptr;
   float* host_loss = nullptr;      // page-locked host float the loss kernel writes (seg_train_step_host)
   float* host_loss_dev = nullptr;  // its device-side address
+  // seg_forward_dataset: rows per chunk (0: not yet chosen) and the chunk's buffers (two for hidden layers in turn, one for a
+  // staged input)
+  int dataset_rows = 0;
+  void* dataset_ws[2] = {nullptr, nullptr};
+  void* dataset_x = nullptr;
   // seg_train_step_host_async: copy stream, two device buffers for the batch in flight and the next one
   cudaStream_t copy_stream = nullptr;
   void* async_x[2] = {nullptr, nullptr};
@@ -301,6 +306,21 @@ seg_status launch_loss(seg_handle* h, int batch, const int32_t* cls) {
   return SEG_OK;
 }
 
+// Forward product of layer l over `batch` rows of (a_prev, ld_prev), output into the handle's own activation buffer.
+GemmDesc forward_desc(seg_handle* h, int l, const void* a_prev, int64_t ld_prev, int batch) {
+  const LayerInfo& L = h->layers[l];
+  const bool last = (l == h->n_layers - 1);
+  GemmDesc g{};
+  g.A = a_prev; g.a_sm = ld_prev; g.a_sk = 1; g.a_dt = h->act_dt;
+  g.B = weights_op(h, l); g.b_sk = 1; g.b_sn = L.ldw; g.b_dt = h->op_dt;
+  g.C = h->act[l + 1]; g.ldc = h->ld_act[l + 1]; g.c_dt = h->act_dtype[l + 1];
+  g.M = batch; g.N = L.out; g.K = L.in;
+  g.c_round = (last && h->is_final) ? RND_NONE : h->act_round;
+  g.epi = EPI_BIAS_ACT; g.relu = (!last || h->last_relu) ? 1 : 0;
+  g.bias = h->params + L.b_off;
+  return g;
+}
+
 // Forward products of all layers, reading layer 0's input from (a_prev, ld_prev).  With loss_cls not
 // null the segment's loss follows: inside the last product's epilogue where the tensor-core path can
 // take it, as a separate launch otherwise.
@@ -308,16 +328,8 @@ seg_status launch_loss(seg_handle* h, int batch, const int32_t* cls) {
 seg_status forward_layers(seg_handle* h, const void* a_prev, int64_t ld_prev, int batch, bool first_early,
                           const int32_t* loss_cls = nullptr) {
   for (int l = 0; l < h->n_layers; ++l) {
-    const LayerInfo& L = h->layers[l];
     const bool last = (l == h->n_layers - 1);
-    GemmDesc g{};
-    g.A = a_prev; g.a_sm = ld_prev; g.a_sk = 1; g.a_dt = h->act_dt;
-    g.B = weights_op(h, l); g.b_sk = 1; g.b_sn = L.ldw; g.b_dt = h->op_dt;
-    g.C = h->act[l + 1]; g.ldc = h->ld_act[l + 1]; g.c_dt = h->act_dtype[l + 1];
-    g.M = batch; g.N = L.out; g.K = L.in;
-    g.c_round = (last && h->is_final) ? RND_NONE : h->act_round;
-    g.epi = EPI_BIAS_ACT; g.relu = (!last || h->last_relu) ? 1 : 0;
-    g.bias = h->params + L.b_off;
+    GemmDesc g = forward_desc(h, l, a_prev, ld_prev, batch);
     g.b_early = (l > 0 || first_early) ? 1 : 0;
     const bool want_loss = last && loss_cls != nullptr;
     if (want_loss && !h->is_final && h->use_tc && h->fuse_loss) {
@@ -665,7 +677,7 @@ seg_status seg_forward(seg_handle* h, const void* x, int32_t batch, void* y) {
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
   if (SmallPrepared* w = small_for(h, batch)) {   // small fp32 segment: all layers in one launch, the last one's output also into y
     Launch l(h, K_FWD);
-    SEG_TRY(h, launch_small_forward(*w, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), h->stream),
+    SEG_TRY(h, launch_small_forward(*w, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), true, h->stream),
             "small-segment forward launch");
     ++h->family_launches[FAM_SIMT];
     h->last_batch = batch;
@@ -1036,6 +1048,59 @@ seg_status seg_train_epochs(seg_handle* h, const void* x, const int32_t* cls, in
   return SEG_OK;
 }
 
+// True when rows of the segment's input (output) at this address are whole 16-byte groups, as tensor copies need them.
+static bool rows_aligned(const void* p, int width, size_t esz) {
+  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (width * esz) % 16 == 0;
+}
+
+// Rows per chunk of a long forward pass: a response does not depend on how its rows are grouped, and products over the
+// training batch alone often leave half of the SMs without a tile in their last round (1024 x 2048 outputs: 32 tiles of
+// 256 x 256 on 74 CTA pairs).  The multiple of 256 with the smallest estimated time per row; at most 8192 rows and 128 MB a buffer.
+static int choose_dataset_rows(const seg_handle* h) {
+  int64_t widest = 1;
+  for (int l = 0; l <= h->n_layers; ++l) widest = std::max(widest, h->ld_act[l]);
+  const int64_t most = std::min<int64_t>(8192, (128ll << 20) / (widest * 4));
+  int best = 0;
+  double best_us = 1e30;
+  for (int rows = 256; rows <= most; rows += 256) {
+    double us = 0;
+    for (const LayerInfo& L : h->layers)
+      us += h->use_tc ? gemm_tc_estimate_us(rows, L.out, L.in, h->precision == SEG_TF32)
+                      : 3.0 + ffma_estimate_us(rows, L.out, L.in);
+    if (us / rows < best_us * 0.99) { best_us = us / rows; best = rows; }
+  }
+  return best;
+}
+
+// Forward pass of `rows` rows through the chunk buffers, the last layer's output into y.
+static seg_status forward_chunk(seg_handle* h, const void* x, int rows, void* y) {
+  const int L = h->n_layers;
+  const size_t esz = elem_size(h->act_dt), osz = elem_size(h->act_dtype[L]);
+  const void* a = x;
+  int64_t ld = h->widths[0];
+  bool early = false;
+  if (h->precision == SEG_TF32 || !rows_aligned(x, h->widths[0], esz)) {
+    Launch l(h, K_COPY);
+    SEG_TRY(h, launch_copy2d(h->dataset_x, h->act_dt, h->ld_act[0], x, h->act_dt, h->widths[0], rows, h->widths[0], h->act_round,
+                             h->stream), "input staging");
+    a = h->dataset_x; ld = h->ld_act[0]; early = true;
+  }
+  const bool direct = rows_aligned(y, h->widths[L], osz);
+  for (int l = 0; l < L; ++l) {
+    GemmDesc g = forward_desc(h, l, a, ld, rows);
+    if (l == L - 1 && direct) { g.C = y; g.ldc = h->widths[L]; }
+    else g.C = h->dataset_ws[l & 1];
+    g.b_early = (l > 0 || early) ? 1 : 0;
+    seg_status st = run_gemm(h, g, K_FWD, h->stream);
+    if (st != SEG_OK) return st;
+    a = g.C; ld = g.ldc;
+  }
+  if (direct) return SEG_OK;
+  Launch l(h, K_COPY);
+  SEG_TRY(h, launch_copy2d(y, h->act_dtype[L], h->widths[L], a, h->act_dtype[L], ld, rows, h->widths[L], RND_NONE, h->stream), "output copy");
+  return SEG_OK;
+}
+
 seg_status seg_forward_dataset(seg_handle* h, const void* x, int64_t n, int32_t batch, void* y) {
   if (!h || !x || !y) return SEG_ERR_INVALID_ARG;
   DeviceGuard guard(h);
@@ -1043,10 +1108,48 @@ seg_status seg_forward_dataset(seg_handle* h, const void* x, int64_t n, int32_t 
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
   const size_t in_bytes = (size_t)h->widths[0] * elem_size(h->act_dt);
   const size_t out_bytes = (size_t)h->widths[h->n_layers] * elem_size(h->act_dtype[h->n_layers]);
-  for (int64_t i = 0; i < n; i += batch) {
+  auto xr = [&](int64_t i) { return reinterpret_cast<const char*>(x) + (size_t)i * in_bytes; };
+  auto yr = [&](int64_t i) { return reinterpret_cast<char*>(y) + (size_t)i * out_bytes; };
+  // the last chunk of `batch` rows (or the partial one) goes through the handle's own buffers, where seg_get_activation looks;
+  // the rows before it are grouped as the GPU likes them
+  const int64_t head = n - (n % batch ? n % batch : batch);
+  int64_t done = 0;
+  if (h->small_fused) {
+    while (done < head) {
+      const int rows = (int)std::min<int64_t>(head - done, 1 << 20);
+      SmallPrepared* w = small_for(h, rows);
+      if (!w) break;
+      Launch l(h, K_FWD);
+      SEG_TRY(h, launch_small_forward(*w, reinterpret_cast<const float*>(xr(done)), reinterpret_cast<float*>(yr(done)), false, h->stream),
+              "small-segment forward launch");
+      ++h->family_launches[FAM_SIMT];
+      done += rows;
+    }
+  } else if (head > batch) {
+    if (h->dataset_rows == 0) {
+      const int rows = choose_dataset_rows(h);
+      int64_t widest = 0;
+      for (int l = 1; l <= h->n_layers; ++l) widest = std::max<int64_t>(widest, h->ld_act[l] * elem_size(h->act_dtype[l]));
+      char *b0 = nullptr, *b1 = nullptr, *bx = nullptr;
+      seg_status st;
+      if ((st = dev_alloc(h, &b0, (size_t)(rows * widest), false)) != SEG_OK || (st = dev_alloc(h, &b1, (size_t)(rows * widest), false)) != SEG_OK ||
+          (st = dev_alloc(h, &bx, (size_t)rows * h->ld_act[0] * elem_size(h->act_dt), true)) != SEG_OK) return st;
+      h->dataset_ws[0] = b0; h->dataset_ws[1] = b1; h->dataset_x = bx;
+      h->dataset_rows = rows;
+    }
+    // equal chunks of at most dataset_rows rows, whole 256-row tiles each
+    const int64_t chunks = (head + h->dataset_rows - 1) / h->dataset_rows;
+    const int64_t rows = std::min<int64_t>(h->dataset_rows, round_up((head + chunks - 1) / chunks, 256));
+    while (done < head) {
+      const int b = (int)std::min<int64_t>(rows, head - done);
+      seg_status st = forward_chunk(h, xr(done), b, yr(done));
+      if (st != SEG_OK) return st;
+      done += b;
+    }
+  }
+  for (int64_t i = done; i < n; i += batch) {
     const int b = (int)std::min<int64_t>(batch, n - i);
-    seg_status st = seg_forward(h, reinterpret_cast<const char*>(x) + (size_t)i * in_bytes, b,
-                                reinterpret_cast<char*>(y) + (size_t)i * out_bytes);
+    seg_status st = seg_forward(h, xr(i), b, yr(i));
     if (st != SEG_OK) return st;
   }
   return SEG_OK;

@@ -48,7 +48,7 @@ struct SmallPlan {
   int ks;                      // features per CTA (C > 1) or the input width rounded up to 4 (C = 1): row pitch of the x tile
   int late;                    // chain weights share the x and W_0 tiles' memory and are loaded once the first layer is done
   int streamed;                // chain weights go through two slots instead of one slot each
-  int forward_only;
+  int forward_only;            // 1: forward pass that also stores every layer's output; 2: only the last layer's, into y
   int off_x, off_w0, off_send, off_recv, off_bias, off_tgt, off_dz[2];
   int off_act[kSmallMaxLayers + 1], off_slot[kSmallMaxLayers];
   int floats;
@@ -355,7 +355,7 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
     o.N = p.widths[l + 1]; o.pa = up(o.N, 4);
     o.last = l == L - 1; o.relu = !o.last || p.last_relu;
     o.a_s = act_s(l + 1);
-    o.ld = p.ld_act[l + 1]; o.a_g = p.act[l + 1] + (int64_t)row0 * o.ld;
+    o.ld = p.ld_act[l + 1]; o.a_g = q.forward_only == 2 ? nullptr : p.act[l + 1] + (int64_t)row0 * o.ld;
     o.ld_y = o.N; o.y_g = (o.last && y != nullptr) ? y + (int64_t)row0 * o.N : nullptr;
     o.dz_g = p.dz[l] + (int64_t)row0 * o.ld;
     return o;
@@ -368,7 +368,7 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
     if (o.relu) v = fmaxf(v, 0.f);
     if (n >= o.N) v = 0.f;
     const bool store = r < nv && n < o.N;
-    if (store) o.a_g[r * o.ld + n] = v;
+    if (store && o.a_g != nullptr) o.a_g[r * o.ld + n] = v;
     if (store && o.y_g != nullptr) o.y_g[r * o.ld_y + n] = v;
     if (o.last && want_targets) {
       float g = 0.f;
@@ -1062,10 +1062,10 @@ cudaError_t launch_small_fwd_bwd(SmallPrepared& w, const float* x, const int32_t
   return launch_chain(a, s);
 }
 
-cudaError_t launch_small_forward(SmallPrepared& w, const float* x, float* y, cudaStream_t s) {
+cudaError_t launch_small_forward(SmallPrepared& w, const float* x, float* y, bool keep, cudaStream_t s) {
   ChainArgs& a = w.a;
   a.x = x; a.cls = nullptr; a.gather = nullptr; a.loss_to = nullptr; a.y = y;
-  a.q.forward_only = 1;
+  a.q.forward_only = keep ? 1 : 2;
   return launch_chain(a, s);
 }
 
