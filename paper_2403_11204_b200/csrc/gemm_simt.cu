@@ -144,7 +144,10 @@ gemm_simt_kernel(GemmDesc g, int k_per_split) {
 // shared-memory loads; a plain 8 x 8 loop measures 60-64 % of the FFMA peak, the packed one 64-71 %.
 enum Form : int { FORM_NT = 0, FORM_NN = 1, FORM_TN = 2 };   // operands k-fast / k-fast, k-fast / n-fast, m-fast / n-fast
 constexpr int FT = 64, FK = 32;                             // tile edge, k per stage
-constexpr int FGROUPS = 4, FTHREADS = 64 * FGROUPS + 32;    // four k groups of 64 threads, one copying warp
+constexpr int FGROUPS = 4, FTHREADS = 64 * FGROUPS;         // four k groups of 64 threads
+// NN and TN have a ninth warp for the copies (71 % of the FFMA peak at 2048^3 in TN form; 61 % when a computing warp issues them);
+// NT does without: nine warps leave a thread 168 registers, its 64 pairs of sums need more (53 % against 46 % with plain FFMA).
+__host__ __device__ constexpr int ffma_threads(int form) { return FTHREADS + (form == 0 ? 0 : 32); }
 constexpr int FSTAGES = 6, FSTAGE_FLOATS = 2 * FT * FK;     // 16 KiB per stage
 constexpr int FPART = FT + 8;                               // row pitch of a partial tile: conflict-free stores in every form
 constexpr int FRING_FLOATS = FSTAGES * FSTAGE_FLOATS;
@@ -163,7 +166,7 @@ __device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) { asm("fma.rn.f
 struct FfmaEpi { void* C; int64_t ldc, ldmask; int c_round, epi, relu; const float* bias; const float* mask; };
 
 template <int FORM>
-__global__ void __launch_bounds__(FTHREADS, 1)
+__global__ void __launch_bounds__(ffma_threads(FORM), 1)
 gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N, int K, int S,
                  int k_per_cta, FfmaEpi e, int* dev_status) {
   extern __shared__ uint8_t raw[];
@@ -185,30 +188,34 @@ gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
   pdl_wait();
   pdl_trigger();
   const int grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
-  f32x2 acc[8][4];                                          // NN, TN: pairs of columns
-  float accf[8][8];                                         // NT
+  // NT: pairs along k (even and odd partial sums of all 64 outputs); NN, TN: pairs of columns
+  constexpr int NJ = FORM == FORM_NT ? 8 : 4;
+  f32x2 acc[8][NJ];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) accf[i][j] = 0.f;
+    for (int j = 0; j < NJ; ++j) acc[i][j] = 0ull;
+  auto load = [&](int s) {                                  // by the issuing thread
+    const int st = s % FSTAGES, k = k0 + s * FK;
+    float* a = sm + st * FSTAGE_FLOATS;
+    float* b = a + FT * FK;
+    bar_expect(full + st, FSTAGE_FLOATS * 4);
+    if constexpr (FORM == FORM_TN) tensor_load(a, &map_a, m0, k, full + st); else tensor_load(a, &map_a, k, m0, full + st);
+    if constexpr (FORM == FORM_NT) tensor_load(b, &map_b, k, n0, full + st); else tensor_load(b, &map_b, n0, k, full + st);
+  };
+  constexpr bool COPY_WARP = ffma_threads(FORM) > FTHREADS;
+  if (!COPY_WARP && warp == 0) {
+    if (elect_one())
+      for (int s = 0; s < min(steps, FSTAGES); ++s) load(s);
   }
-  if (warp == 2 * FGROUPS) {
-    // ---------------- copies ----------------
-    if (elect_one()) {
+  if (COPY_WARP && warp == 2 * FGROUPS) {
+    if (elect_one())
       for (int s = 0; s < steps; ++s) {
-        const int st = s % FSTAGES, k = k0 + s * FK;
-        if (s >= FSTAGES) bar_wait(empty + st, (uint32_t)(s / FSTAGES - 1) & 1u, dev_status);
-        float* a = sm + st * FSTAGE_FLOATS;
-        float* b = a + FT * FK;
-        bar_expect(full + st, FSTAGE_FLOATS * 4);
-        if constexpr (FORM == FORM_TN) tensor_load(a, &map_a, m0, k, full + st); else tensor_load(a, &map_a, k, m0, full + st);
-        if constexpr (FORM == FORM_NT) tensor_load(b, &map_b, k, n0, full + st); else tensor_load(b, &map_b, n0, k, full + st);
+        if (s >= FSTAGES) bar_wait(empty + s % FSTAGES, (uint32_t)(s / FSTAGES - 1) & 1u, dev_status);
+        load(s);
       }
-    }
   } else {
-    // ---------------- arithmetic: this group's 8 of every stage's 32 k ----------------
+    // this group's 8 of every stage's 32 k
     for (int s = 0; s < steps; ++s) {
       const int st = s % FSTAGES;
       const float* a_s = sm + st * FSTAGE_FLOATS;
@@ -218,23 +225,19 @@ gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
       for (int h = 0; h < 2; ++h) {
         const int c = 2 * grp + h;                          // four k: c * 4 ..
         if constexpr (FORM == FORM_NT) {
-          // k-fast tiles: rows of 32 k, 128-byte swizzle (16-byte group c of row r at c ^ (r & 7)).  Plain FFMA: pairs along k would
-          // need twice the accumulators, more than the 168 registers nine warps leave a thread
-          float4 a[8];
+          // k-fast tiles: rows of 32 k, 128-byte swizzle (16-byte group c of row r at c ^ (r & 7)); a 16-byte load is two pairs
+          ulonglong2 a[8];
           const float* ar = a_s + ty * FK + ((c ^ ty) << 2);
           const float* br = b_s + tx * FK + ((c ^ tx) << 2);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) a[i] = lds4(ar + i * 8 * FK);
+          for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(ar + i * 8 * FK);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float4 b = lds4(br + j * 8 * FK);
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(br + j * 8 * FK);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              accf[i][j] = fmaf(a[i].x, b.x, accf[i][j]);
-              accf[i][j] = fmaf(a[i].y, b.y, accf[i][j]);
-              accf[i][j] = fmaf(a[i].z, b.z, accf[i][j]);
-              accf[i][j] = fmaf(a[i].w, b.w, accf[i][j]);
-            }
+            for (int i = 0; i < 8; ++i) fma2(acc[i][j], a[i].x, b.x);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) fma2(acc[i][j], a[i].y, b.y);
           }
         } else {
           // n-fast B: rows of 64 n; packed multiply-adds over pairs of columns 4 tx .. and 32 + 4 tx ..
@@ -272,17 +275,24 @@ gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         __syncwarp();
         if (lane == 0) bar_arrive(empty + st);
       }
+      if (!COPY_WARP && warp == 0 && s + FSTAGES < steps) {
+        if (elect_one()) { bar_wait(empty + st, (uint32_t)(s / FSTAGES) & 1u, dev_status); load(s + FSTAGES); }
+      }
     }
   }
   __syncthreads();                                          // the ring is free: partial tiles [group][64][72] take its place
-  if (warp < 2 * FGROUPS) {
+  if (!COPY_WARP || warp < 2 * FGROUPS) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int m = FORM == FORM_TN ? (i >> 2) * 32 + 4 * ty + (i & 3) : ty + 8 * i;
       float* d = sm + (grp * FT + m) * FPART;
       if constexpr (FORM == FORM_NT) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) d[tx + 8 * j] = accf[i][j];
+        for (int j = 0; j < 8; ++j) {
+          float lo, hi;
+          unpack2(acc[i][j], lo, hi);
+          d[tx + 8 * j] = lo + hi;
+        }
       } else {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -304,7 +314,7 @@ gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     return v;
   };
   if (S > 1) {
-    if (tid < 64 * FGROUPS) {
+    if (!COPY_WARP || tid < FTHREADS) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int row = (tid >> 4) + 16 * u, c = tid & 15, owner = row / slice;
@@ -315,7 +325,7 @@ gemm_ffma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     cluster_arrive_release();
     cluster_wait_acquire();
   }
-  if (tid >= 64 * FGROUPS) return;
+  if (COPY_WARP && tid >= FTHREADS) return;
   float* C = reinterpret_cast<float*>(e.C);
   const bool wide = (e.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0;
   const bool mask_wide = (e.ldmask & 3) == 0 && (reinterpret_cast<uintptr_t>(e.mask) & 15u) == 0;
@@ -399,7 +409,7 @@ cudaError_t launch_ffma(const CUtensorMap& ma, const CUtensorMap& mb, const Gemm
   e.C = g.C; e.ldc = g.ldc; e.ldmask = g.ldmask; e.c_round = g.c_round; e.epi = g.epi; e.relu = g.relu;
   e.bias = g.bias; e.mask = reinterpret_cast<const float*>(g.mask);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * S)); cfg.blockDim = dim3(FTHREADS); cfg.dynamicSmemBytes = FSMEM; cfg.stream = s;
+  cfg.gridDim = dim3((unsigned)(tiles * S)); cfg.blockDim = dim3(ffma_threads(FORM)); cfg.dynamicSmemBytes = FSMEM; cfg.stream = s;
   cudaLaunchAttribute attr[2];
   int n = 0;
   if (g_use_pdl) {

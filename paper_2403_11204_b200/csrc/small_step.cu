@@ -89,12 +89,15 @@ __device__ __forceinline__ void dot_chunk(float (&v)[VP], const float* A, int pa
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
     const float4 a = lds4(A + r * pa);
+    // component by component: the CT sums in between hide the latency of a multiply-add on the same sum
 #pragma unroll
-    for (int j = 0; j < CT; ++j) {
-      float t = v[r * CT + j];
-      t = fmaf(a.x, w[j].x, t); t = fmaf(a.y, w[j].y, t); t = fmaf(a.z, w[j].z, t); t = fmaf(a.w, w[j].w, t);
-      v[r * CT + j] = t;
-    }
+    for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.x, w[j].x, v[r * CT + j]);
+#pragma unroll
+    for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.y, w[j].y, v[r * CT + j]);
+#pragma unroll
+    for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.z, w[j].z, v[r * CT + j]);
+#pragma unroll
+    for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.w, w[j].w, v[r * CT + j]);
   }
 }
 template <int RT, int CT, int VP>
@@ -198,11 +201,13 @@ __device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float*
     for (int r = 0; r < RT; ++r) {
       const float4 a = lds4(A + r * pz + 4 * c);            // zero between N and the end of the chunk
 #pragma unroll
-      for (int j = 0; j < CT; ++j) {
-        float t = v[r * CT + j];
-        t = fmaf(a.x, w[0][j], t); t = fmaf(a.y, w[1][j], t); t = fmaf(a.z, w[2][j], t); t = fmaf(a.w, w[3][j], t);
-        v[r * CT + j] = t;
-      }
+      for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.x, w[0][j], v[r * CT + j]);
+#pragma unroll
+      for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.y, w[1][j], v[r * CT + j]);
+#pragma unroll
+      for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.z, w[2][j], v[r * CT + j]);
+#pragma unroll
+      for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.w, w[3][j], v[r * CT + j]);
     }
   };
   const int full = chunks >> 2;
