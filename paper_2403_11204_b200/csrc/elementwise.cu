@@ -195,7 +195,7 @@ update_kernel(UpdateArgs u, int bias_blocks, int bias_cols) {
     // small batches: 8 columns x 32 row lanes per block, so that the walk over the batch is only batch / 32
     // loads deep and these blocks finish inside the streaming part even when the layer is small;
     // large batches: 32 columns x 8 row lanes (whole 64- or 128-byte row segments per warp)
-    __shared__ float part[32][33];
+    __shared__ float part[256];
     const int cols = bias_cols, lanes = 256 / bias_cols;
     const int c = threadIdx.x % cols, rl = threadIdx.x / cols;
     const int col = blockIdx.x * cols + c;
@@ -211,11 +211,11 @@ update_kernel(UpdateArgs u, int bias_blocks, int bias_cols) {
         for (int b = rl; b < u.batch; b += lanes) acc += dz[(int64_t)b * u.ld_dz + col];
       }
     }
-    part[rl][c] = acc;
+    part[rl * cols + c] = acc;
     __syncthreads();
     if (rl == 0 && col < u.n_bias) {
       float g = 0.f;
-      for (int r = 0; r < lanes; ++r) g += part[r][c];
+      for (int r = 0; r < lanes; ++r) g += part[r * cols + c];
       const int64_t i = u.bias_off + col;
       u.g_bias[col] = g;
       float p = u.p[i], m = 0.f, v = 0.f;

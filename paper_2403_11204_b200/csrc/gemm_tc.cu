@@ -65,6 +65,7 @@ constexpr int A_TILE_BYTES = BLOCK_M * TILE_ROW_BYTES; // 16 KiB per stage
 constexpr int NUM_THREADS = 192;                       // TMA warp, MMA warp, four epilogue warps
 constexpr int UPDATE_WARPS = 8;                        // fused-update variants: eight more warps stream the optimizer update
 constexpr int NUM_THREADS_FUSED = NUM_THREADS + 32 * UPDATE_WARPS;
+constexpr int NUM_THREADS_PAIR = NUM_THREADS + 128;    // CTA-pair kernel: eight epilogue warps
 constexpr int SMEM_BUDGET = 192 * 1024;                // operand ring
 constexpr int SMEM_EXTRA = 2048;                       // alignment slack + barriers
 constexpr int HALF_SM_MAX_KB = 16;                     // k-blocks up to which the persistent kernel gives up ring depth for it
@@ -78,6 +79,7 @@ constexpr int HALF_SM_SMEM = 113 * 1024;               // two CTAs of this size 
 // old footprint the steps gain 1-3.5 %.
 constexpr int STAGE_OUT_WARP_BYTES = 32 * 64;          // one buffer of one warp
 constexpr int STAGE_OUT_BYTES = 4 * 2 * STAGE_OUT_WARP_BYTES;   // 16 KiB
+constexpr int PAIR_STAGE_OUT_BYTES = STAGE_OUT_BYTES;           // eight epilogue warps with one buffer each
 constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;
 
 // ---- PTX wrappers ------------------------------------------------------------------------------
@@ -154,6 +156,8 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
 }
 // at most one of this thread's bulk stores may still be reading its shared-memory source
 __device__ __forceinline__ void tma_store_wait_source_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+// none of them may
+__device__ __forceinline__ void tma_store_wait_source() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // all of this thread's bulk stores are complete
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
@@ -402,15 +406,16 @@ __device__ __forceinline__ void epilogue_store(const EpilogueArgs& e, float (&v)
 // piece j of row r at position j ^ ((r >> 1) & 3) - the 64-byte swizzle, which the output tensor map expects and which
 // makes the warp's stores conflict-free - and one bulk tensor store per buffer writes the 32-row box; rows and columns
 // beyond the matrix are clipped by the store.  Before a buffer is written, the store issued from it two stores earlier
-// has finished reading it (at most one store is left pending).
+// has finished reading it (at most one store is left pending).  With BUFS = 1 the warp has one buffer, drained before each use.
+template <int BUFS = 2>
 __device__ __forceinline__ void epilogue_store_staged(const EpilogueArgs& e, const CUtensorMap* map_c, uint8_t* warp_stage,
                                                       float (&v)[32], const EpiSide& s, int lane, int row0, int col0,
                                                       int n_total, int n_rows, int chunk) {
   epilogue_values(e, v, s, col0, n_total);
   const int x = (lane >> 1) & 3;
   if (e.c_dt == DT_BF16) {
-    uint8_t* buf = warp_stage + (chunk & 1) * STAGE_OUT_WARP_BYTES;
-    if (lane == 0) tma_store_wait_source_but_one();
+    uint8_t* buf = warp_stage + (BUFS == 2 ? (chunk & 1) * STAGE_OUT_WARP_BYTES : 0);
+    if (lane == 0) { if (BUFS == 2) tma_store_wait_source_but_one(); else tma_store_wait_source(); }
     __syncwarp();
     uint8_t* rowp = buf + lane * 64;
 #pragma unroll
@@ -431,8 +436,8 @@ __device__ __forceinline__ void epilogue_store_staged(const EpilogueArgs& e, con
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (col0 + 16 * h >= n_total) break;                              // uniform: nothing of this half is inside the matrix
-      uint8_t* buf = warp_stage + h * STAGE_OUT_WARP_BYTES;
-      if (lane == 0) tma_store_wait_source_but_one();
+      uint8_t* buf = warp_stage + (BUFS == 2 ? h * STAGE_OUT_WARP_BYTES : 0);
+      if (lane == 0) { if (BUFS == 2) tma_store_wait_source_but_one(); else tma_store_wait_source(); }
       __syncwarp();
       uint8_t* rowp = buf + lane * 64;
 #pragma unroll
@@ -1133,7 +1138,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-constexpr int PAIR_TILE_M = 256, PAIR_TILE_N = 256;
+constexpr int PAIR_TILE_M = 256, PAIR_TILE_N = 256;                   // columns: at most; a launch may take fewer
 constexpr int PAIR_HALF_N = PAIR_TILE_N / 2;
 constexpr int PAIR_B_BYTES = PAIR_HALF_N * TILE_ROW_BYTES;            // 16 KiB: this CTA's half of B
 constexpr int PAIR_STAGE_BYTES = A_TILE_BYTES + PAIR_B_BYTES;         // 32 KiB per CTA per k-block
@@ -1142,23 +1147,26 @@ constexpr int PAIR_STAGES_STAGED = 5;      // with it: ring + staging stay withi
 constexpr int PAIR_SMEM = PAIR_STAGES * PAIR_STAGE_BYTES + SMEM_EXTRA;   // upper bound of both layouts
 
 template <bool TF32, bool A_MN, bool B_MN, bool FUSED = false>
-__global__ void __launch_bounds__(FUSED ? NUM_THREADS_FUSED : NUM_THREADS, 1)
+__global__ void __launch_bounds__(FUSED ? NUM_THREADS_FUSED : NUM_THREADS_PAIR, 1)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                     const __grid_constant__ CUtensorMap map_c, int M, int N, int K, EpilogueArgs epi, int* dev_status,
-                    int group_m, int n_stages) {
+                    int group_m, int n_stages, int tile_n) {
   const int STAGES = n_stages;
+  const int half_n = tile_n >> 1;                      // columns of B each CTA of the pair stages
   constexpr int BLOCK_K = TF32 ? 32 : 64;
   constexpr int UMMA_K = TF32 ? 8 : 16;
   constexpr int CHUNK = TF32 ? 32 : 64;
   constexpr int MN_CHUNK_BYTES = BLOCK_K * TILE_ROW_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * PAIR_TILE_N;      // two 256-column accumulators per CTA
+  // Epilogue warps: two per quarter of the TMEM lanes, each taking every other 32-column chunk of the tile
+  constexpr int EPI_WARPS = FUSED ? 4 : 8, EPI_PER_QUARTER = EPI_WARPS / 4;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* smem_a = smem;
   uint8_t* smem_b = smem + STAGES * A_TILE_BYTES;
   uint8_t* stage_out = smem + STAGES * PAIR_STAGE_BYTES;               // 1024-byte aligned
-  uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + (epi.staged ? STAGE_OUT_BYTES : 0));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + (epi.staged ? PAIR_STAGE_OUT_BYTES : 0));
   // bars[0..S) full (used in the even CTA), [S..2S) empty, [2S..2S+2) tmem_full, [2S+2..2S+4) tmem_empty (even CTA)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -1177,7 +1185,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     prefetch_tensormap(&map_b);
     prefetch_tensormap(&map_c);
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 8); }   // 4 warps x 2 CTAs
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 2 * EPI_WARPS); }   // both CTAs
     *abort_flag = 0;
     *tiles_done = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1192,7 +1200,9 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
   // index arithmetic, the first tile's coordinates included: ahead of the dependency wait
   const int tiles_m = (M + PAIR_TILE_M - 1) / PAIR_TILE_M;
-  const int tiles_n = (N + PAIR_TILE_N - 1) / PAIR_TILE_N;
+  const int tiles_n = (N + tile_n - 1) / tile_n;
+  const int b_chunks = (half_n + CHUNK - 1) / CHUNK;   // MN-major B: whole 128-byte chunks are loaded
+  const uint32_t stage_tx = 2u * (uint32_t)(A_TILE_BYTES + (B_MN ? b_chunks * MN_CHUNK_BYTES : half_n * TILE_ROW_BYTES));
   const int n_tiles = tiles_m * tiles_n;
   const int num_k = (K + BLOCK_K - 1) / BLOCK_K;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
@@ -1211,11 +1221,11 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         int m_idx, n_idx;
         if (t == pair) { m_idx = first_m; n_idx = first_n; } else tile_coords(t, tiles_m, tiles_n, group_m, m_idx, n_idx);
         const int m0 = m_idx * PAIR_TILE_M + (int)rank * BLOCK_M;
-        const int n0 = n_idx * PAIR_TILE_N + (int)rank * PAIR_HALF_N;
+        const int n0 = n_idx * tile_n + (int)rank * half_n;
         for (int kb = 0; kb < num_k; ++kb) {
           if (fills < STAGES) ++fills;
           else if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, dev_status)) { ok = false; break; }
-          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), (uint32_t)(2 * PAIR_STAGE_BYTES));
+          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), stage_tx);
           const uint32_t fb = map_to_cta(full_bar(stage), 0);
           const uint32_t a_dst = smem_u32(smem_a + stage * A_TILE_BYTES);
           const uint32_t b_dst = smem_u32(smem_b + stage * PAIR_B_BYTES);
@@ -1228,8 +1238,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             tma_load_2d_pair(a_dst, &map_a, k0, m0, fb);
           }
           if constexpr (B_MN) {
-#pragma unroll
-            for (int c = 0; c < PAIR_HALF_N / CHUNK; ++c)
+            for (int c = 0; c < b_chunks; ++c)
               tma_load_2d_pair(b_dst + c * MN_CHUNK_BYTES, &map_b, n0 + c * CHUNK, k0, fb);
           } else {
             tma_load_2d_pair(b_dst, &map_b, k0, n0, fb);
@@ -1242,9 +1251,9 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // ---------------- MMA issuer: the even CTA only ----------------
     if (rank == 0 && elect_one()) {
       constexpr uint32_t fmt = TF32 ? 2u : 1u;
-      constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((A_MN ? 1u : 0u) << 15) |
-                                 ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(PAIR_TILE_N >> 3) << 17) |
-                                 ((uint32_t)(PAIR_TILE_M >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((A_MN ? 1u : 0u) << 15) |
+                             ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(tile_n >> 3) << 17) |
+                             ((uint32_t)(PAIR_TILE_M >> 4) << 24);
       constexpr uint32_t a_lbo = A_MN ? MN_CHUNK_BYTES : 16, b_lbo = B_MN ? MN_CHUNK_BYTES : 16;
       constexpr uint32_t a_kstep = A_MN ? UMMA_K * TILE_ROW_BYTES : 32;
       constexpr uint32_t b_kstep = B_MN ? UMMA_K * TILE_ROW_BYTES : 32;
@@ -1276,33 +1285,35 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
     }
-  } else if (warp < NUM_THREADS / 32) {
+  } else if (warp < 2 + EPI_WARPS) {
     // ---------------- epilogue warps: each CTA drains its own 128 rows ----------------
-    const int quarter = warp & 3;
+    const int quarter = warp & 3, part = (warp - 2) >> 2;    // (a warp reads the TMEM lanes of its index modulo 4)
+    uint8_t* my_stage_out = stage_out + (FUSED ? quarter * 2 : part * 4 + quarter) * STAGE_OUT_WARP_BYTES;
     int acc = 0; uint32_t acc_phase = 0;
     bool ok = true;
     for (int t = pair; t < n_tiles && ok; t += n_pairs) {
       int m_idx, n_idx;
       if (t == pair) { m_idx = first_m; n_idx = first_n; } else tile_coords(t, tiles_m, tiles_n, group_m, m_idx, n_idx);
       const int m0 = m_idx * PAIR_TILE_M + (int)rank * BLOCK_M;
-      const int n0 = n_idx * PAIR_TILE_N;
+      const int n0 = n_idx * tile_n, n_end = min(N, n0 + tile_n);
       const int row = m0 + quarter * 32 + lane;
       EpiSide side, side_next;
-      epilogue_prefetch(epi, side, row, row < M, n0, N);
+      epilogue_prefetch(epi, side, row, row < M, n0 + part * 32, N);
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, dev_status)) { ok = false; break; }
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < PAIR_TILE_N / 32; ++c) {
+      for (int c = part; c < PAIR_TILE_N / 32; c += EPI_PER_QUARTER) {
         const int col0 = n0 + c * 32;
-        if (col0 >= N) break;
-        if (c + 1 < PAIR_TILE_N / 32) epilogue_prefetch(epi, side_next, row, row < M, col0 + 32, N);
+        if (col0 >= n_end) break;
+        if (c + EPI_PER_QUARTER < PAIR_TILE_N / 32) epilogue_prefetch(epi, side_next, row, row < M, col0 + 32 * EPI_PER_QUARTER, N);
         float v[32];
         tmem_load_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * PAIR_TILE_N + c * 32), v);
-        if (FUSED || !epi.staged) {        // (the update warps read the tile back with ordinary loads: ordinary stores)
-          if (row < M) epilogue_store(epi, v, side, row, col0, N);
+        // per-lane stores: where the update warps read the tile back with ordinary loads, and for the half chunk at the end
+        // of a tile that is no multiple of 32 wide (a bf16 box of the bulk store has 32 columns)
+        if (FUSED || !epi.staged || (epi.c_dt == DT_BF16 && col0 + 32 > n_end && n_end < N)) {
+          if (row < M) epilogue_store(epi, v, side, row, col0, n_end);
         } else {
-          epilogue_store_staged(epi, &map_c, stage_out + quarter * 2 * STAGE_OUT_WARP_BYTES, v, side, lane,
-                                m0 + quarter * 32, col0, N, M, c);
+          epilogue_store_staged<FUSED ? 2 : 1>(epi, &map_c, my_stage_out, v, side, lane, m0 + quarter * 32, col0, n_end, M, c / EPI_PER_QUARTER);
         }
         side = side_next;
       }
@@ -1326,7 +1337,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         int m_idx, n_idx;
         if (t == pair) { m_idx = first_m; n_idx = first_n; } else tile_coords(t, tiles_m, tiles_n, group_m, m_idx, n_idx);
         const int m0 = m_idx * PAIR_TILE_M + (int)rank * BLOCK_M;
-        const int n0 = n_idx * PAIR_TILE_N;
+        const int n0 = n_idx * tile_n;          // (256 columns in this variant)
         update_tile<PAIR_TILE_N>(epi.upd, reinterpret_cast<const float*>(epi.C), epi.ldc, m0, n0, M, N, uw, lane,
                                  inv_bc1, inv_bc2);
       }
@@ -1384,6 +1395,7 @@ bool g_allow_splitk = true;
 bool g_allow_pairs = true;
 bool g_allow_fused_update = true;
 bool g_staged_epilogue = true;      // SEG_NO_STAGED_EPILOGUE: per-lane stores instead of shared-memory staging + bulk stores
+int g_pair_tile_n = PAIR_TILE_N;  // SEG_PAIR_TILE_N: columns of a pair's tile where SEG_PAIR_MIN_TILES forces pairs (a multiple of 16 up to 256)
 long g_pair_min_tiles = 0;      // SEG_PAIR_MIN_TILES: CTA pairs exactly from this many 256 x 256 tiles on (0: cost model)
 
 // 2-D tensor map over a row-major matrix: `inner` contiguous elements per row, `outer` rows,
@@ -1540,17 +1552,17 @@ int pick_split(int M, int N, int K, bool tf32) {
 
 template <bool TF32, bool A_MN, bool B_MN, bool FUSED = false>
 cudaError_t launch_pair_variant(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const GemmDesc& g,
-                                const EpilogueArgs& e, int* dev_status, cudaStream_t s) {
+                                const EpilogueArgs& e, int tile_n, int* dev_status, cudaStream_t s) {
   auto kern = gemm_tc_pair_kernel<TF32, A_MN, B_MN, FUSED>;
   static std::atomic<bool> attr_set_dev[kMaxDevices];      // the attribute is per device
   if (cudaError_t err = ensure_dynamic_smem(kern, PAIR_SMEM, attr_set_dev); err != cudaSuccess) return err;
-  const int tiles = ((g.M + PAIR_TILE_M - 1) / PAIR_TILE_M) * ((g.N + PAIR_TILE_N - 1) / PAIR_TILE_N);
+  const int tiles = ((g.M + PAIR_TILE_M - 1) / PAIR_TILE_M) * ((g.N + tile_n - 1) / tile_n);
   const int pairs = std::min(tiles, num_sms() / 2);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
-  cfg.blockDim = dim3(FUSED ? NUM_THREADS_FUSED : NUM_THREADS, 1, 1);
+  cfg.blockDim = dim3(FUSED ? NUM_THREADS_FUSED : NUM_THREADS_PAIR, 1, 1);
   const int n_stages = e.staged ? PAIR_STAGES_STAGED : PAIR_STAGES;
-  cfg.dynamicSmemBytes = n_stages * PAIR_STAGE_BYTES + (e.staged ? STAGE_OUT_BYTES : 0) + SMEM_EXTRA;
+  cfg.dynamicSmemBytes = n_stages * PAIR_STAGE_BYTES + (e.staged ? PAIR_STAGE_OUT_BYTES : 0) + SMEM_EXTRA;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1558,19 +1570,19 @@ cudaError_t launch_pair_variant(const CUtensorMap& ma, const CUtensorMap& mb, co
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
-  const int group_m = pick_group_m((g.M + PAIR_TILE_M - 1) / PAIR_TILE_M, (g.N + PAIR_TILE_N - 1) / PAIR_TILE_N, pairs,
-                                   PAIR_TILE_M, PAIR_TILE_N, g.K, TF32 ? 4 : 2);
-  return cudaLaunchKernelEx(&cfg, kern, ma, mb, mc, g.M, g.N, g.K, e, dev_status, group_m, n_stages);
+  const int group_m = pick_group_m((g.M + PAIR_TILE_M - 1) / PAIR_TILE_M, (g.N + tile_n - 1) / tile_n, pairs,
+                                   PAIR_TILE_M, tile_n, g.K, TF32 ? 4 : 2);
+  return cudaLaunchKernelEx(&cfg, kern, ma, mb, mc, g.M, g.N, g.K, e, dev_status, group_m, n_stages, tile_n);
 }
 
 template <bool TF32>
 cudaError_t launch_pair_majors(bool a_mn, bool b_mn, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc,
-                               const GemmDesc& g, const EpilogueArgs& e, int* dev_status, cudaStream_t s) {
-  if (!a_mn && !b_mn) return launch_pair_variant<TF32, false, false>(ma, mb, mc, g, e, dev_status, s);
-  if (!a_mn && b_mn) return launch_pair_variant<TF32, false, true>(ma, mb, mc, g, e, dev_status, s);
+                               const GemmDesc& g, const EpilogueArgs& e, int tile_n, int* dev_status, cudaStream_t s) {
+  if (!a_mn && !b_mn) return launch_pair_variant<TF32, false, false>(ma, mb, mc, g, e, tile_n, dev_status, s);
+  if (!a_mn && b_mn) return launch_pair_variant<TF32, false, true>(ma, mb, mc, g, e, tile_n, dev_status, s);
   if (a_mn && b_mn) {
-    if (e.upd.enabled) return launch_pair_variant<TF32, true, true, true>(ma, mb, mc, g, e, dev_status, s);
-    return launch_pair_variant<TF32, true, true>(ma, mb, mc, g, e, dev_status, s);
+    if (e.upd.enabled) return launch_pair_variant<TF32, true, true, true>(ma, mb, mc, g, e, tile_n, dev_status, s);
+    return launch_pair_variant<TF32, true, true>(ma, mb, mc, g, e, tile_n, dev_status, s);
   }
   return cudaErrorNotSupported;
 }
@@ -1608,9 +1620,15 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput) {
       us = rounds * t + (double)(2 * tiles) * t / num_sms();
     }
     if (g_pair_min_tiles > 0) {                            // diagnostic override: pairs from that many tiles on
-      if (tiles >= g_pair_min_tiles) best = Choice{1, PAIR_HALF_N, us};
+      if (tiles >= g_pair_min_tiles) best = Choice{1, g_pair_tile_n / 2, us};
     } else if (us < best.us) {
       best = Choice{1, PAIR_HALF_N, us};
+    }
+    // Fewer than half as many 256-column tiles as pairs: tiles of 128 columns give every pair one (a k-block takes 0.18 us instead
+    // of 0.30).  1024 x 2048 x 4096: 18.3 us against 25.8 with 256 columns and 19.6 with one CTA per 128 x 128 tile.
+    if (g_pair_min_tiles == 0 && !throughput && 2 * tiles <= pairs) {
+      const double us128 = num_k * 0.18 + 4.5;
+      if (us128 < best.us) best = Choice{1, PAIR_HALF_N / 2, us128};
     }
   }
   return best;
@@ -1634,6 +1652,8 @@ bool gemm_tc_init() {
     if (env && env[0] == '1') g_allow_pairs = false;
     env = getenv("SEG_PAIR_MIN_TILES");
     if (env) g_pair_min_tiles = atol(env);
+    env = getenv("SEG_PAIR_TILE_N");
+    if (env && atoi(env) >= 32 && atoi(env) <= PAIR_TILE_N && atoi(env) % 16 == 0) g_pair_tile_n = atoi(env);
     env = getenv("SEG_NO_STAGED_EPILOGUE");
     if (env && env[0] == '1') g_staged_epilogue = false;
     g_init_ok = true;
@@ -1768,8 +1788,8 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   }
   if (family) *family = pairs ? FAM_TC_PAIR : (split > 1 ? FAM_TC_SPLITK : FAM_TC_SINGLE);
   if (pairs) {
-    return tf32 ? launch_pair_majors<true>(a_mn, b_mn, ma, mb, mc, g, e, dev_status, s)
-                : launch_pair_majors<false>(a_mn, b_mn, ma, mb, mc, g, e, dev_status, s);
+    return tf32 ? launch_pair_majors<true>(a_mn, b_mn, ma, mb, mc, g, e, 2 * block_n, dev_status, s)
+                : launch_pair_majors<false>(a_mn, b_mn, ma, mb, mc, g, e, 2 * block_n, dev_status, s);
   }
   if (split > 1) {
     return tf32 ? launch_splitk_majors<true>(a_mn, b_mn, ma, mb, g, e, split, dev_status, s)

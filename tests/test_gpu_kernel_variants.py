@@ -32,6 +32,16 @@ def test_tensor_core_cases_with_forced_kernel_selection(env):
     assert res.returncode == 0, res.stdout[-3000:] + res.stderr[-1000:]
 
 
+@pytest.mark.parametrize("tile_n", ["32", "128", "208", "240"])
+def test_tensor_core_cases_with_narrower_pair_tiles(tile_n):
+    """CTA pairs on tiles of fewer than 256 columns: whole 128-byte chunks of B, a chunk of which only a part is used, and an output
+    chunk cut at the tile's edge inside the matrix."""
+    child_env = dict(os.environ, SEG_PAIR_MIN_TILES="1", SEG_PAIR_TILE_N=tile_n)
+    res = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_parity.py", "-m", "gpu", "-q", "-x",
+                          "-k", "tensor_core"], cwd=ROOT, env=child_env, capture_output=True, text=True, timeout=900)
+    assert res.returncode == 0, res.stdout[-3000:] + res.stderr[-1000:]
+
+
 @pytest.mark.parametrize("env", [{"SEG_NO_SMALL_FUSED": "1"}, {"SEG_NO_GRAPH": "1"}, {"SEG_NO_PDL": "1"}])
 def test_fp32_cases_with_switches(env):
     """The fp32 cases once more: launch by launch (no two-launch step for small segments), and the two-launch step
