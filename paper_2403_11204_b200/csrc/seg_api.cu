@@ -78,6 +78,8 @@ struct seg_handle {
   std::vector<void*> act;          // index 1..L
   std::vector<int64_t> ld_act;     // index 0..L
   std::vector<int> act_dtype;      // index 1..L
+  char* act_block = nullptr;       // x_stage, act[] and dzbuf[] live in this block
+  size_t act_block_bytes = 0;
   void* x_stage = nullptr;
   int32_t* cls_stage = nullptr;
   std::vector<void*> dzbuf;        // index 0..L-1
@@ -134,11 +136,7 @@ struct seg_handle {
   int32_t* host_cls = nullptr;
   float* host_loss = nullptr;      // page-locked host float the loss kernel writes (seg_train_step_host)
   float* host_loss_dev = nullptr;  // its device-side address
-  // seg_forward_dataset: rows per chunk (0: not yet chosen) and the chunk's buffers (two for hidden layers in turn, one for a
-  // staged input)
-  int dataset_rows = 0;
-  void* dataset_ws[2] = {nullptr, nullptr};
-  void* dataset_x = nullptr;
+  int dataset_rows[4] = {-1, -1, -1, -1};   // seg_forward_dataset: rows per chunk (-1: not yet chosen), see choose_dataset_rows
   // seg_train_step_host_async: copy stream, two device buffers for the batch in flight and the next one
   cudaStream_t copy_stream = nullptr;
   void* async_x[2] = {nullptr, nullptr};
@@ -508,22 +506,18 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
     h->ld_act[l] = round_up(h->widths[l] + (h->small_fused ? 1 : 0), 8);
   }
   if (h->is_final) h->act_dtype[h->n_layers] = DT_F32;
-  for (int l = 1; l <= h->n_layers; ++l) {
-    char* p = nullptr;
-    const size_t bytes = (size_t)h->max_batch * h->ld_act[l] * elem_size(h->act_dtype[l]);
-    if ((st = dev_alloc(h, &p, bytes, true)) != SEG_OK) return bail(st);
-    h->act[l] = p;
-  }
   {
-    char* p = nullptr;
-    if ((st = dev_alloc(h, &p, (size_t)h->max_batch * h->ld_act[0] * elem_size(h->act_dt), true)) != SEG_OK) return bail(st);
-    h->x_stage = p;
-  }
-  h->dzbuf.assign(h->n_layers, nullptr);
-  for (int l = 0; l < h->n_layers; ++l) {
-    char* p = nullptr;
-    if ((st = dev_alloc(h, &p, (size_t)h->max_batch * h->ld_act[l + 1] * elem_size(h->act_dt), true)) != SEG_OK) return bail(st);
-    h->dzbuf[l] = p;
+    // staged input, activations and dZ in one block: a long forward pass uses all of it for its chunks (seg_forward_dataset)
+    h->dzbuf.assign(h->n_layers, nullptr);
+    auto bytes = [&](int l, int dt) { return (size_t)round_up((int64_t)h->max_batch * h->ld_act[l] * (int64_t)elem_size(dt), 1024); };
+    size_t total = bytes(0, h->act_dt);
+    for (int l = 1; l <= h->n_layers; ++l) total += bytes(l, h->act_dtype[l]) + bytes(l, h->act_dt);
+    if ((st = dev_alloc(h, &h->act_block, total, true)) != SEG_OK) return bail(st);
+    h->act_block_bytes = total;
+    char* p = h->act_block;
+    h->x_stage = p; p += bytes(0, h->act_dt);
+    for (int l = 1; l <= h->n_layers; ++l) { h->act[l] = p; p += bytes(l, h->act_dtype[l]); }
+    for (int l = 0; l < h->n_layers; ++l) { h->dzbuf[l] = p; p += bytes(l + 1, h->act_dt); }
   }
   if ((st = dev_alloc(h, &h->cls_stage, h->max_batch, true)) != SEG_OK) return bail(st);
   if ((st = dev_alloc(h, &h->loss_slot, 1, true)) != SEG_OK) return bail(st);
@@ -1053,49 +1047,62 @@ static bool rows_aligned(const void* p, int width, size_t esz) {
   return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (width * esz) % 16 == 0;
 }
 
-// Rows per chunk of a long forward pass: a response does not depend on how its rows are grouped, and products over the
-// training batch alone often leave half of the SMs without a tile in their last round (1024 x 2048 outputs: 32 tiles of
-// 256 x 256 on 74 CTA pairs).  The multiple of 256 with the smallest estimated time per row; at most 8192 rows and 128 MB a buffer.
-static int choose_dataset_rows(const seg_handle* h) {
-  int64_t widest = 1;
-  for (int l = 0; l <= h->n_layers; ++l) widest = std::max(widest, h->ld_act[l]);
-  const int64_t most = std::min<int64_t>(8192, (128ll << 20) / (widest * 4));
-  int best = 0;
-  double best_us = 1e30;
-  for (int rows = 256; rows <= most; rows += 256) {
-    double us = 0;
-    for (const LayerInfo& L : h->layers)
-      us += h->use_tc ? gemm_tc_estimate_us(rows, L.out, L.in, h->precision == SEG_TF32)
-                      : 3.0 + ffma_estimate_us(rows, L.out, L.in);
-    if (us / rows < best_us * 0.99) { best_us = us / rows; best = rows; }
-  }
-  return best;
+// A chunk of a long forward pass: the outputs of its hidden layers take turns in two buffers, a staged input and an output the
+// products cannot write into the caller's buffer have one each, all inside the handle's block of training buffers (a training
+// step or an ordinary forward pass writes every one of them before it reads it).
+struct ChunkPlan { bool staged, direct; int rows; size_t buf[2], out, total; };   // bytes per row of each buffer
+static ChunkPlan chunk_plan(const seg_handle* h, bool staged, bool direct) {
+  ChunkPlan c{staged, direct, 0, {0, 0}, 0, 0};
+  const int L = h->n_layers;
+  for (int l = 0; l + 1 < L; ++l) c.buf[l & 1] = std::max<size_t>(c.buf[l & 1], h->ld_act[l + 1] * elem_size(h->act_dtype[l + 1]));
+  if (!direct) c.out = h->ld_act[L] * elem_size(h->act_dtype[L]);
+  c.total = c.buf[0] + c.buf[1] + c.out + (staged ? h->ld_act[0] * elem_size(h->act_dt) : 0);
+  return c;
 }
 
-// Forward pass of `rows` rows through the chunk buffers, the last layer's output into y.
-static seg_status forward_chunk(seg_handle* h, const void* x, int rows, void* y) {
+// Rows per chunk: a response does not depend on how its rows are grouped, and products over the training batch alone often
+// leave half of the SMs without a tile in their last round (1024 x 2048 outputs: 32 tiles of 256 x 256 on 74 CTA pairs).  The
+// multiple of 256 with the smallest estimated time per row that fits the block, 8192 at most; 0: not even 256 rows fit.
+static int choose_dataset_rows(seg_handle* h, const ChunkPlan& c) {
+  int& rows = h->dataset_rows[(c.staged ? 2 : 0) + (c.direct ? 1 : 0)];
+  if (rows >= 0) return rows;
+  const int64_t most = c.total == 0 ? 8192 : std::min<int64_t>(8192, (int64_t)(h->act_block_bytes / c.total));
+  rows = 0;
+  double best_us = 1e30;
+  for (int r = 256; r <= most; r += 256) {
+    double us = 0;
+    for (const LayerInfo& L : h->layers)
+      us += h->use_tc ? gemm_tc_estimate_us(r, L.out, L.in, h->precision == SEG_TF32) : 3.0 + ffma_estimate_us(r, L.out, L.in);
+    if (us / r < best_us * 0.99) { best_us = us / r; rows = r; }
+  }
+  return rows;
+}
+
+// Forward pass of `rows` rows in the chunk buffers, the last layer's output into y.  The buffers are sized for `most` rows.
+static seg_status forward_chunk(seg_handle* h, const ChunkPlan& c, int most, const void* x, int rows, void* y) {
   const int L = h->n_layers;
-  const size_t esz = elem_size(h->act_dt), osz = elem_size(h->act_dtype[L]);
+  char* buf[2] = {h->act_block, h->act_block + (size_t)most * c.buf[0]};
+  char* out = buf[1] + (size_t)most * c.buf[1];
+  char* xs = out + (size_t)most * c.out;
   const void* a = x;
   int64_t ld = h->widths[0];
-  bool early = false;
-  if (h->precision == SEG_TF32 || !rows_aligned(x, h->widths[0], esz)) {
+  if (c.staged) {
     Launch l(h, K_COPY);
-    SEG_TRY(h, launch_copy2d(h->dataset_x, h->act_dt, h->ld_act[0], x, h->act_dt, h->widths[0], rows, h->widths[0], h->act_round,
-                             h->stream), "input staging");
-    a = h->dataset_x; ld = h->ld_act[0]; early = true;
+    SEG_TRY(h, launch_copy2d(xs, h->act_dt, h->ld_act[0], x, h->act_dt, h->widths[0], rows, h->widths[0], h->act_round, h->stream),
+            "input staging");
+    a = xs; ld = h->ld_act[0];
   }
-  const bool direct = rows_aligned(y, h->widths[L], osz);
   for (int l = 0; l < L; ++l) {
     GemmDesc g = forward_desc(h, l, a, ld, rows);
-    if (l == L - 1 && direct) { g.C = y; g.ldc = h->widths[L]; }
-    else g.C = h->dataset_ws[l & 1];
-    g.b_early = (l > 0 || early) ? 1 : 0;
+    if (l < L - 1) g.C = buf[l & 1];
+    else if (c.direct) { g.C = y; g.ldc = h->widths[L]; }
+    else g.C = out;
+    g.b_early = (l > 0 || c.staged) ? 1 : 0;
     seg_status st = run_gemm(h, g, K_FWD, h->stream);
     if (st != SEG_OK) return st;
     a = g.C; ld = g.ldc;
   }
-  if (direct) return SEG_OK;
+  if (c.direct) return SEG_OK;
   Launch l(h, K_COPY);
   SEG_TRY(h, launch_copy2d(y, h->act_dtype[L], h->widths[L], a, h->act_dtype[L], ld, rows, h->widths[L], RND_NONE, h->stream), "output copy");
   return SEG_OK;
@@ -1126,25 +1133,19 @@ seg_status seg_forward_dataset(seg_handle* h, const void* x, int64_t n, int32_t 
       done += rows;
     }
   } else if (head > batch) {
-    if (h->dataset_rows == 0) {
-      const int rows = choose_dataset_rows(h);
-      int64_t widest = 0;
-      for (int l = 1; l <= h->n_layers; ++l) widest = std::max<int64_t>(widest, h->ld_act[l] * elem_size(h->act_dtype[l]));
-      char *b0 = nullptr, *b1 = nullptr, *bx = nullptr;
-      seg_status st;
-      if ((st = dev_alloc(h, &b0, (size_t)(rows * widest), false)) != SEG_OK || (st = dev_alloc(h, &b1, (size_t)(rows * widest), false)) != SEG_OK ||
-          (st = dev_alloc(h, &bx, (size_t)rows * h->ld_act[0] * elem_size(h->act_dt), true)) != SEG_OK) return st;
-      h->dataset_ws[0] = b0; h->dataset_ws[1] = b1; h->dataset_x = bx;
-      h->dataset_rows = rows;
-    }
-    // equal chunks of at most dataset_rows rows, whole 256-row tiles each
-    const int64_t chunks = (head + h->dataset_rows - 1) / h->dataset_rows;
-    const int64_t rows = std::min<int64_t>(h->dataset_rows, round_up((head + chunks - 1) / chunks, 256));
-    while (done < head) {
-      const int b = (int)std::min<int64_t>(rows, head - done);
-      seg_status st = forward_chunk(h, xr(done), b, yr(done));
-      if (st != SEG_OK) return st;
-      done += b;
+    const bool staged = h->precision == SEG_TF32 || !rows_aligned(x, h->widths[0], elem_size(h->act_dt));
+    const ChunkPlan c = chunk_plan(h, staged, rows_aligned(y, h->widths[h->n_layers], elem_size(h->act_dtype[h->n_layers])));
+    const int most = choose_dataset_rows(h, c);
+    if (most > batch) {
+      // equal chunks of at most that many rows, whole 256-row tiles each
+      const int64_t chunks = (head + most - 1) / most;
+      const int64_t rows = std::min<int64_t>(most, round_up((head + chunks - 1) / chunks, 256));
+      while (done < head) {
+        const int b = (int)std::min<int64_t>(rows, head - done);
+        seg_status st = forward_chunk(h, c, most, xr(done), b, yr(done));
+        if (st != SEG_OK) return st;
+        done += b;
+      }
     }
   }
   for (int64_t i = done; i < n; i += batch) {

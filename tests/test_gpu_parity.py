@@ -551,3 +551,23 @@ def test_small_segment_shapes(widths, final, batch):
     x2, cls2 = batch_arrays(w, batch, widths[0], seed=3)
     compare_step(gpu, ora, x2, cls2, "fp32", TOL["fp32"])
     gpu.close()
+
+
+@pytest.mark.parametrize("widths,final,precision,tol", [([784, 320, 200, 72], False, "bf16", 2e-2), ([72, 136, 264, 47], True, "bf16", 2e-2),
+                                                        ([100, 320, 200, 72], False, "tf32", 2e-3), ([200, 160, 96], False, "fp32", 1e-4),
+                                                        ([90, 160, 47], True, "fp32", 1e-4), ([33, 60, 47], True, "fp32", 1e-4)])
+def test_response_over_a_set_in_larger_chunks(widths, final, precision, tol):
+    """seg_forward_dataset groups rows as the GPU likes them: every row must match the oracle's response, the last partial
+    batch's activations stay readable, and a training step afterwards is the oracle's."""
+    w = wl.WORKLOADS["tiny"]
+    batch, n = 192, 1500
+    gpu, ora = make_pair(widths, 47, final, precision, "sgd", 0.01, batch)
+    x, cls = batch_arrays(w, n, widths[0], precision=precision)
+    xt, _ = to_device(x, cls, precision)
+    y = gpu.forward_dataset(xt, batch)
+    gpu.poll()
+    ref = ora.forward(x)[-1]
+    assert rel_err(y.float().cpu().numpy(), ref) < tol
+    assert rel_err(gpu.activation(len(widths) - 1).cpu().numpy(), ref[n - n % batch:]) < tol
+    compare_step(gpu, ora, x[:batch], cls[:batch], precision, tol)
+    gpu.close()
