@@ -592,11 +592,11 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
       ++h->launches;
       if (launch_small_ones(p.act[l], p.ld_act[l], p.widths[l], h->max_batch, h->stream) != cudaSuccess) return bail(SEG_ERR_CUDA);
     }
-    CUtensorMap maps[4 * kSmallMaxLayers];
+    CUtensorMap maps[3 * kSmallMaxLayers];
     CUtensorMap* dev_maps = nullptr;
     if (!small_step_maps(p, h->max_batch, maps)) return bail(SEG_ERR_CUDA);
-    if ((st = dev_alloc(h, &dev_maps, 4 * kSmallMaxLayers, false)) != SEG_OK) return bail(st);
-    if (cudaMemcpyAsync(dev_maps, maps, sizeof(CUtensorMap) * 4 * h->n_layers, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+    if ((st = dev_alloc(h, &dev_maps, 3 * kSmallMaxLayers, false)) != SEG_OK) return bail(st);
+    if (cudaMemcpyAsync(dev_maps, maps, sizeof(CUtensorMap) * 3 * h->n_layers, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
       return bail(SEG_ERR_CUDA);
     p.maps = dev_maps;
   }

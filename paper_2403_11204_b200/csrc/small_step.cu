@@ -16,7 +16,7 @@
 //      order: bit-reproducible).  Activations, dZ and the staged input also go to global memory for the second
 //      kernel.  Forward-only calls (seg_forward) run the same kernel up to the last layer's output.
 //   2. small_wgrad_update_kernel: tiles of (all outputs) x NT inputs of dW_l = dZ_l^T [A_{l-1} | 1] for all layers
-//      in one grid; a cluster of S CTAs splits the batch of one tile, tensor copies bring 32 rows of both operands
+//      in one grid; a cluster of S CTAs splits the batch of one tile, tensor copies bring 64 rows of both operands
 //      per stage, threads hold 8 x NT/8 register tiles, the partial tiles are combined as a reduce-scatter through
 //      distributed shared memory (fixed order), and every CTA applies the optimizer to the rows it received.  The
 //      column of ones, which yields the bias gradient, is kept in the padding of the activation buffers.
@@ -578,7 +578,7 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
 }
 
 // ---- weight gradients of all layers, bias gradients and the update ---------------------------------
-constexpr int WK = 32, W_STAGES = 6;                        // batch rows per stage, stages at most
+constexpr int WBOX = 32, WK = 64, W_STAGES = 3;             // batch rows per tensor copy and per stage, stages at most
 
 __host__ __device__ inline int wgrad_tiles(int in, int nt) { return (in + 1 + nt - 1) / nt; }
 
@@ -613,15 +613,18 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
   float* ringA = sm;                                        // [stage][WK][MT]
   float* ringB = sm + stages * WK * MT;                     // [stage][WK][NT]
   float* recv = sm + wgrad_ring_floats(MT, NT, stages);     // [source CTA][MT / S rows][NT]
-  const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(p.maps) + 4 * l;
+  const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(p.maps) + 3 * l;
   const CUtensorMap* map_a = maps;                          // (m = o, k = b) at dz[b * ld + o]
-  const CUtensorMap* map_b = maps + (NT == 64 ? 1 : NT == 32 ? 2 : 3);   // (k = b, n = i) at act[b * ld + i]; column `in` holds ones
-  const uint32_t stage_bytes = (uint32_t)(WK * (MT + NT) * 4);
+  const CUtensorMap* map_b = maps + (NT == 32 ? 1 : 2);   // (k = b, n = i) at act[b * ld + i]; column `in` holds ones
+  const uint32_t box_bytes = (uint32_t)(WBOX * (MT + NT) * 4);
   auto load = [&](int step) {                               // by the issuing thread
-    const int s = step % stages;
-    bar_expect(full + s, stage_bytes);
-    tensor_load(ringA + s * WK * MT, map_a, 0, k_begin + step * WK, full + s);
-    tensor_load(ringB + s * WK * NT, map_b, n0, k_begin + step * WK, full + s);
+    const int s = step % stages, boxes = min(WK / WBOX, (rows - step * WK + WBOX - 1) / WBOX);
+    bar_expect(full + s, (uint32_t)boxes * box_bytes);
+    for (int b = 0; b < boxes; ++b) {
+      const int r = b * WBOX;
+      tensor_load(ringA + (s * WK + r) * MT, map_a, 0, k_begin + step * WK + r, full + s);
+      tensor_load(ringB + (s * WK + r) * NT, map_b, n0, k_begin + step * WK + r, full + s);
+    }
   };
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) { bar_init(full + i, 1); bar_init(empty + i, SS_WARPS); }
@@ -640,11 +643,11 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
   if (blockIdx.x == 0)
     for (int i = tid; i < n_partials; i += SS_THREADS) lpart += p.loss_partials[i];
 
-  float acc[8][CN];
+  uint64_t acc2[4][CN];                                     // rows 2i and 2i + 1
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < CN; ++j) acc2[i][j] = 0;
   for (int step = 0; step < steps; ++step) {
     const int s = step % stages;
     bar_wait(full + s, (uint32_t)(step / stages) & 1u, p.dev_status);
@@ -654,13 +657,10 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
       const float* b_s = ringB + (s * WK + grp) * NT + (CN == 2 ? 2 : 4) * tx;
 #pragma unroll 4
       for (int k = grp; k < kmax; k += G, a_s += G * MT, b_s += G * NT) {
-        const float4 a0 = lds4(a_s), a1 = lds4(a_s + 4);
-        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(a_s), a1 = *reinterpret_cast<const ulonglong2*>(a_s + 4);
+        const uint64_t a[4] = {a0.x, a0.y, a1.x, a1.y};
         float b[CN];
-        if constexpr (CN == 8) {
-          const float4 b0 = lds4(b_s), b1 = lds4(b_s + 32);
-          b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
-        } else if constexpr (CN == 4) {
+        if constexpr (CN == 4) {
           const float4 b0 = lds4(b_s);
           b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
         } else {
@@ -668,9 +668,12 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
           b[0] = b0.x; b[1] = b0.y;
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int j = 0; j < CN; ++j) {
+          uint64_t bb;
+          asm("mov.b64 %0, {%1, %1};" : "=l"(bb) : "f"(b[j]));
 #pragma unroll
-          for (int j = 0; j < CN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+          for (int i = 0; i < 4; ++i) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[i][j]) : "l"(a[i]), "l"(bb));
+        }
       }
     }
     if (step + stages < steps) {                            // the stage is needed again
@@ -684,15 +687,18 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
       }
     }
   }
+  float acc[8][CN];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < CN; ++j)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[2 * i][j]), "=f"(acc[2 * i + 1][j]) : "l"(acc2[i][j]));
   __syncthreads();                                          // the ring is free: partial tiles [group][MT][NT] take its place
   if (grp < G) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       float* d = sm + (grp * MT + ty * 8 + i) * NT;
-      if constexpr (CN == 8) {
-        *reinterpret_cast<float4*>(d + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        *reinterpret_cast<float4*>(d + 32 + 4 * tx) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
-      } else if constexpr (CN == 4) {
+      if constexpr (CN == 4) {
         *reinterpret_cast<float4*>(d + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
       } else {
         *reinterpret_cast<float2*>(d + 2 * tx) = make_float2(acc[i][0], acc[i][1]);
@@ -807,6 +813,8 @@ __global__ void small_ones_kernel(float* a, int64_t ld, int col, int rows) {
 // Clusters of C CTAs the GPU runs at once with one CTA per SM (cudaOccupancyMaxActiveClusters on a B200: 148, 74, 33, 15 - a
 // cluster lives inside one GPC, and what a GPC has beyond a multiple of C stays idle).
 int resident_clusters(int C) { return C == 1 ? 148 : C == 2 ? 74 : C == 4 ? 33 : 15; }
+// The same with two CTAs per SM.
+int resident_clusters_2(int C) { return C == 1 ? 296 : C == 2 ? 148 : C == 4 ? 71 : 33; }
 
 constexpr int kRowChoices[] = {1, 2, 4, 6, 8, 10, 12, 16};
 int split_columns(int N1) { return N1 <= 32 ? 2 : N1 <= 64 ? 4 : N1 <= 80 ? 5 : 8; }   // columns per lane in the split first layer
@@ -967,20 +975,26 @@ size_t wgrad_smem_bytes(const SmallStep& p, int nt, int stages) {
   return b;
 }
 
-// Tile width and batch split of the second kernel with the smallest estimate: a wave of CTAs costs its fixed latencies once
-// per CTA an SM has to run, its arithmetic at the rate the register tile reaches (8 x 8 best, 8 x 2 bound by shared-memory loads).
+// Tile width and batch split of the second kernel with the smallest estimate: a wave of CTAs costs its fixed latencies, its
+// arithmetic at the rate the register tile reaches (8 x 2 bound by shared-memory loads, 8 x 4 by FFMA issue) and the exchange.
+// The constants follow from timing all splits of six networks at 64 to 1410 rows: at most 6 % off the best of them, most
+// exactly it.  Eight warps per SM are bound by latency, so a grid of two CTAs per SM wins although each redoes the fixed part:
+// 784-80-60 at 1410 rows 28.2 us per step with 32 columns x 8 CTAs (224 CTAs), 29.8 with 64 x 8 (120), which also lost
+// everywhere else and is not built.
 void plan_wgrad(SmallPrepared* w) {
   const SmallStep& p = w->a.p;
   double best_t = 1e30;
-  for (int nt : {64, 32, 16}) {
+  for (int nt : {32, 16}) {
     int tiles = 0, mt = 8;
     for (int l = 0; l < p.n_layers; ++l) { tiles += wgrad_tiles(p.widths[l], nt); mt = std::max(mt, up(p.widths[l + 1], 8)); }
-    const double rate = nt == 64 ? 90.0 : nt == 32 ? 80.0 : 60.0;      // multiply-adds per cycle and SM
     for (int S : {1, 2, 4, 8}) {
       if (S > 1 && p.batch < 8 * S) continue;
       const int rows = (p.batch + S - 1) / S;
-      const int load = (tiles + resident_clusters(S) - 1) / resident_clusters(S);
-      const double t = (S > 1 ? 1500.0 : 500.0) + load * (1500.0 + rows * (double)mt * nt / rate + mt * nt / 8.0 * (1.0 + 1.0 / S));
+      const bool pairs = tiles > resident_clusters(S);               // two CTAs share an SM
+      const int waves = pairs ? (tiles + resident_clusters_2(S) - 1) / resident_clusters_2(S) : 1;
+      const double rate = pairs ? (nt == 32 ? 61.5 : 50.5) : (nt == 32 ? 87.0 : 65.0);   // multiply-adds per cycle and CTA
+      const double exchange = S == 1 ? 500.0 : S == 2 ? 450.0 : S == 4 ? 950.0 : 1500.0;
+      const double t = exchange + waves * (700.0 + rows * (double)mt * nt / rate + mt * nt / 12.0 * (1.0 + 1.0 / S));
       if (t < best_t) { best_t = t; w->nt = nt; w->S = S; w->tiles = tiles; w->rows = rows; }
     }
   }
@@ -1003,7 +1017,6 @@ cudaError_t launch_wgrad(SmallPrepared& w, cudaStream_t s) {
 
 template <int OPT>
 cudaError_t launch_wgrad(SmallPrepared& w, cudaStream_t s) {
-  if (w.nt == 64) return launch_wgrad<OPT, 64>(w, s);
   if (w.nt == 32) return launch_wgrad<OPT, 32>(w, s);
   return launch_wgrad<OPT, 16>(w, s);
 }
@@ -1044,12 +1057,12 @@ bool small_can_train(const SmallPrepared& w) { return chain_grid(w.a.p, w.a.q) <
 
 bool small_step_maps(const SmallStep& p, int max_batch, CUtensorMap* maps) {
   for (int l = 0; l < p.n_layers; ++l) {
-    CUtensorMap* m = maps + 4 * l;
+    CUtensorMap* m = maps + 3 * l;
     const uint32_t mt = (uint32_t)up(p.widths[l + 1], 8);
-    if (!make_map_f32(m, p.dz[l], mt, (uint64_t)max_batch, (uint64_t)p.ld_act[l + 1] * 4, mt, WK)) return false;
-    const uint32_t nts[3] = {64, 32, 16};
-    for (int i = 0; i < 3; ++i)
-      if (!make_map_f32(m + 1 + i, p.act[l], (uint64_t)p.widths[l] + 1, (uint64_t)max_batch, (uint64_t)p.ld_act[l] * 4, nts[i], WK)) return false;
+    if (!make_map_f32(m, p.dz[l], mt, (uint64_t)max_batch, (uint64_t)p.ld_act[l + 1] * 4, mt, WBOX)) return false;
+    const uint32_t nts[2] = {32, 16};
+    for (int i = 0; i < 2; ++i)
+      if (!make_map_f32(m + 1 + i, p.act[l], (uint64_t)p.widths[l] + 1, (uint64_t)max_batch, (uint64_t)p.ld_act[l] * 4, nts[i], WBOX)) return false;
   }
   return true;
 }

@@ -535,7 +535,7 @@ def test_default_stream_step_is_captured_and_replayed(widths, precision, batch):
 
 @pytest.mark.parametrize("widths,final", [([784, 128, 128, 128, 47], True), ([1024, 128, 128, 128, 128], False),
                                           ([128, 128, 128, 128, 128], False), ([129, 1, 47], True), ([300, 81, 33], False),
-                                          ([513, 97, 128, 5], False), ([260, 17, 128], False), ([1, 1], False)])
+                                          ([513, 97, 128, 5], False), ([260, 17, 128], False), ([784, 80, 60], False), ([1, 1], False)])
 @pytest.mark.parametrize("batch", [1, 7, 200, 1411])
 def test_small_segment_shapes(widths, final, batch):
     """Edges of the two-launch step: weights that pass through two slots or wait for the first layer's tiles, first layers
