@@ -133,7 +133,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // those instructions take their operands from uniform registers, and only behind elect.sync does the compiler know that one
 // thread is active and issue them directly; behind `lane == 0` it wraps each in a loop over the active threads.  Measured:
 // eight expect-and-copy pairs are issued in 92 cycles against 474; 1024-row responses of 784-4096-4096-2048 take 2561 us
-// against 2782 (33 chunks), a step of 512-1024-768-512 (bf16, batch 512) 54.3 us against 61.2.
+// against 2782 (33 chunks), a step of 512-1024-768-512 (bf16, batch 512) 54.3 us against 61.2, and the split-K kernel's
+// three sends to its peers bring a step of 784-1024-1024-512 (TF32, batch 256) from 57.5 to 56.8.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
@@ -1051,12 +1052,14 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the bulk copies
       cluster_wait();                                                // every peer's receive barrier exists
       asm volatile("bar.sync 1, 128;" ::: "memory");                 // the four epilogue warps
-      if (warp == 2 && lane == 0) {
-        for (uint32_t dest = 0; dest < (uint32_t)split; ++dest) {
-          if (dest == rank) continue;
-          const uint32_t src = smem_u32(send + (int)dest * w * BLOCK_M);
-          const uint32_t dst = map_to_cta(smem_u32(recv + (int)rank * w * BLOCK_M), dest);
-          bulk_copy_to_peer(dst, src, slice_bytes, map_to_cta(recv_bar, dest));
+      if (warp == 2) {
+        if (elect_one()) {
+          for (uint32_t d = 1; d < (uint32_t)split; ++d) {
+            const uint32_t dest = (rank + d) & (uint32_t)(split - 1);
+            const uint32_t src = smem_u32(send + (int)dest * w * BLOCK_M);
+            const uint32_t dst = map_to_cta(smem_u32(recv + (int)rank * w * BLOCK_M), dest);
+            bulk_copy_to_peer(dst, src, slice_bytes, map_to_cta(recv_bar, dest));
+          }
         }
       }
       ok = mbar_wait(recv_bar, 0, abort_flag, dev_status);
