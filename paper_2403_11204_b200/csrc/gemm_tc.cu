@@ -6,10 +6,10 @@
 //   wgrad    C = dZ^T A    : both operands MN-major (contraction over the batch)
 // with bf16 operands (kind::f16) or TF32 operands (kind::tf32) and fp32 accumulation in TMEM.
 //
-// CTA = 6 warps.  Warp 0 lane 0 issues TMA loads into a ring of shared-memory stages; warp 1 owns
-// the TMEM allocation and its lane 0 issues the MMAs; warps 2..5 drain the accumulator (each warp
-// reads its own 32 TMEM lanes), apply the epilogue and store.  Two accumulator buffers in TMEM let
-// the epilogue of tile i overlap the main loop of tile i+1.
+// CTA = 6 warps (10 in the CTA-pair kernel).  A thread of warp 0 issues TMA loads into a ring of
+// shared-memory stages; warp 1 owns the TMEM allocation and one of its threads issues the MMAs; the other
+// four (eight) warps drain the accumulator (a warp reads its own 32 TMEM lanes), apply the epilogue and
+// store.  Two accumulator buffers in TMEM let the epilogue of tile i overlap the main loop of tile i+1.
 //
 // Shared-memory operand tiles use the 128-byte swizzle.  K-major tile: rows of 128 bytes (64 bf16
 // or 32 TF32 along K), 8-row groups 1024 bytes apart.  MN-major tile: chunks of 64 bf16 / 32 TF32
@@ -19,11 +19,12 @@
 // 32-byte atoms (4-row groups 512 bytes apart), in the tensor map and in the descriptor alike.
 //
 // Small problems (few output tiles, long K) use gemm_tc_splitk_kernel instead: a thread-block
-// cluster of 2, 4 or 8 CTAs shares one 128 x 64 output tile, each CTA contracts its own slice of K
+// cluster of 2 or 4 CTAs shares one 128 x 64 output tile, each CTA contracts its own slice of K
 // into TMEM, and the partial tiles are combined through distributed shared memory as a
 // reduce-scatter (every CTA bulk-copies column slice j of its partial into CTA j's shared memory;
-// CTA j adds what it received and runs the epilogue on that slice).  One SM's shared-memory fill rate bounds a single CTA's main loop, so spreading K over a
-// cluster shortens exactly the part of the kernel that grows with the problem.
+// CTA j adds what it received and runs the epilogue on that slice).  One SM's shared-memory fill rate
+// bounds a single CTA's main loop, so spreading K over a cluster shortens exactly the part of the
+// kernel that grows with the problem.
 //
 // Large problems use gemm_tc_pair_kernel: two CTAs of a cluster share one 256 x 256 output tile
 // through tcgen05.mma.cta_group::2.  Each CTA stages its own 128 rows of A and its own 128 columns

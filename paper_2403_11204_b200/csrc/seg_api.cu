@@ -4,11 +4,14 @@
 // Device memory layout of a handle
 //   params / grads / state1 / state2 : one flat fp32 range each, identical layout
 //       [W_0 | b_0 | W_1 | b_1 | ...], every tensor starting on a 256-byte boundary, W_l stored
-//       [out][ldw] with ldw = in rounded up to 8 elements (16-byte rows for TMA); padding stays 0.
+//       [out][ldw] with ldw = in rounded up to 8 elements (16-byte rows for TMA; small fp32 segments:
+//       small_weight_pitch(in), whose rows also stay clear of each other's banks); padding stays 0.
 //   params_op : the same layout in the operand dtype (bf16, or TF32-rounded fp32).
 //   act[l], l = 1..L : [max_batch][ld_l] stored outputs (bf16 or fp32; final logits fp32).
 //   dzbuf[l]         : dZ of layer l, [max_batch][ld_{l+1}] (one per layer: the weight-gradient
 //                      branch reads dZ_l while the main branch already produces dZ_{l-1}).
+//   act, dzbuf and the staged input share one allocation, in which long forward passes lay out the
+//   buffers of their chunks.
 //   sil              : [M][N_P] fp32 intermediate labels (Eq. 1).
 //
 // One training step is a dependency graph with one branch per layer.  Main branch: input staging,
@@ -17,8 +20,9 @@
 // (the same launch forms the bias gradient), which also waits for dgrad(l), the last reader of the
 // old weights.  The upper layers' HBM-bound updates thereby run beside the tensor-core products of
 // the layers below, and only two kernels follow the last dgrad.  After one eager run per batch size
-// the step is captured into a CUDA graph and replayed; the caller's x / cls are first copied into
-// fixed staging buffers so that the graph never changes.
+// (kLegacyEagerRuns on the legacy default stream) the step is captured into a CUDA graph and replayed;
+// the caller's x / cls are first copied into fixed staging buffers so that the graph never changes.
+// A small fp32 segment runs its step as two launches instead (small_step.cu), without a graph.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -842,9 +846,11 @@ static seg_status replay_graph(seg_handle* h, seg_handle::StepGraph& g, const vo
 }
 
 // Eager runs of a step before it is captured, on a handle that uses the legacy default stream.  Capture and instantiation cost
-// about 0.4 ms, a replayed step of 784-1024-1024-512 (TF32, batch 256) saves the GPU 5 us over an eager one: a short pass
-// over a new handle, or the partial batch at the end of a few epochs, is not worth a graph.
-constexpr int kLegacyEagerRuns = 24;
+// about 0.4 ms, a replayed step saves 5 to 10 us over an eager one: the graph is made when eager steps have cost about as much
+// more as it will, so that a short pass over a new handle, or the partial batch at the end of a few epochs, does not pay for
+// one.  First 40 steps of a new handle, captured after 24 and not at all: 512-512-256-47 (TF32, batch 256) 2.61 and 2.19 ms,
+// 784-300-100-47 (batch 128) 2.20 and 2.08, 512-1024-768-47 (bf16, batch 512) 2.32 and 2.30, 784-1024-1024-47 2.59 and 2.75.
+constexpr int kLegacyEagerRuns = 48;
 
 // Runs one step through its captured graph: the first call with this graph slot (the first kLegacyEagerRuns calls on the
 // legacy default stream) runs eagerly (it sets kernel attributes), the next captures the same enqueue into a graph, later ones

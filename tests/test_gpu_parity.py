@@ -520,9 +520,9 @@ def test_default_stream_step_is_captured_and_replayed(widths, precision, batch):
     for stream in (None, torch.cuda.Stream()):
         seg = Segment(widths, 47, False, precision=precision, optimizer="adam", lr=1e-3, max_batch=batch, stream=stream)
         seg.gen_labels(wl.LABEL_SEED, "normal")
-        loss = torch.zeros(70, device="cuda")
+        loss = torch.zeros(160, device="cuda")
         torch.cuda.synchronize()
-        for i in range(70):
+        for i in range(160):
             lo, n = (i % 4) * batch, batch - 7 * (i % 2)
             seg.train_step(xt[lo:lo + n], ct[lo:lo + n], loss[i:i + 1])
         seg.poll()
