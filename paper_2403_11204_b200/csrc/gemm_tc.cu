@@ -1341,7 +1341,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         int m_idx, n_idx;
         if (t == pair) { m_idx = first_m; n_idx = first_n; } else tile_coords(t, tiles_m, tiles_n, group_m, m_idx, n_idx);
         const int m0 = m_idx * PAIR_TILE_M + (int)rank * BLOCK_M;
-        const int n0 = n_idx * tile_n;          // (256 columns in this variant)
+        const int n0 = n_idx * PAIR_TILE_N;     // this variant is launched with whole tiles only
         update_tile<PAIR_TILE_N>(epi.upd, reinterpret_cast<const float*>(epi.C), epi.ldc, m0, n0, M, N, uw, lane,
                                  inv_bc1, inv_bc2);
       }
@@ -1557,6 +1557,7 @@ int pick_split(int M, int N, int K, bool tf32) {
 template <bool TF32, bool A_MN, bool B_MN, bool FUSED = false>
 cudaError_t launch_pair_variant(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const GemmDesc& g,
                                 const EpilogueArgs& e, int tile_n, int* dev_status, cudaStream_t s) {
+  if (FUSED && tile_n != PAIR_TILE_N) return cudaErrorInvalidValue;   // its update warps walk tiles of that width
   auto kern = gemm_tc_pair_kernel<TF32, A_MN, B_MN, FUSED>;
   static std::atomic<bool> attr_set_dev[kMaxDevices];      // the attribute is per device
   if (cudaError_t err = ensure_dynamic_smem(kern, PAIR_SMEM, attr_set_dev); err != cudaSuccess) return err;
@@ -1595,8 +1596,9 @@ cudaError_t launch_pair_majors(bool a_mn, bool b_mn, const CUtensorMap& ma, cons
 // which one SM's shared memory is filled (about 64 bytes per clock, measured: 24 KiB of operands per
 // k-block take 0.2 us, 32 KiB 0.27 us, 48 KiB 0.4 us); a CTA pair stages 32 KiB per CTA for the work
 // a single CTA needs 48 KiB for.  Persistent kernels run ceil(tiles / CTAs) rounds of num_k k-blocks.
+// fused_update: the kernel also applies the optimizer, whose warps walk pair tiles of 256 columns.
 struct Choice { int kind; int block_n; double us; };      // kind 0: single CTA, 1: CTA pair
-Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput) {
+Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_update) {
   const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64);
   const int tiles_m = (M + BLOCK_M - 1) / BLOCK_M;
   Choice best{0, 64, 1e30};
@@ -1624,13 +1626,13 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput) {
       us = rounds * t + (double)(2 * tiles) * t / num_sms();
     }
     if (g_pair_min_tiles > 0) {                            // diagnostic override: pairs from that many tiles on
-      if (tiles >= g_pair_min_tiles) best = Choice{1, g_pair_tile_n / 2, us};
+      if (tiles >= g_pair_min_tiles) best = Choice{1, (fused_update ? PAIR_TILE_N : g_pair_tile_n) / 2, us};
     } else if (us < best.us) {
       best = Choice{1, PAIR_HALF_N, us};
     }
     // Fewer than half as many 256-column tiles as pairs: tiles of 128 columns give every pair one (a k-block takes 0.18 us instead
     // of 0.30).  1024 x 2048 x 4096: 18.3 us against 25.8 with 256 columns and 19.6 with one CTA per 128 x 128 tile.
-    if (g_pair_min_tiles == 0 && !throughput && 2 * tiles <= pairs) {
+    if (g_pair_min_tiles == 0 && !throughput && !fused_update && 2 * tiles <= pairs) {
       const double us128 = num_k * 0.18 + 4.5;
       if (us128 < best.us) best = Choice{1, PAIR_HALF_N / 2, us128};
     }
@@ -1711,7 +1713,7 @@ cudaError_t launch_wait_selftest(int* dev_status, uint64_t limit_ns, cudaStream_
 // per row with short loops over its row in shared memory (about the cost of the launch it saves, and
 // it gives up the split over K) - and stays a launch of its own.
 double gemm_tc_estimate_us(int M, int N, int K, bool tf32) {
-  return 3.0 + pick_kernel(M, N, K, tf32, false).us;         // + launch, first loads and drain
+  return 3.0 + pick_kernel(M, N, K, tf32, false, false).us;         // + launch, first loads and drain
 }
 
 int gemm_tc_fused_loss_partials(int M, int N, int K, bool tf32) {
@@ -1762,7 +1764,7 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
     return cudaErrorInvalidValue;                           // the caller asks gemm_tc_fused_loss_partials first
   const bool throughput = g.off_critical_path != 0;
   const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 1;
-  const Choice choice = pick_kernel(g.M, g.N, g.K, tf32, throughput);
+  const Choice choice = pick_kernel(g.M, g.N, g.K, tf32, throughput, g.upd.enabled != 0);
   const bool pairs = (split == 1) && choice.kind == 1;
   const int block_n = split > 1 ? SPLITK_BLOCK_N : choice.block_n;
   const uint32_t block_k = tf32 ? 32 : 64, chunk = tf32 ? 32 : 64;

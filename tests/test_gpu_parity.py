@@ -333,6 +333,23 @@ def test_single_step_tensor_core_backend(widths, final, precision, optimizer, ba
     gpu.close()
 
 
+@pytest.mark.parametrize("widths,precision,batch", [([784, 2048], "tf32", 2048), ([784, 2048], "bf16", 4096)])
+def test_fused_update_where_the_cost_model_prefers_narrow_pair_tiles(widths, precision, batch, monkeypatch):
+    """Layer 0's weight gradient at these sizes would run on CTA-pair tiles of 128 columns; with the optimizer inside the
+    product it must keep tiles the update warps walk exactly once."""
+    if any(os.environ.get(k) for k in ("SEG_PAIR_MIN_TILES", "SEG_NO_SPLITK", "SEG_NO_PAIRS")):
+        pytest.skip("the kernel selection is forced in this process")
+    monkeypatch.setenv("SEG_FUSED_UPDATE", "1")
+    w = wl.WORKLOADS["tiny"]
+    gpu, ora = make_pair(widths, 47, False, precision, "momentum", 0.01, batch, gemm_backend="tcgen05")
+    x, cls = batch_arrays(w, batch, widths[0], precision=precision)
+    compare_step(gpu, ora, x, cls, precision, TOL[precision])
+    assert gpu.product_launches()["fused_update"] == 1
+    # first step from a zero momentum buffer: the buffer is the gradient, bit for bit, unless an element was updated twice
+    assert bits_equal(gpu.opt_state(0, 0)[0].cpu().numpy(), gpu.grads(0)[0].cpu().numpy())
+    gpu.close()
+
+
 def test_product_family_counters_tell_the_backends_apart():
     """seg_product_launches is what the tensor-core tests rely on to show that tcgen05 kernels ran, so it is
     checked from both sides: a bf16 handle on the automatic or the tensor-core backend counts its five
