@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <atomic>
 #include <new>
+#include <type_traits>
 
 #include "async_copy.cuh"
 #include "common.cuh"
@@ -83,12 +84,13 @@ __device__ __forceinline__ void element_of(int i, int b, int& row, int& col) {
 
 // v[r * CT + j] += sum over this lane's chunks (four k each) of A[r][4c ..] . W[n_j][4c ..]; A rows `pa` apart, wp[j] the row
 // of column n_j.  The lanes' chunks are c0, c0 + step, ...; all lanes make the same number of rounds (a lane without a chunk
-// left multiplies by zero), so that a warp never splits.
+// left multiplies zeros by zeros: a value it does not own may be infinite), so that a warp never splits.
 template <int RT, int CT, int VP>
-__device__ __forceinline__ void dot_chunk(float (&v)[VP], const float* A, int pa, const float4 (&w)[CT]) {
+__device__ __forceinline__ void dot_chunk(float (&v)[VP], const float* A, int pa, const float4 (&w)[CT], bool own = true) {
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
-    const float4 a = lds4(A + r * pa);
+    float4 a = lds4(A + r * pa);
+    if (!own) a = make_float4(0.f, 0.f, 0.f, 0.f);
     // component by component: the CT sums in between hide the latency of a multiply-add on the same sum
 #pragma unroll
     for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.x, w[j].x, v[r * CT + j]);
@@ -120,7 +122,7 @@ __device__ __forceinline__ void dot_rows(float (&v)[VP], const float* A, int pa,
       w[j] = lds4(wp[j] + 4 * c);
       if (!ok) w[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    dot_chunk<RT, CT, VP>(v, A + 4 * c, pa, w);
+    dot_chunk<RT, CT, VP>(v, A + 4 * c, pa, w, ok);
   }
 }
 
@@ -182,13 +184,16 @@ __device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float*
     er[i] += rp * RT;
     if (ek[i] >= 0) es[i] = side(er[i], ek[i]);
   }
-  // chunks of four n in rounds of four lane groups, as in dot_rows: in the last round a lane beyond N multiplies by zero
-  const int chunks = (N + 3) >> 2;
-  auto round = [&](int c, bool ok) {
+  // chunks of four n in rounds of four lane groups, as in dot_rows: in the last round, which also holds a chunk that N cuts,
+  // what lies beyond N is zeros on both sides
+  auto round = [&](int c, auto last) {
+    const bool own = !decltype(last)::value || 4 * c < N;
+    if (decltype(last)::value) c = min(c, (N - 1) >> 2);
     float w[4][CT];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const float* row = wk + min(4 * c + u, N - 1) * pw;
+      const bool ok = !decltype(last)::value || (own && 4 * c + u < N);
+      const float* row = wk + (decltype(last)::value ? min(4 * c + u, N - 1) : 4 * c + u) * pw;
       if constexpr (CT == 4) { const float4 t = lds4(row); w[u][0] = t.x; w[u][1] = t.y; w[u][2] = t.z; w[u][3] = t.w; }
       else if constexpr (CT == 2) { const float2 t = *reinterpret_cast<const float2*>(row); w[u][0] = t.x; w[u][1] = t.y; }
       else w[u][0] = row[0];
@@ -199,7 +204,8 @@ __device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float*
     }
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
-      const float4 a = lds4(A + r * pz + 4 * c);            // zero between N and the end of the chunk
+      float4 a = lds4(A + r * pz + 4 * c);                  // zero between N and the end of the chunk
+      if (!own) a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.x, w[0][j], v[r * CT + j]);
 #pragma unroll
@@ -210,10 +216,10 @@ __device__ __forceinline__ void link_dgrad(const float* dZ, int pz, const float*
       for (int j = 0; j < CT; ++j) v[r * CT + j] = fmaf(a.w, w[3][j], v[r * CT + j]);
     }
   };
-  const int full = chunks >> 2;
+  const int full = N >> 4;
 #pragma unroll 2
-  for (int i = 0; i < full; ++i) round(4 * i + sl, true);
-  if (full * 4 < chunks) round(min(4 * full + sl, chunks - 1), 4 * full + sl < chunks);
+  for (int i = 0; i < full; ++i) round(4 * i + sl, std::false_type{});
+  if ((N & 15) != 0) round(4 * full + sl, std::true_type{});
   reduce_scatter<V, 4>(v, lane);
 #pragma unroll
   for (int i = 0; i < H; ++i)

@@ -570,6 +570,50 @@ def test_small_segment_shapes(widths, final, batch):
     gpu.close()
 
 
+@pytest.mark.parametrize("widths", [[20, 12], [784, 40], [300, 16], [33, 47], [784, 128, 64], [20, 24, 12]])
+def test_infinite_features_of_a_small_segment(widths):
+    """One infinite feature per row, every feature in turn: the outputs are the infinities (and, behind a second layer, the
+    NaNs) of the definition, for contractions that do not fill the lanes' last round."""
+    import torch
+    from paper_2403_11204_b200.binding import Segment
+    k = widths[0]
+    seg = Segment(widths, 47, False, precision="fp32", max_batch=k, last_relu=False)
+    x = torch.rand(k, k, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    x.fill_diagonal_(float("inf"))
+    y = seg.forward(x)
+    seg.poll()
+    a = x.double()
+    for l in range(len(widths) - 1):
+        W, b = seg.params(l)
+        a = a @ W.double().T + b.double()
+        if l < len(widths) - 2:
+            a = a.clamp(min=0)
+    assert torch.equal(y.isnan(), a.isnan())
+    keep = ~a.isnan()
+    assert torch.equal(y[keep], a[keep].float())
+    seg.close()
+
+
+def test_infinite_gradient_of_a_small_segment():
+    """An infinite weight in the last row of a layer whose width no lane group divides, and an infinite target of one output:
+    every gradient element below is the definition's infinity or zero, none NaN."""
+    import torch
+    from paper_2403_11204_b200.binding import Segment
+    for n_out in (5, 21, 33):
+        seg = Segment([8, 12, n_out], 3, False, precision="fp32", max_batch=1, last_relu=False)
+        seg.gen_labels(1)
+        W0, b0 = torch.full((12, 8), 0.25, device="cuda"), torch.zeros(12, device="cuda")
+        W1, b1 = torch.full((n_out, 12), 0.5, device="cuda"), torch.zeros(n_out, device="cuda")
+        W1[-1, 3] = float("inf")
+        seg.set_params(0, W0, b0)
+        seg.set_params(1, W1, b1)
+        seg.train_step(torch.ones(1, 8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda"))
+        seg.poll()
+        dW, db = seg.grads(0)                            # dZ_1 = inf everywhere: the last output's error is infinite
+        assert bool(torch.isposinf(dW).all()) and bool(torch.isposinf(db).all()), n_out
+        seg.close()
+
+
 @pytest.mark.parametrize("widths,final,precision,tol", [([784, 320, 200, 72], False, "bf16", 2e-2), ([72, 136, 264, 47], True, "bf16", 2e-2),
                                                         ([100, 320, 200, 72], False, "tf32", 2e-3), ([200, 160, 96], False, "fp32", 1e-4),
                                                         ([90, 160, 47], True, "fp32", 1e-4), ([33, 60, 47], True, "fp32", 1e-4)])
