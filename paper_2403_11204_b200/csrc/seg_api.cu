@@ -128,6 +128,7 @@ struct seg_handle {
   bool fork_enabled = true;        // run the gradient and update branches on their own streams
   bool small_fused = false;        // small fp32 segment: the whole step runs as two launches (SEG_NO_SMALL_FUSED=1: off)
   SmallStep small{};               // its description, filled by seg_create (batch is set per launch)
+  SmallMaps small_maps{};
   std::map<int, SmallPrepared*> small_by_batch;
   bool fuse_update = false;        // SEG_FUSED_UPDATE=1: apply the optimizer inside the weight-gradient product where the
                                    // kernel can (measured slower than the separate update launch, see gemm_tc.cu)
@@ -379,7 +380,7 @@ SmallPrepared* small_for(seg_handle* h, int batch) {
   if (!w) {
     SmallStep p = h->small;
     p.batch = batch;
-    w = small_prepare(p);
+    w = small_prepare(p, h->small_maps);
   }
   return w;
 }
@@ -596,13 +597,7 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
       ++h->launches;
       if (launch_small_ones(p.act[l], p.ld_act[l], p.widths[l], h->max_batch, h->stream) != cudaSuccess) return bail(SEG_ERR_CUDA);
     }
-    CUtensorMap maps[3 * kSmallMaxLayers];
-    CUtensorMap* dev_maps = nullptr;
-    if (!small_step_maps(p, h->max_batch, maps)) return bail(SEG_ERR_CUDA);
-    if ((st = dev_alloc(h, &dev_maps, 3 * kSmallMaxLayers, false)) != SEG_OK) return bail(st);
-    if (cudaMemcpyAsync(dev_maps, maps, sizeof(CUtensorMap) * 3 * h->n_layers, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
-      return bail(SEG_ERR_CUDA);
-    p.maps = dev_maps;
+    if (!small_step_maps(p, h->max_batch, &h->small_maps)) return bail(SEG_ERR_CUDA);
   }
   if (cudaEventCreate(&h->ev_start) != cudaSuccess || cudaEventCreate(&h->ev_stop) != cudaSuccess)
     return bail(SEG_ERR_CUDA);

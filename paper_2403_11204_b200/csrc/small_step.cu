@@ -596,7 +596,8 @@ __host__ __device__ inline int wgrad_ring_floats(int mt, int nt, int stages) {
 
 template <int OPT, int NT>
 __global__ void __launch_bounds__(SS_THREADS, 2)
-small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_per_cta, int n_partials, int stages) {
+small_wgrad_update_kernel(const __grid_constant__ SmallStep p, const __grid_constant__ SmallMaps maps, int S, int rows_per_cta,
+                          int n_partials, int stages) {
   constexpr int CN = NT / 8;                                // columns per thread
   constexpr int CPR = NT / 4;                               // 16-byte groups per row of B
   extern __shared__ __align__(128) float sm[];
@@ -619,9 +620,8 @@ small_wgrad_update_kernel(const __grid_constant__ SmallStep p, int S, int rows_p
   float* ringA = sm;                                        // [stage][WK][MT]
   float* ringB = sm + stages * WK * MT;                     // [stage][WK][NT]
   float* recv = sm + wgrad_ring_floats(MT, NT, stages);     // [source CTA][MT / S rows][NT]
-  const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(p.maps) + 3 * l;
-  const CUtensorMap* map_a = maps;                          // (m = o, k = b) at dz[b * ld + o]
-  const CUtensorMap* map_b = maps + (NT == 32 ? 1 : 2);   // (k = b, n = i) at act[b * ld + i]; column `in` holds ones
+  const CUtensorMap* map_a = maps.m + 3 * l;                // (m = o, k = b) at dz[b * ld + o]
+  const CUtensorMap* map_b = map_a + (NT == 32 ? 1 : 2);    // (k = b, n = i) at act[b * ld + i]; column `in` holds ones
   const uint32_t box_bytes = (uint32_t)(WBOX * (MT + NT) * 4);
   auto load = [&](int step) {                               // by the issuing thread
     const int s = step % stages, boxes = min(WK / WBOX, (rows - step * WK + WBOX - 1) / WBOX);
@@ -927,6 +927,7 @@ struct ChainArgs {
 // own buffers, tiles of the second kernel.
 struct SmallPrepared {
   ChainArgs a;
+  SmallMaps maps;
   int nt, S, tiles, rows, stages;
   size_t wgrad_smem;
 };
@@ -1017,7 +1018,7 @@ cudaError_t launch_wgrad(SmallPrepared& w, cudaStream_t s) {
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(small_wgrad_update_kernel<OPT, NT>), SS_SMEM_LIMIT, allowed);
   if (e != cudaSuccess) return e;
   int n_partials = chain_grid(w.a.p, w.a.q);
-  void* args[] = {&w.a.p, &w.S, &w.rows, &n_partials, &w.stages};
+  void* args[] = {&w.a.p, &w.maps, &w.S, &w.rows, &n_partials, &w.stages};
   return launch_clustered(small_wgrad_update_kernel<OPT, NT>, w.tiles * w.S, w.S, w.wgrad_smem, s, args);
 }
 
@@ -1036,9 +1037,10 @@ bool small_step_supported(int n_layers, const int* widths) {
   return true;
 }
 
-SmallPrepared* small_prepare(const SmallStep& p) {
+SmallPrepared* small_prepare(const SmallStep& p, const SmallMaps& maps) {
   SmallPrepared* w = new (std::nothrow) SmallPrepared();
   if (!w) return nullptr;
+  w->maps = maps;
   ChainArgs& a = w->a;
   a.p = p;
   bool ok = plan_small(p, &a.q);
@@ -1061,9 +1063,9 @@ void small_release(SmallPrepared* w) { delete w; }
 
 bool small_can_train(const SmallPrepared& w) { return chain_grid(w.a.p, w.a.q) <= loss_max_partials(); }
 
-bool small_step_maps(const SmallStep& p, int max_batch, CUtensorMap* maps) {
+bool small_step_maps(const SmallStep& p, int max_batch, SmallMaps* maps) {
   for (int l = 0; l < p.n_layers; ++l) {
-    CUtensorMap* m = maps + 3 * l;
+    CUtensorMap* m = maps->m + 3 * l;
     const uint32_t mt = (uint32_t)up(p.widths[l + 1], 8);
     if (!make_map_f32(m, p.dz[l], mt, (uint64_t)max_batch, (uint64_t)p.ld_act[l + 1] * 4, mt, WBOX)) return false;
     const uint32_t nts[2] = {32, 16};

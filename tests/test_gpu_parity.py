@@ -570,6 +570,18 @@ def test_small_segment_shapes(widths, final, batch):
     gpu.close()
 
 
+def test_small_segments_created_where_others_were_destroyed():
+    """Handles of changing shapes one after the other: each gets device memory an earlier one has freed, and its step must
+    not see anything of that one's buffers."""
+    w = wl.WORKLOADS["tiny"]
+    for widths, final, batch in [([784, 80, 60], False, 200), ([60, 60, 60, 47], True, 200), ([300, 81, 33], False, 40),
+                                 ([784, 80, 60], False, 90), ([40, 24, 47], True, 7)] * 3:
+        gpu, ora = make_pair(widths, 47, final, "fp32", "momentum", 0.01, batch)
+        x, cls = batch_arrays(w, batch, widths[0])
+        compare_step(gpu, ora, x, cls, "fp32", TOL["fp32"])
+        gpu.close()
+
+
 @pytest.mark.parametrize("widths", [[20, 12], [784, 40], [300, 16], [33, 47], [784, 128, 64], [20, 24, 12]])
 def test_infinite_features_of_a_small_segment(widths):
     """One infinite feature per row, every feature in turn: the outputs are the infinities (and, behind a second layer, the
