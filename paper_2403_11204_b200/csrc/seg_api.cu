@@ -664,11 +664,21 @@ seg_status seg_gen_labels(seg_handle* h, uint64_t seed, int32_t dist, float kapp
   return SEG_OK;
 }
 
+// True when the rows a forward pass reads and the rows it writes share memory.  The kernels that write y while other rows of x
+// are still being read then stand back for the layer-by-layer pass, which puts y down after its last read of x.
+static bool rows_overlap(const seg_handle* h, const void* x, const void* y, int64_t n) {
+  const uintptr_t x0 = reinterpret_cast<uintptr_t>(x), y0 = reinterpret_cast<uintptr_t>(y);
+  const uintptr_t xb = (uintptr_t)n * h->widths[0] * elem_size(h->act_dt);
+  const uintptr_t yb = (uintptr_t)n * h->widths[h->n_layers] * elem_size(h->act_dtype[h->n_layers]);
+  return x0 < y0 + yb && y0 < x0 + xb;
+}
+
 seg_status seg_forward(seg_handle* h, const void* x, int32_t batch, void* y) {
   if (!h || !x || !y) return SEG_ERR_INVALID_ARG;
   DeviceGuard guard(h);
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
-  if (SmallPrepared* w = small_for(h, batch)) {   // small fp32 segment: all layers in one launch, the last one's output also into y
+  SmallPrepared* w = rows_overlap(h, x, y, batch) ? nullptr : small_for(h, batch);
+  if (w) {                         // small fp32 segment: all layers in one launch, the last one's output also into y
     Launch l(h, K_FWD);
     SEG_TRY(h, launch_small_forward(*w, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), true, h->stream),
             "small-segment forward launch");
@@ -1120,7 +1130,8 @@ seg_status seg_forward_dataset(seg_handle* h, const void* x, int64_t n, int32_t 
   auto yr = [&](int64_t i) { return reinterpret_cast<char*>(y) + (size_t)i * out_bytes; };
   // the last chunk of `batch` rows (or the partial one) goes through the handle's own buffers, where seg_get_activation looks;
   // the rows before it are grouped as the GPU likes them
-  const int64_t head = n - (n % batch ? n % batch : batch);
+  // (over x itself: batch by batch)
+  const int64_t head = rows_overlap(h, x, y, n) ? 0 : n - (n % batch ? n % batch : batch);
   int64_t done = 0;
   if (h->small_fused) {
     while (done < head) {

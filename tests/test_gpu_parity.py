@@ -582,6 +582,27 @@ def test_small_segments_created_where_others_were_destroyed():
         gpu.close()
 
 
+@pytest.mark.parametrize("widths,precision,tol", [([64, 64], "fp32", 1e-4), ([784, 80, 60], "fp32", 1e-4), ([128, 40, 128], "fp32", 1e-4),
+                                                  ([256, 256], "bf16", 2e-2), ([160, 160], "fp32", 1e-4), ([256, 320, 128], "tf32", 2e-3)])
+def test_response_written_over_its_input(widths, precision, tol):
+    """seg_forward and seg_forward_dataset with y at x's address (responses no wider than the input rows): the input is read
+    before the response takes its place."""
+    import torch
+    w = wl.WORKLOADS["tiny"]
+    batch, n = 600, 2500
+    gpu, ora = make_pair(widths, 47, False, precision, "sgd", 0.01, batch)
+    x, _ = batch_arrays(w, n, widths[0], precision=precision)
+    xt, _ = to_device(x, np.zeros(n), precision)
+    ref = ora.forward(x)[-1]
+    for rows, call in ((batch, lambda t: gpu.forward(t, t)), (n, lambda t: gpu.forward_dataset(t, batch, t))):
+        t = xt[:rows].clone()
+        call(t)
+        gpu.poll()
+        got = t.view(-1)[:rows * widths[-1]].view(rows, widths[-1]).float().cpu().numpy()
+        assert rel_err(got, ref[:rows]) < tol, (rows, widths)
+    gpu.close()
+
+
 @pytest.mark.parametrize("widths", [[20, 12], [784, 40], [300, 16], [33, 47], [784, 128, 64], [20, 24, 12]])
 def test_infinite_features_of_a_small_segment(widths):
     """One infinite feature per row, every feature in turn: the outputs are the infinities (and, behind a second layer, the
