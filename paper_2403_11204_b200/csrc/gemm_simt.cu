@@ -12,7 +12,8 @@
 // stages, 8 x 8 outputs per thread.  The 64 threads that hold a tile exist four times in a CTA (each group takes a quarter of
 // every stage's K) and S CTAs of a cluster split K again, so that few tiles still fill the GPU; the partial tiles meet in
 // shared memory and, as a reduce-scatter, in distributed shared memory, in a fixed order.  gemm_simt_kernel serves what tensor
-// copies cannot take (rows that are no whole 16-byte groups) and bf16 operands on the FFMA backend.
+// copies cannot take (rows that are no whole 16-byte groups), bf16 operands on the FFMA backend, and the fp32 products it is
+// the faster one for (strided_is_faster).
 #include <algorithm>
 #include <atomic>
 
@@ -424,6 +425,41 @@ cudaError_t launch_ffma(const CUtensorMap& ma, const CUtensorMap& mb, const Gemm
   return cudaLaunchKernelEx(&cfg, kern, ma, mb, g.M, g.N, g.K, S, kp, e, dev_status);
 }
 
+// The split of K the strided kernel takes: while it adds CTAs the GPU has room for and leaves every split at least 4 k-steps.
+struct StridedSplit { int splits, k_per_split; };
+StridedSplit strided_split(int tiles, int K, int slots) {
+  int splits = 1;
+  if (tiles <= slots) splits = std::max(1, std::min(std::min(148 / tiles, slots / tiles), K / (4 * BK)));
+  const int k_per_split = std::max(BK, ((K + splits - 1) / splits + BK - 1) / BK * BK);
+  return {std::max(1, (K + k_per_split - 1) / k_per_split), k_per_split};
+}
+
+// Estimated cycles of an fp32 product in each of the two kernels.  Which one takes it (strided_is_faster): two kinds of products
+// are the strided kernel's - few tiles over a very long contraction (the weight gradient of narrow layers over a large batch, very
+// wide inputs), which it cuts into up to 148 pieces where a cluster cuts 8, and many tiles over a short one, where two of its CTAs
+// share an SM and the other kernel's fixed cost of 6500 to 8500 cycles per tile is most of its time.  Strided against tensor
+// copies, us: weight gradient of 64 x 64 over 16384 / 65536 rows 29 / 50 against 56 / 207, forward 65536 x 256 over K = 8 / 64 /
+// 128 78 / 117 / 205 against 111 / 138 / 189, dgrad 65536 x 784 over K = 8 / 64 / 128 297 / 410 / 660 against 555 / 637 / 793.
+// The constants follow from 552 products timed in both kernels: none of them goes to one that is over 5 % and 0.6 us behind.
+double copies_cycles(Form form, int tiles, int K) {
+  const int S = ffma_split(tiles, K);
+  const int resident = S == 1 ? 148 : S == 2 ? 74 : S == 4 ? 33 : 15, kp = ((K + S - 1) / S + FK - 1) / FK * FK;
+  const double fixed = (form == FORM_NT ? 6500.0 : form == FORM_NN ? 8500.0 : 7000.0) + (S > 1 ? 1000.0 : 0.0);
+  return (double)((tiles + resident - 1) / resident) * (fixed + 46.0 * kp);
+}
+double strided_cycles(int tiles, int K, int slots) {
+  const StridedSplit sp = strided_split(tiles, K, slots);
+  const int64_t ctas = (int64_t)tiles * sp.splits;
+  const double t = ctas > 148 ? (double)((ctas + 295) / 296) * (4800.0 + 168.0 * sp.k_per_split) : 6000.0 + 107.0 * sp.k_per_split;
+  return t + (sp.splits > 1 ? 200.0 * sp.splits : 0.0);
+}
+// Not for a few per cent, though: its CTAs take more of the SMs from the products of other branches (weight gradients, TN, run
+// beside the dgrad chain).  Whole steps of 81 fp32 cases against tensor copies alone: 0.986 of the time with these factors, 0.995
+// with 0.75 for all three forms, 1.004 with 0.75 for TN and 0 for the others; the worst case 1.05, 1.14 and 1.13.
+bool strided_is_faster(Form form, int tiles, int K, int slots) {
+  return strided_cycles(tiles, K, slots) < (form == FORM_TN ? 0.75 : 0.93) * copies_cycles(form, tiles, K);
+}
+
 // cudaErrorNotSupported: operands that tensor copies cannot take (the strided kernel serves them).
 cudaError_t try_ffma(const GemmDesc& g, int* dev_status, cudaStream_t s) {
   if (g.a_dt != DT_F32 || g.b_dt != DT_F32 || g.c_dt != DT_F32 || g.M <= 0 || g.N <= 0 || g.K <= 0 || g.c_round == RND_BF16)
@@ -462,19 +498,14 @@ int gemm_simt_slots(int M, int N, int K) {
 cudaError_t launch_gemm_simt(const GemmDesc& g, int* dev_status, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   if (g.a_dt != g.b_dt) return cudaErrorInvalidValue;
-  if (cudaError_t e = try_ffma(g, dev_status, s); e != cudaErrorNotSupported) return e;
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
-  // split K while that adds CTAs the GPU has room for and leaves every split at least 4 k-steps
-  const int tiles = (int)(grid.x * grid.y);
-  int splits = 1;
-  if (g.simt_scratch != nullptr && g.simt_counters != nullptr && tiles <= g.simt_slots) {
-    splits = std::min(std::min(148 / tiles, g.simt_slots / tiles), g.K / (4 * BK));
-    if (splits < 1) splits = 1;
-  }
-  int k_per_split = ((g.K + splits - 1) / splits + BK - 1) / BK * BK;
-  if (k_per_split < BK) k_per_split = BK;
-  splits = g.K > 0 ? (g.K + k_per_split - 1) / k_per_split : 1;
-  grid.z = (unsigned)std::max(splits, 1);
+  const int tiles = (int)(grid.x * grid.y), slots = g.simt_scratch != nullptr && g.simt_counters != nullptr ? g.simt_slots : 0;
+  const Form form = g.a_sk != 1 ? FORM_TN : (g.b_sk == 1 && g.b_sn != 1) ? FORM_NT : FORM_NN;
+  if (!strided_is_faster(form, tiles, g.K, slots))
+    if (cudaError_t e = try_ffma(g, dev_status, s); e != cudaErrorNotSupported) return e;
+  const StridedSplit sp = strided_split(tiles, g.K, slots);
+  const int k_per_split = sp.k_per_split;
+  grid.z = (unsigned)sp.splits;
   if (g.a_dt == DT_F32 && g.c_dt == DT_F32) launch_k(gemm_simt_kernel<float, float>, dim3(grid), dim3(256), 0, s, g, k_per_split);
   else if (g.a_dt == DT_BF16 && g.c_dt == DT_BF16)
     launch_k(gemm_simt_kernel<__nv_bfloat16, __nv_bfloat16>, dim3(grid), dim3(256), 0, s, g, k_per_split);

@@ -570,6 +570,18 @@ def test_small_segment_shapes(widths, final, batch):
     gpu.close()
 
 
+@pytest.mark.parametrize("widths,final,batch", [([16, 160, 8], False, 20000), ([8, 300, 47], True, 9001), ([9000, 64, 136], False, 40),
+                                                ([33000, 5, 130], False, 3), ([130, 64, 64], False, 16384)])
+def test_fp32_products_of_extreme_shapes(widths, final, batch):
+    """Few output tiles over a long contraction and many over a short one, on both sides of the choice between the two kernels."""
+    w = wl.WORKLOADS["tiny"]
+    gpu, ora = make_pair(widths, 47, final, "fp32", "momentum", 0.01, batch)
+    for n, seed in ((batch, wl.DATA_SEED), (max(1, batch // 7), 5)):
+        x, cls = batch_arrays(w, n, widths[0], seed=seed)
+        compare_step(gpu, ora, x, cls, "fp32", TOL["fp32"])
+    gpu.close()
+
+
 def test_small_segments_created_where_others_were_destroyed():
     """Handles of changing shapes one after the other: each gets device memory an earlier one has freed, and its step must
     not see anything of that one's buffers."""
