@@ -487,6 +487,13 @@ double ffma_estimate_us(int M, int N, int K) {
   return cycles / 1900.0;
 }
 
+// The copy: a launch of about 3 us and 8 bytes per element at about 3 TB/s.  784-80-60 at 8192 rows, us: 85 with the strided first
+// layer, 62 with aligned rows.
+bool fp32_staging_pays(int M, int N, int K, int slots) {
+  const int tiles = ((M + FT - 1) / FT) * ((N + FT - 1) / FT);
+  return strided_cycles(tiles, K, slots) / 1900.0 > copies_cycles(FORM_NT, tiles, K) / 1900.0 + 3.0 + 8.0 * M * K / 3e6;
+}
+
 // Partial tiles the split of an M x N x K product would use with an unlimited workspace (0: no split).
 int gemm_simt_slots(int M, int N, int K) {
   const int tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);

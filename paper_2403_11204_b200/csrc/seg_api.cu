@@ -261,13 +261,15 @@ void* weights_op(seg_handle* h, int l) {
   return base + h->layers[l].w_off * elem_size(h->params_op ? h->op_dt : DT_F32);
 }
 
-// Returns the pointer / pitch the first product reads x from, staging it when the caller's
-// buffer cannot be used directly (TF32 rounding, or rows that are not 16-byte multiples).
+// Returns the pointer / pitch the first product reads x from, staging it when the caller's buffer cannot be used
+// directly (TF32 rounding, or rows that are not 16-byte multiples) or, in fp32, when aligned rows pay for the copy.
 seg_status prepare_input(seg_handle* h, const void* x, int batch, const void** x_use, int64_t* ld) {
   const int w0 = h->widths[0];
   const bool aligned = ((reinterpret_cast<uintptr_t>(x) & 15u) == 0) &&
                        ((w0 * elem_size(h->act_dt)) % 16 == 0);
-  if (h->precision != SEG_TF32 && (aligned || !h->use_tc)) {
+  const bool stage = h->precision == SEG_TF32 ||
+                     (!aligned && (h->use_tc || (h->precision == SEG_FP32 && fp32_staging_pays(batch, h->widths[1], w0, h->simt_slots[0]))));
+  if (!stage) {
     *x_use = x; *ld = w0;
     return SEG_OK;
   }
@@ -375,7 +377,6 @@ seg_status refresh_operand_copy(seg_handle* h, int64_t off, int64_t n) {
 
 // The prepared launches of a small fp32 segment for this batch size; nullptr: the segment runs layer by layer.
 SmallPrepared* small_for(seg_handle* h, int batch) {
-  if (!h->small_fused) return nullptr;
   SmallPrepared*& w = h->small_by_batch[batch];
   if (!w) {
     SmallStep p = h->small;
@@ -677,7 +678,10 @@ seg_status seg_forward(seg_handle* h, const void* x, int32_t batch, void* y) {
   if (!h || !x || !y) return SEG_ERR_INVALID_ARG;
   DeviceGuard guard(h);
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
-  SmallPrepared* w = rows_overlap(h, x, y, batch) ? nullptr : small_for(h, batch);
+  SmallPrepared* w = nullptr;
+  if (h->small_fused && !rows_overlap(h, x, y, batch) &&
+      batch <= small_max_rows(h->small, false, small_input_by_tensor(reinterpret_cast<const float*>(x), nullptr, h->widths[0])))
+    w = small_for(h, batch);
   if (w) {                         // small fp32 segment: all layers in one launch, the last one's output also into y
     Launch l(h, K_FWD);
     SEG_TRY(h, launch_small_forward(*w, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), true, h->stream),
@@ -954,7 +958,10 @@ static seg_status train_step_impl(seg_handle* h, const void* x, const int32_t* c
   if (batch < 1 || batch > h->max_batch) return SEG_ERR_SHAPE;
   if (!h->is_final && !h->have_labels) return SEG_ERR_STATE;
   seg_status st = SEG_OK;
-  SmallPrepared* small = small_for(h, batch);
+  SmallPrepared* small = nullptr;
+  if (h->small_fused &&
+      batch <= small_max_rows(h->small, true, small_input_by_tensor(reinterpret_cast<const float*>(x), gather, h->widths[0])))
+    small = small_for(h, batch);
   if (small && small_can_train(*small)) {
     st = small_step(h, *small, batch, x, cls, loss_out ? loss_out : h->loss_slot, gather);
   } else if (h->profile || !h->graphs_enabled) {
@@ -1133,8 +1140,9 @@ seg_status seg_forward_dataset(seg_handle* h, const void* x, int64_t n, int32_t 
   // (over x itself: batch by batch)
   const int64_t head = rows_overlap(h, x, y, n) ? 0 : n - (n % batch ? n % batch : batch);
   int64_t done = 0;
+  const bool by_tensor = small_input_by_tensor(reinterpret_cast<const float*>(x), nullptr, h->widths[0]);
   if (h->small_fused) {
-    while (done < head) {
+    while (done < head && batch < small_dataset_batch(h->small, by_tensor)) {
       const int rows = (int)std::min<int64_t>(head - done, 1 << 20);
       SmallPrepared* w = small_for(h, rows);
       if (!w) break;

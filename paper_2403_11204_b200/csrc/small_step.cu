@@ -24,6 +24,7 @@
 // when they do not (measured), so r rows x c columns cost 2 r + 4 c cycles of loads per r c cycles of FFMA issue and
 // four k.
 #include <cuda.h>
+#include <limits.h>
 
 #include <algorithm>
 #include <atomic>
@@ -822,6 +823,8 @@ int resident_clusters(int C) { return C == 1 ? 148 : C == 2 ? 74 : C == 4 ? 33 :
 // The same with two CTAs per SM.
 int resident_clusters_2(int C) { return C == 1 ? 296 : C == 2 ? 148 : C == 4 ? 71 : 33; }
 
+int cluster_of(int n0) { return n0 <= 128 ? 1 : n0 <= 256 ? 2 : n0 <= 512 ? 4 : 8; }   // CTAs per cluster: at most 128 features each
+
 constexpr int kRowChoices[] = {1, 2, 4, 6, 8, 10, 12, 16};
 int split_columns(int N1) { return N1 <= 32 ? 2 : N1 <= 64 ? 4 : N1 <= 80 ? 5 : 8; }   // columns per lane in the split first layer
 
@@ -829,7 +832,7 @@ int split_columns(int N1) { return N1 <= 32 ? 2 : N1 <= 64 ? 4 : N1 <= 80 ? 5 : 
 bool layout_small(const SmallStep& p, int R, SmallPlan* q) {
   const int L = p.n_layers, n0 = p.widths[0], N1 = p.widths[1];
   q->R = R;
-  q->C = n0 <= 128 ? 1 : n0 <= 256 ? 2 : n0 <= 512 ? 4 : 8;        // at most 128 features per CTA
+  q->C = cluster_of(n0);
   const int first = q->C > 1 ? 1 : 0, n_slots = L - first;
   q->ks = q->C > 1 ? pitch_of((n0 + q->C - 1) / q->C) : up(n0, 4);
   int slot_max = 0, slot_sum = 0;
@@ -1062,6 +1065,28 @@ SmallPrepared* small_prepare(const SmallStep& p, const SmallMaps& maps) {
 void small_release(SmallPrepared* w) { delete w; }
 
 bool small_can_train(const SmallPrepared& w) { return chain_grid(w.a.p, w.a.q) <= loss_max_partials(); }
+
+// A batch runs in waves of 16 rows per CTA (1920 rows with clusters of 8, 2368 with one CTA per block of rows); past a few of
+// them the layer-by-layer products, whose tiles share a layer's weights among 64 rows, catch up.  Rows that cannot be loaded by a
+// tensor copy (by_tensor false: plain loads of a warp per row) make a wave longer.  us, this path / layer by layer:
+//   forward   784-80-60 at 1536 / 3072 / 8192 rows 17/24 32/36 79/63, 784-128-128-64 31/28 55/42 127/78, 60-60-60-47 7/17 12/18 30/20;
+//             without tensor copies 31/40 60/56 148/85, 45/38 80/62 187/101, 8/19 14/20 34/24
+//   training  784-80-60 at 2048 / 8192 / 16384 rows 46/56 143/148 272/298, 784-128-128-64 at 2048 / 4096 / 8192 75/75 136/113 241/204,
+//             300-81-33 34/43 66/60 125/98, 60-60-60-47 22/47 38/59 72/81; without tensor copies 784-80-60 62/60 103/92 213/160,
+//             784-128-128-64 91/78 169/119 323/218, 300-81-33 39/44 77/62 147/102, 60-60-60-47 23/47 40/60 75/82
+int small_max_rows(const SmallStep& p, bool train, bool by_tensor) {
+  const int C = cluster_of(p.widths[0]), wave = 16 * C * resident_clusters(C);
+  if (!train) return by_tensor ? (C == 1 ? 2 * wave : wave) : (C == 8 ? wave / 2 : wave);
+  if (C == 1 || (by_tensor && (C == 2 || (C == 8 && p.widths[1] <= 96)))) return INT_MAX;   // (one loss partial per CTA: 16384 rows)
+  return by_tensor ? 2 * wave : C == 2 ? 3 * wave : wave;
+}
+// A whole data set in one launch takes many waves at a constant time per row, which the layer-by-layer pass undercuts in batches
+// of this many rows (784-80-60: 8.7 ns per row against 8.8 in batches of 4096; 60-60-60-47: 3.4 against 4.4 and, at 8192, 2.4;
+// without tensor copies 784-80-60 17.7 against 14 in batches of 2048).
+int small_dataset_batch(const SmallStep& p, bool by_tensor) {
+  const int C = cluster_of(p.widths[0]);
+  return C == 1 ? 8192 : by_tensor || C < 8 ? 4096 : 2048;
+}
 
 bool small_step_maps(const SmallStep& p, int max_batch, SmallMaps* maps) {
   for (int l = 0; l < p.n_layers; ++l) {

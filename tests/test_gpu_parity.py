@@ -582,6 +582,43 @@ def test_fp32_products_of_extreme_shapes(widths, final, batch):
     gpu.close()
 
 
+@pytest.mark.parametrize("widths,final,rows", [([784, 100, 60], False, 1920), ([300, 81, 33], False, 2112), ([60, 60, 47], True, 2368)])
+def test_small_segment_batches_on_both_sides_of_the_route_limits(widths, final, rows):
+    """Batches that stay with the launches of a small segment and batches that go layer by layer, in turn on one handle (a large
+    one must leave what the next small one relies on), from aligned and from unaligned input, and long responses."""
+    import torch
+    w = wl.WORKLOADS["tiny"]
+    most = 4 * rows + 2500
+    gpu, ora = make_pair(widths, 47, final, "fp32", "momentum", 0.01, most)
+    x, cls = batch_arrays(w, most, widths[0])
+    xt, ct = to_device(x, cls, "fp32")
+    xu = torch.zeros(x.size + 1, device="cuda")[1:].view(most, widths[0])    # four bytes off a 16-byte boundary
+    xu.copy_(xt)
+    def step(t, n):
+        gpu.train_step(t[:n], ct[:n])
+        acts = {l: gpu.activation(l).cpu().numpy() for l in range(1, ora.n_layers + 1)}
+        # among a million units a pre-activation can lie within its fp32 rounding error of zero (outputs agree to 3e-7 of the
+        # largest), and a flipped unit moves 1/n of a gradient: there the oracle follows the stored sign
+        ora.train_step(x[:n], cls[:n], lambda l, z, m: np.where(np.abs(z) <= 1e-6 * np.max(np.abs(z)), acts[l] > 0, m))
+        for l in range(ora.n_layers):
+            for got, ref in zip(gpu.grads(l) + gpu.params(l), (ora.dW[l], ora.db[l], ora.W[l], ora.b[l])):
+                assert rel_err(got.cpu().numpy(), ref) < TOL["fp32"], (n, l)
+
+    for n in (rows, rows + 1, 130, most, 40):
+        step(xt, n)
+    for n in (rows // 2, rows // 2 + 1, rows, rows + 1, 2 * rows + 1, most, 70):
+        ref = ora.forward(x[:n])[-1]
+        for t in (xt, xu):
+            assert rel_err(gpu.forward(t[:n]).cpu().numpy(), ref) < 1e-4, n
+    for batch in (64, 2048, 4096, most):
+        for t in (xt, xu):
+            assert rel_err(gpu.forward_dataset(t, batch).cpu().numpy(), ora.forward(x)[-1]) < 1e-4, batch
+    for n in (rows, most, 33):
+        step(xu, n)
+    gpu.poll()
+    gpu.close()
+
+
 def test_small_segments_created_where_others_were_destroyed():
     """Handles of changing shapes one after the other: each gets device memory an earlier one has freed, and its step must
     not see anything of that one's buffers."""
