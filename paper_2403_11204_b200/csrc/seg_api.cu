@@ -129,7 +129,10 @@ struct seg_handle {
   bool small_fused = false;        // small fp32 segment: the whole step runs as two launches (SEG_NO_SMALL_FUSED=1: off)
   SmallStep small{};               // its description, filled by seg_create (batch is set per launch)
   SmallMaps small_maps{};
-  std::map<int, SmallPrepared*> small_by_batch;
+  // its launches for the row counts used last (a set of any length may pass through seg_forward_dataset: the oldest gives way)
+  static constexpr int kSmallKept = 16;
+  struct SmallKept { int rows = 0; uint64_t used = 0; SmallPrepared* w = nullptr; } small_kept[kSmallKept];
+  uint64_t small_uses = 0;
   bool fuse_update = false;        // SEG_FUSED_UPDATE=1: apply the optimizer inside the weight-gradient product where the
                                    // kernel can (measured slower than the separate update launch, see gemm_tc.cu)
   float* sil = nullptr;
@@ -377,13 +380,18 @@ seg_status refresh_operand_copy(seg_handle* h, int64_t off, int64_t n) {
 
 // The prepared launches of a small fp32 segment for this batch size; nullptr: the segment runs layer by layer.
 SmallPrepared* small_for(seg_handle* h, int batch) {
-  SmallPrepared*& w = h->small_by_batch[batch];
-  if (!w) {
-    SmallStep p = h->small;
-    p.batch = batch;
-    w = small_prepare(p, h->small_maps);
+  seg_handle::SmallKept* oldest = h->small_kept;
+  for (seg_handle::SmallKept& k : h->small_kept) {
+    if (k.w && k.rows == batch) { k.used = ++h->small_uses; return k.w; }
+    if (k.used < oldest->used) oldest = &k;
   }
-  return w;
+  if (oldest->w) small_release(oldest->w);       // its launches have their own copy of the arguments
+  SmallStep p = h->small;
+  p.batch = batch;
+  oldest->w = small_prepare(p, h->small_maps);
+  oldest->rows = batch;
+  oldest->used = ++h->small_uses;
+  return oldest->w;
 }
 
 // Small fp32 segment: staging, forward, loss and the dgrad chain in one launch, every weight and bias gradient with its
@@ -637,7 +645,7 @@ seg_status seg_destroy(seg_handle* h) {
   for (cudaEvent_t e : h->ev_done) if (e) cudaEventDestroy(e);
   for (cudaStream_t ls : h->lstream) if (ls) cudaStreamDestroy(ls);
   for (void* p : h->allocations) cudaFree(p);
-  for (auto& kv : h->small_by_batch) if (kv.second) small_release(kv.second);
+  for (seg_handle::SmallKept& k : h->small_kept) if (k.w) small_release(k.w);
   if (h->host_loss) cudaFreeHost(h->host_loss);
   for (int i = 0; i < 2; ++i) {
     if (h->ev_copied[i]) cudaEventDestroy(h->ev_copied[i]);

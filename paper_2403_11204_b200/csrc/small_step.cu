@@ -1058,7 +1058,6 @@ SmallPrepared* small_prepare(const SmallStep& p, const SmallMaps& maps) {
                         (uint32_t)q.ks, (uint32_t)p.widths[1]);
   }
   if (!ok) { delete w; return nullptr; }
-  plan_wgrad(w);
   return w;
 }
 
@@ -1121,6 +1120,7 @@ cudaError_t launch_small_forward(SmallPrepared& w, const float* x, float* y, boo
 }
 
 cudaError_t launch_small_wgrad_update(SmallPrepared& w, cudaStream_t s) {
+  if (w.tiles == 0) plan_wgrad(&w);              // the first training step of this batch size
   switch (w.a.p.optimizer) {
     case SEG_SGD: return launch_wgrad<SEG_SGD>(w, s);
     case SEG_SGD_MOMENTUM: return launch_wgrad<SEG_SGD_MOMENTUM>(w, s);

@@ -619,6 +619,33 @@ def test_small_segment_batches_on_both_sides_of_the_route_limits(widths, final, 
     gpu.close()
 
 
+def test_response_sets_of_many_lengths_leave_nothing_behind():
+    """A handle that answers sets of ever new lengths keeps the launches of the last few only: host memory stays where it is,
+    and a length that comes back is answered as before."""
+    import resource
+    import torch
+    from paper_2403_11204_b200.binding import Segment
+    seg = Segment([4, 4], 3, False, precision="fp32", max_batch=1)
+    x = torch.rand(20000, 4, device="cuda")
+    y = torch.empty_like(x)
+    first = seg.forward_dataset(x[:777], 1).clone()
+
+    def resident():
+        with open("/proc/self/statm") as f:
+            return int(f.read().split()[1]) * resource.getpagesize()
+    for n in range(2, 2000):
+        seg.forward_dataset(x[:n], 1, y[:n])
+    torch.cuda.synchronize()
+    before = resident()
+    for n in range(2000, 20000):
+        seg.forward_dataset(x[:n], 1, y[:n])
+    torch.cuda.synchronize()
+    assert resident() - before < 8 << 20                 # one plan is about 3 KiB: 18,000 of them would be 50 MiB
+    assert torch.equal(seg.forward_dataset(x[:777], 1), first)
+    seg.poll()
+    seg.close()
+
+
 def test_small_segments_created_where_others_were_destroyed():
     """Handles of changing shapes one after the other: each gets device memory an earlier one has freed, and its step must
     not see anything of that one's buffers."""
