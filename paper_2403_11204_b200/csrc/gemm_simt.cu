@@ -143,7 +143,6 @@ gemm_simt_kernel(GemmDesc g, int k_per_split) {
 // ---- fp32 products by tensor copies and packed FFMA ------------------------------------------------------
 // What bounds it: FFMA issue.  The packed form (fma.rn.f32x2, two multiply-adds per issue slot) leaves issue slots for the
 // shared-memory loads; a plain 8 x 8 loop measures 60-64 % of the FFMA peak, the packed one 64-71 %.
-enum Form : int { FORM_NT = 0, FORM_NN = 1, FORM_TN = 2 };   // operands k-fast / k-fast, k-fast / n-fast, m-fast / n-fast
 constexpr int FT = 64, FK = 32;                             // tile edge, k per stage
 constexpr int FGROUPS = 4, FTHREADS = 64 * FGROUPS;         // four k groups of 64 threads
 // NN and TN have a ninth warp for the copies (71 % of the FFMA peak at 2048^3 in TN form; 61 % when a computing warp issues them);
@@ -500,6 +499,11 @@ int gemm_simt_slots(int M, int N, int K) {
   if (tiles < 1 || tiles > 148) return 0;
   const int splits = std::min(148 / tiles, K / (4 * BK));
   return splits > 1 ? tiles * splits : 0;
+}
+
+int fp32_slots(Form form, int M, int N, int K) {
+  const int slots = gemm_simt_slots(M, N, K);
+  return strided_is_faster(form, ((M + FT - 1) / FT) * ((N + FT - 1) / FT), K, slots) ? slots : 0;
 }
 
 cudaError_t launch_gemm_simt(const GemmDesc& g, int* dev_status, cudaStream_t s) {

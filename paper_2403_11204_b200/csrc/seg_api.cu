@@ -562,18 +562,26 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
     if (env && env[0] == '1') h->fuse_update = true;
   }
   if (!h->use_tc) {
-    // split-K workspaces of the FFMA path, sized for the products each one serves at max_batch
+    // Split-K workspaces of the strided kernel, sized for the products each one serves at max_batch.  fp32 products go to it
+    // where it is the faster one, which a few rows over a wide layer can be and max_batch rows not; so does a forward pass
+    // from rows that tensor copies cannot take, except in a small segment, whose own kernel takes those.
     h->simt_scratch.assign(h->n_layers, nullptr);
     h->simt_counters.assign(h->n_layers, nullptr);
     h->simt_slots.assign(h->n_layers, 0);
     const int B = h->max_batch;
+    const bool fp32 = h->act_dt == DT_F32 && gemm_tc_init();
     for (int l = 0; l < h->n_layers; ++l) {
       const int in = h->widths[l], out = h->widths[l + 1];
-      const int wg = gemm_simt_slots(out, in, B);
-      if (l > 0) h->simt_slots[l] = wg;
-      else h->simt_slots[0] = std::max(h->simt_slots[0], wg);
-      h->simt_slots[0] = std::max(h->simt_slots[0], gemm_simt_slots(B, out, in));            // forward
-      if (l > 0) h->simt_slots[0] = std::max(h->simt_slots[0], gemm_simt_slots(B, in, out)); // dgrad
+      h->simt_slots[l] = std::max(h->simt_slots[l], fp32 ? fp32_slots(FORM_TN, out, in, B) : gemm_simt_slots(out, in, B));
+      int most = 0;                                            // forward and dgrad, on the main branch
+      for (int64_t m = fp32 ? 64 : B; ; m = std::min<int64_t>(2 * m, B)) {
+        const int rows = (int)std::min<int64_t>(m, B);
+        most = std::max(most, fp32 ? fp32_slots(FORM_NT, rows, out, in) : gemm_simt_slots(rows, out, in));
+        if (l > 0) most = std::max(most, fp32 ? fp32_slots(FORM_NN, rows, in, out) : gemm_simt_slots(rows, in, out));
+        if (rows == B) break;
+      }
+      if (fp32 && l == 0 && h->precision == SEG_FP32 && !h->small_fused) most = std::max(most, gemm_simt_slots(B, out, in));
+      h->simt_slots[0] = std::max(h->simt_slots[0], most);
     }
     for (int l = 0; l < h->n_layers; ++l) {
       if (h->simt_slots[l] == 0) continue;

@@ -646,6 +646,19 @@ def test_response_sets_of_many_lengths_leave_nothing_behind():
     seg.close()
 
 
+@pytest.mark.parametrize("widths,batch", [([784, 80, 60], 1410), ([512, 512, 256, 64], 1024)])
+def test_fp32_handles_hold_no_workspace_they_do_not_use(widths, batch):
+    """Device memory of an fp32 handle: parameters, gradients and momentum, staged input, activations and dZ, labels - and at
+    most one layer's split workspace for a forward pass from unaligned rows."""
+    from paper_2403_11204_b200.binding import Segment
+    seg = Segment(widths, 47, False, precision="fp32", optimizer="momentum", max_batch=batch)
+    flat = sum((i + 20) * o + 2 * 64 for i, o in zip(widths, widths[1:])) + sum(widths[1:])
+    need = 4 * (3 * flat + batch * (widths[0] + 16) + batch * 2 * sum(w + 16 for w in widths[1:]) + 47 * widths[-1])
+    unaligned = 148 * 64 * 64 * 4 if max(widths[1:]) > 128 else 0
+    assert seg.mem_bytes()[0] <= need + unaligned + 64 * 1024
+    seg.close()
+
+
 def test_small_segments_created_where_others_were_destroyed():
     """Handles of changing shapes one after the other: each gets device memory an earlier one has freed, and its step must
     not see anything of that one's buffers."""
