@@ -44,7 +44,7 @@
  *                         shared memory and bulk tensor stores)
  *   SEG_PAIR_MIN_TILES=n  use CTA pairs exactly when a product has n or more tiles of 256 x 256
  *                         (default: a cost model of the main loop chooses)
- *   SEG_PAIR_TILE_N=n     columns of such a forced pair's tile, a multiple of 16 from 32 to 256 (default: 256)
+ *   SEG_PAIR_TILE_N=128   such forced pairs take tiles of 128 columns, except where they also apply the update (default: 256)
  *   SEG_DEBUG=1           report on stderr when a step could not be captured into a graph
  */
 #ifndef SEG_H_

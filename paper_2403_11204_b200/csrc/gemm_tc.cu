@@ -1142,7 +1142,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-constexpr int PAIR_TILE_M = 256, PAIR_TILE_N = 256;                   // columns: at most; a launch may take fewer
+constexpr int PAIR_TILE_M = 256, PAIR_TILE_N = 256;                   // columns: a launch may take half of them
 constexpr int PAIR_HALF_N = PAIR_TILE_N / 2;
 constexpr int PAIR_B_BYTES = PAIR_HALF_N * TILE_ROW_BYTES;            // 16 KiB: this CTA's half of B
 constexpr int PAIR_STAGE_BYTES = A_TILE_BYTES + PAIR_B_BYTES;         // 32 KiB per CTA per k-block
@@ -1205,8 +1205,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   // index arithmetic, the first tile's coordinates included: ahead of the dependency wait
   const int tiles_m = (M + PAIR_TILE_M - 1) / PAIR_TILE_M;
   const int tiles_n = (N + tile_n - 1) / tile_n;
-  const int b_chunks = (half_n + CHUNK - 1) / CHUNK;   // MN-major B: whole 128-byte chunks are loaded
-  const uint32_t stage_tx = 2u * (uint32_t)(A_TILE_BYTES + (B_MN ? b_chunks * MN_CHUNK_BYTES : half_n * TILE_ROW_BYTES));
+  const uint32_t stage_tx = 2u * (uint32_t)(A_TILE_BYTES + half_n * TILE_ROW_BYTES);
   const int n_tiles = tiles_m * tiles_n;
   const int num_k = (K + BLOCK_K - 1) / BLOCK_K;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
@@ -1242,7 +1241,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             tma_load_2d_pair(a_dst, &map_a, k0, m0, fb);
           }
           if constexpr (B_MN) {
-            for (int c = 0; c < b_chunks; ++c)
+            for (int c = 0; c < half_n / CHUNK; ++c)
               tma_load_2d_pair(b_dst + c * MN_CHUNK_BYTES, &map_b, n0 + c * CHUNK, k0, fb);
           } else {
             tma_load_2d_pair(b_dst, &map_b, k0, n0, fb);
@@ -1312,9 +1311,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (c + EPI_PER_QUARTER < PAIR_TILE_N / 32) epilogue_prefetch(epi, side_next, row, row < M, col0 + 32 * EPI_PER_QUARTER, N);
         float v[32];
         tmem_load_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * PAIR_TILE_N + c * 32), v);
-        // per-lane stores: where the update warps read the tile back with ordinary loads, and for the half chunk at the end
-        // of a tile that is no multiple of 32 wide (a bf16 box of the bulk store has 32 columns)
-        if (FUSED || !epi.staged || (epi.c_dt == DT_BF16 && col0 + 32 > n_end && n_end < N)) {
+        if (FUSED || !epi.staged) {        // (the update warps read the tile back with ordinary loads: ordinary stores)
           if (row < M) epilogue_store(epi, v, side, row, col0, n_end);
         } else {
           epilogue_store_staged<FUSED ? 2 : 1>(epi, &map_c, my_stage_out, v, side, lane, m0 + quarter * 32, col0, n_end, M, c / EPI_PER_QUARTER);
@@ -1399,7 +1396,7 @@ bool g_allow_splitk = true;
 bool g_allow_pairs = true;
 bool g_allow_fused_update = true;
 bool g_staged_epilogue = true;      // SEG_NO_STAGED_EPILOGUE: per-lane stores instead of shared-memory staging + bulk stores
-int g_pair_tile_n = PAIR_TILE_N;  // SEG_PAIR_TILE_N: columns of a pair's tile where SEG_PAIR_MIN_TILES forces pairs (a multiple of 16 up to 256)
+int g_pair_tile_n = PAIR_TILE_N;  // SEG_PAIR_TILE_N: columns of a pair's tile where SEG_PAIR_MIN_TILES forces pairs (128 or 256)
 long g_pair_min_tiles = 0;      // SEG_PAIR_MIN_TILES: CTA pairs exactly from this many 256 x 256 tiles on (0: cost model)
 
 // 2-D tensor map over a row-major matrix: `inner` contiguous elements per row, `outer` rows,
@@ -1659,7 +1656,7 @@ bool gemm_tc_init() {
     env = getenv("SEG_PAIR_MIN_TILES");
     if (env) g_pair_min_tiles = atol(env);
     env = getenv("SEG_PAIR_TILE_N");
-    if (env && atoi(env) >= 32 && atoi(env) <= PAIR_TILE_N && atoi(env) % 16 == 0) g_pair_tile_n = atoi(env);
+    if (env && atoi(env) == PAIR_HALF_N) g_pair_tile_n = PAIR_HALF_N;
     env = getenv("SEG_NO_STAGED_EPILOGUE");
     if (env && env[0] == '1') g_staged_epilogue = false;
     g_init_ok = true;
