@@ -45,7 +45,7 @@
  *   SEG_PAIR_MIN_TILES=n  use CTA pairs exactly when a product has n or more tiles of 256 x 256
  *                         (default: a cost model of the main loop chooses)
  *   SEG_PAIR_TILE_N=128   such forced pairs take tiles of 128 columns, except where they also apply the update (default: 256)
- *   SEG_DEBUG=1           report on stderr when a step could not be captured into a graph
+ *   SEG_DEBUG=1           report on stderr when a step was captured into a graph, and when it could not be
  */
 #ifndef SEG_H_
 #define SEG_H_

@@ -913,7 +913,8 @@ static seg_status run_step_captured(seg_handle* h, seg_handle::StepGraph& g, seg
     h->capture_stream = nullptr;
   }
   const cudaStream_t record_on = legacy && h->capture_stream ? h->capture_stream : user_stream;
-  if (cudaStreamBeginCapture(record_on, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+  if (cudaError_t b = cudaStreamBeginCapture(record_on, cudaStreamCaptureModeThreadLocal); b != cudaSuccess) {
+    if (getenv("SEG_DEBUG")) fprintf(stderr, "seg: step capture failed (begin-capture '%s')\n", cudaGetErrorString(b));
     cudaGetLastError();
     h->graphs_enabled = false;
     return enqueue(h->fork_enabled);
@@ -936,6 +937,7 @@ static seg_status run_step_captured(seg_handle* h, seg_handle::StepGraph& g, seg
       for (int f = 0; f < FAM_COUNT; ++f) g.family_peer[f] = peer->family_launches[f] - fam_before_peer[f];
     }
     restore_counts();
+    if (getenv("SEG_DEBUG")) fprintf(stderr, "seg: step captured (%llu kernels)\n", (unsigned long long)(g.kernels + g.kernels_peer));
     return replay_graph(h, g, x, cls, loss_to, gather);
   }
   // capture did not work here: run eagerly from now on

@@ -1,5 +1,7 @@
 """Helpers shared by the GPU parity tests: build the CUDA segment and the oracle segment from
 one description, feed both the same seeded arrays, and compare tensor by tensor."""
+import os
+
 import numpy as np
 
 from oracle import rng as orng
@@ -19,11 +21,11 @@ DIST_CODE = {"uniform_kappa": orng.DIST_UNIFORM_KAPPA, "normal": orng.DIST_NORMA
 
 def make_pair(widths, n_classes, is_final, precision, optimizer, lr, max_batch, segment_id=0,
               oracle_precision=None, gemm_backend="auto", label_dist="normal", kappa=10.0,
-              label_seed=wl.LABEL_SEED, init_seed=wl.INIT_SEED, momentum=0.9, last_relu=None):
+              label_seed=wl.LABEL_SEED, init_seed=wl.INIT_SEED, momentum=0.9, last_relu=None, stream=None):
     from paper_2403_11204_b200.binding import Segment
     gpu = Segment(widths, n_classes, is_final, precision=precision, optimizer=optimizer, lr=lr,
                   momentum=momentum, max_batch=max_batch, segment_id=segment_id, init_seed=init_seed,
-                  gemm_backend=gemm_backend, last_relu=last_relu)
+                  gemm_backend=gemm_backend, last_relu=last_relu, stream=stream)
     ora = make_oracle(widths, n_classes, is_final, oracle_precision or precision, optimizer, lr, segment_id,
                       label_dist, kappa, label_seed, init_seed, momentum, last_relu)
     if not is_final:
@@ -104,6 +106,17 @@ def sync_from_oracle(gpu, ora):
         if ora.optimizer == "adam":
             gpu.set_opt_state(l, 1, torch.from_numpy(ora.state2[l]).cuda(), torch.from_numpy(ora.state2[n + l]).cuda())
     gpu.set_step(ora.t)
+
+
+def captured_steps(capfd):
+    """Steps captured into graphs since the last call, as the library reports them under SEG_DEBUG=1; none may have failed."""
+    err = capfd.readouterr().err
+    assert "capture failed" not in err, err
+    return err.count("seg: step captured")
+
+
+def expected_captures(n):
+    return 0 if os.environ.get("SEG_NO_GRAPH") == "1" else n
 
 
 def bits_equal(a, b):

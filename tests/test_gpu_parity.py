@@ -11,8 +11,8 @@ from oracle import rng as orng
 from paper_2403_11204_b200 import workloads as wl
 import os
 
-from parity_util import (batch_arrays, bits_equal, compare_step, make_oracle, make_pair, rel_err, sync_from_oracle,
-                         to_device)
+from parity_util import (batch_arrays, bits_equal, captured_steps, compare_step, expected_captures, make_oracle, make_pair, rel_err,
+                         sync_from_oracle, to_device)
 
 pytestmark = pytest.mark.gpu
 
@@ -350,7 +350,7 @@ def test_fused_update_where_the_cost_model_prefers_narrow_pair_tiles(widths, pre
     gpu.close()
 
 
-def test_product_family_counters_tell_the_backends_apart():
+def test_product_family_counters_tell_the_backends_apart(monkeypatch, capfd):
     """seg_product_launches is what the tensor-core tests rely on to show that tcgen05 kernels ran, so it is
     checked from both sides: a bf16 handle on the automatic or the tensor-core backend counts its five
     products (2 forward, 2 weight-gradient, 1 dgrad) as tensor-core launches and none as FFMA; the same
@@ -361,8 +361,10 @@ def test_product_family_counters_tell_the_backends_apart():
     from paper_2403_11204_b200.binding import Segment
     x = torch.rand(8, 24, device="cuda").to(torch.bfloat16)
     cls = torch.zeros(8, dtype=torch.int32, device="cuda")
+    monkeypatch.setenv("SEG_DEBUG", "1")
+    torch.cuda.synchronize()
     for backend in ("auto", "tcgen05", "simt"):
-        seg = Segment([24, 16, 8], 47, False, precision="bf16", max_batch=8, gemm_backend=backend)
+        seg = Segment([24, 16, 8], 47, False, precision="bf16", max_batch=8, gemm_backend=backend, stream=torch.cuda.Stream())
         seg.gen_labels(1)
         for _ in range(4):                               # eager, captured and replayed steps all count
             seg.train_step(x, cls)
@@ -370,26 +372,32 @@ def test_product_family_counters_tell_the_backends_apart():
         fam = seg.product_launches()
         tc = fam["tc_single"] + fam["tc_splitk"] + fam["tc_pair"]
         assert (fam["ffma"], tc) == ((20, 0) if backend == "simt" else (0, 20)), (backend, fam)
+        assert captured_steps(capfd) == expected_captures(1)
         seg.close()
 
 
-def test_replayed_step_reports_its_own_batch_size():
+def test_replayed_step_reports_its_own_batch_size(monkeypatch, capfd):
     """A step replayed from its captured graph must leave the handle knowing that step's batch size:
     seg_get_activation after it copies exactly that many rows (guard rows behind the buffer stay
     untouched), also when a forward pass at a larger batch ran in between."""
     import torch
     w = wl.WORKLOADS["tiny"]
     A, B = 24, 64
-    gpu, ora = make_pair([784, 128, 64], 47, False, "fp32", "sgd", 0.01, B)
+    monkeypatch.setenv("SEG_DEBUG", "1")
+    # a stream of its own (captured from the second run on) and a layer too wide for the two-launch step, which has no graph
+    gpu, ora = make_pair([784, 160, 64], 47, False, "fp32", "sgd", 0.01, B, stream=torch.cuda.Stream())
     x, cls = batch_arrays(w, B, 784)
     xt, ct = to_device(x, cls, "fp32")
+    torch.cuda.synchronize()
     for _ in range(3):                                   # eager, capture, replay at batch A
         gpu.train_step(xt[:A], ct[:A])
         ora.train_step(x[:A], cls[:A])
+    assert captured_steps(capfd) == expected_captures(1)
     gpu.forward(xt)                                      # batch B in between
     gpu.train_step(xt[:A], ct[:A])                       # replayed
     ora.loss_and_grads(x[:A], cls[:A])
     buf = torch.full((A + 8, 64), -7.0, device="cuda")   # A rows for the call, 8 guard rows behind them
+    torch.cuda.synchronize()
     st = gpu.lib.seg_get_activation(gpu.h, 2, buf.data_ptr())
     assert st == 0
     gpu.poll()
@@ -525,15 +533,17 @@ def test_handles_created_and_used_from_two_threads():
 
 
 @pytest.mark.parametrize("widths,precision,batch", [([72, 200, 136, 64], "tf32", 96), ([200, 160, 96], "fp32", 50)])
-def test_default_stream_step_is_captured_and_replayed(widths, precision, batch):
+def test_default_stream_step_is_captured_and_replayed(widths, precision, batch, monkeypatch, capfd):
     """A handle on the legacy default stream, whose step is captured on a stream of the handle's own after a number of eager
-    runs, must end with the bits of a handle on an ordinary stream; batch size, input and loss address change on the way."""
+    runs, must end with the bits of a handle on an ordinary stream; batch size, input and loss address change on the way.
+    Both handles capture both batch sizes."""
     import torch
     from paper_2403_11204_b200.binding import Segment
     w = wl.WORKLOADS["tiny"]
     x, cls = batch_arrays(w, 4 * batch, widths[0])
     xt, ct = to_device(x, cls, precision)
     results = []
+    monkeypatch.setenv("SEG_DEBUG", "1")
     for stream in (None, torch.cuda.Stream()):
         seg = Segment(widths, 47, False, precision=precision, optimizer="adam", lr=1e-3, max_batch=batch, stream=stream)
         seg.gen_labels(wl.LABEL_SEED, "normal")
@@ -546,6 +556,7 @@ def test_default_stream_step_is_captured_and_replayed(widths, precision, batch):
         out = [loss.cpu().numpy()] + [t.cpu().numpy() for l in range(len(widths) - 1) for t in seg.params(l)]
         results.append(out)
         seg.close()
+        assert captured_steps(capfd) == expected_captures(2)
     for a, b in zip(*results):
         assert bits_equal(a, b)
 
