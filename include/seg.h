@@ -184,7 +184,8 @@ SEG_API seg_status seg_train_step_host_async(seg_handle* h, const void* x_host, 
 
 /* Forward pass only (the response handed to the next segment, Section 2):
  *   y [batch][widths[n_layers]]: float for FP32/TF32 and for the logits of a final
- *   segment, bf16 for a non-final BF16 segment.                                           */
+ *   segment, bf16 for a non-final BF16 segment.  y may share memory with x: x is read before
+ *   the response takes its place.                                                           */
 SEG_API seg_status seg_forward(seg_handle* h, const void* x, int32_t batch, void* y);
 
 /* Epoch driver (Section 2, both phases): trains the segment for `epochs` passes over a
@@ -197,8 +198,11 @@ SEG_API seg_status seg_train_epochs(seg_handle* h, const void* x, const int32_t*
                                     int32_t batch, int32_t epochs, float* losses);
 
 /* The stored response of a trained segment over a whole data set (Section 2: the left
- * partition's final response, which is the next partition's input): seg_forward over
- * consecutive chunks of `batch` rows.  y [n][widths[n_layers]], dtype as for seg_forward. */
+ * partition's final response, which is the next partition's input).  y [n][widths[n_layers]],
+ * dtype as for seg_forward.  The last chunk of `batch` rows (or the partial one) is a
+ * seg_forward: seg_get_activation afterwards refers to it.  How the rows before it are grouped
+ * is the library's choice; a row's response equals seg_forward's up to the rounding of a
+ * different order of summation, not bit for bit.                                            */
 SEG_API seg_status seg_forward_dataset(seg_handle* h, const void* x, int64_t n, int32_t batch, void* y);
 
 /* Recovery step (Section 5, "recovery epochs"): after both partitions are trained, the

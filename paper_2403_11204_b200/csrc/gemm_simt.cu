@@ -141,12 +141,14 @@ gemm_simt_kernel(GemmDesc g, int k_per_split) {
 }
 
 // ---- fp32 products by tensor copies and packed FFMA ------------------------------------------------------
-// What bounds it: FFMA issue.  The packed form (fma.rn.f32x2, two multiply-adds per issue slot) leaves issue slots for the
-// shared-memory loads; a plain 8 x 8 loop measures 60-64 % of the FFMA peak, the packed one 64-71 %.
+// What bounds it: FFMA issue beside the loads of 8 x 8 tiles from shared memory.  Packed multiply-adds (fma.rn.f32x2, two per
+// issue slot) leave slots for the loads.  At 2048^3 / 4096^3: NT 37.6 / 39.7 TFLOP/s, NN 42.2 / 43.6, TN 49.2 / 51.2, 53 to 72 %
+// of the 71.5 that a loop of multiply-adds alone reaches.
 constexpr int FT = 64, FK = 32;                             // tile edge, k per stage
 constexpr int FGROUPS = 4, FTHREADS = 64 * FGROUPS;         // four k groups of 64 threads
-// NN and TN have a ninth warp for the copies (71 % of the FFMA peak at 2048^3 in TN form; 61 % when a computing warp issues them);
-// NT does without: nine warps leave a thread 168 registers, its 64 pairs of sums need more (53 % against 46 % with plain FFMA).
+// NN and TN have a ninth warp that issues the tensor copies (TN at 2048^3 falls from 49 to 43 TFLOP/s when a computing warp issues
+// them); NT does without: nine warps leave a thread 168 registers, its 64 pairs of sums need more (38 TFLOP/s against 33 with
+// the ninth warp and plain multiply-adds).
 __host__ __device__ constexpr int ffma_threads(int form) { return FTHREADS + (form == 0 ? 0 : 32); }
 constexpr int FSTAGES = 6, FSTAGE_FLOATS = 2 * FT * FK;     // 16 KiB per stage
 constexpr int FPART = FT + 8;                               // row pitch of a partial tile: conflict-free stores in every form
@@ -487,7 +489,7 @@ double ffma_estimate_us(int M, int N, int K) {
 }
 
 // The copy: a launch of about 3 us and 8 bytes per element at about 3 TB/s.  784-80-60 at 8192 rows, us: 85 with the strided first
-// layer, 62 with aligned rows.
+// layer, 72 with the copy (63 from aligned rows).
 bool fp32_staging_pays(int M, int N, int K, int slots) {
   const int tiles = ((M + FT - 1) / FT) * ((N + FT - 1) / FT);
   return strided_cycles(tiles, K, slots) / 1900.0 > copies_cycles(FORM_NT, tiles, K) / 1900.0 + 3.0 + 8.0 * M * K / 3e6;

@@ -1627,8 +1627,8 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_u
     } else if (us < best.us) {
       best = Choice{1, PAIR_HALF_N, us};
     }
-    // Fewer than half as many 256-column tiles as pairs: tiles of 128 columns give every pair one (a k-block takes 0.18 us instead
-    // of 0.30).  1024 x 2048 x 4096: 18.3 us against 25.8 with 256 columns and 19.6 with one CTA per 128 x 128 tile.
+    // Fewer than half as many 256-column tiles as pairs: tiles of 128 columns give every pair one (a k-block takes 0.18 us; of
+    // 256 columns 0.267 where tiles fill the GPU, as above, and 0.30 where half of the pairs have none).  1024 x 2048 x 4096: 18.3 us against 25.8 with 256 columns and 19.6 with one CTA per 128 x 128 tile.
     if (g_pair_min_tiles == 0 && !throughput && !fused_update && 2 * tiles <= pairs) {
       const double us128 = num_k * 0.18 + 4.5;
       if (us128 < best.us) best = Choice{1, PAIR_HALF_N / 2, us128};

@@ -875,6 +875,9 @@ static seg_status replay_graph(seg_handle* h, seg_handle::StepGraph& g, const vo
 // more as it will, so that a short pass over a new handle, or the partial batch at the end of a few epochs, does not pay for
 // one.  First 40 steps of a new handle, captured after 24 and not at all: 512-512-256-47 (TF32, batch 256) 2.61 and 2.19 ms,
 // 784-300-100-47 (batch 128) 2.20 and 2.08, 512-1024-768-47 (bf16, batch 512) 2.32 and 2.30, 784-1024-1024-47 2.59 and 2.75.
+// Longer runs: 300 steps of these four 14.3, 14.6, 15.3 and 17.6 ms, without a graph 15.1, 16.6, 16.6 and 19.7.  On a stream of
+// the caller's own the second run is captured: short runs pay a quarter of a millisecond there, longer ones have their gain from
+// the start (16 / 40 / 100 steps of the first 1.18 / 2.22 / 4.91 ms, without a graph 0.94 / 2.31 / 5.08).
 constexpr int kLegacyEagerRuns = 48;
 
 // Runs one step through its captured graph: the first call with this graph slot (the first kLegacyEagerRuns calls on the

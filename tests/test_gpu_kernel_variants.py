@@ -38,8 +38,8 @@ def test_tensor_core_cases_with_forced_kernel_selection(env):
 
 @pytest.mark.parametrize("env", [{"SEG_NO_SMALL_FUSED": "1"}, {"SEG_NO_GRAPH": "1"}, {"SEG_NO_PDL": "1"}])
 def test_fp32_cases_with_switches(env):
-    """The fp32 cases once more: launch by launch (no two-launch step for small segments), and the two-launch step
-    without the captured graph and without programmatic dependent launches."""
+    """The fp32 cases once more: launch by launch (no two-launch step for small segments), wider segments without the
+    captured graph, and all without programmatic dependent launches."""
     child_env = dict(os.environ, **env)
     res = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_parity.py", "-m", "gpu", "-q", "-x",
                           "-k", "fp32 or tiny or reproducible or replayed or class_index"], cwd=ROOT, env=child_env,
