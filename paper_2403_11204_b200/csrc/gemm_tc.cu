@@ -56,12 +56,12 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "tc_ops.cuh"
 
 namespace segk {
 namespace {
 
 constexpr int BLOCK_M = 128;
-constexpr int TILE_ROW_BYTES = 128;                    // one swizzle row
 constexpr int A_TILE_BYTES = BLOCK_M * TILE_ROW_BYTES; // 16 KiB per stage
 constexpr int NUM_THREADS = 192;                       // TMA warp, MMA warp, four epilogue warps
 constexpr int UPDATE_WARPS = 8;                        // fused-update variants: eight more warps stream the optimizer update
@@ -81,143 +81,6 @@ constexpr int HALF_SM_SMEM = 113 * 1024;               // two CTAs of this size 
 constexpr int STAGE_OUT_WARP_BYTES = 32 * 64;          // one buffer of one warp
 constexpr int STAGE_OUT_BYTES = 4 * 2 * STAGE_OUT_WARP_BYTES;   // 16 KiB
 constexpr int PAIR_STAGE_OUT_BYTES = STAGE_OUT_BYTES;           // eight epilogue warps with one buffer each
-constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;
-
-// ---- PTX wrappers ------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_timer_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait.  Returns false when the wait was abandoned (own time-out or another role's abort).
-// The product kernels pass the compile-time limit; the self-test kernel passes a short one.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          int* dev_status, uint64_t limit_ns = WAIT_LIMIT_NS) {
-  uint32_t spins = 0;
-  uint64_t t0 = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 0xFFu) == 0u) {
-      if (*abort_flag) return false;
-      const uint64_t now = global_timer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) {
-        *abort_flag = 1;
-        atomicOr(dev_status, (int)DEV_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
-}
-// True for exactly one thread of a converged warp.  The threads that issue TMA loads, MMAs and commits are chosen with it:
-// those instructions take their operands from uniform registers, and only behind elect.sync does the compiler know that one
-// thread is active and issue them directly; behind `lane == 0` it wraps each in a loop over the active threads.  Measured:
-// eight expect-and-copy pairs are issued in 92 cycles against 474; 1024-row responses of 784-4096-4096-2048 take 2561 us
-// against 2782 (33 chunks), a step of 512-1024-768-512 (bf16, batch 512) 54.3 us against 61.2, and the split-K kernel's
-// three sends to its peers bring a step of 784-1024-1024-512 (TF32, batch 256) from 57.5 to 56.8.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar) : "memory");
-}
-// bulk tensor store shared -> global of one box (clipped to the tensor's extent), tracked by the thread's bulk groups
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c0), "r"(c1) : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// at most one of this thread's bulk stores may still be reading its shared-memory source
-__device__ __forceinline__ void tma_store_wait_source_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-// none of them may
-__device__ __forceinline__ void tma_store_wait_source() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// all of this thread's bulk stores are complete
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols) : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-template <bool TF32>
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  if constexpr (TF32) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  }
-}
-// 32 lanes x 32 columns of fp32: thread i of the warp receives row (lane base + i), 32 columns.
-__device__ __forceinline__ void tmem_load_32x32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Shared-memory matrix descriptor (sm_100 format): start address, leading / stride byte offsets
-// in 16-byte units, descriptor version 1, 128-byte swizzle.
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes,
-                                                   uint32_t layout_type) {
-  uint64_t d = 0;
-  d |= (uint64_t)((smem_addr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;   // descriptor version
-  d |= (uint64_t)layout_type << 61;   // 2: 128-byte swizzle; 1: 128-byte swizzle, 32-byte atoms
-  return d;
-}
 
 // Tile order of the persistent kernels.  Tiles are numbered in groups of `group_m` rows of tiles: inside a
 // group the row index runs fastest, then the column index, and the groups follow each other.  The CTAs (or pairs)
@@ -449,73 +312,6 @@ __device__ __forceinline__ void epilogue_store_staged(const EpilogueArgs& e, con
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0 && row0 < n_rows) tma_store_2d(map_c, smem_u32(buf), col0 + 16 * h, row0);
-    }
-  }
-}
-
-// ---- fused loss (last forward product of a non-final segment) -----------------------------------
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  return v;
-}
-
-// Targets of n_cols (<= 32) consecutive columns of one row: row cls[row] of the label matrix, whose
-// pitch is n_p.  Fetched ahead of the accumulator like the other side inputs.
-template <int NV = 32>
-__device__ __forceinline__ void loss_prefetch_target(const LossFuse& l, EpiSide& t, int row, bool row_ok, int col0,
-                                                     int n_cols, int n_p) {
-  if (n_cols <= 0 || !row_ok) return;
-  const float* trow = l.sil + (int64_t)__ldg(l.cls + row) * n_p + col0;
-  if (((n_cols & 3) == 0) && ((reinterpret_cast<uintptr_t>(trow) & 15u) == 0)) {
-#pragma unroll
-    for (int j = 0; j < NV; j += 4) {
-      if (j < n_cols) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(trow + j));
-        t.w[j] = q.x; t.w[j + 1] = q.y; t.w[j + 2] = q.z; t.w[j + 3] = q.w;
-      }
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) if (j < n_cols) t.w[j] = __float_as_uint(__ldg(trow + j));
-  }
-}
-
-// Mean-squared-error part of the epilogue for columns [col0, n_end): stores the output, then
-// dZ = gscale (a - t) [a > 0], and adds (a - t)^2 to the thread's loss sum; a is the output as it
-// is stored (after rounding to the storage type).
-template <int NV>
-__device__ __forceinline__ void epilogue_store_mse(const EpilogueArgs& e, float (&v)[NV], const EpiSide& s,
-                                                   const EpiSide& t, int row, int col0, int n_end, float& lacc) {
-  epilogue_values(e, v, s, col0, n_end);
-  store_row_segment(e.C, e.c_dt, e.ldc, v, row, col0, n_end);
-  const int n_valid = min(NV, n_end - col0);
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    if (j < n_valid) {
-      const float a = (e.c_dt == DT_BF16) ? round_bf16_rne(v[j]) : v[j];
-      const float d = a - __uint_as_float(t.w[j]);
-      lacc = fmaf(d, d, lacc);
-      float g = d * e.loss.gscale;
-      if (e.loss.relu_mask && !(a > 0.f)) g = 0.f;
-      v[j] = apply_round(g, e.loss.dz_round);
-    }
-  }
-  store_row_segment(e.loss.dz, e.loss.dz_dt, e.loss.ld_dz, v, row, col0, n_end);
-}
-
-// End of a CTA's epilogue: the four epilogue warps leave their loss sums in shared memory; the last
-// warp to arrive adds them in warp order and publishes the CTA's partial (the step's last update launch adds the
-// partials in index order: bit-reproducible).  No barrier is used, so a warp that gave up a bounded wait cannot block the others.
-__device__ __forceinline__ void loss_finish(const LossFuse& l, float lacc, int quarter, int lane, volatile float* slots,
-                                            unsigned int* warp_counter) {
-  const float w = warp_sum_f(lacc);
-  if (lane == 0) {
-    slots[quarter] = w;
-    __threadfence_block();
-    if (atomicAdd(warp_counter, 1u) == 3u) {
-      __threadfence_block();
-      l.partials[blockIdx.x] = ((slots[0] + slots[1]) + slots[2]) + slots[3];
     }
   }
 }
@@ -851,30 +647,76 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t rank) {
   uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank)); return r;
 }
-// bulk copy from this CTA's shared memory into a peer's; completes (by bytes) on the peer's mbarrier
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster_addr, uint32_t src_local_addr,
-                                                  uint32_t bytes, uint32_t bar_cluster_addr) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst_cluster_addr), "r"(src_local_addr), "r"(bytes), "r"(bar_cluster_addr) : "memory");
-}
 constexpr int SPLITK_BLOCK_N = 64;
-// Three stages, and the send buffer takes the ring's place once the accumulator is complete: 106 KiB per CTA, so that two CTAs
-// share an SM.  What that buys is not this kernel's own time but its neighbours': the next kernel's prologue runs beside it, and
-// a weight gradient on another branch no longer keeps the dgrad chain's clusters waiting for whole SMs.
+// Three stages: 106 KiB per CTA, so that two CTAs share an SM.  What that buys is not this kernel's own time but its neighbours':
+// the next kernel's prologue runs beside it, and a weight gradient on another branch does not keep the dgrad chain's clusters
+// waiting for whole SMs.
 constexpr int SPLITK_STAGES = 3;
 constexpr int SPLITK_STAGE_BYTES = A_TILE_BYTES + SPLITK_BLOCK_N * TILE_ROW_BYTES;       // 24 KiB
-constexpr int SPLITK_RECV_BYTES = 8 * (SPLITK_BLOCK_N / 8) * BLOCK_M * 4;                // [src][col in slice][row] fp32, 32 KiB
+constexpr int SPLITK_RECV_BYTES = SPLITK_BLOCK_N * BLOCK_M * 4;                          // [src][row][pieces of the slice], 32 KiB
 constexpr int SPLITK_SMEM = SPLITK_STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES + SMEM_EXTRA;
-static_assert(SPLITK_STAGES * SPLITK_STAGE_BYTES >= SPLITK_RECV_BYTES, "the send buffer fits into the ring");
+constexpr int SPLITK_THREADS = 320, SPLITK_EPI_THREADS = 256;                            // eight epilogue warps
+constexpr int CE_SPLIT = 4;                                // CTAs per cluster of a product that forms the cross-entropy too
 
-// One 128 x 64 output tile per cluster; CTA r of the cluster contracts k-blocks [r*kpc, (r+1)*kpc).
-template <bool TF32, bool A_MN, bool B_MN, int SPLIT, bool LOSS = false>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+// 16 bytes (8 bytes) into a peer's shared memory; they complete (by bytes) on the peer's mbarrier.
+__device__ __forceinline__ void send_to_peer(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send_to_peer(uint32_t addr, uint32_t bar, float a, float b) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
+}
+
+// Up to four consecutive columns of one row.
+__device__ __forceinline__ float4 load_piece(const float* src, int n, bool wide) {
+  if (wide) return __ldg(reinterpret_cast<const float4*>(src));
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (n > 0) v.x = __ldg(src);
+  if (n > 1) v.y = __ldg(src + 1);
+  if (n > 2) v.z = __ldg(src + 2);
+  if (n > 3) v.w = __ldg(src + 3);
+  return v;
+}
+__device__ __forceinline__ void store_piece(void* base, int dt, int64_t at, const float (&v)[4], int n, bool wide) {
+  if (dt == DT_BF16) {
+    __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(base) + at;
+    if (wide) {
+      __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+      uint2 q;
+      q.x = *reinterpret_cast<uint32_t*>(&lo); q.y = *reinterpret_cast<uint32_t*>(&hi);
+      *reinterpret_cast<uint2*>(d) = q;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) if (j < n) d[j] = __float2bfloat16_rn(v[j]);
+    }
+  } else {
+    float* d = reinterpret_cast<float*>(base) + at;
+    if (wide) *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+    else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) if (j < n) d[j] = v[j];
+    }
+  }
+}
+
+// One 128 x 64 output tile per cluster (SPLIT = 1: per CTA, nothing to exchange); CTA r of the cluster contracts k-blocks
+// [r*kpc, (r+1)*kpc).
+//
+// The exchange.  A warp holds 32 rows x 32 columns of the partial tile and sends each piece of four columns straight from its
+// registers to the CTA that owns them (st.async, counted by the owner's barrier; pieces of a row swizzled, so that the eight lanes
+// of a phase reach different banks); a thread of the owner then finishes pieces of rows that follow each other, four to sixteen to
+// a row, so that outputs, masks and targets move in row segments of 64 to 256 bytes.
+template <bool TF32, bool A_MN, bool B_MN, int SPLIT, int LOSS = LOSS_NONE>
+__global__ void __launch_bounds__(SPLITK_THREADS, 2)
 gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                       int M, int N, int K, EpilogueArgs epi, int* dev_status) {
   constexpr int split = SPLIT;                             // CTAs per cluster
   constexpr int W = SPLITK_BLOCK_N / SPLIT;                // columns of the tile each CTA owns after the exchange
-  static_assert(W == 32 || W == 16 || W == 8, "slice width");
+  static_assert(W == 64 || W == 32 || W == 16, "slice width");
+  constexpr int PPR = W / 4;                               // pieces per row of the slice
+  constexpr int PER_THREAD = BLOCK_M * PPR / SPLITK_EPI_THREADS;
+  constexpr int ROW_STEP = SPLITK_EPI_THREADS / PPR;       // rows between a thread's pieces
   constexpr int BLOCK_N = SPLITK_BLOCK_N;
   constexpr int STAGES = SPLITK_STAGES;
   constexpr int B_TILE_BYTES = BLOCK_N * TILE_ROW_BYTES;
@@ -888,22 +730,23 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* smem_a = smem;
   uint8_t* smem_b = smem + STAGES * A_TILE_BYTES;
-  float* recv = reinterpret_cast<float*>(smem + STAGES * SPLITK_STAGE_BYTES);                      // [src][col in slice][row]
-  float* send = reinterpret_cast<float*>(smem);                        // [dest][col in slice][row], in the ring's place
+  uint8_t* recv = smem + STAGES * SPLITK_STAGE_BYTES;      // [src][row][piece]
+  float2* stats = reinterpret_cast<float2*>(smem);         // LOSS_CE: [src][row] maximum and sum, in the ring's place (who sends them has had this CTA's sums)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES);
-  // bars[0..S) full, [S..2S) empty, [2S] accumulator complete, [2S+1] partial slices received
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
+  // bars[0..S) full, [S..2S) empty, [2S] accumulator complete, [2S+1] partial slices received, [2S+2] row statistics received
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 3);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile float* loss_slots = reinterpret_cast<volatile float*>(reinterpret_cast<uint8_t*>(bars) + 256);
-  unsigned int* loss_warps = reinterpret_cast<unsigned int*>(reinterpret_cast<uint8_t*>(bars) + 272);
+  volatile float* loss_slots = reinterpret_cast<volatile float*>(reinterpret_cast<uint8_t*>(bars) + 128);
+  unsigned int* loss_warps = reinterpret_cast<unsigned int*>(reinterpret_cast<uint8_t*>(bars) + 192);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
+  const uint32_t rank = split > 1 ? cluster_ctarank() : 0u;
   const uint32_t bar_base = smem_u32(bars);
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   const uint32_t acc_bar = bar_base + 8u * (2 * STAGES);
   const uint32_t recv_bar = bar_base + 8u * (2 * STAGES + 1);
+  const uint32_t stats_bar = bar_base + 8u * (2 * STAGES + 2);
 
   if (threadIdx.x == 0) {
     prefetch_tensormap(&map_a);       // descriptor fetch overlaps the rest of the prologue
@@ -911,17 +754,19 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(acc_bar, 1);
     mbar_init(recv_bar, 1);
+    mbar_init(stats_bar, 1);
     *abort_flag = 0;
     *loss_warps = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // this CTA will receive one column slice (BLOCK_N / split columns x 128 rows, fp32) from every peer
-    mbar_arrive_expect_tx(recv_bar, (uint32_t)((split - 1) * (BLOCK_N / split) * BLOCK_M * 4));
+    if (split > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)((split - 1) * W * BLOCK_M * 4));
+    if (LOSS == LOSS_CE) mbar_arrive_expect_tx(stats_bar, (uint32_t)((split - 1) * BLOCK_M * 8));
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
   tc_fence_before();
   __syncthreads();
-  cluster_arrive();                   // "my barriers are initialised"; the matching wait sits in front of the
+  if (split > 1) cluster_arrive();    // "my barriers are initialised"; the matching wait sits in front of the
   tc_fence_after();                   // first remote access (the slice exchange), off the main loop's path
   const uint32_t tmem_base = *tmem_slot;
   // tile and k-range of this CTA: index arithmetic only, done while the previous kernel drains
@@ -1007,97 +852,225 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         else mbar_arrive(acc_bar);          // nothing to contract: the epilogue treats the partial as zero
       }
     }
+    __syncwarp();
+    asm volatile("bar.sync 2, 288;" ::: "memory");         // the epilogue warps have drained the accumulator
+    tc_fence_after();
+    tmem_dealloc(tmem_base, TMEM_COLS);
   } else {
     // ---------------- epilogue warps: reduce-scatter across the cluster, then the usual epilogue ------------
     if (warp == 2 && elect_one()) {                        // first: the B tiles of the main loop (see above)
       int stage = 0; uint32_t phase = 0;
       for (int kb = kb_begin; kb < kb_end; ++kb) {
-        // the first pass over the ring finds every stage free: no wait (a wait that passes at once still costs a
-        // couple of hundred cycles of the issuing thread)
         if (kb - kb_begin >= STAGES && !mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, dev_status)) break;
         if (kb - kb_begin >= early) load_b(stage, kb);
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
     __syncwarp();
-    const int quarter = warp & 3;
-    const int row_in_tile = quarter * 32 + lane;
-    const int row = m0 + row_in_tile;
-    constexpr int w = W;                                   // columns owned by each CTA: 32, 16 or 8
-    const int own_col0 = n0 + (int)rank * w;
-    EpiSide side, tgt;                                     // side inputs of this CTA's slice, fetched ahead
-    epilogue_prefetch<W>(epi, side, row, row < M, own_col0, min(N, own_col0 + w));
-    if constexpr (LOSS) loss_prefetch_target<W>(epi.loss, tgt, row, row < M, own_col0, min(w, N - own_col0), N);
-    float lacc = 0.f;
-    bool ok = mbar_wait(acc_bar, 0, abort_flag, dev_status);
-    tc_fence_after();
-    const uint32_t slice_bytes = (uint32_t)(w * BLOCK_M * 4);
-    float own[W];                                          // this CTA's slice of the tile
+    // this thread's pieces of the CTA's slice: rows er + i * ROW_STEP, the same four columns each
+    const int ut = threadIdx.x - 64, ep = ut % PPR, er = ut / PPR;
+    const int col = n0 + (int)rank * W + 4 * ep, n_cols = min(4, N - col);   // <= 0: beyond the matrix
+    const bool whole = n_cols == 4;
+    // what the epilogue needs from memory, fetched ahead of the accumulator
+    const bool c_wide = whole && (epi.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(epi.C) & 15u) == 0;
+    const bool m_wide = whole && (epi.ldmask & 3) == 0 && (reinterpret_cast<uintptr_t>(epi.mask) & 15u) == 0;
+    float4 bias4 = make_float4(0.f, 0.f, 0.f, 0.f), side[PER_THREAD];
+    if (epi.epi == EPI_BIAS_ACT && n_cols > 0)
+      bias4 = load_piece(epi.bias + col, n_cols, whole && (reinterpret_cast<uintptr_t>(epi.bias + col) & 15u) == 0);
+    int cls[PER_THREAD];
 #pragma unroll
-    for (int j = 0; j < W; ++j) own[j] = 0.f;
-    if (ok) {
-#pragma unroll 1
-      for (int c = 0; c < BLOCK_N / 32; ++c) {
-        float v[32];
-        if (my_k > 0) {
-          tmem_load_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(c * 32), v);
+    for (int i = 0; i < PER_THREAD; ++i) {
+      const int row = m0 + er + i * ROW_STEP;
+      side[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      cls[i] = 0;
+      if (row >= M) continue;
+      if (epi.epi == EPI_MASK && n_cols > 0) {             // the stored activations that give the ReLU mask
+        if (epi.c_dt == DT_F32) {
+          side[i] = load_piece(reinterpret_cast<const float*>(epi.mask) + (int64_t)row * epi.ldmask + col, n_cols, m_wide);
         } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = 0.f;
-        }
-        // column c*32+j belongs to CTA (c*32+j)/w; the send buffer is [dest][col in slice][row], which is
-        // simply [column][row]: consecutive lanes write consecutive floats
-#pragma unroll
-        for (int j = 0; j < 32; ++j) send[(c * 32 + j) * BLOCK_M + row_in_tile] = v[j];
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the bulk copies
-      cluster_wait();                                                // every peer's receive barrier exists
-      asm volatile("bar.sync 1, 128;" ::: "memory");                 // the four epilogue warps
-      if (warp == 2) {
-        if (elect_one()) {
-          for (uint32_t d = 1; d < (uint32_t)split; ++d) {
-            const uint32_t dest = (rank + d) & (uint32_t)(split - 1);
-            const uint32_t src = smem_u32(send + (int)dest * w * BLOCK_M);
-            const uint32_t dst = map_to_cta(smem_u32(recv + (int)rank * w * BLOCK_M), dest);
-            bulk_copy_to_peer(dst, src, slice_bytes, map_to_cta(recv_bar, dest));
+          const unsigned short* m = reinterpret_cast<const unsigned short*>(epi.mask) + (int64_t)row * epi.ldmask + col;
+          uint2 q = make_uint2(0u, 0u);
+          if (m_wide) q = __ldg(reinterpret_cast<const uint2*>(m));
+          else {
+            if (n_cols > 0) q.x = __ldg(m);
+            if (n_cols > 1) q.x |= (uint32_t)__ldg(m + 1) << 16;
+            if (n_cols > 2) q.y = __ldg(m + 2);
+            if (n_cols > 3) q.y |= (uint32_t)__ldg(m + 3) << 16;
           }
+          side[i] = make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xFFFF0000u), __uint_as_float(q.y << 16),
+                                __uint_as_float(q.y & 0xFFFF0000u));
         }
       }
-      ok = mbar_wait(recv_bar, 0, abort_flag, dev_status);
-    } else {
+      if constexpr (LOSS != LOSS_NONE) cls[i] = __ldg(epi.loss.cls + row);
+      if (LOSS == LOSS_MSE && n_cols > 0) {                // the label row of the sample's class
+        const float* t = epi.loss.sil + (int64_t)cls[i] * N + col;
+        side[i] = load_piece(t, n_cols, whole && (reinterpret_cast<uintptr_t>(t) & 15u) == 0);
+      }
+    }
+    float lacc = 0.f;
+    bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_bar, 0, abort_flag, dev_status));
+    tc_fence_after();
+    if (ok) {
+      // a warp reads the TMEM lanes of its index modulo 4; the two warps of a quarter take half of the columns each
+      const int quarter = warp & 3, half = (warp - 2) >> 2, row = quarter * 32 + lane;
+      float v[32];
+      if (my_k > 0) {
+        tmem_load_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 32), v);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = 0.f;
+      }
+      tc_fence_before();
+      if (split > 1) cluster_wait();                       // every peer's receive barrier exists
+      const uint32_t share = (uint32_t)(((int)rank * BLOCK_M + row) * PPR) * 16u;   // this CTA's share of the row, in any CTA
+      const int sw = W == 16 ? (row >> 1) & 3 : row & 7;
+      constexpr int OWNERS = W >= 32 ? 1 : 32 / W, RUN = W >= 32 ? 8 : PPR;   // owners of this warp's 32 columns, pieces for each
+#pragma unroll
+      for (int o = 0; o < OWNERS; ++o) {
+        const uint32_t owner = split == 1 ? 0u : (uint32_t)(half * OWNERS + o);
+        const uint32_t dst = split == 1 ? 0u : map_to_cta(smem_u32(recv) + share, owner);
+        const uint32_t bar = split == 1 ? 0u : map_to_cta(recv_bar, owner);
+        const int c0 = split == 1 ? half * 8 : 0;
+#pragma unroll
+        for (int c = 0; c < RUN; ++c) {
+          const float* x = v + o * W + 4 * c;
+          const uint32_t at = (uint32_t)((c0 + c) ^ sw) * 16u;
+          if (owner == rank) *reinterpret_cast<float4*>(recv + share + at) = make_float4(x[0], x[1], x[2], x[3]);
+          else send_to_peer(dst + at, bar, x[0], x[1], x[2], x[3]);
+        }
+      }
+    } else if (split > 1) {
       cluster_wait();
     }
-    cluster_arrive();                   // "I have received everything": completes under the epilogue, waited for at the end
+    asm volatile("bar.arrive 2, 288;" ::: "memory");       // drained: warp 1 gives the tensor memory back
+    asm volatile("bar.sync 1, 256;" ::: "memory");         // the own share is in place
+    if (split > 1) ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(recv_bar, 0, abort_flag, dev_status));
+    float x[PER_THREAD][4];
+#pragma unroll
+    for (int i = 0; i < PER_THREAD; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[i][j] = 0.f;
     if (ok) {
 #pragma unroll
-      for (int cs = 0; cs < W; ++cs) own[cs] = send[((int)rank * w + cs) * BLOCK_M + row_in_tile];
-      for (int src = 0; src < split; ++src) {
-        if ((uint32_t)src == rank) continue;
+      for (int i = 0; i < PER_THREAD; ++i) {
+        const int row = er + i * ROW_STEP;
+        const int sw = W == 16 ? (row >> 1) & 3 : row & 7;
+        const uint8_t* at = recv + (row * PPR + (ep ^ sw)) * 16;
+        float4 s = *reinterpret_cast<const float4*>(at);
 #pragma unroll
-        for (int cs = 0; cs < W; ++cs) own[cs] += recv[(src * w + cs) * BLOCK_M + row_in_tile];
+        for (int src = 1; src < split; ++src) {
+          const float4 t = *reinterpret_cast<const float4*>(at + src * BLOCK_M * PPR * 16);
+          s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+        }
+        x[i][0] = s.x; x[i][1] = s.y; x[i][2] = s.z; x[i][3] = s.w;
+        if (epi.epi == EPI_BIAS_ACT) {
+          x[i][0] += bias4.x; x[i][1] += bias4.y; x[i][2] += bias4.z; x[i][3] += bias4.w;
+          if (epi.relu) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[i][j] = fmaxf(x[i][j], 0.f);
+          }
+        } else if (epi.epi == EPI_MASK) {
+          if (!(side[i].x > 0.f)) x[i][0] = 0.f;
+          if (!(side[i].y > 0.f)) x[i][1] = 0.f;
+          if (!(side[i].z > 0.f)) x[i][2] = 0.f;
+          if (!(side[i].w > 0.f)) x[i][3] = 0.f;
+        }
+        if (epi.c_round == RND_TF32) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[i][j] = round_tf32_rne(x[i][j]);
+        }
+        if (m0 + row < M && n_cols > 0) store_piece(epi.C, epi.c_dt, (int64_t)(m0 + row) * epi.ldc + col, x[i], n_cols, c_wide);
       }
-      if (row < M && own_col0 < N) {
-        if constexpr (LOSS) epilogue_store_mse(epi, own, side, tgt, row, own_col0, min(N, own_col0 + w), lacc);
-        else epilogue_store(epi, own, side, row, own_col0, min(N, own_col0 + w));
-      }
-      if constexpr (LOSS) loss_finish(epi.loss, lacc, quarter, lane, loss_slots, loss_warps);
     }
-    tc_fence_before();
+    const bool dz_wide = whole && (epi.loss.ld_dz & 3) == 0 && (reinterpret_cast<uintptr_t>(epi.loss.dz) & 15u) == 0;
+    if constexpr (LOSS == LOSS_MSE) {
+      // dZ = gscale (a - t) [a > 0] and the sum of (a - t)^2; a is the output as it is stored
+#pragma unroll
+      for (int i = 0; i < PER_THREAD; ++i) {
+        const int row = m0 + er + i * ROW_STEP;
+        if (!ok || row >= M || n_cols <= 0) continue;
+        const float t[4] = {side[i].x, side[i].y, side[i].z, side[i].w};
+        float g[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float a = epi.c_dt == DT_BF16 ? round_bf16_rne(x[i][j]) : x[i][j];
+          const float d = a - t[j];
+          if (j < n_cols) lacc = fmaf(d, d, lacc);
+          g[j] = (epi.loss.relu_mask && !(a > 0.f)) ? 0.f : d * epi.loss.gscale;
+          g[j] = apply_round(g[j], epi.loss.dz_round);
+        }
+        store_piece(epi.loss.dz, epi.loss.dz_dt, (int64_t)row * epi.loss.ld_dz + col, g, n_cols, dz_wide);
+      }
+    }
+    if constexpr (LOSS == LOSS_CE) {
+      // Softmax cross-entropy of rows that this cluster holds whole (N <= 64): every CTA's maximum and sum of exponentials over its
+      // columns, 8 bytes per row, go to its peers; dZ = (softmax - onehot) / B, loss = log(sum) - (z_class - maximum).
+#pragma unroll
+      for (int i = 0; i < PER_THREAD; ++i) {
+        const int row = er + i * ROW_STEP;
+        float mx = -INFINITY, se = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (j < n_cols) mx = fmaxf(mx, x[i][j]);
+#pragma unroll
+        for (int o = PPR / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+        const float ref = mx == -INFINITY ? 0.f : mx;      // a slice of -infinity alone adds nothing
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (j < n_cols) se += expf(x[i][j] - ref);
+#pragma unroll
+        for (int o = PPR / 2; o > 0; o >>= 1) se += __shfl_xor_sync(0xFFFFFFFFu, se, o);
+        if (ok && ep < split) {                             // lane ep of the row tells CTA ep
+          float2* at = stats + rank * BLOCK_M + row;
+          if (ep == (int)rank) *at = make_float2(mx, se);
+          else send_to_peer(map_to_cta(smem_u32(at), (uint32_t)ep), map_to_cta(stats_bar, (uint32_t)ep), mx, se);
+        }
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");       // the own statistics are in place
+      ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(stats_bar, 0, abort_flag, dev_status));
+#pragma unroll
+      for (int i = 0; i < PER_THREAD; ++i) {
+        const int r = er + i * ROW_STEP, row = m0 + r;
+        if (!ok || row >= M || n_cols <= 0) continue;
+        float2 st[split];
+        float mx = -INFINITY, se = 0.f;
+#pragma unroll
+        for (int src = 0; src < split; ++src) { st[src] = stats[src * BLOCK_M + r]; mx = fmaxf(mx, st[src].x); }
+#pragma unroll
+        for (int src = 0; src < split; ++src) se += st[src].y * expf(st[src].x - mx);
+        const float inv_se = 1.0f / se;
+        float g[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float a = x[i][j];
+          g[j] = (expf(a - mx) * inv_se - (col + j == cls[i] ? 1.f : 0.f)) * epi.loss.gscale;
+          if (epi.loss.relu_mask && !(a > 0.f)) g[j] = 0.f;
+          g[j] = apply_round(g[j], epi.loss.dz_round);
+          if (j < n_cols && col + j == cls[i]) lacc += logf(se) - (a - mx);
+        }
+        store_piece(epi.loss.dz, epi.loss.dz_dt, (int64_t)row * epi.loss.ld_dz + col, g, n_cols, dz_wide);
+      }
+    }
+    if constexpr (LOSS != LOSS_NONE) {
+      const float w = warp_sum(lacc);
+      if (ok && lane == 0) {
+        loss_slots[warp - 2] = w;
+        __threadfence_block();
+        if (atomicAdd(loss_warps, 1u) == SPLITK_EPI_THREADS / 32 - 1) {    // the last warp adds them up, in warp order
+          __threadfence_block();
+          float t = 0.f;
+          for (int i = 0; i < SPLITK_EPI_THREADS / 32; ++i) t += loss_slots[i];
+          epi.loss.partials[blockIdx.x] = t;
+        }
+      }
+    }
   }
 
+  // Nothing of this CTA is read by its peers, and it has received what they send: it may leave before them.
   __syncwarp();
+  if (split > 1 && warp < 2) cluster_wait();
   if (*abort_flag) {
-    for (int i = 0; i < 64; ++i) __nanosleep(20000);
+    // a wait was given up: leave time for copies in flight to land, and for peers to send or give up (their waits are bounded)
+    for (int i = 0; i < 4000; ++i) __nanosleep(1000000);
   }
-  if (warp < 2) {                     // the producer and MMA warps complete the first cluster phase and arrive for the second here
-    cluster_wait();
-    cluster_arrive();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
-  cluster_wait();                     // no CTA leaves before its peers have what it sent them
 }
 
 
@@ -1491,7 +1464,7 @@ cudaError_t launch_majors(bool a_mn, bool b_mn, const CUtensorMap& ma, const CUt
 }
 
 
-template <bool TF32, bool A_MN, bool B_MN, int SPLIT, bool LOSS = false>
+template <bool TF32, bool A_MN, bool B_MN, int SPLIT, int LOSS = LOSS_NONE>
 cudaError_t launch_splitk_cluster(const CUtensorMap& ma, const CUtensorMap& mb, const GemmDesc& g,
                                   const EpilogueArgs& e, int* dev_status, cudaStream_t s) {
   constexpr int split = SPLIT;
@@ -1501,25 +1474,31 @@ cudaError_t launch_splitk_cluster(const CUtensorMap& ma, const CUtensorMap& mb, 
   const int tiles = ((g.M + BLOCK_M - 1) / BLOCK_M) * ((g.N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(tiles * split), 1, 1);
-  cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+  cfg.blockDim = dim3(SPLITK_THREADS, 1, 1);
   cfg.dynamicSmemBytes = SPLITK_SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
+  int n = 0;
+  if (split > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)split; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+  }
+  if (g_use_pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, ma, mb, g.M, g.N, g.K, e, dev_status);
 }
 
-template <bool TF32, bool A_MN, bool B_MN, bool LOSS = false>
+template <bool TF32, bool A_MN, bool B_MN, int LOSS = LOSS_NONE>
 cudaError_t launch_splitk_variant(const CUtensorMap& ma, const CUtensorMap& mb, const GemmDesc& g,
                                   const EpilogueArgs& e, int split, int* dev_status, cudaStream_t s) {
   switch (split) {
+    case 1: return launch_splitk_cluster<TF32, A_MN, B_MN, 1, LOSS>(ma, mb, g, e, dev_status, s);
     case 2: return launch_splitk_cluster<TF32, A_MN, B_MN, 2, LOSS>(ma, mb, g, e, dev_status, s);
     case 4: return launch_splitk_cluster<TF32, A_MN, B_MN, 4, LOSS>(ma, mb, g, e, dev_status, s);
-    default: return cudaErrorNotSupported;                  // pick_split chooses 2 or 4
+    default: return cudaErrorNotSupported;                  // pick_split chooses 1, 2 or 4
   }
 }
 
@@ -1527,28 +1506,13 @@ template <bool TF32>
 cudaError_t launch_splitk_majors(bool a_mn, bool b_mn, const CUtensorMap& ma, const CUtensorMap& mb,
                                  const GemmDesc& g, const EpilogueArgs& e, int split, int* dev_status, cudaStream_t s) {
   if (!a_mn && !b_mn) {
-    if (e.loss.enabled) return launch_splitk_variant<TF32, false, false, true>(ma, mb, g, e, split, dev_status, s);
+    if (e.loss.enabled == LOSS_MSE) return launch_splitk_variant<TF32, false, false, LOSS_MSE>(ma, mb, g, e, split, dev_status, s);
+    if (e.loss.enabled == LOSS_CE) return launch_splitk_cluster<TF32, false, false, CE_SPLIT, LOSS_CE>(ma, mb, g, e, dev_status, s);
     return launch_splitk_variant<TF32, false, false>(ma, mb, g, e, split, dev_status, s);
   }
   if (!a_mn && b_mn) return launch_splitk_variant<TF32, false, true>(ma, mb, g, e, split, dev_status, s);
   if (a_mn && b_mn) return launch_splitk_variant<TF32, true, true>(ma, mb, g, e, split, dev_status, s);
   return cudaErrorNotSupported;
-}
-
-// Split K over a cluster when the 128 x 64 tiles alone would leave most SMs idle and K is long
-// enough that the main loop, not the fixed cost, dominates.  Returns 1 for "do not split".
-int pick_split(int M, int N, int K, bool tf32) {
-  const int tiles = ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
-  const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64);
-  // measured: a k-block costs about 0.27 us of one SM's shared-memory fill time, the cluster exchange about 2 us
-  int best = 1;
-  double best_us = 0.27 * num_k;
-  for (int sp : {2, 4}) {
-    if (tiles * sp > num_sms()) break;
-    const double us = 0.27 * ((num_k + sp - 1) / sp) + 2.0;
-    if (us < best_us - 0.5) { best = sp; best_us = us; }
-  }
-  return best;
 }
 
 template <bool TF32, bool A_MN, bool B_MN, bool FUSED = false>
@@ -1637,6 +1601,23 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_u
   return best;
 }
 
+// CTAs per 128 x 64 tile of the split-K kernel (1, 2 or 4), or 0 where a persistent kernel takes the product.  A k-block costs a
+// CTA about 0.27 us (its ring holds three), the exchange about 1 us; a persistent kernel finishes its only tile about 1.5 us later.
+int pick_split(int M, int N, int K, bool tf32) {
+  const int tiles = ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
+  const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64);
+  const Choice other = pick_kernel(M, N, K, tf32, false, false);
+  if (g_pair_min_tiles > 0 && other.kind == 1) return 0;    // CTA pairs are forced
+  int best = 0;
+  double best_us = other.us + 1.5;
+  for (int sp : {1, 2, 4}) {
+    if (tiles * sp > num_sms()) break;
+    const double us = 0.27 * ((num_k + sp - 1) / sp) + (sp > 1 ? 1.0 : 0.0);
+    if (us < best_us) { best = sp; best_us = us; }
+  }
+  return best;
+}
+
 }  // namespace
 
 bool gemm_tc_init() {
@@ -1713,10 +1694,11 @@ double gemm_tc_estimate_us(int M, int N, int K, bool tf32) {
   return 3.0 + pick_kernel(M, N, K, tf32, false, false).us;         // + launch, first loads and drain
 }
 
-int gemm_tc_fused_loss_partials(int M, int N, int K, bool tf32) {
+int gemm_tc_fused_loss_partials(int kind, int M, int N, int K, bool tf32) {
   if (!g_init_ok || !g_allow_splitk) return 0;
-  const int split = pick_split(M, N, K, tf32);
-  return split > 1 ? split * ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N) : 0;
+  const int tiles_m = (M + BLOCK_M - 1) / BLOCK_M;
+  if (kind == LOSS_CE) return N <= SPLITK_BLOCK_N && CE_SPLIT * tiles_m <= num_sms() ? CE_SPLIT * tiles_m : 0;
+  return pick_split(M, N, K, tf32) * tiles_m * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
 }
 
 // The fused update lives in the persistent kernels (one CTA or a CTA pair per tile); products small enough to
@@ -1731,8 +1713,8 @@ bool gemm_tc_can_fuse_update(const GemmDesc& g) {
   if ((g.a_sk * esz) % 16 != 0 || (g.b_sk * esz) % 16 != 0) return false;
   if ((reinterpret_cast<uintptr_t>(g.C) & 15u) || (g.ldc & 3)) return false;
   const bool throughput = g.off_critical_path != 0;
-  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 1;
-  return split == 1;
+  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 0;
+  return split <= 1;
 }
 
 cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, int* family) {
@@ -1756,14 +1738,15 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   if ((a_pitch * esz) % 16 != 0 || (b_pitch * esz) % 16 != 0) return cudaErrorNotSupported;
   if (a_pitch * (int64_t)esz >= (1ll << 40) || b_pitch * (int64_t)esz >= (1ll << 40)) return cudaErrorNotSupported;
 
-  const bool fuse_loss = (g.epi == EPI_BIAS_ACT) && g.loss.enabled != 0;
-  if (fuse_loss && (a_mn || b_mn || gemm_tc_fused_loss_partials(g.M, g.N, g.K, tf32) == 0))
+  const int fuse_loss = g.epi == EPI_BIAS_ACT ? g.loss.enabled : LOSS_NONE;
+  if (fuse_loss && (a_mn || b_mn || gemm_tc_fused_loss_partials(fuse_loss, g.M, g.N, g.K, tf32) == 0))
     return cudaErrorInvalidValue;                           // the caller asks gemm_tc_fused_loss_partials first
   const bool throughput = g.off_critical_path != 0;
-  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 1;
+  int split = fuse_loss == LOSS_CE ? CE_SPLIT : (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 0;
+  if (g.upd.enabled && split == 1) split = 0;               // the persistent kernels' variant
   const Choice choice = pick_kernel(g.M, g.N, g.K, tf32, throughput, g.upd.enabled != 0);
-  const bool pairs = (split == 1) && choice.kind == 1;
-  const int block_n = split > 1 ? SPLITK_BLOCK_N : choice.block_n;
+  const bool pairs = (split == 0) && choice.kind == 1;
+  const int block_n = split > 0 ? SPLITK_BLOCK_N : choice.block_n;
   const uint32_t block_k = tf32 ? 32 : 64, chunk = tf32 ? 32 : 64;
   CUtensorMap ma, mb;
   bool ok;
@@ -1777,15 +1760,15 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   EpilogueArgs e;
   e.C = g.C; e.ldc = g.ldc; e.c_dt = g.c_dt; e.c_round = g.c_round; e.epi = g.epi; e.relu = g.relu;
   e.bias = g.bias; e.mask = g.mask; e.ldmask = g.ldmask; e.b_early = g.b_early;
-  e.loss = g.loss; e.loss.enabled = fuse_loss ? 1 : 0;
+  e.loss = g.loss; e.loss.enabled = fuse_loss;
   e.upd = g.upd;
   e.staged = (g_staged_epilogue && !e.upd.enabled) ? 1 : 0;
-  if (e.upd.enabled && (split > 1 || !a_mn || !b_mn || g.epi != EPI_PLAIN || g.c_dt != DT_F32))
+  if (e.upd.enabled && (split > 0 || !a_mn || !b_mn || g.epi != EPI_PLAIN || g.c_dt != DT_F32))
     return cudaErrorInvalidValue;                           // the caller asks gemm_tc_can_fuse_update first
 
   // output map of the persistent kernels' staged epilogue (the split-K kernel stores its column slices itself)
   CUtensorMap mc;
-  if (split == 1) {
+  if (split == 0) {
     if ((reinterpret_cast<uintptr_t>(g.C) & 15u) || (g.ldc * (g.c_dt == DT_F32 ? 4 : 2)) % 16 != 0) return cudaErrorNotSupported;
     if (!make_output_map(&mc, g.c_dt == DT_F32, g.C, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldc)) return cudaErrorNotSupported;
   }
@@ -1794,7 +1777,7 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
     return tf32 ? launch_pair_majors<true>(a_mn, b_mn, ma, mb, mc, g, e, 2 * block_n, dev_status, s)
                 : launch_pair_majors<false>(a_mn, b_mn, ma, mb, mc, g, e, 2 * block_n, dev_status, s);
   }
-  if (split > 1) {
+  if (split > 0) {
     return tf32 ? launch_splitk_majors<true>(a_mn, b_mn, ma, mb, g, e, split, dev_status, s)
                 : launch_splitk_majors<false>(a_mn, b_mn, ma, mb, g, e, split, dev_status, s);
   }

@@ -283,15 +283,15 @@ seg_status prepare_input(seg_handle* h, const void* x, int batch, const void** x
   return SEG_OK;
 }
 
-// Description of a non-final segment's loss for fusion into its last forward product.
+// Description of a segment's loss for fusion into its last forward product.
 LossFuse loss_fuse_desc(seg_handle* h, int batch, const int32_t* cls) {
   const int L = h->n_layers;
   LossFuse f{};
-  f.enabled = 1;
+  f.enabled = h->is_final ? LOSS_CE : LOSS_MSE;
   f.cls = cls; f.sil = h->sil;
   f.dz = h->dzbuf[L - 1]; f.ld_dz = h->ld_act[L]; f.dz_dt = h->act_dt; f.dz_round = h->act_round;
   f.relu_mask = h->last_relu ? 1 : 0;
-  f.gscale = 2.0f / (float)((int64_t)batch * h->widths[L]);
+  f.gscale = h->is_final ? 1.0f / (float)batch : 2.0f / (float)((int64_t)batch * h->widths[L]);
   f.partials = h->loss_partials;
   return f;
 }
@@ -340,8 +340,8 @@ seg_status forward_layers(seg_handle* h, const void* a_prev, int64_t ld_prev, in
     GemmDesc g = forward_desc(h, l, a_prev, ld_prev, batch);
     g.b_early = (l > 0 || first_early) ? 1 : 0;
     const bool want_loss = last && loss_cls != nullptr;
-    if (want_loss && !h->is_final && h->use_tc && h->fuse_loss) {
-      const int n = gemm_tc_fused_loss_partials(g.M, g.N, g.K, h->precision == SEG_TF32);
+    if (want_loss && h->use_tc && h->fuse_loss) {
+      const int n = gemm_tc_fused_loss_partials(h->is_final ? LOSS_CE : LOSS_MSE, g.M, g.N, g.K, h->precision == SEG_TF32);
       if (n > 0 && n <= loss_max_partials()) { g.loss = loss_fuse_desc(h, batch, loss_cls); h->n_loss_partials = n; }
     }
     bool used_tc = false;
