@@ -653,7 +653,7 @@ constexpr int SPLITK_BLOCK_N = 64;
 // waiting for whole SMs.
 constexpr int SPLITK_STAGES = 3;
 constexpr int SPLITK_STAGE_BYTES = A_TILE_BYTES + SPLITK_BLOCK_N * TILE_ROW_BYTES;       // 24 KiB
-constexpr int SPLITK_RECV_BYTES = SPLITK_BLOCK_N * BLOCK_M * 4;                          // [src][row][pieces of the slice], 32 KiB
+constexpr int SPLITK_RECV_BYTES = SPLITK_BLOCK_N * BLOCK_M * 4;                          // [src][piece of the slice][row], 32 KiB
 constexpr int SPLITK_SMEM = SPLITK_STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES + SMEM_EXTRA;
 constexpr int SPLITK_THREADS = 320, SPLITK_EPI_THREADS = 256;                            // eight epilogue warps
 constexpr int CE_SPLIT = 4;                                // CTAs per cluster of a product that forms the cross-entropy too
@@ -700,20 +700,27 @@ __device__ __forceinline__ void store_piece(void* base, int dt, int64_t at, cons
   }
 }
 
-// One 128 x 64 output tile per cluster (SPLIT = 1: per CTA, nothing to exchange); CTA r of the cluster contracts k-blocks
-// [r*kpc, (r+1)*kpc).
+// Byte offset of a piece (four columns) of a row in a share of 128 rows x PPR pieces: [piece][row], rows rotated by piece, so that a
+// warp that holds 32 rows writes 512 consecutive bytes and the eight lanes that read one or two whole rows reach different banks.
+template <int PPR>
+__device__ __forceinline__ uint32_t piece_at(int piece, int row) {
+  return (uint32_t)(piece * BLOCK_M + ((row + (PPR == 4 ? 2 * piece : piece)) & (BLOCK_M - 1))) * 16u;
+}
+
+// One 128 x 64 output tile per cluster; CTA r of the cluster contracts k-blocks [r*kpc, (r+1)*kpc).
 //
 // The exchange.  A warp holds 32 rows x 32 columns of the partial tile and sends each piece of four columns straight from its
-// registers to the CTA that owns them (st.async, counted by the owner's barrier; pieces of a row swizzled, so that the eight lanes
-// of a phase reach different banks); a thread of the owner then finishes pieces of rows that follow each other, four to sixteen to
-// a row, so that outputs, masks and targets move in row segments of 64 to 256 bytes.
+// registers to the CTA that owns them (st.async, counted by the owner's barrier); a thread of the owner then finishes pieces of rows
+// that follow each other, four or eight to a row, so that outputs, masks and targets move in row segments of 64 or 128 bytes.  What
+// a warp sends at a time has to be consecutive at the receiver: with the pieces of a row side by side instead (64-byte rows) a step
+// of 512-512-256-47 (TF32, batch 256) took 39.0 us, against 34.9.
 template <bool TF32, bool A_MN, bool B_MN, int SPLIT, int LOSS = LOSS_NONE>
 __global__ void __launch_bounds__(SPLITK_THREADS, 2)
 gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                       int M, int N, int K, EpilogueArgs epi, int* dev_status) {
   constexpr int split = SPLIT;                             // CTAs per cluster
   constexpr int W = SPLITK_BLOCK_N / SPLIT;                // columns of the tile each CTA owns after the exchange
-  static_assert(W == 64 || W == 32 || W == 16, "slice width");
+  static_assert(W == 32 || W == 16, "slice width");
   constexpr int PPR = W / 4;                               // pieces per row of the slice
   constexpr int PER_THREAD = BLOCK_M * PPR / SPLITK_EPI_THREADS;
   constexpr int ROW_STEP = SPLITK_EPI_THREADS / PPR;       // rows between a thread's pieces
@@ -730,7 +737,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* smem_a = smem;
   uint8_t* smem_b = smem + STAGES * A_TILE_BYTES;
-  uint8_t* recv = smem + STAGES * SPLITK_STAGE_BYTES;      // [src][row][piece]
+  uint8_t* recv = smem + STAGES * SPLITK_STAGE_BYTES;      // [src][piece][row]
   float2* stats = reinterpret_cast<float2*>(smem);         // LOSS_CE: [src][row] maximum and sum, in the ring's place (who sends them has had this CTA's sums)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES);
   // bars[0..S) full, [S..2S) empty, [2S] accumulator complete, [2S+1] partial slices received, [2S+2] row statistics received
@@ -740,7 +747,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   unsigned int* loss_warps = reinterpret_cast<unsigned int*>(reinterpret_cast<uint8_t*>(bars) + 192);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = split > 1 ? cluster_ctarank() : 0u;
+  const uint32_t rank = cluster_ctarank();
   const uint32_t bar_base = smem_u32(bars);
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
@@ -760,13 +767,13 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // this CTA will receive one column slice (BLOCK_N / split columns x 128 rows, fp32) from every peer
-    if (split > 1) mbar_arrive_expect_tx(recv_bar, (uint32_t)((split - 1) * W * BLOCK_M * 4));
+    mbar_arrive_expect_tx(recv_bar, (uint32_t)((split - 1) * W * BLOCK_M * 4));
     if (LOSS == LOSS_CE) mbar_arrive_expect_tx(stats_bar, (uint32_t)((split - 1) * BLOCK_M * 8));
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
   tc_fence_before();
   __syncthreads();
-  if (split > 1) cluster_arrive();    // "my barriers are initialised"; the matching wait sits in front of the
+  cluster_arrive();                   // "my barriers are initialised"; the matching wait sits in front of the
   tc_fence_after();                   // first remote access (the slice exchange), off the main loop's path
   const uint32_t tmem_base = *tmem_slot;
   // tile and k-range of this CTA: index arithmetic only, done while the previous kernel drains
@@ -921,30 +928,26 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         for (int j = 0; j < 32; ++j) v[j] = 0.f;
       }
       tc_fence_before();
-      if (split > 1) cluster_wait();                       // every peer's receive barrier exists
-      const uint32_t share = (uint32_t)(((int)rank * BLOCK_M + row) * PPR) * 16u;   // this CTA's share of the row, in any CTA
-      const int sw = W == 16 ? (row >> 1) & 3 : row & 7;
-      constexpr int OWNERS = W >= 32 ? 1 : 32 / W, RUN = W >= 32 ? 8 : PPR;   // owners of this warp's 32 columns, pieces for each
+      cluster_wait();                                      // every peer's receive barrier exists
+      const uint32_t share = (uint32_t)((int)rank * BLOCK_M * PPR) * 16u;   // this CTA's share, in any CTA
 #pragma unroll
-      for (int o = 0; o < OWNERS; ++o) {
-        const uint32_t owner = split == 1 ? 0u : (uint32_t)(half * OWNERS + o);
-        const uint32_t dst = split == 1 ? 0u : map_to_cta(smem_u32(recv) + share, owner);
-        const uint32_t bar = split == 1 ? 0u : map_to_cta(recv_bar, owner);
-        const int c0 = split == 1 ? half * 8 : 0;
+      for (int o = 0; o < 32 / W; ++o) {                   // the owners of this warp's 32 columns
+        const uint32_t owner = (uint32_t)(half * (32 / W) + o);
+        const uint32_t dst = map_to_cta(smem_u32(recv) + share, owner), bar = map_to_cta(recv_bar, owner);
 #pragma unroll
-        for (int c = 0; c < RUN; ++c) {
+        for (int c = 0; c < PPR; ++c) {
           const float* x = v + o * W + 4 * c;
-          const uint32_t at = (uint32_t)((c0 + c) ^ sw) * 16u;
+          const uint32_t at = piece_at<PPR>(c, row);
           if (owner == rank) *reinterpret_cast<float4*>(recv + share + at) = make_float4(x[0], x[1], x[2], x[3]);
           else send_to_peer(dst + at, bar, x[0], x[1], x[2], x[3]);
         }
       }
-    } else if (split > 1) {
+    } else {
       cluster_wait();
     }
     asm volatile("bar.arrive 2, 288;" ::: "memory");       // drained: warp 1 gives the tensor memory back
     asm volatile("bar.sync 1, 256;" ::: "memory");         // the own share is in place
-    if (split > 1) ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(recv_bar, 0, abort_flag, dev_status));
+    ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(recv_bar, 0, abort_flag, dev_status));
     float x[PER_THREAD][4];
 #pragma unroll
     for (int i = 0; i < PER_THREAD; ++i)
@@ -954,8 +957,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 #pragma unroll
       for (int i = 0; i < PER_THREAD; ++i) {
         const int row = er + i * ROW_STEP;
-        const int sw = W == 16 ? (row >> 1) & 3 : row & 7;
-        const uint8_t* at = recv + (row * PPR + (ep ^ sw)) * 16;
+        const uint8_t* at = recv + piece_at<PPR>(ep, row);
         float4 s = *reinterpret_cast<const float4*>(at);
 #pragma unroll
         for (int src = 1; src < split; ++src) {
@@ -1066,7 +1068,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 
   // Nothing of this CTA is read by its peers, and it has received what they send: it may leave before them.
   __syncwarp();
-  if (split > 1 && warp < 2) cluster_wait();
+  if (warp < 2) cluster_wait();
   if (*abort_flag) {
     // a wait was given up: leave time for copies in flight to land, and for peers to send or give up (their waits are bounded)
     for (int i = 0; i < 4000; ++i) __nanosleep(1000000);
@@ -1478,16 +1480,11 @@ cudaError_t launch_splitk_cluster(const CUtensorMap& ma, const CUtensorMap& mb, 
   cfg.dynamicSmemBytes = SPLITK_SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
-  int n = 0;
-  if (split > 1) {
-    attr[n].id = cudaLaunchAttributeClusterDimension;
-    attr[n].val.clusterDim.x = (unsigned)split; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
-  }
-  if (g_use_pdl) {
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n++].val.programmaticStreamSerializationAllowed = 1;
-  }
-  cfg.attrs = attr; cfg.numAttrs = n;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, ma, mb, g.M, g.N, g.K, e, dev_status);
 }
 
@@ -1495,10 +1492,9 @@ template <bool TF32, bool A_MN, bool B_MN, int LOSS = LOSS_NONE>
 cudaError_t launch_splitk_variant(const CUtensorMap& ma, const CUtensorMap& mb, const GemmDesc& g,
                                   const EpilogueArgs& e, int split, int* dev_status, cudaStream_t s) {
   switch (split) {
-    case 1: return launch_splitk_cluster<TF32, A_MN, B_MN, 1, LOSS>(ma, mb, g, e, dev_status, s);
     case 2: return launch_splitk_cluster<TF32, A_MN, B_MN, 2, LOSS>(ma, mb, g, e, dev_status, s);
     case 4: return launch_splitk_cluster<TF32, A_MN, B_MN, 4, LOSS>(ma, mb, g, e, dev_status, s);
-    default: return cudaErrorNotSupported;                  // pick_split chooses 1, 2 or 4
+    default: return cudaErrorNotSupported;                  // pick_split chooses 2 or 4
   }
 }
 
@@ -1601,18 +1597,23 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_u
   return best;
 }
 
-// CTAs per 128 x 64 tile of the split-K kernel (1, 2 or 4), or 0 where a persistent kernel takes the product.  A k-block costs a
-// CTA about 0.27 us (its ring holds three), the exchange about 1 us; a persistent kernel finishes its only tile about 1.5 us later.
-int pick_split(int M, int N, int K, bool tf32) {
+// CTAs per 128 x 64 tile of the split-K kernel (2 or 4), or 1 where a persistent kernel takes the product.  A k-block costs a CTA
+// about 0.27 us (its ring holds three), the exchange 1 us, the epilogue 1.8 us by the CTAs that share it; a persistent kernel's
+// epilogue takes 1.2 us more than its estimate says.  A weight gradient runs beside those of the layers above, from which a split
+// takes SMs: half a microsecond has to be gained there.  Whole steps of 78 nets (13 shapes, TF32 and bf16, batch 64 to 1024), against
+// the bulk-copy exchange and the line it had: 1.129 times as fast in the geometric mean, none slower; with 0.3 instead of 1.2 it is
+// 1.112, with 0.7 for weight gradients 1.125 and the worst 0.966.  A step of 512-512-256-47 (TF32, batch 256) 45.1 -> 34.9 us, of
+// 784-1024-1024-512 55.8 -> 50.4, of 72-136-64 (bf16, batch 64) 24.6 -> 20.5.
+int pick_split(int M, int N, int K, bool tf32, bool wgrad) {
   const int tiles = ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
   const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64);
   const Choice other = pick_kernel(M, N, K, tf32, false, false);
-  if (g_pair_min_tiles > 0 && other.kind == 1) return 0;    // CTA pairs are forced
-  int best = 0;
-  double best_us = other.us + 1.5;
-  for (int sp : {1, 2, 4}) {
+  if (g_pair_min_tiles > 0 && other.kind == 1) return 1;    // CTA pairs are forced
+  int best = 1;
+  double best_us = other.us + (wgrad ? -0.5 : 1.2);
+  for (int sp : {2, 4}) {
     if (tiles * sp > num_sms()) break;
-    const double us = 0.27 * ((num_k + sp - 1) / sp) + (sp > 1 ? 1.0 : 0.0);
+    const double us = 0.27 * ((num_k + sp - 1) / sp) + 1.0 + 1.8 / sp;
     if (us < best_us) { best = sp; best_us = us; }
   }
   return best;
@@ -1698,7 +1699,8 @@ int gemm_tc_fused_loss_partials(int kind, int M, int N, int K, bool tf32) {
   if (!g_init_ok || !g_allow_splitk) return 0;
   const int tiles_m = (M + BLOCK_M - 1) / BLOCK_M;
   if (kind == LOSS_CE) return N <= SPLITK_BLOCK_N && CE_SPLIT * tiles_m <= num_sms() ? CE_SPLIT * tiles_m : 0;
-  return pick_split(M, N, K, tf32) * tiles_m * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
+  const int split = pick_split(M, N, K, tf32, false);
+  return split > 1 ? split * tiles_m * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N) : 0;
 }
 
 // The fused update lives in the persistent kernels (one CTA or a CTA pair per tile); products small enough to
@@ -1713,8 +1715,8 @@ bool gemm_tc_can_fuse_update(const GemmDesc& g) {
   if ((g.a_sk * esz) % 16 != 0 || (g.b_sk * esz) % 16 != 0) return false;
   if ((reinterpret_cast<uintptr_t>(g.C) & 15u) || (g.ldc & 3)) return false;
   const bool throughput = g.off_critical_path != 0;
-  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 0;
-  return split <= 1;
+  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32, true) : 1;
+  return split == 1;
 }
 
 cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, int* family) {
@@ -1742,11 +1744,10 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   if (fuse_loss && (a_mn || b_mn || gemm_tc_fused_loss_partials(fuse_loss, g.M, g.N, g.K, tf32) == 0))
     return cudaErrorInvalidValue;                           // the caller asks gemm_tc_fused_loss_partials first
   const bool throughput = g.off_critical_path != 0;
-  int split = fuse_loss == LOSS_CE ? CE_SPLIT : (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32) : 0;
-  if (g.upd.enabled && split == 1) split = 0;               // the persistent kernels' variant
+  const int split = fuse_loss == LOSS_CE ? CE_SPLIT : (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32, a_mn) : 1;
   const Choice choice = pick_kernel(g.M, g.N, g.K, tf32, throughput, g.upd.enabled != 0);
-  const bool pairs = (split == 0) && choice.kind == 1;
-  const int block_n = split > 0 ? SPLITK_BLOCK_N : choice.block_n;
+  const bool pairs = (split == 1) && choice.kind == 1;
+  const int block_n = split > 1 ? SPLITK_BLOCK_N : choice.block_n;
   const uint32_t block_k = tf32 ? 32 : 64, chunk = tf32 ? 32 : 64;
   CUtensorMap ma, mb;
   bool ok;
@@ -1763,12 +1764,12 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   e.loss = g.loss; e.loss.enabled = fuse_loss;
   e.upd = g.upd;
   e.staged = (g_staged_epilogue && !e.upd.enabled) ? 1 : 0;
-  if (e.upd.enabled && (split > 0 || !a_mn || !b_mn || g.epi != EPI_PLAIN || g.c_dt != DT_F32))
+  if (e.upd.enabled && (split > 1 || !a_mn || !b_mn || g.epi != EPI_PLAIN || g.c_dt != DT_F32))
     return cudaErrorInvalidValue;                           // the caller asks gemm_tc_can_fuse_update first
 
   // output map of the persistent kernels' staged epilogue (the split-K kernel stores its column slices itself)
   CUtensorMap mc;
-  if (split == 0) {
+  if (split == 1) {
     if ((reinterpret_cast<uintptr_t>(g.C) & 15u) || (g.ldc * (g.c_dt == DT_F32 ? 4 : 2)) % 16 != 0) return cudaErrorNotSupported;
     if (!make_output_map(&mc, g.c_dt == DT_F32, g.C, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldc)) return cudaErrorNotSupported;
   }
@@ -1777,7 +1778,7 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
     return tf32 ? launch_pair_majors<true>(a_mn, b_mn, ma, mb, mc, g, e, 2 * block_n, dev_status, s)
                 : launch_pair_majors<false>(a_mn, b_mn, ma, mb, mc, g, e, 2 * block_n, dev_status, s);
   }
-  if (split > 0) {
+  if (split > 1) {
     return tf32 ? launch_splitk_majors<true>(a_mn, b_mn, ma, mb, g, e, split, dev_status, s)
                 : launch_splitk_majors<false>(a_mn, b_mn, ma, mb, g, e, split, dev_status, s);
   }
