@@ -6,10 +6,9 @@
 //   wgrad    C = dZ^T A    : both operands MN-major (contraction over the batch)
 // with bf16 operands (kind::f16) or TF32 operands (kind::tf32) and fp32 accumulation in TMEM.
 //
-// CTA = 6 warps (10 in the CTA-pair kernel).  A thread of warp 0 issues TMA loads into a ring of
-// shared-memory stages; warp 1 owns the TMEM allocation and one of its threads issues the MMAs; the other
-// four (eight) warps drain the accumulator (a warp reads its own 32 TMEM lanes), apply the epilogue and
-// store.  Two accumulator buffers in TMEM let the epilogue of tile i overlap the main loop of tile i+1.
+// CTA = 10 warps.  A thread of warp 0 issues TMA loads into a ring of shared-memory stages; warp 1 owns the
+// TMEM allocation and one of its threads issues the MMAs; the other eight warps drain the accumulator (a warp
+// reads its own 32 TMEM lanes), apply the epilogue and store.  Two accumulator buffers in TMEM let the epilogue of tile i overlap the main loop of tile i+1.
 //
 // Shared-memory operand tiles use the 128-byte swizzle.  K-major tile: rows of 128 bytes (64 bf16
 // or 32 TF32 along K), 8-row groups 1024 bytes apart.  MN-major tile: chunks of 64 bf16 / 32 TF32
@@ -21,8 +20,8 @@
 // Small problems (few output tiles, long K) use gemm_tc_splitk_kernel instead: a thread-block
 // cluster of 2 or 4 CTAs shares one 128 x 64 output tile, each CTA contracts its own slice of K
 // into TMEM, and the partial tiles are combined through distributed shared memory as a
-// reduce-scatter (every CTA bulk-copies column slice j of its partial into CTA j's shared memory;
-// CTA j adds what it received and runs the epilogue on that slice).  One SM's shared-memory fill rate
+// reduce-scatter (every CTA sends column slice j of its partial from its registers into CTA j's shared
+// memory; CTA j adds what it received and runs the epilogue on that slice, the loss of the segment's last layer included).  One SM's shared-memory fill rate
 // bounds a single CTA's main loop, so spreading K over a cluster shortens exactly the part of the
 // kernel that grows with the problem.
 //
@@ -63,15 +62,15 @@ namespace {
 
 constexpr int BLOCK_M = 128;
 constexpr int A_TILE_BYTES = BLOCK_M * TILE_ROW_BYTES; // 16 KiB per stage
-constexpr int NUM_THREADS = 192;                       // TMA warp, MMA warp, four epilogue warps
+constexpr int NUM_THREADS = 320;                       // TMA warp, MMA warp, eight epilogue warps
 constexpr int UPDATE_WARPS = 8;                        // fused-update variants: eight more warps stream the optimizer update
-constexpr int NUM_THREADS_FUSED = NUM_THREADS + 32 * UPDATE_WARPS;
-constexpr int NUM_THREADS_PAIR = NUM_THREADS + 128;    // CTA-pair kernel: eight epilogue warps
+constexpr int FUSED_UPDATE_WARP0 = 6;                  // there four epilogue warps
+constexpr int NUM_THREADS_FUSED = 32 * (FUSED_UPDATE_WARP0 + UPDATE_WARPS);
 constexpr int SMEM_BUDGET = 192 * 1024;                // operand ring
 constexpr int SMEM_EXTRA = 2048;                       // alignment slack + barriers
 constexpr int HALF_SM_MAX_KB = 16;                     // k-blocks up to which the persistent kernel gives up ring depth for it
 constexpr int HALF_SM_SMEM = 113 * 1024;               // two CTAs of this size fit on an SM (228 KiB, 1 KiB of it per CTA reserved)
-// Output staging of the persistent kernels: every epilogue warp owns two buffers of 32 rows x 64 bytes (32 bf16 or 16
+// Output staging of the persistent kernels: each of the eight epilogue warps owns a buffer of 32 rows x 64 bytes (32 bf16 or 16
 // fp32 columns), written with the shared-memory swizzle of the output tensor map and drained by bulk tensor stores, so
 // that global memory sees whole 64-byte row segments instead of 32 separate 16-byte pieces.  16 KiB in all, taken out
 // of the operand ring's 192 KiB (one stage fewer): the CTA's footprint must not grow.  Measured: with the staging area
@@ -79,8 +78,7 @@ constexpr int HALF_SM_SMEM = 113 * 1024;               // two CTAs of this size 
 // and every training step 3-5 % SLOWER, and 8 KiB of unused padding alone did the same to the old kernels; within the
 // old footprint the steps gain 1-3.5 %.
 constexpr int STAGE_OUT_WARP_BYTES = 32 * 64;          // one buffer of one warp
-constexpr int STAGE_OUT_BYTES = 4 * 2 * STAGE_OUT_WARP_BYTES;   // 16 KiB
-constexpr int PAIR_STAGE_OUT_BYTES = STAGE_OUT_BYTES;           // eight epilogue warps with one buffer each
+constexpr int STAGE_OUT_BYTES = 8 * STAGE_OUT_WARP_BYTES;   // 16 KiB
 
 // Tile order of the persistent kernels.  Tiles are numbered in groups of `group_m` rows of tiles: inside a
 // group the row index runs fastest, then the column index, and the groups follow each other.  The CTAs (or pairs)
@@ -266,23 +264,20 @@ __device__ __forceinline__ void epilogue_store(const EpilogueArgs& e, float (&v)
   store_row_segment(e.C, e.c_dt, e.ldc, v, row, col0, n_total);
 }
 
-// The same epilogue through shared memory: the lane's 32 columns go to row `lane` of the warp's staging buffers, 64 bytes
-// per row and buffer (all 32 bf16 columns, or 16 fp32 columns: an fp32 chunk takes both buffers), in 16-byte pieces,
+// The same epilogue through shared memory: the lane's 32 columns go to row `lane` of the warp's staging buffer, 64 bytes
+// per row (all 32 bf16 columns, or 16 fp32 columns: an fp32 chunk takes two turns), in 16-byte pieces,
 // piece j of row r at position j ^ ((r >> 1) & 3) - the 64-byte swizzle, which the output tensor map expects and which
-// makes the warp's stores conflict-free - and one bulk tensor store per buffer writes the 32-row box; rows and columns
-// beyond the matrix are clipped by the store.  Before a buffer is written, the store issued from it two stores earlier
-// has finished reading it (at most one store is left pending).  With BUFS = 1 the warp has one buffer, drained before each use.
-template <int BUFS = 2>
+// makes the warp's stores conflict-free - and one bulk tensor store per turn writes the 32-row box; rows and columns
+// beyond the matrix are clipped by the store.  Before the buffer is written, the store issued from it has finished reading it.
 __device__ __forceinline__ void epilogue_store_staged(const EpilogueArgs& e, const CUtensorMap* map_c, uint8_t* warp_stage,
                                                       float (&v)[32], const EpiSide& s, int lane, int row0, int col0,
-                                                      int n_total, int n_rows, int chunk) {
+                                                      int n_total, int n_rows) {
   epilogue_values(e, v, s, col0, n_total);
   const int x = (lane >> 1) & 3;
   if (e.c_dt == DT_BF16) {
-    uint8_t* buf = warp_stage + (BUFS == 2 ? (chunk & 1) * STAGE_OUT_WARP_BYTES : 0);
-    if (lane == 0) { if (BUFS == 2) tma_store_wait_source_but_one(); else tma_store_wait_source(); }
+    if (lane == 0) tma_store_wait_source();
     __syncwarp();
-    uint8_t* rowp = buf + lane * 64;
+    uint8_t* rowp = warp_stage + lane * 64;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       __nv_bfloat162 p0 = __floats2bfloat162_rn(v[8 * j], v[8 * j + 1]);
@@ -296,22 +291,21 @@ __device__ __forceinline__ void epilogue_store_staged(const EpilogueArgs& e, con
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // generic writes -> visible to the bulk store
     __syncwarp();
-    if (lane == 0 && row0 < n_rows) tma_store_2d(map_c, smem_u32(buf), col0, row0);
+    if (lane == 0 && row0 < n_rows) tma_store_2d(map_c, smem_u32(warp_stage), col0, row0);
   } else {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (col0 + 16 * h >= n_total) break;                              // uniform: nothing of this half is inside the matrix
-      uint8_t* buf = warp_stage + (BUFS == 2 ? h * STAGE_OUT_WARP_BYTES : 0);
-      if (lane == 0) { if (BUFS == 2) tma_store_wait_source_but_one(); else tma_store_wait_source(); }
+      if (lane == 0) tma_store_wait_source();
       __syncwarp();
-      uint8_t* rowp = buf + lane * 64;
+      uint8_t* rowp = warp_stage + lane * 64;
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         *reinterpret_cast<float4*>(rowp + ((j ^ x) << 4)) =
             make_float4(v[16 * h + 4 * j], v[16 * h + 4 * j + 1], v[16 * h + 4 * j + 2], v[16 * h + 4 * j + 3]);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      if (lane == 0 && row0 < n_rows) tma_store_2d(map_c, smem_u32(buf), col0 + 16 * h, row0);
+      if (lane == 0 && row0 < n_rows) tma_store_2d(map_c, smem_u32(warp_stage), col0 + 16 * h, row0);
     }
   }
 }
@@ -422,7 +416,7 @@ __device__ __forceinline__ void update_tile(const FusedUpdate& f, const float* g
 }
 
 template <bool TF32, bool A_MN, bool B_MN, int BLOCK_N, bool FUSED = false>
-__global__ void __launch_bounds__(FUSED ? NUM_THREADS_FUSED : NUM_THREADS, 1)
+__global__ void __launch_bounds__(FUSED ? NUM_THREADS_FUSED : NUM_THREADS, !FUSED && BLOCK_N == 64 ? 2 : 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_c, int M, int N, int K, EpilogueArgs epi, int* dev_status, int group_m,
                int n_stages) {
@@ -433,6 +427,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   constexpr int CHUNK = TF32 ? 32 : 64;            // elements per 128-byte row along M/N (MN-major)
   constexpr int MN_CHUNK_BYTES = BLOCK_K * TILE_ROW_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BLOCK_N;
+  // Epilogue warps: two per quarter of the TMEM lanes, each taking every other 32-column chunk of the tile (four warps took 3.3 us for
+  // a 128 x 64 tile; steps of 1024-1024-1024-1024 in TF32, batch 1024: 110.9 us with four, 106.3 with eight, 78 nets 1.015 times as fast)
+  constexpr int EPI_WARPS = FUSED ? 4 : 8, EPI_PER_QUARTER = EPI_WARPS / 4;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -457,7 +454,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     prefetch_tensormap(&map_b);
     prefetch_tensormap(&map_c);
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 4); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), EPI_WARPS); }
     *abort_flag = 0;
     *tiles_done = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -569,9 +566,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
     }
-  } else if (warp < NUM_THREADS / 32) {
+  } else if (warp < 2 + EPI_WARPS) {
     // ---------------- epilogue warps ----------------
-    const int quarter = warp & 3;          // TMEM lanes 32*quarter .. +31 belong to this warp
+    const int quarter = warp & 3, part = (warp - 2) >> 2;    // (a warp reads the TMEM lanes of its index modulo 4)
+    uint8_t* my_stage_out = stage_out + (part * 4 + quarter) * STAGE_OUT_WARP_BYTES;
     int acc = 0; uint32_t acc_phase = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
@@ -580,23 +578,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const int m0 = m_idx * BLOCK_M, n0 = n_idx * BLOCK_N;
       const int row = m0 + quarter * 32 + lane;
       EpiSide side, side_next;
-      epilogue_prefetch(epi, side, row, row < M, n0, N);   // before the wait: latency off the critical path
+      epilogue_prefetch(epi, side, row, row < M, n0 + part * 32, N);   // before the wait: latency off the critical path
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, dev_status)) { ok = false; break; }
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < BLOCK_N / 32; ++c) {
+      for (int c = part; c < BLOCK_N / 32; c += EPI_PER_QUARTER) {
         const int col0 = n0 + c * 32;
         if (col0 >= N) break;              // uniform across the CTA
-        if (c + 1 < BLOCK_N / 32) epilogue_prefetch(epi, side_next, row, row < M, col0 + 32, N);
+        constexpr bool MORE = BLOCK_N / 32 > EPI_PER_QUARTER;
+        if (MORE && c + EPI_PER_QUARTER < BLOCK_N / 32)
+          epilogue_prefetch(epi, side_next, row, row < M, col0 + 32 * EPI_PER_QUARTER, N);
         float v[32];
         tmem_load_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BLOCK_N + c * 32), v);
         if (FUSED || !epi.staged) {        // (the update warps read the tile back with ordinary loads: ordinary stores)
           if (row < M) epilogue_store(epi, v, side, row, col0, N);
         } else {
-          epilogue_store_staged(epi, &map_c, stage_out + quarter * 2 * STAGE_OUT_WARP_BYTES, v, side, lane,
-                                m0 + quarter * 32, col0, N, M, c);
+          epilogue_store_staged(epi, &map_c, my_stage_out, v, side, lane, m0 + quarter * 32, col0, N, M);
         }
-        side = side_next;
+        if (MORE) side = side_next;
       }
       tc_fence_before();
       __syncwarp();
@@ -607,8 +606,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (lane == 0) tma_store_wait_all();   // the staging buffers are read, and the output written, before the CTA leaves
   } else if constexpr (FUSED) {
     // ---------------- update warps: the optimizer on every tile this CTA has stored ----------------
-    if (warp >= NUM_THREADS / 32) {
-      const int uw = warp - NUM_THREADS / 32;
+    if (warp >= FUSED_UPDATE_WARP0) {
+      const int uw = warp - FUSED_UPDATE_WARP0;
       float inv_bc1 = 1.0f, inv_bc2 = 1.0f;
       if (epi.upd.optimizer == SEG_ADAM) { inv_bc1 = 1.0f / __ldg(epi.upd.bc); inv_bc2 = 1.0f / __ldg(epi.upd.bc + 1); }
       unsigned int needed = 0;
@@ -1126,7 +1125,7 @@ constexpr int PAIR_STAGES_STAGED = 5;      // with it: ring + staging stay withi
 constexpr int PAIR_SMEM = PAIR_STAGES * PAIR_STAGE_BYTES + SMEM_EXTRA;   // upper bound of both layouts
 
 template <bool TF32, bool A_MN, bool B_MN, bool FUSED = false>
-__global__ void __launch_bounds__(FUSED ? NUM_THREADS_FUSED : NUM_THREADS_PAIR, 1)
+__global__ void __launch_bounds__(FUSED ? NUM_THREADS_FUSED : NUM_THREADS, 1)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                     const __grid_constant__ CUtensorMap map_c, int M, int N, int K, EpilogueArgs epi, int* dev_status,
                     int group_m, int n_stages, int tile_n) {
@@ -1145,7 +1144,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   uint8_t* smem_a = smem;
   uint8_t* smem_b = smem + STAGES * A_TILE_BYTES;
   uint8_t* stage_out = smem + STAGES * PAIR_STAGE_BYTES;               // 1024-byte aligned
-  uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + (epi.staged ? PAIR_STAGE_OUT_BYTES : 0));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + (epi.staged ? STAGE_OUT_BYTES : 0));
   // bars[0..S) full (used in the even CTA), [S..2S) empty, [2S..2S+2) tmem_full, [2S+2..2S+4) tmem_empty (even CTA)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -1266,7 +1265,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   } else if (warp < 2 + EPI_WARPS) {
     // ---------------- epilogue warps: each CTA drains its own 128 rows ----------------
     const int quarter = warp & 3, part = (warp - 2) >> 2;    // (a warp reads the TMEM lanes of its index modulo 4)
-    uint8_t* my_stage_out = stage_out + (FUSED ? quarter * 2 : part * 4 + quarter) * STAGE_OUT_WARP_BYTES;
+    uint8_t* my_stage_out = stage_out + (part * 4 + quarter) * STAGE_OUT_WARP_BYTES;
     int acc = 0; uint32_t acc_phase = 0;
     bool ok = true;
     for (int t = pair; t < n_tiles && ok; t += n_pairs) {
@@ -1289,7 +1288,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (FUSED || !epi.staged) {        // (the update warps read the tile back with ordinary loads: ordinary stores)
           if (row < M) epilogue_store(epi, v, side, row, col0, n_end);
         } else {
-          epilogue_store_staged<FUSED ? 2 : 1>(epi, &map_c, my_stage_out, v, side, lane, m0 + quarter * 32, col0, n_end, M, c / EPI_PER_QUARTER);
+          epilogue_store_staged(epi, &map_c, my_stage_out, v, side, lane, m0 + quarter * 32, col0, n_end, M);
         }
         side = side_next;
       }
@@ -1302,8 +1301,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     if (lane == 0) tma_store_wait_all();   // the staging buffers are read, and the output written, before the CTA leaves
   } else if constexpr (FUSED) {
     // ---------------- update warps: the optimizer on this CTA's 128 rows of every tile of the pair ----------------
-    if (warp >= NUM_THREADS / 32) {
-      const int uw = warp - NUM_THREADS / 32;
+    if (warp >= FUSED_UPDATE_WARP0) {
+      const int uw = warp - FUSED_UPDATE_WARP0;
       float inv_bc1 = 1.0f, inv_bc2 = 1.0f;
       if (epi.upd.optimizer == SEG_ADAM) { inv_bc1 = 1.0f / __ldg(epi.upd.bc); inv_bc2 = 1.0f / __ldg(epi.upd.bc + 1); }
       unsigned int needed = 0;
@@ -1522,9 +1521,9 @@ cudaError_t launch_pair_variant(const CUtensorMap& ma, const CUtensorMap& mb, co
   const int pairs = std::min(tiles, num_sms() / 2);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
-  cfg.blockDim = dim3(FUSED ? NUM_THREADS_FUSED : NUM_THREADS_PAIR, 1, 1);
+  cfg.blockDim = dim3(FUSED ? NUM_THREADS_FUSED : NUM_THREADS, 1, 1);
   const int n_stages = e.staged ? PAIR_STAGES_STAGED : PAIR_STAGES;
-  cfg.dynamicSmemBytes = n_stages * PAIR_STAGE_BYTES + (e.staged ? PAIR_STAGE_OUT_BYTES : 0) + SMEM_EXTRA;
+  cfg.dynamicSmemBytes = n_stages * PAIR_STAGE_BYTES + (e.staged ? STAGE_OUT_BYTES : 0) + SMEM_EXTRA;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1599,21 +1598,22 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_u
 
 // CTAs per 128 x 64 tile of the split-K kernel (2 or 4), or 1 where a persistent kernel takes the product.  A k-block costs a CTA
 // about 0.27 us (its ring holds three), the exchange 1 us, the epilogue 1.8 us by the CTAs that share it; a persistent kernel's
-// epilogue takes 1.2 us more than its estimate says.  A weight gradient runs beside those of the layers above, from which a split
-// takes SMs: half a microsecond has to be gained there.  Whole steps of 78 nets (13 shapes, TF32 and bf16, batch 64 to 1024), against
-// the bulk-copy exchange and the line it had: 1.129 times as fast in the geometric mean, none slower; with 0.3 instead of 1.2 it is
-// 1.112, with 0.7 for weight gradients 1.125 and the worst 0.966.  A step of 512-512-256-47 (TF32, batch 256) 45.1 -> 34.9 us, of
-// 784-1024-1024-512 55.8 -> 50.4, of 72-136-64 (bf16, batch 64) 24.6 -> 20.5.
+// epilogue takes 0.6 us more than its estimate says.  Every CTA also takes its share of the GPU from what runs beside the product,
+// the upper layers' weight gradients or another segment: 1.5 us for all SMs; a weight gradient, which runs beside others by itself,
+// has to gain half a microsecond on top.  Whole steps of 90 nets (15 shapes, TF32 and bf16, batch 64 to 1024), geometric mean of the
+// speed against the bulk-copy exchange, four epilogue warps and the line they had: 1.150 with one handle (worst 0.99), 1.131 with
+// three handles on streams of their own (worst 0.96); without the share of the GPU 1.152 and 1.114 (worst 0.92).
 int pick_split(int M, int N, int K, bool tf32, bool wgrad) {
   const int tiles = ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
-  const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64);
+  const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64), sms = num_sms();
   const Choice other = pick_kernel(M, N, K, tf32, false, false);
   if (g_pair_min_tiles > 0 && other.kind == 1) return 1;    // CTA pairs are forced
+  auto share_us = [&](int ctas) { return 1.5 * std::min(ctas, sms) / sms; };
   int best = 1;
-  double best_us = other.us + (wgrad ? -0.5 : 1.2);
+  double best_us = other.us + share_us(tiles) + (wgrad ? -0.5 : 0.6);
   for (int sp : {2, 4}) {
-    if (tiles * sp > num_sms()) break;
-    const double us = 0.27 * ((num_k + sp - 1) / sp) + 1.0 + 1.8 / sp;
+    if (tiles * sp > sms) break;
+    const double us = 0.27 * ((num_k + sp - 1) / sp) + 1.0 + 1.8 / sp + share_us(tiles * sp);
     if (us < best_us) { best = sp; best_us = us; }
   }
   return best;
@@ -1680,17 +1680,13 @@ cudaError_t launch_wait_selftest(int* dev_status, uint64_t limit_ns, cudaStream_
   return cudaGetLastError();
 }
 
-// The mean-squared-error loss of a non-final segment is fused into the split-K kernel, the one that
-// serves the small, latency-bound products: there it replaces a launch on the critical path for about
-// 3 us of extra epilogue (paper_shaped: -3 us per step).  In the single-CTA kernel of mid-sized
-// products the same epilogue measured slower than the separate loss launch (bf16_wide 1024x2048x4096:
-// 44 us against 25 + 14 us under ncu), and the CTA-pair kernel serves large products, where a separate
-// loss launch costs next to nothing.  Softmax cross-entropy was tried in the epilogue of the single-CTA
-// kernel in three forms - one thread per row of at most 64 logits unrolled in registers (3-4 times slower
-// than the separate warp-per-row kernel), the tile left in shared memory with each warp walking its 32
-// rows, lanes over the classes (slower still: 32 dependent reduction chains per warp), and one thread
-// per row with short loops over its row in shared memory (about the cost of the launch it saves, and
-// it gives up the split over K) - and stays a launch of its own.
+// The losses are fused into the split-K kernel, the one that serves the small, latency-bound products, where they replace a launch on
+// the critical path: the mean-squared error wherever that kernel runs the last product, the softmax cross-entropy where one tile
+// holds whole rows (at most 64 classes), with four CTAs to a tile whatever K is, since the epilogue is the longer part (a step of
+// 512-512-256-47 in TF32, batch 256: 46.6 -> 42.2 us together with the exchange from registers).  In the persistent kernels the same epilogues measured slower than the
+// separate loss launch (mean-squared error, 1024x2048x4096: 44 us against 25 + 14 under ncu; cross-entropy with one thread per row or
+// one warp per 32 rows: slower by up to four times), and the CTA-pair kernel serves large products, where a separate loss launch
+// costs next to nothing.
 double gemm_tc_estimate_us(int M, int N, int K, bool tf32) {
   return 3.0 + pick_kernel(M, N, K, tf32, false, false).us;         // + launch, first loads and drain
 }

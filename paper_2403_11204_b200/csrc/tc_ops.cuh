@@ -86,9 +86,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
                ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c0), "r"(c1) : "memory");
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
-// at most one of this thread's bulk stores may still be reading its shared-memory source
-__device__ __forceinline__ void tma_store_wait_source_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-// none of them may
+// none of this thread's bulk stores may still be reading its shared-memory source
 __device__ __forceinline__ void tma_store_wait_source() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // all of this thread's bulk stores are complete
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
