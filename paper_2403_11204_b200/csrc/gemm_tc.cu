@@ -908,6 +908,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         }
       }
       if constexpr (LOSS != LOSS_NONE) cls[i] = __ldg(epi.loss.cls + row);
+      if (LOSS == LOSS_CE) cls[i] = min(max(cls[i], 0), N - 1);   // (a recovery step's are clamped to the left segment's classes)
       if (LOSS == LOSS_MSE && n_cols > 0) {                // the label row of the sample's class
         const float* t = epi.loss.sil + (int64_t)cls[i] * N + col;
         side[i] = load_piece(t, n_cols, whole && (reinterpret_cast<uintptr_t>(t) & 15u) == 0);

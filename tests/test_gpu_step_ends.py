@@ -62,3 +62,26 @@ def test_classes_of_minus_infinity(precision, n_classes, monkeypatch):
         gpu.close()
     for a, b in zip(*out):
         assert rel_err(a, b) <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision", ["tf32", "fp32"])
+def test_recovery_clamps_classes_to_the_right_segments(precision):
+    """A left segment of more classes than the right one has: an index beyond the right segment's counts as its last class, whichever
+    kernel forms the loss."""
+    import torch
+    from paper_2403_11204_b200 import binding
+    from paper_2403_11204_b200.binding import Segment
+    x, cls = arrays(150, 72, 47, precision)
+    out = []
+    for c in (cls, np.minimum(cls, 9)):
+        left = Segment([72, 200, 136], 47, False, precision=precision, optimizer="sgd", lr=0.01, max_batch=150)
+        right = Segment([136, 160, 10], 10, True, precision=precision, optimizer="sgd", lr=0.01, max_batch=150, segment_id=1)
+        left.gen_labels(1, "normal")
+        loss = torch.zeros(1, device="cuda")
+        binding.recovery_step(left, right, torch.from_numpy(x).cuda(), torch.from_numpy(c.astype(np.int32)).cuda(), loss)
+        left.poll()
+        out.append([loss.cpu().numpy()] + [t.cpu().numpy() for l in range(2) for t in left.grads(l)])
+        left.close()
+        right.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
