@@ -296,8 +296,7 @@ LossFuse loss_fuse_desc(seg_handle* h, int batch, const int32_t* cls) {
   return f;
 }
 
-// The segment's loss as a launch of its own (the final segment's softmax cross-entropy always; the
-// intermediate-label loss when the last forward product could not take it).
+// The segment's loss as a launch of its own, where the last forward product could not take it (LossFuse).
 seg_status launch_loss(seg_handle* h, int batch, const int32_t* cls) {
   const int L = h->n_layers;
   Launch l(h, K_LOSS, h->stream);
