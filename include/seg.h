@@ -268,11 +268,12 @@ SEG_API seg_status seg_product_launches(const seg_handle* h, uint64_t* counts);
  * a class index outside [0, M), SEG_ERR_CUDA on a CUDA error.  The record is cleared.       */
 SEG_API seg_status seg_poll_status(seg_handle* h);
 
-/* Self-test of the bounded wait every product kernel uses: launches one small block that waits,
- * with the product kernels' own wait routine, on a barrier nothing ever arrives at, for at most
- * limit_ns nanoseconds (1,000 .. 1,000,000,000; SEG_ERR_INVALID_ARG otherwise).  The wait runs
- * out, the block records it in the handle's status word and returns; the next seg_poll_status
- * reports SEG_ERR_DEVICE_TIMEOUT and the handle stays usable.  Nothing faults or hangs.        */
+/* Self-test of the bounded wait every product kernel uses: launches a cluster of two small blocks,
+ * the first of which waits, with the product kernels' own wait routine and for at most limit_ns
+ * nanoseconds (1,000 .. 1,000,000,000; SEG_ERR_INVALID_ARG otherwise), for something the second sends
+ * it only after that wait has run out.  The first block stays for it, as the blocks of a split product
+ * do, and records the time-out in the handle's status word when it has arrived; the next
+ * seg_poll_status reports SEG_ERR_DEVICE_TIMEOUT and the handle stays usable.  Nothing faults or hangs. */
 SEG_API seg_status seg_selftest_bounded_wait(seg_handle* h, uint64_t limit_ns);
 
 /* Hand-off between segments that live on different devices (Section 2.1: each partition trains on

@@ -625,10 +625,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
   // ---------------- teardown ----------------
   __syncwarp();
-  if (*abort_flag) {
-    // give copies and MMAs still in flight time to land before shared memory and TMEM are released
-    for (int i = 0; i < 64; ++i) __nanosleep(20000);
-  }
+  if (*abort_flag) linger();          // copies and MMAs still in flight land before shared memory and TMEM are released
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -645,6 +642,17 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // address of the same shared-memory location in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t rank) {
   uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank)); return r;
+}
+// End of a CTA into whose shared memory its peers send, by every warp, behind the cluster's first barrier phase.  Nothing of it is read
+// by the peers, so where all its waits passed it has received what they send and leaves before them.  Where a wait was given up, a
+// peer may still send: the CTA stays until every other thread of the cluster has exited or come here too (their waits are bounded,
+// and the barrier counts threads that have not exited), and then until what was sent last has landed.
+__device__ __forceinline__ void cluster_leave(volatile int* abort_flag) {
+  if (__any_sync(0xFFFFFFFFu, *abort_flag != 0)) {
+    cluster_arrive();
+    cluster_wait();
+    linger();
+  }
 }
 constexpr int SPLITK_BLOCK_N = 64;
 // Three stages: 106 KiB per CTA, so that two CTAs share an SM.  What that buys is not this kernel's own time but its neighbours':
@@ -860,6 +868,8 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     }
     __syncwarp();
     asm volatile("bar.sync 2, 288;" ::: "memory");         // the epilogue warps have drained the accumulator
+    if (*abort_flag) linger();                             // or given up waiting for MMAs that may still write it
+    __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, TMEM_COLS);
   } else {
@@ -1066,13 +1076,9 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     }
   }
 
-  // Nothing of this CTA is read by its peers, and it has received what they send: it may leave before them.
   __syncwarp();
   if (warp < 2) cluster_wait();
-  if (*abort_flag) {
-    // a wait was given up: leave time for copies in flight to land, and for peers to send or give up (their waits are bounded)
-    for (int i = 0; i < 4000; ++i) __nanosleep(1000000);
-  }
+  cluster_leave(abort_flag);
 }
 
 
@@ -1322,9 +1328,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 
   // ---------------- teardown ----------------
   __syncwarp();
-  if (*abort_flag) {
-    for (int i = 0; i < 64; ++i) __nanosleep(20000);
-  }
+  if (*abort_flag) linger();
   tc_fence_before();
   __syncthreads();
   cluster_arrive();                   // the pair releases its tensor memory together, after both are done
@@ -1662,22 +1666,47 @@ bool make_map_f32(CUtensorMap* map, const void* base, uint64_t inner, uint64_t o
 
 // ---- self-test of the bounded wait ---------------------------------------------------------------
 namespace {
-__global__ void __launch_bounds__(32)
+// Two blocks of a cluster, as in the split-K kernel.  The first waits, with the limit, for a send that the second makes only once it has
+// been told that the wait ran out; the time-out is recorded when the send has landed in the shared memory of the first, which has to be
+// there still.  The second block's own wait is bounded too.
+constexpr float SELFTEST_SENT = 47.f;
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32)
 wait_selftest_kernel(int* dev_status, uint64_t limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_flag;
+  __shared__ __align__(16) float late[4];
+  __shared__ uint64_t bars[2];               // the late send; "the wait has run out"
+  __shared__ int abort_flag, ran_out;
+  const uint32_t rank = cluster_ctarank(), late_bar = smem_u32(&bars[0]), told_bar = smem_u32(&bars[1]);
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    mbar_init(smem_u32(&bar), 1);
+    ran_out = 0;
+    late[0] = 0.f;
+    mbar_init(late_bar, 1);
+    mbar_init(told_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // nothing ever arrives at this barrier: the wait below ends only through its own time limit
-    mbar_wait(smem_u32(&bar), 0, &abort_flag, dev_status, limit_ns);
+    if (rank == 0) mbar_arrive_expect_tx(late_bar, 16);
   }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();                            // both blocks' barriers exist
+  if (threadIdx.x == 0) {
+    if (rank == 0) {
+      mbar_wait(late_bar, 0, &abort_flag, &ran_out, limit_ns);
+      mbar_arrive_cluster(map_to_cta(told_bar, 1));
+    } else if (mbar_wait(told_bar, 0, &abort_flag, &ran_out, limit_ns + WAIT_LIMIT_NS)) {
+      linger(100000);                        // the first block is at its end by now
+      send_to_peer(map_to_cta(smem_u32(late), 0), map_to_cta(late_bar, 0), SELFTEST_SENT, 0.f, 0.f, 0.f);
+    }
+  }
+  __syncwarp();
+  cluster_leave(&abort_flag);
+  if (rank == 0 && threadIdx.x == 0 && ran_out == DEV_TIMEOUT && mbar_try_wait(late_bar, 0) &&
+      *const_cast<volatile float*>(late) == SELFTEST_SENT)
+    atomicOr(dev_status, (int)DEV_TIMEOUT);
 }
 }  // namespace
 
 cudaError_t launch_wait_selftest(int* dev_status, uint64_t limit_ns, cudaStream_t s) {
-  wait_selftest_kernel<<<1, 32, 0, s>>>(dev_status, limit_ns);
+  wait_selftest_kernel<<<2, 32, 0, s>>>(dev_status, limit_ns);
   return cudaGetLastError();
 }
 

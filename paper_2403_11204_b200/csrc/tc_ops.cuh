@@ -40,6 +40,13 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
+// At least LINGER_NS (which __nanosleep, free to return at once, does not promise), and bounded: the time that a block which gave up a
+// wait leaves its copies and MMAs in flight to land before it gives up the memory they use.
+constexpr uint64_t LINGER_NS = 2000000ull;
+__device__ __forceinline__ void linger(uint64_t ns = LINGER_NS) {
+  const uint64_t t0 = global_timer_ns();
+  for (int i = 0; i < 65536 && global_timer_ns() - t0 < ns; ++i) __nanosleep(20000);
+}
 // Bounded wait.  Returns false when the wait was abandoned (own time-out or another role's abort).
 // The product kernels pass the compile-time limit; the self-test kernel passes a short one.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,

@@ -85,3 +85,26 @@ def test_recovery_clamps_classes_to_the_right_segments(precision):
         right.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("limit_ns", [1_000, 1_000_000, 50_000_000])
+def test_a_block_that_gave_up_stays_for_its_peer_and_no_longer(limit_ns):
+    """The end of a split product's block whose wait ran out: a peer that sends only afterwards still finds its shared memory (the
+    time-out is recorded once that send has landed), and it does not outstay the peer by more than milliseconds."""
+    import time
+    import torch
+    from paper_2403_11204_b200.binding import SegError
+    gpu, ora = make_pair([264, 160, 47], 47, True, "tf32", "sgd", 0.01, 70)
+    x, cls = arrays(70, 264, 47, "tf32")
+    torch.cuda.synchronize()
+    for _ in range(2):                               # the first call loads the kernel
+        t0 = time.perf_counter()
+        gpu.selftest_bounded_wait(limit_ns)
+        with pytest.raises(SegError) as e:
+            gpu.poll()
+        took = time.perf_counter() - t0
+        assert e.value.status == 7
+    assert limit_ns * 1e-9 <= took <= limit_ns * 1e-9 + 0.25
+    gpu.poll()
+    compare_step(gpu, ora, x, cls, "tf32", TOL["tf32"])
+    gpu.close()
