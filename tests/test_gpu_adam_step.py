@@ -43,3 +43,34 @@ def test_adam_step_against_64_bits(precision, eps, scale):
     assert P[3, 5] == W0[3, 5] and np.isinf(V[3, 5])
     np.testing.assert_allclose(M, m1, rtol=0, atol=4 * U * (np.abs(m0) + np.abs(gw)).max())
     seg.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_adam_step_outside_the_range_of_its_fast_form(precision):
+    """A second moment below zero, however small, has no root; a denominator near the end of fp32's range still divides."""
+    import torch
+    from paper_2403_11204_b200.binding import Segment
+    widths, batch = [157, 200], 64
+    x = torch.rand(batch, widths[0], device="cuda")
+    cls = torch.zeros(batch, device="cuda", dtype=torch.int32)
+    for eps in (1e-8, 1e-3, 3e38):
+        seg = Segment(widths, 47, False, precision=precision, optimizer="adam", lr=1.0, eps=eps, max_batch=batch, init_seed=2)
+        seg.gen_labels(1, "normal")
+        W, b = [t.clone() for t in seg.params(0)]
+        m, v = torch.full_like(W, 2e38 if eps > 1 else 0.5), torch.zeros_like(W)
+        v[5, :6] = -torch.tensor([1e-41, 2e-38, 1e-36, 1e-33, 1e-20, 1.0], device="cuda")
+        b[:] = 1.0
+        b[5] = -1.0                                            # never fires: no gradient is added to that row's moments
+        seg.set_params(0, torch.zeros_like(W), b)
+        seg.set_opt_state(0, 0, m, torch.zeros_like(b))
+        seg.set_opt_state(0, 1, v, torch.zeros_like(b))
+        seg.set_step(1 << 20)                                  # bias corrections of one
+        seg.train_step(x.to(torch.bfloat16) if precision == "bf16" else x, cls)
+        seg.poll()
+        g, P = seg.grads(0)[0], seg.params(0)[0]
+        assert torch.all(g[5] == 0) and torch.any(g != 0)
+        assert torch.all(torch.isnan(P) == (v < 0))
+        if eps > 1:
+            want = -(0.9 * m + 0.1 * g).double() / eps         # -0.6: the root of v is nothing beside eps
+            assert torch.all((P.double() - want)[v >= 0].abs() <= 1e-6)
+        seg.close()
