@@ -156,6 +156,15 @@ constexpr int FRING_FLOATS = FSTAGES * FSTAGE_FLOATS;
 constexpr size_t FSMEM = 1024 + (size_t)(FRING_FLOATS + FT * FT) * sizeof(float);
 static_assert(FGROUPS * FT * FPART <= FRING_FLOATS, "the partial tiles take the ring's place");
 
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
+
 struct FfmaEpi { void* C; int64_t ldc, ldmask; int c_round, epi, relu; const float* bias; const float* mask; };
 
 template <int FORM>

@@ -127,44 +127,6 @@ __device__ __forceinline__ void dot_rows(float (&v)[VP], const float* A, int pa,
   }
 }
 
-// The same with packed multiply-adds, even and odd k in the halves of a pair: half the issue slots, so that the loads of one of a
-// scheduler's two warps go out beside the arithmetic of the other.  784-80-60 at batch 1410 (12 x 5 sums per lane): 28.65 -> 28.25 us
-// per step; at 8 x 8 sums (784-128-128-64 at batch 64) nothing, and beyond 60 the pairs crowd the registers: those keep the plain form.
-template <int RT, int CT, int VP>
-__device__ __forceinline__ void dot_rows_packed(float (&v)[VP], const float* A, int pa, const float* const (&wp)[CT], int c0, int chunks, int step) {
-  f32x2 acc[RT * CT];
-#pragma unroll
-  for (int i = 0; i < RT * CT; ++i) acc[i] = 0ull;
-  auto chunk = [&](int c, bool own) {
-    ulonglong2 w[CT];
-#pragma unroll
-    for (int j = 0; j < CT; ++j) {
-      w[j] = *reinterpret_cast<const ulonglong2*>(wp[j] + 4 * c);
-      if (!own) w[j] = make_ulonglong2(0ull, 0ull);
-    }
-#pragma unroll
-    for (int r = 0; r < RT; ++r) {
-      ulonglong2 a = *reinterpret_cast<const ulonglong2*>(A + r * pa + 4 * c);
-      if (!own) a = make_ulonglong2(0ull, 0ull);
-#pragma unroll
-      for (int j = 0; j < CT; ++j) fma2(acc[r * CT + j], a.x, w[j].x);
-#pragma unroll
-      for (int j = 0; j < CT; ++j) fma2(acc[r * CT + j], a.y, w[j].y);
-    }
-  };
-  const int full = chunks / step;
-  int c = c0;
-#pragma unroll 1
-  for (int i = 0; i < full; ++i, c += step) chunk(c, true);
-  if (full * step < chunks) chunk(min(c, chunks - 1), c < chunks);
-#pragma unroll
-  for (int i = 0; i < RT * CT; ++i) {
-    float lo, hi;
-    unpack2(acc[i], lo, hi);
-    v[i] = lo + hi;
-  }
-}
-
 // A forward link for R rows: every element n < N (rounded up to 4) of A W^T.  Warp = (half of the rows, block of 8 * CT columns),
 // lane = (column, quarter of the contraction).  side(r, n) is what the element's epilogue needs from shared memory, fetched
 // ahead of the arithmetic; emit(r, n, value, side) finishes the element.
@@ -458,8 +420,7 @@ small_fwd_bwd_kernel(const __grid_constant__ SmallStep p, const float* __restric
       if (elect_one()) tensor_store(&map_stage, xs, k0, rb0);
     }
     const int kc = max(0, min(q.ks, n0 - k0) + 3) >> 2;     // 16-byte groups that hold features
-    if constexpr (V <= 60) dot_rows_packed<R, CT0, VP>(v, xs + owner * R * q.ks, q.ks, wp, 2 * kw + (lane >> 4), kc, 2 * KW);
-    else dot_rows<R, CT0, VP>(v, xs + owner * R * q.ks, q.ks, wp, 2 * kw + (lane >> 4), kc, 2 * KW);
+    dot_rows<R, CT0, VP>(v, xs + owner * R * q.ks, q.ks, wp, 2 * kw + (lane >> 4), kc, 2 * KW);
     reduce_scatter<V, 2>(v, lane);
     // [owner][kw][row][column] in the send buffer, the own rows' share straight into the receive buffer
     float* out = owner == rank ? sm + q.off_recv + (size_t)(rank * KW + kw) * R * N4 : sm + q.off_send + (size_t)(owner * KW + kw) * R * N4;
