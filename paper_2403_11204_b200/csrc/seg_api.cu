@@ -608,7 +608,7 @@ seg_status seg_create(const seg_config* cfg, seg_handle** out) {
     p.sil = h->sil; p.cls_stage = h->cls_stage;
     p.loss_partials = h->loss_partials; p.loss_dst = h->loss_dst;
     p.t = h->step_dev; p.bc = h->bc_dev; p.dev_status = h->dev_status;
-    p.lr = h->lr; p.momentum = h->momentum; p.beta1 = h->beta1; p.beta2 = h->beta2; p.eps = h->eps;
+    p.lr = h->lr; p.momentum = h->momentum; p.beta1 = h->beta1; p.beta2 = h->beta2; p.eps = h->eps; p.adam_least = adam_least(h->eps);
     for (int l = 0; l < h->n_layers; ++l) {
       ++h->launches;
       if (launch_small_ones(p.act[l], p.ld_act[l], p.widths[l], h->max_batch, h->stream) != cudaSuccess) return bail(SEG_ERR_CUDA);
@@ -801,7 +801,7 @@ static seg_status enqueue_backward(seg_handle* h, int batch, bool forked, const 
       f.s1 = h->state1 ? h->state1 + lo : nullptr; f.s2 = h->state2 ? h->state2 + lo : nullptr;
       f.p_op = reinterpret_cast<char*>(h->params_op) + lo * elem_size(h->op_dt);
       f.op_dt = h->op_dt; f.op_round = h->op_round; f.optimizer = h->optimizer;
-      f.lr = h->lr; f.momentum = h->momentum; f.beta1 = h->beta1; f.beta2 = h->beta2; f.eps = h->eps;
+      f.lr = h->lr; f.momentum = h->momentum; f.beta1 = h->beta1; f.beta2 = h->beta2; f.eps = h->eps; f.adam_least = adam_least(h->eps);
       f.bc = h->bc_dev;
     }
     bool w_on_tc = false;
@@ -818,7 +818,7 @@ static seg_status enqueue_backward(seg_handle* h, int batch, bool forked, const 
     u.n = fused ? 0 : Ly.b_off - lo; u.optimizer = h->optimizer;
     u.dz = dz_l; u.dz_dt = h->act_dt; u.ld_dz = ld_dz; u.batch = batch; u.n_bias = Ly.out;
     u.bias_off = Ly.b_off - lo; u.g_bias = h->grads + Ly.b_off;
-    u.lr = h->lr; u.momentum = h->momentum; u.beta1 = h->beta1; u.beta2 = h->beta2; u.eps = h->eps;
+    u.lr = h->lr; u.momentum = h->momentum; u.beta1 = h->beta1; u.beta2 = h->beta2; u.eps = h->eps; u.adam_least = adam_least(h->eps);
     u.bc = h->bc_dev;
     if (l == 0) {
       u.loss_partials = loss_of->loss_partials; u.n_loss = loss_of->n_loss_partials; u.loss_dst = h->loss_dst;
