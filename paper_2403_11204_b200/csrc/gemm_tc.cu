@@ -1605,20 +1605,25 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_u
 // about 0.27 us (its ring holds three), the exchange 1 us, the epilogue 1.8 us by the CTAs that share it; a persistent kernel's
 // epilogue takes 0.6 us more than its estimate says.  Every CTA also takes its share of the GPU from what runs beside the product,
 // the upper layers' weight gradients or another segment: 1.5 us for all SMs; a weight gradient, which runs beside others by itself,
-// has to gain half a microsecond on top.  Whole steps of 90 nets (15 shapes, TF32 and bf16, batch 64 to 1024), geometric mean of the
-// speed against the bulk-copy exchange, four epilogue warps and the line they had: 1.150 with one handle (worst 0.99), 1.131 with
-// three handles on streams of their own (worst 0.96); without the share of the GPU 1.152 and 1.114 (worst 0.92).
-int pick_split(int M, int N, int K, bool tf32, bool wgrad) {
+// has to gain half a microsecond on top.  A bf16 forward product costs 0.2 us more as clusters of two: without that the last layer of
+// 144-336-992-336 at batch 1024 (48 tiles, 16 k-blocks) takes 96 SMs, one handle's step 44.4 us instead of 45.1, but each of three
+// handles' 25.3 instead of 23.2 (24.3 before there were such clusters), and of 200-400-1000-400 49.1 instead of 49.5 and 28.7 instead
+// of 27.6; in TF32 the same product gains either way (three handles 37.2 -> 33.4).  Whole steps of 210 nets (21 shapes, TF32 and bf16,
+// batch 64 to 1024), geometric mean of the speed against the bulk-copy exchange, four epilogue warps and the line they had: 1.156 with
+// one handle (worst 1.00), 1.132 with three handles on streams of their own (worst 0.995; 0.960 without the 0.2).  Without the share of
+// the GPU, 90 of these nets: 1.152 and 1.114 (worst 0.92).
+int pick_split(int M, int N, int K, bool tf32, Form form) {
   const int tiles = ((M + BLOCK_M - 1) / BLOCK_M) * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N);
   const int num_k = (K + (tf32 ? 32 : 64) - 1) / (tf32 ? 32 : 64), sms = num_sms();
   const Choice other = pick_kernel(M, N, K, tf32, false, false);
   if (g_pair_min_tiles > 0 && other.kind == 1) return 1;    // CTA pairs are forced
   auto share_us = [&](int ctas) { return 1.5 * std::min(ctas, sms) / sms; };
   int best = 1;
-  double best_us = other.us + share_us(tiles) + (wgrad ? -0.5 : 0.6);
+  double best_us = other.us + share_us(tiles) + (form == FORM_TN ? -0.5 : 0.6);
   for (int sp : {2, 4}) {
     if (tiles * sp > sms) break;
-    const double us = 0.27 * ((num_k + sp - 1) / sp) + 1.0 + 1.8 / sp + share_us(tiles * sp);
+    double us = 0.27 * ((num_k + sp - 1) / sp) + 1.0 + 1.8 / sp + share_us(tiles * sp);
+    if (sp == 2 && form == FORM_NT && !tf32) us += 0.2;
     if (us < best_us) { best = sp; best_us = us; }
   }
   return best;
@@ -1725,7 +1730,7 @@ int gemm_tc_fused_loss_partials(int kind, int M, int N, int K, bool tf32) {
   if (!g_init_ok || !g_allow_splitk) return 0;
   const int tiles_m = (M + BLOCK_M - 1) / BLOCK_M;
   if (kind == LOSS_CE) return N <= SPLITK_BLOCK_N && CE_SPLIT * tiles_m <= num_sms() ? CE_SPLIT * tiles_m : 0;
-  const int split = pick_split(M, N, K, tf32, false);
+  const int split = pick_split(M, N, K, tf32, FORM_NT);
   return split > 1 ? split * tiles_m * ((N + SPLITK_BLOCK_N - 1) / SPLITK_BLOCK_N) : 0;
 }
 
@@ -1741,7 +1746,7 @@ bool gemm_tc_can_fuse_update(const GemmDesc& g) {
   if ((g.a_sk * esz) % 16 != 0 || (g.b_sk * esz) % 16 != 0) return false;
   if ((reinterpret_cast<uintptr_t>(g.C) & 15u) || (g.ldc & 3)) return false;
   const bool throughput = g.off_critical_path != 0;
-  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32, true) : 1;
+  const int split = (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32, FORM_TN) : 1;
   return split == 1;
 }
 
@@ -1770,7 +1775,8 @@ cudaError_t launch_gemm_tc(const GemmDesc& g, int* dev_status, cudaStream_t s, i
   if (fuse_loss && (a_mn || b_mn || gemm_tc_fused_loss_partials(fuse_loss, g.M, g.N, g.K, tf32) == 0))
     return cudaErrorInvalidValue;                           // the caller asks gemm_tc_fused_loss_partials first
   const bool throughput = g.off_critical_path != 0;
-  const int split = fuse_loss == LOSS_CE ? CE_SPLIT : (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32, a_mn) : 1;
+  const Form form = a_mn ? FORM_TN : b_mn ? FORM_NN : FORM_NT;
+  const int split = fuse_loss == LOSS_CE ? CE_SPLIT : (g_allow_splitk && !throughput) ? pick_split(g.M, g.N, g.K, tf32, form) : 1;
   const Choice choice = pick_kernel(g.M, g.N, g.K, tf32, throughput, g.upd.enabled != 0);
   const bool pairs = (split == 1) && choice.kind == 1;
   const int block_n = split > 1 ? SPLITK_BLOCK_N : choice.block_n;

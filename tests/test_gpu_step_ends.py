@@ -108,3 +108,17 @@ def test_a_block_that_gave_up_stays_for_its_peer_and_no_longer(limit_ns):
     gpu.poll()
     compare_step(gpu, ora, x, cls, "tf32", TOL["tf32"])
     gpu.close()
+
+
+@pytest.mark.parametrize("batch", [900, 1024])
+def test_a_short_bf16_forward_product_does_not_take_clusters_of_two(batch):
+    """The last layer of 144-336-992-336 (48 tiles, 16 k-blocks) would take 96 SMs as clusters of two, which three handles beside each
+    other pay for; the dgrad of the same shape and the weight gradient of layer 0 are split."""
+    import torch
+    from paper_2403_11204_b200.binding import Segment
+    seg = Segment([144, 336, 992, 336], 47, False, precision="bf16", optimizer="sgd", lr=1e-3, max_batch=batch)
+    seg.gen_labels(1, "normal")
+    seg.train_step(torch.rand(batch, 144, device="cuda").to(torch.bfloat16), torch.zeros(batch, device="cuda", dtype=torch.int32))
+    seg.poll()
+    assert seg.product_launches()["tc_splitk"] == 2
+    seg.close()
