@@ -8,7 +8,8 @@
 //
 // CTA = 10 warps.  A thread of warp 0 issues TMA loads into a ring of shared-memory stages; warp 1 owns the
 // TMEM allocation and one of its threads issues the MMAs; the other eight warps drain the accumulator (a warp
-// reads its own 32 TMEM lanes), apply the epilogue and store.  Two accumulator buffers in TMEM let the epilogue of tile i overlap the main loop of tile i+1.
+// reads its own 32 TMEM lanes), apply the epilogue and store.  Two accumulator buffers in TMEM let the
+// epilogue of tile i overlap the main loop of tile i+1.
 //
 // Shared-memory operand tiles use the 128-byte swizzle.  K-major tile: rows of 128 bytes (64 bf16
 // or 32 TF32 along K), 8-row groups 1024 bytes apart.  MN-major tile: chunks of 64 bf16 / 32 TF32
@@ -21,8 +22,8 @@
 // cluster of 2 or 4 CTAs shares one 128 x 64 output tile, each CTA contracts its own slice of K
 // into TMEM, and the partial tiles are combined through distributed shared memory as a
 // reduce-scatter (every CTA sends column slice j of its partial from its registers into CTA j's shared
-// memory; CTA j adds what it received and runs the epilogue on that slice, the loss of the segment's last layer included).  One SM's shared-memory fill rate
-// bounds a single CTA's main loop, so spreading K over a cluster shortens exactly the part of the
+// memory; CTA j adds what it received and runs the epilogue on that slice, the loss of the segment's last
+// layer included).  One SM's shared-memory fill rate bounds a single CTA's main loop, so spreading K over a cluster shortens exactly the part of the
 // kernel that grows with the problem.
 //
 // Large problems use gemm_tc_pair_kernel: two CTAs of a cluster share one 256 x 256 output tile
@@ -124,17 +125,16 @@ struct SmemLayout {
 // global-memory latency is off the critical path.
 struct EpiSide { uint32_t w[32]; };
 
-template <int NV = 32>
 __device__ __forceinline__ void epilogue_prefetch(const EpilogueArgs& e, EpiSide& s, int row, bool row_ok,
                                                   int col0, int n_total) {
-  const int n_valid = min(NV, n_total - col0);
+  const int n_valid = min(32, n_total - col0);
   if (n_valid <= 0) return;
   const bool whole = (n_valid & 7) == 0;
   if (e.epi == EPI_BIAS_ACT) {
     const float* brow = e.bias + col0;
     if (whole && ((reinterpret_cast<uintptr_t>(brow) & 15u) == 0)) {
 #pragma unroll
-      for (int j = 0; j < NV; j += 4) {
+      for (int j = 0; j < 32; j += 4) {
         if (j < n_valid) {
           const uint4 b = __ldg(reinterpret_cast<const uint4*>(brow + j));
           s.w[j] = b.x; s.w[j + 1] = b.y; s.w[j + 2] = b.z; s.w[j + 3] = b.w;
@@ -142,14 +142,14 @@ __device__ __forceinline__ void epilogue_prefetch(const EpilogueArgs& e, EpiSide
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) if (j < n_valid) s.w[j] = __float_as_uint(__ldg(brow + j));
+      for (int j = 0; j < 32; ++j) if (j < n_valid) s.w[j] = __float_as_uint(__ldg(brow + j));
     }
   } else if (e.epi == EPI_MASK && row_ok) {
     if (e.c_dt == DT_BF16) {
       const unsigned short* mrow = reinterpret_cast<const unsigned short*>(e.mask) + (int64_t)row * e.ldmask + col0;
       if (whole && ((reinterpret_cast<uintptr_t>(mrow) & 15u) == 0)) {
 #pragma unroll
-        for (int j = 0; j < NV; j += 8) {
+        for (int j = 0; j < 32; j += 8) {
           if (j < n_valid) {
             const uint4 q = __ldg(reinterpret_cast<const uint4*>(mrow + j));
             s.w[j / 2] = q.x; s.w[j / 2 + 1] = q.y; s.w[j / 2 + 2] = q.z; s.w[j / 2 + 3] = q.w;
@@ -157,7 +157,7 @@ __device__ __forceinline__ void epilogue_prefetch(const EpilogueArgs& e, EpiSide
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < NV; j += 2) {
+        for (int j = 0; j < 32; j += 2) {
           uint32_t lo = 0u, hi = 0u;
           if (j < n_valid) lo = __ldg(mrow + j);
           if (j + 1 < n_valid) hi = __ldg(mrow + j + 1);
@@ -168,7 +168,7 @@ __device__ __forceinline__ void epilogue_prefetch(const EpilogueArgs& e, EpiSide
       const float* mrow = reinterpret_cast<const float*>(e.mask) + (int64_t)row * e.ldmask + col0;
       if (whole && ((reinterpret_cast<uintptr_t>(mrow) & 15u) == 0)) {
 #pragma unroll
-        for (int j = 0; j < NV; j += 4) {
+        for (int j = 0; j < 32; j += 4) {
           if (j < n_valid) {
             const uint4 m = __ldg(reinterpret_cast<const uint4*>(mrow + j));
             s.w[j] = m.x; s.w[j + 1] = m.y; s.w[j + 2] = m.z; s.w[j + 3] = m.w;
@@ -176,7 +176,7 @@ __device__ __forceinline__ void epilogue_prefetch(const EpilogueArgs& e, EpiSide
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < NV; ++j) if (j < n_valid) s.w[j] = __float_as_uint(__ldg(mrow + j));
+        for (int j = 0; j < 32; ++j) if (j < n_valid) s.w[j] = __float_as_uint(__ldg(mrow + j));
       }
     }
   }
@@ -186,48 +186,46 @@ __device__ __forceinline__ void epilogue_prefetch(const EpilogueArgs& e, EpiSide
 // Columns are stored in groups of 8 with 16-byte accesses when the group count is whole and the
 // row segment is 16-byte aligned (every lane touches its own row, so wide accesses are what keeps
 // the number of memory wavefronts down); ragged or unaligned segments fall back to scalar stores.
-template <int NV>
-__device__ __forceinline__ void epilogue_values(const EpilogueArgs& e, float (&v)[NV], const EpiSide& s, int col0,
+__device__ __forceinline__ void epilogue_values(const EpilogueArgs& e, float (&v)[32], const EpiSide& s, int col0,
                                                 int n_total) {
-  const int n_valid = min(NV, n_total - col0);
+  const int n_valid = min(32, n_total - col0);
   if (e.epi == EPI_BIAS_ACT) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) if (j < n_valid) v[j] += __uint_as_float(s.w[j]);
+    for (int j = 0; j < 32; ++j) if (j < n_valid) v[j] += __uint_as_float(s.w[j]);
     if (e.relu) {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) v[j] = fmaxf(v[j], 0.f);
+      for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j], 0.f);
     }
   } else if (e.epi == EPI_MASK) {
     if (e.c_dt == DT_BF16) {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) {
+      for (int j = 0; j < 32; ++j) {
         // a bf16 is positive iff its sign bit is clear and it is not zero
         const uint32_t bits = (s.w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
         if (j < n_valid && !(bits != 0u && bits < 0x8000u)) v[j] = 0.f;
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < NV; ++j)
+      for (int j = 0; j < 32; ++j)
         if (j < n_valid && !(__uint_as_float(s.w[j]) > 0.f)) v[j] = 0.f;
     }
   }
   if (e.c_round == RND_TF32) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = round_tf32_rne(v[j]);
+    for (int j = 0; j < 32; ++j) v[j] = round_tf32_rne(v[j]);
   }
 }
 
 // Stores up to 32 consecutive columns of one row into a [rows][ld] matrix of dtype dt.
-template <int NV>
-__device__ __forceinline__ void store_row_segment(void* base, int dt, int64_t ld, const float (&v)[NV], int row,
+__device__ __forceinline__ void store_row_segment(void* base, int dt, int64_t ld, const float (&v)[32], int row,
                                                   int col0, int n_total) {
-  const int n_valid = min(NV, n_total - col0);
+  const int n_valid = min(32, n_total - col0);
   const bool whole = (n_valid & 7) == 0;
   if (dt == DT_BF16) {
     __nv_bfloat16* crow = reinterpret_cast<__nv_bfloat16*>(base) + (int64_t)row * ld + col0;
     if (whole && ((reinterpret_cast<uintptr_t>(crow) & 15u) == 0)) {
 #pragma unroll
-      for (int j = 0; j < NV; j += 8) {
+      for (int j = 0; j < 32; j += 8) {
         if (j < n_valid) {
           uint4 q;
           __nv_bfloat162 p0 = __floats2bfloat162_rn(v[j], v[j + 1]);
@@ -241,24 +239,23 @@ __device__ __forceinline__ void store_row_segment(void* base, int dt, int64_t ld
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) if (j < n_valid) crow[j] = __float2bfloat16_rn(v[j]);
+      for (int j = 0; j < 32; ++j) if (j < n_valid) crow[j] = __float2bfloat16_rn(v[j]);
     }
   } else {
     float* crow = reinterpret_cast<float*>(base) + (int64_t)row * ld + col0;
     if (whole && ((reinterpret_cast<uintptr_t>(crow) & 15u) == 0)) {
 #pragma unroll
-      for (int j = 0; j < NV; j += 4) {
+      for (int j = 0; j < 32; j += 4) {
         if (j < n_valid) *reinterpret_cast<float4*>(crow + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) if (j < n_valid) crow[j] = v[j];
+      for (int j = 0; j < 32; ++j) if (j < n_valid) crow[j] = v[j];
     }
   }
 }
 
-template <int NV>
-__device__ __forceinline__ void epilogue_store(const EpilogueArgs& e, float (&v)[NV], const EpiSide& s, int row,
+__device__ __forceinline__ void epilogue_store(const EpilogueArgs& e, float (&v)[32], const EpiSide& s, int row,
                                                int col0, int n_total) {
   epilogue_values(e, v, s, col0, n_total);
   store_row_segment(e.C, e.c_dt, e.ldc, v, row, col0, n_total);
@@ -584,7 +581,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll 1
       for (int c = part; c < BLOCK_N / 32; c += EPI_PER_QUARTER) {
         const int col0 = n0 + c * 32;
-        if (col0 >= N) break;              // uniform across the CTA
+        if (col0 >= N) break;              // uniform across the warp
         constexpr bool MORE = BLOCK_N / 32 > EPI_PER_QUARTER;
         if (MORE && c + EPI_PER_QUARTER < BLOCK_N / 32)
           epilogue_prefetch(epi, side_next, row, row < M, col0 + 32 * EPI_PER_QUARTER, N);
@@ -745,7 +742,8 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   uint8_t* smem_a = smem;
   uint8_t* smem_b = smem + STAGES * A_TILE_BYTES;
   uint8_t* recv = smem + STAGES * SPLITK_STAGE_BYTES;      // [src][piece][row]
-  float2* stats = reinterpret_cast<float2*>(smem);         // LOSS_CE: [src][row] maximum and sum, in the ring's place (who sends them has had this CTA's sums)
+  // LOSS_CE: [src][row] maximum and sum, in the ring's place (who sends them has had this CTA's sums)
+  float2* stats = reinterpret_cast<float2*>(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * SPLITK_STAGE_BYTES + SPLITK_RECV_BYTES);
   // bars[0..S) full, [S..2S) empty, [2S] accumulator complete, [2S+1] partial slices received, [2S+2] row statistics received
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 3);
@@ -1557,6 +1555,8 @@ cudaError_t launch_pair_majors(bool a_mn, bool b_mn, const CUtensorMap& ma, cons
 // which one SM's shared memory is filled (about 64 bytes per clock, measured: 24 KiB of operands per
 // k-block take 0.2 us, 32 KiB 0.27 us, 48 KiB 0.4 us); a CTA pair stages 32 KiB per CTA for the work
 // a single CTA needs 48 KiB for.  Persistent kernels run ceil(tiles / CTAs) rounds of num_k k-blocks.
+// The single-CTA kernel's costs per tile (0.4 + bn / 128; 3.5 + bn / 48) were fitted when four warps drained a tile and are not fitted
+// to the eight it has now; pick_split's 0.6 us is what its tiles take beyond the former.
 // fused_update: the kernel also applies the optimizer, whose warps walk pair tiles of 256 columns.
 struct Choice { int kind; int block_n; double us; };      // kind 0: single CTA, 1: CTA pair
 Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_update) {
@@ -1592,7 +1592,8 @@ Choice pick_kernel(int M, int N, int K, bool tf32, bool throughput, bool fused_u
       best = Choice{1, PAIR_HALF_N, us};
     }
     // Fewer than half as many 256-column tiles as pairs: tiles of 128 columns give every pair one (a k-block takes 0.18 us; of
-    // 256 columns 0.267 where tiles fill the GPU, as above, and 0.30 where half of the pairs have none).  1024 x 2048 x 4096: 18.3 us against 25.8 with 256 columns and 19.6 with one CTA per 128 x 128 tile.
+    // 256 columns 0.267 where tiles fill the GPU, as above, and 0.30 where half of the pairs have none).  1024 x 2048 x 4096: 18.3 us
+    // against 25.8 with 256 columns and 19.6 with one CTA per 128 x 128 tile.
     if (g_pair_min_tiles == 0 && !throughput && !fused_update && 2 * tiles <= pairs) {
       const double us128 = num_k * 0.18 + 4.5;
       if (us128 < best.us) best = Choice{1, PAIR_HALF_N / 2, us128};
@@ -1715,17 +1716,17 @@ cudaError_t launch_wait_selftest(int* dev_status, uint64_t limit_ns, cudaStream_
   return cudaGetLastError();
 }
 
-// The losses are fused into the split-K kernel, the one that serves the small, latency-bound products, where they replace a launch on
-// the critical path: the mean-squared error wherever that kernel runs the last product, the softmax cross-entropy where one tile
-// holds whole rows (at most 64 classes), with four CTAs to a tile whatever K is, since the epilogue is the longer part (a step of
-// 512-512-256-47 in TF32, batch 256: 46.6 -> 42.2 us together with the exchange from registers).  In the persistent kernels the same epilogues measured slower than the
-// separate loss launch (mean-squared error, 1024x2048x4096: 44 us against 25 + 14 under ncu; cross-entropy with one thread per row or
-// one warp per 32 rows: slower by up to four times), and the CTA-pair kernel serves large products, where a separate loss launch
-// costs next to nothing.
 double gemm_tc_estimate_us(int M, int N, int K, bool tf32) {
   return 3.0 + pick_kernel(M, N, K, tf32, false, false).us;         // + launch, first loads and drain
 }
 
+// The losses are fused into the split-K kernel, the one that serves the small, latency-bound products, where they replace a launch on
+// the critical path: the mean-squared error wherever that kernel runs the last product, the softmax cross-entropy where one tile
+// holds whole rows (at most 64 classes), with four CTAs to a tile whatever K is, since the epilogue is the longer part (a step of
+// 512-512-256-47 in TF32, batch 256: 46.6 -> 42.2 us together with the exchange from registers).  In the persistent kernels the same
+// epilogues measured slower than the separate loss launch (mean-squared error, 1024x2048x4096: 44 us against 25 + 14 under ncu;
+// cross-entropy with one thread per row or one warp per 32 rows: slower by up to four times), and the CTA-pair kernel serves large
+// products, where a separate loss launch costs next to nothing.
 int gemm_tc_fused_loss_partials(int kind, int M, int N, int K, bool tf32) {
   if (!g_init_ok || !g_allow_splitk) return 0;
   const int tiles_m = (M + BLOCK_M - 1) / BLOCK_M;

@@ -71,8 +71,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // those instructions take their operands from uniform registers, and only behind elect.sync does the compiler know that one
 // thread is active and issue them directly; behind `lane == 0` it wraps each in a loop over the active threads.  Measured:
 // eight expect-and-copy pairs are issued in 92 cycles against 474; 1024-row responses of 784-4096-4096-2048 take 2561 us
-// against 2782 (33 chunks), a step of 512-1024-768-512 (bf16, batch 512) 54.3 us against 61.2, and the split-K kernel's
-// three sends to its peers bring a step of 784-1024-1024-512 (TF32, batch 256) from 57.5 to 56.8.
+// against 2782 (33 chunks), a step of 512-1024-768-512 (bf16, batch 512) 54.3 us against 61.2.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
